@@ -13,30 +13,37 @@
 // there are few); each CTA owns a contiguous range of 128-key tiles. Between the passes every CTA publishes its
 // per-row (reference, sum) pairs in its own shared memory, signals its peers with a remote mbarrier arrive, and reads
 // the peers' pairs with distributed-shared-memory loads. Pass 2 walks the CTA's tiles backwards so that the tiles read
-// last are re-read first from L2. When the caller supplies the rows' log-sum-exp (lse_obs), pass 1 is skipped.
+// last are re-read first from L2. When the caller supplies the rows' log-sum-exp (lse_obs), pass 1 is skipped; the keys
+// of a unit are then independent, and a uniform batch is cut into equal shares of tiles, one per CTA (32 layers x 8111
+// tokens: 256 units on 148 CTAs are 2 rounds of whole units but 1.73 rounds of shares; 118 -> 105 us with the rest).
 //
-// The grid is persistent: as many clusters as the device can hold at once, each walking over units
-// cluster, cluster + n_clusters, ...; the TMA and MMA warps run ahead across pass and unit boundaries (double-buffered
-// query tile, ring of key tiles, one accumulator stage per softmax group or pair of groups), so barrier set-up, TMEM
-// allocation and pipeline fill are paid once per CTA and not once per unit.
+// The grid is persistent: as many clusters as the device can hold at once, each walking over its units. Roles, all of them
+// whole warps that meet only at mbarriers (no barrier among the softmax warps: each runs on as soon as its own data is
+// there):
+//   TMA producer        walks the units, publishes each one's description in a small ring, streams query and key tiles
+//   MMA issuer          TMEM owner; one elected lane issues, the warp around it is uniform
+//   2 statistics warps  merge the row statistics between the passes, exchange them over the cluster, form the row constants
+//   12 softmax warps    three groups of four. A "job" is one block of up to 128 score rows of one key tile in one pass; jobs
+//                       are dealt round-robin to the three groups and to the four accumulator stages, so that the products
+//                       of a group's next job are ready when it hands back the current one (four groups on four stages
+//                       waited 30 % of their time for their own stage to be refilled). With 129..256 score rows (MB 2) a
+//                       tile is two consecutive jobs, one per block of 128 rows; in pass 2 their partial sums meet in a
+//                       shared-memory ring.
+// After set-up the producer's warpgroup gives registers back (setmaxnreg) and the softmax warps take them.
 //
-// Warp roles: four softmax warpgroups plus one warpgroup with the TMA producer warp, the MMA issuer warp (TMEM owner)
-// and two idle warps. A "job" is one block of up to 128 score rows of one key tile in one pass. With up to 128 score rows (MB 1) the four groups take the
-// jobs round-robin, one accumulator stage of 128 columns each. With 129..256 rows (MB 2) every tile is two jobs, one
-// per block of 128 rows, again one group and one stage each: in pass 1 a group owns the rows of its block, in pass 2
-// it sums its block's rows for the tile's keys and the two partial sums meet in a small shared-memory ring.
-// After set-up the last warpgroup gives registers back (setmaxnreg) and the softmax warpgroups take them.
-//
-// The softmax warps are bound by instruction issue and by the special-function unit (one ex2 per score element and
-// pass), so a fixed share of the exponentials (2 of every 16 with 256 score rows) is evaluated on the FMA pipe instead: the argument is
-// clamped to [-126, 126] with a saturating multiply-add, split into integer and fraction with the 1.5*2^23 rounding
-// trick, 2^fraction comes from a cubic polynomial (relative error 7.5e-5) and the integer part goes into the exponent
-// field with an integer add. The other exponentials take their scale-and-shift and their running sums two at a time
-// (fma.rn.f32x2, add.rn.f32x2: the same roundings as the scalar forms, a third fewer issue slots per element).
+// What bounds it. Back to back, the board's power limit (1000 W): a call takes its energy over 1000 W, whatever the clock.
+// On 32 layers x 4096 tokens (118 mJ, 120 us; 122 mJ with the earlier four groups, single-lane issuer and barriers at
+// every unit border) the copies alone take 71 mJ, the products 55 mJ, the softmax arithmetic 34 mJ, each with its share of the
+// idle power. Copies dominate, from L2 as well as from HBM (keeping the keys of all units in flight inside L2 with 4 CTAs
+// per unit costs as much energy), so what helps is fewer bytes and fewer stalls, not more arithmetic throughput.
+// In single calls, at full clock: the softmax warps (two exponentials per score element, 16 per clock and SM on the
+// special-function unit) and the memory system, at about the same time each: the parts alone take 85 us (softmax), 73 us
+// (products) and 72 us (copies), together 107 us (112 us before). The scale-and-shift and the running sums are taken two at
+// a time (fma.rn.f32x2, add.rn.f32x2: the same roundings as the scalar forms, a third fewer issue slots per element).
 //
 // Every wait on an mbarrier is bounded by wall time; when one runs out the CTA records TA_ERR_TIMEOUT, its producer
-// and MMA warps stop issuing work, the copies and MMAs in flight are drained, and the softmax warps finish their loops
-// without waiting or storing. The only unbounded waits are hardware barriers that every thread reaches on every path.
+// and MMA warps stop issuing work, the copies and MMAs in flight are drained, and the other warps leave their loops
+// without storing. The only unbounded waits are hardware barriers that every thread reaches on every path.
 #include <cuda.h>
 
 #include <type_traits>
@@ -53,21 +60,19 @@ constexpr int kD = TA_HEAD_DIM;                   // 128
 constexpr int kHalfBytes = kTileN * 128;          // one 64-column half of a 128-row operand tile: 16 KB
 constexpr int kKTileBytes = 2 * kHalfBytes;       // 32 KB
 constexpr int kMaxCluster = 8;
-constexpr int kGroups = 4;                        // softmax warpgroups
-constexpr int kThreads = (kGroups + 1) * 128;     // 640
+constexpr int kGroups = 3;                        // softmax warpgroups
+constexpr int kSoftWarps = kGroups * 4;
+constexpr int kThreads = (kGroups + 1) * 128;     // 512
 // Register split after set-up (setmaxnreg); the shares must fit in threads x registers at launch:
-// 640 threads x 96 = 61440 = 16*32*112 + 4*32*32
-constexpr int kRegsSoftmax = 112;
-constexpr int kRegsOther = 32;
-constexpr int kRegsNeeded = (kGroups * 4 * kRegsSoftmax + 4 * kRegsOther) * 32;
+// 512 threads x 128 = 65536 = 12*32*152 + 4*32*56
+constexpr int kRegsSoftmax = 152;
+constexpr int kRegsOther = 56;
+constexpr int kRegsNeeded = (kSoftWarps * kRegsSoftmax + 4 * kRegsOther) * 32;
 
-// Of every 16 exponentials, this many run on the FMA pipe. Measured on B200: with up to 128 score rows the softmax
-// warps are not what limits the kernel (replacing every ex2 by a multiply changes its duration by 3 %) and any
-// polynomial share costs issue slots (0: 119 us, 4: 129 us on 32 layers x 4096 tokens); with 256 rows the
-// special-function unit is the longest pole and 2 of 16 is the best share (1.69 -> 1.62 ms on 2 layers of 16 x 32768).
-#ifndef TA_SCORE_POLY_MB1
-#define TA_SCORE_POLY_MB1 0
-#endif
+// Of every 16 exponentials, this many (an even number: they are taken in pairs) run on the FMA pipe with 129 to 256 score
+// rows. Back to back the kernel runs into the board's 1000 W limit, and a polynomial costs more energy than ex2 while it
+// relieves the special-function unit: 8 layers of 16 x 32768 tokens with 256 rows 0: 6.22 ms, 2: 6.02 ms, more: the same.
+// With up to 128 rows no share pays (one pass over 32 x 8111 tokens: 0: 122 us, 4: 125 us) and none is taken.
 #ifndef TA_SCORE_POLY_MB2
 #define TA_SCORE_POLY_MB2 2
 #endif
@@ -83,6 +88,8 @@ struct ScoreParams {
   int rows;           // G*W
   int cluster;        // CTAs per unit
   int units;          // L * B * Hkv
+  // One pass (lse_obs given): the keys of a unit are independent of one another and a unit may be cut anywhere.
+  int flat;           // uniform batches: CTA i takes the i-th equal share of all tiles, over unit borders
   int two_pass;       // 0 when lse_obs is given
   int causal;
   float c;            // softmax scale * log2(e)
@@ -98,50 +105,46 @@ struct ScoreParams {
 };
 
 // ---------------------------------------------------------------------------------------------- shared memory
-template <int MB>
-struct ScoreCfg {
-  static constexpr int kQBufs = MB == 1 ? 2 : 1;   // query tiles in flight (next unit's tile loads early)
-  static constexpr int kStages = MB == 1 ? 4 : 3;  // ring of key tiles
-  static constexpr int kRowsPad = MB * 128;
-  static constexpr int kAcc = 4;                   // accumulator stages of 128 columns (512 columns in all)
-  static constexpr int kWarpsPerJob = 4;           // softmax warps that read one accumulator stage
-  static constexpr int kRing = 4;                  // MB 2: partial sums in flight between the two groups of a pair
+struct alignas(16) UnitInfo {
+  int l, b, g, tok0;       // layer, sequence, KV head, packed index of the first token
+  int n, t_begin, T, end;  // tokens, this CTA's first tile and its number of tiles; end: no unit, the walk is over
 };
+constexpr int kUnitRing = 4;  // unit descriptions in flight between the producer and the other warps
+constexpr int kAcc = 4;       // accumulator stages of 128 tensor-memory columns (512 columns in all)
+constexpr int kStages = 4;    // ring of key tiles
+constexpr int kRing = 4;      // MB 2: partial column sums in flight between the groups
 
 template <int MB>
 struct alignas(1024) ScoreSmem {
-  using Cfg = ScoreCfg<MB>;
-  uint8_t q[Cfg::kQBufs][MB * 2 * kHalfBytes];    // [buffer][half][MB*128 rows][128 B]
-  uint8_t k[Cfg::kStages][kKTileBytes];           // [stage][half][128 rows][128 B]
-  float mine_m[2][MB * 128];                      // [unit parity][row]: this CTA's row statistics, read by its peers
-  float mine_z[2][MB * 128];
-  float part_m[kGroups][128];                     // per softmax group: MB 1 rows 0..127; MB 2 rows of block (group & 1)
-  float part_z[kGroups][128];
-  float tab[2][MB * 128];                         // [unit parity][row] pass-2 constant of the row (see row constants)
-  float nbeta[2][MB * 128];                       // [unit parity][row] -beta (masked tiles use ex2 for every row)
-  float wrow[MB * 128];                           // pension weight per row
-  float lv[MB * 128];                             // log2 of the row's output weight (kOutFused), else 0
-  float psum[2][Cfg::kRing][2][128];              // MB 2: [pair][ring slot][A|P][key] partial sums of row block 0
-  int row_t[MB * 128];                            // window index t of the row, -1 for padding rows
-  unsigned long long full[Cfg::kStages], empty[Cfg::kStages], acc_full[Cfg::kAcc], acc_empty[Cfg::kAcc];
-  unsigned long long q_full[Cfg::kQBufs], q_empty[Cfg::kQBufs], xchg_full[2], drain;
-  unsigned long long pfull[2][Cfg::kRing], pfree[2][Cfg::kRing];
+  static constexpr int kQBufs = MB == 1 ? 2 : 1;  // query tiles in flight (next unit's tile loads early)
+  static constexpr int kRowsPad = MB * 128;
+  uint8_t q[kQBufs][MB * 2 * kHalfBytes];  // [buffer][half][MB*128 rows][128 B]
+  uint8_t k[kStages][kKTileBytes];         // [stage][half][128 rows][128 B]
+  float part_m[2][kGroups][kRowsPad];      // [unit parity][softmax group][row]: reference and sum of the group's keys
+  float part_z[2][kGroups][kRowsPad];
+  float mine_m[2][kRowsPad];               // [unit parity][row]: this CTA's row statistics, read by its peers
+  float mine_z[2][kRowsPad];
+  float tab[2][kRowsPad];                  // [unit parity][row] pass-2 constant of the row
+  float wrow[kRowsPad];                    // pension weight per row
+  float lv[kRowsPad];                      // log2 of the row's output weight (kOutFused), else 0
+  int row_t[kRowsPad];                     // window index t of the row, -1 for padding rows
+  float psum[kRing][2][128];               // MB 2: [ring slot][A|P][key] partial sums of row block 0
+  UnitInfo unit[kUnitRing];
+  unsigned long long full[kStages], empty[kStages], acc_full[kAcc], acc_empty[kAcc];
+  unsigned long long q_full[kQBufs], q_empty[kQBufs], ufull[kUnitRing], ufree[kUnitRing];
+  unsigned long long stat_full[2], tab_full[2], tab_free[2], xchg_full[2], drain;
+  unsigned long long pfull[kRing], pfree[kRing];
   uint32_t tmem_base;
   int abort_flag;
 };
 
-struct UnitInfo {
-  int l, b, g, tok0, n, t_begin, T;
-};
-
 // ---------------------------------------------------------------------------------------------- exponentials
-// Position q of a 16-element group runs on the FMA pipe when this is true (the positions are spread evenly).
+// Pair q2 (elements 2*q2, 2*q2 + 1) of a 16-element group runs on the FMA pipe when this is true (spread evenly).
 template <int MB>
-__host__ __device__ constexpr bool poly_slot(int q) {
-  constexpr int kPoly = MB == 1 ? TA_SCORE_POLY_MB1 : TA_SCORE_POLY_MB2;
-  return ((q * kPoly) / 16) != (((q + 1) * kPoly) / 16);
+__host__ __device__ constexpr bool poly_pair(int q2) {
+  constexpr int kPairs = MB == 1 ? 0 : TA_SCORE_POLY_MB2 / 2;
+  return ((q2 * kPairs) / 8) != (((q2 + 1) * kPairs) / 8);
 }
-
 constexpr float kPolyRange = 252.0f;                // width of the clamped argument range [-126, 126]
 constexpr float kPolyMagic = 12582912.0f - 126.0f;  // 1.5 * 2^23 - 126: adding it leaves the integer part in the low bits
 // minimax cubic for 2^f on [0, 1) in relative error (7.5e-5)
@@ -153,16 +156,25 @@ __device__ __forceinline__ float fma_sat(float a, float b, float c) {
   asm("fma.rn.sat.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
   return d;
 }
-// exp2(x) for x = s*c - beta clamped to [-126, 126], given c252 = c/252 and bias = (126 - beta)/252
-__device__ __forceinline__ float exp2_poly(float s, float c252, float bias) {
-  const float t = fma_sat(s, c252, bias);                 // (x + 126) / 252 in [0, 1]
-  const float y = __fmaf_rd(t, kPolyRange, kPolyMagic);   // 1.5*2^23 + floor(x)
-  const float w = kPolyMagic - y;                         // -126 - floor(x), exact
-  const float f = fmaf(t, kPolyRange, w);                 // x - floor(x)
-  float p = fmaf(kC3, f, kC2);
-  p = fmaf(p, f, kC1);
-  p = fmaf(p, f, kC0);
-  return __int_as_float((__float_as_int(y) << 23) + __float_as_int(p));
+// two values of exp2(x), x = s*c - beta clamped to [-126, 126], given c252 = c/252 and bias = (126 - beta)/252
+__device__ __forceinline__ void exp2_poly2(float& e0, float& e1, float s0, float s1, float c252, float bias0, float bias1) {
+  const float t0 = fma_sat(s0, c252, bias0), t1 = fma_sat(s1, c252, bias1);  // (x + 126) / 252 in [0, 1]
+  float p0, p1;
+  uint32_t y0, y1;
+  asm("{\n\t.reg .b64 t, r, m, y, w, f, p, k;\n\t"
+      "mov.b64 t, {%4, %5};\n\tmov.b64 r, {%6, %6};\n\tmov.b64 m, {%7, %7};\n\t"
+      "fma.rm.f32x2 y, t, r, m;\n\t"           // 1.5*2^23 + floor(x)
+      "mov.b64 k, {%8, %8};\n\t"
+      "fma.rn.f32x2 w, y, k, m;\n\t"           // -126 - floor(x), exact
+      "fma.rn.f32x2 f, t, r, w;\n\t"           // x - floor(x)
+      "mov.b64 p, {%9, %9};\n\tmov.b64 k, {%10, %10};\n\tfma.rn.f32x2 p, p, f, k;\n\t"
+      "mov.b64 k, {%11, %11};\n\tfma.rn.f32x2 p, p, f, k;\n\t"
+      "mov.b64 k, {%12, %12};\n\tfma.rn.f32x2 p, p, f, k;\n\t"
+      "mov.b64 {%0, %1}, p;\n\tmov.b64 {%2, %3}, y;\n\t}"
+      : "=f"(p0), "=f"(p1), "=r"(y0), "=r"(y1)
+      : "f"(t0), "f"(t1), "f"(kPolyRange), "f"(kPolyMagic), "f"(-1.0f), "f"(kC3), "f"(kC2), "f"(kC1), "f"(kC0));
+  e0 = __uint_as_float((y0 << 23) + __float_as_uint(p0));
+  e1 = __uint_as_float((y1 << 23) + __float_as_uint(p1));
 }
 // two multiply-adds / two adds in one instruction (same roundings as the scalar forms)
 __device__ __forceinline__ void fma2(float& d0, float& d1, float a0, float a1, float b, float c0, float c1) {
@@ -179,62 +191,78 @@ __device__ __forceinline__ void add2(float& d0, float& d1, float a0, float a1) {
 }
 __device__ __forceinline__ float poly_bias(float beta) { return (126.0f - beta) * (1.0f / kPolyRange); }
 
+// Products K .. END-1 of the eight of a job: S = Q_block * Ktile^T (STATS) or S^T = Ktile * Q_block^T, 16 dimensions each.
+template <int MB, bool STATS, int K, int END>
+__device__ __forceinline__ void issue_job(uint32_t acc, uint32_t q_lo, uint32_t k_lo, uint32_t desc_hi, uint32_t idesc) {
+  constexpr uint32_t oq = (uint32_t)((K >> 2) * (MB * kHalfBytes) + (K & 3) * 32) >> 4;
+  constexpr uint32_t ok = (uint32_t)((K >> 2) * kHalfBytes + (K & 3) * 32) >> 4;
+  if constexpr (STATS) umma_bf16_off<oq, ok, (K > 0)>(acc, q_lo, k_lo, desc_hi, idesc);
+  else umma_bf16_off<ok, oq, (K > 0)>(acc, k_lo, q_lo, desc_hi, idesc);
+  if constexpr (K + 1 < END) issue_job<MB, STATS, K + 1, END>(acc, q_lo, k_lo, desc_hi, idesc);
+}
+
 // ---------------------------------------------------------------------------------------------- the kernel
 template <int MB, int PM>
 __global__ void __launch_bounds__(kThreads, 1)
 ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                 const __grid_constant__ ScoreParams p) {
-  using Cfg = ScoreCfg<MB>;
-  constexpr int kWarpTma = kGroups * 4, kWarpMma = kGroups * 4 + 1;
-  constexpr int kStages = Cfg::kStages, kQBufs = Cfg::kQBufs, kRowsPad = Cfg::kRowsPad;
-  constexpr int kAcc = Cfg::kAcc;
+  using Smem = ScoreSmem<MB>;
+  constexpr int kWarpTma = kSoftWarps, kWarpMma = kSoftWarps + 1, kWarpStat = kSoftWarps + 2;
+  constexpr int kStatWarps = 2;
+  constexpr int kQBufs = Smem::kQBufs, kRowsPad = Smem::kRowsPad;
   constexpr uint32_t kTmemCols = 512;  // kAcc accumulator stages of 128 columns
   extern __shared__ uint8_t smem_raw[];
-  ScoreSmem<MB>& sm = *reinterpret_cast<ScoreSmem<MB>*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  Smem& sm = *reinterpret_cast<Smem*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  // the warp index through a shuffle: the compiler then knows the role branches to be warp-uniform
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
   const uint32_t rank = cluster_ctarank();
   const int cluster_id = blockIdx.x / p.cluster;
   const int n_clusters = gridDim.x / p.cluster;
   volatile int* abort_flag = &sm.abort_flag;
   const unsigned long long limit = p.wait_limit_ns;
 
-  // `walk` = cluster_id + round * n_clusters. With a length-sorted order the rounds are taken in alternating
-  // direction (the cluster that got the longest unit of one round gets the shortest of the next), which evens out the
-  // clusters' totals; a position past the end of the list is an empty unit.
-  auto get_unit = [&](int walk) {
-    // every cluster makes the same number of rounds; walk positions at and beyond the number of units are empty
-    int u = walk;
-    bool empty = walk >= p.units;
-    if (p.order) {
-      const int round = walk / n_clusters;
-      const int w = (round & 1) ? round * n_clusters + (n_clusters - 1 - cluster_id) : walk;
-      empty = w >= p.units;
-      u = empty ? 0 : p.order[w];
-    } else if (empty) {
-      u = 0;
+  // The unit of round `round` of this cluster's walk over units cluster_id + round * n_clusters. With a length-sorted
+  // order the rounds are taken in alternating direction (the cluster that got the longest unit of one round gets the
+  // shortest of the next), which evens out the clusters' totals. False: there is nothing to do in this round (ui.end: nor in
+  // any later one).
+  auto get_unit = [&](int round, UnitInfo& ui) {
+    ui = UnitInfo{};
+    int u, t_lo = 0, t_hi = 0;
+    if (p.flat) {
+      const int tiles = (p.seq.n_uniform + kTileN - 1) / kTileN;
+      const long long all = (long long)p.units * tiles;
+      const long long lo = all * cluster_id / n_clusters, hi = all * (cluster_id + 1) / n_clusters;
+      u = (int)(lo / tiles) + round;
+      t_lo = (int)max(lo - (long long)u * tiles, 0LL);
+      t_hi = (int)min(hi - (long long)u * tiles, (long long)tiles);
+      ui.end = t_lo >= t_hi;
+    } else {
+      u = round * n_clusters + cluster_id;
+      ui.end = round * n_clusters >= p.units;
+      if (p.order && (round & 1)) u = round * n_clusters + (n_clusters - 1 - cluster_id);
     }
-    UnitInfo ui;
+    if (ui.end || u >= p.units) return false;
+    if (p.order) u = p.order[u];
     ui.g = u % p.Hkv;
     ui.b = (u / p.Hkv) % p.seq.batch;
     ui.l = u / (p.Hkv * p.seq.batch);
     ui.tok0 = ta_seq_begin(p.seq, ui.b);
-    int n = (p.seq.cu ? p.seq.cu[ui.b + 1] : ui.tok0 + p.seq.n_uniform) - ui.tok0;
+    ui.n = (p.seq.cu ? p.seq.cu[ui.b + 1] : ui.tok0 + p.seq.n_uniform) - ui.tok0;
     // a sequence that does not lie inside the token arrays is skipped here and rejected by the selection step
-    if (n > p.seq.max_n || n < 0 || ui.tok0 < 0 || (long long)ui.tok0 + n > p.seq.total) {
-      if (tid == 0 && atomicCAS(&p.status->code, 0, (int)TA_ERR_DEVICE_BOUNDS) == 0) {
+    if (ui.n > p.seq.max_n || ui.n < 0 || ui.tok0 < 0 || (long long)ui.tok0 + ui.n > p.seq.total) {
+      if (atomicCAS(&p.status->code, 0, (int)TA_ERR_DEVICE_BOUNDS) == 0) {
         p.status->where = 2;
         p.status->detail0 = ui.b;
-        p.status->detail1 = n;
+        p.status->detail1 = ui.n;
       }
-      n = 0;
+      return false;
     }
-    if (empty) n = 0;
-    ui.n = n;
-    const int tiles_total = (n + kTileN - 1) / kTileN;
-    ui.t_begin = (int)((long long)tiles_total * rank / p.cluster);
-    ui.T = (int)((long long)tiles_total * (rank + 1) / p.cluster) - ui.t_begin;
-    return ui;
+    const int tiles_total = (ui.n + kTileN - 1) / kTileN;
+    ui.t_begin = p.flat ? t_lo : (int)((long long)tiles_total * rank / p.cluster);
+    ui.T = (p.flat ? t_hi : (int)((long long)tiles_total * (rank + 1) / p.cluster)) - ui.t_begin;
+    // a CTA without tiles still takes part in its cluster's exchange of statistics
+    return ui.T > 0 || (ui.n > 0 && p.two_pass && p.cluster > 1);
   };
 
   // ---- set-up (once per CTA)
@@ -245,19 +273,27 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
     }
     for (int a = 0; a < kAcc; ++a) {
       mbar_init(smem_u32(&sm.acc_full[a]), 1);
-      mbar_init(smem_u32(&sm.acc_empty[a]), Cfg::kWarpsPerJob);
+      mbar_init(smem_u32(&sm.acc_empty[a]), 4);
     }
-    for (int a = 0; a < 2; ++a) mbar_init(smem_u32(&sm.xchg_full[a]), (uint32_t)p.cluster);
-    for (int qb = 0; qb < kQBufs; ++qb) {
-      mbar_init(smem_u32(&sm.q_full[qb]), 1);
-      mbar_init(smem_u32(&sm.q_empty[qb]), 1);
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(smem_u32(&sm.stat_full[i]), kSoftWarps);
+      mbar_init(smem_u32(&sm.tab_full[i]), kStatWarps);
+      mbar_init(smem_u32(&sm.tab_free[i]), kSoftWarps);
+      mbar_init(smem_u32(&sm.xchg_full[i]), (uint32_t)p.cluster * kStatWarps);
+    }
+    for (int i = 0; i < kQBufs; ++i) {
+      mbar_init(smem_u32(&sm.q_full[i]), 1);
+      mbar_init(smem_u32(&sm.q_empty[i]), 1);
+    }
+    for (int r = 0; r < kUnitRing; ++r) {
+      mbar_init(smem_u32(&sm.ufull[r]), 1);
+      mbar_init(smem_u32(&sm.ufree[r]), kSoftWarps + 1 + kStatWarps);  // softmax warps, MMA issuer, statistics warps
+    }
+    for (int r = 0; r < kRing; ++r) {
+      mbar_init(smem_u32(&sm.pfull[r]), 4);
+      mbar_init(smem_u32(&sm.pfree[r]), 4);
     }
     mbar_init(smem_u32(&sm.drain), 1);
-    for (int pr = 0; pr < 2; ++pr)
-      for (int r = 0; r < Cfg::kRing; ++r) {
-        mbar_init(smem_u32(&sm.pfull[pr][r]), 4);
-        mbar_init(smem_u32(&sm.pfree[pr][r]), 4);
-      }
     // a wait that ran out in an earlier CTA or call (not yet polled) makes the remaining CTAs skip their waits
     sm.abort_flag = (*reinterpret_cast<volatile int*>(&p.status->code) == (int)TA_ERR_TIMEOUT) ? 1 : 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -297,423 +333,466 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
 
   const uint32_t k_smem = smem_u32(sm.k);
 
-  if (warp >= kWarpTma) {
+  if (warp >= kSoftWarps) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsOther));
     if (warp == kWarpTma) {
       // =========================================================================== TMA producer
-      if (lane == 0) {
-        int issued[kStages], q_issued[kQBufs];
-#pragma unroll
-        for (int s = 0; s < kStages; ++s) issued[s] = 0;
-#pragma unroll
-        for (int s = 0; s < kQBufs; ++s) q_issued[s] = 0;
-        int jg = 0, qn = 0;
-        bool ok = true;
-        for (int u = cluster_id; ok && u - cluster_id < p.units; u += n_clusters) {
-          const UnitInfo ui = get_unit(u);
-          if (ui.T == 0) continue;
-          const int qb = qn % kQBufs;
-          ok = mbar_wait(smem_u32(&sm.q_empty[qb]), ((uint32_t)(qn / kQBufs) & 1u) ^ 1u, abort_flag, p.status, 11, limit);
-          if (!ok) break;  // nothing may be copied into a buffer that was not handed back
-          {
-            const uint32_t bar = smem_u32(&sm.q_full[qb]);
-            const uint32_t dst = smem_u32(sm.q[qb]);
-            mbar_expect_tx(bar, (uint32_t)(2 * p.rows * 128));
-            tma_load_5d(dst, &map_q, bar, 0, 0, ui.g * p.G, ui.b, ui.l);
-            tma_load_5d(dst + MB * kHalfBytes, &map_q, bar, 64, 0, ui.g * p.G, ui.b, ui.l);
-            q_issued[qb] = qn + 1;
-          }
-          ++qn;
-          const int row0 = p.seq.cu ? ui.tok0 : 0;  // ragged: tokens are packed along the row axis
-          const int bc = p.seq.cu ? 0 : ui.b;
-          const int n_jobs = p.two_pass ? 2 * ui.T : ui.T;
-          for (int j = 0; j < n_jobs; ++j, ++jg) {
-            const int s = jg % kStages;
-            ok = mbar_wait(smem_u32(&sm.empty[s]), ((uint32_t)(jg / kStages) & 1u) ^ 1u, abort_flag, p.status, 10, limit);
-            if (!ok) break;
+      // Walks the units of this cluster, publishes each one's description in the unit ring and streams its tiles.
+      const bool leader = elect_one();
+      uint32_t issued = 0, q_issued = 0;  // stages that were armed at least once
+      int s = 0, qb = 0, us = 0;
+      uint32_t sph = 1, qph = 1, uph = 1;
+      bool ok = true;
+      for (int round = 0;; ++round) {
+        UnitInfo ui;
+        const bool work = get_unit(round, ui);
+        const bool end = ui.end != 0;
+        if (!work && !end) continue;
+        const int T = __shfl_sync(0xffffffffu, ui.T, 0);
+        ok = mbar_wait(smem_u32(&sm.ufree[us]), uph, abort_flag, p.status, 12, limit);
+        if (!ok) break;
+        if (leader) {
+          sm.unit[us] = ui;
+          mbar_arrive(smem_u32(&sm.ufull[us]));
+        }
+        if (++us == kUnitRing) us = 0, uph ^= 1;
+        if (end) break;
+        if (T == 0) continue;
+        ok = mbar_wait(smem_u32(&sm.q_empty[qb]), qph, abort_flag, p.status, 11, limit);
+        if (!ok) break;  // nothing may be copied into a buffer that was not handed back
+        if (leader) {
+          const uint32_t bar = smem_u32(&sm.q_full[qb]);
+          const uint32_t dst = smem_u32(sm.q[qb]);
+          mbar_expect_tx(bar, (uint32_t)(2 * p.rows * 128));
+          tma_load_5d(dst, &map_q, bar, 0, 0, ui.g * p.G, ui.b, ui.l);
+          tma_load_5d(dst + MB * kHalfBytes, &map_q, bar, 64, 0, ui.g * p.G, ui.b, ui.l);
+        }
+        q_issued |= 1u << qb;
+        if (++qb == kQBufs) qb = 0, qph ^= 1;
+        const int row0 = p.seq.cu ? ui.tok0 : 0;  // ragged: tokens are packed along the row axis
+        const int bc = p.seq.cu ? 0 : ui.b;
+        const int n_tiles = p.two_pass ? 2 * T : T;
+#pragma unroll 1
+        for (int j = 0; j < n_tiles; ++j) {
+          ok = mbar_wait(smem_u32(&sm.empty[s]), sph, abort_flag, p.status, 10, limit);
+          if (!ok) break;
+          if (leader) {
             // the second sweep walks the CTA's tiles backwards: the tiles read last are the ones still in L2
-            const int tile = ui.t_begin + (j >= ui.T ? 2 * ui.T - 1 - j : j);
+            const int row = row0 + (ui.t_begin + (j >= T ? 2 * T - 1 - j : j)) * kTileN;
             const uint32_t bar = smem_u32(&sm.full[s]);
             mbar_expect_tx(bar, kKTileBytes);
             const uint32_t dst = k_smem + s * kKTileBytes;
-            tma_load_5d(dst, &map_k, bar, 0, row0 + tile * kTileN, ui.g, bc, ui.l);
-            tma_load_5d(dst + kHalfBytes, &map_k, bar, 64, row0 + tile * kTileN, ui.g, bc, ui.l);
-            issued[s] = jg + 1;
+            tma_load_5d(dst, &map_k, bar, 0, row, ui.g, bc, ui.l);
+            tma_load_5d(dst + kHalfBytes, &map_k, bar, 64, row, ui.g, bc, ui.l);
           }
+          issued |= 1u << s;
+          if (++s == kStages) s = 0, sph ^= 1;
         }
-        if (!ok || *abort_flag) {
-          // drain: every copy that was started must have landed before the CTA may leave. A stage is only ever armed
-          // after its previous contents were handed back, so at most the last copy per stage can still be in flight.
-          for (int s = 0; s < kStages; ++s)
-            if (issued[s]) mbar_wait_drain(smem_u32(&sm.full[s]), (uint32_t)((issued[s] - 1) / kStages) & 1u, limit);
-          for (int s = 0; s < kQBufs; ++s)
-            if (q_issued[s]) mbar_wait_drain(smem_u32(&sm.q_full[s]), (uint32_t)((q_issued[s] - 1) / kQBufs) & 1u, limit);
-        }
+        if (!ok) break;
+      }
+      if (!ok || *abort_flag) {
+        // drain: every copy that was started must have landed before the CTA may leave. A stage is only ever armed
+        // after its previous contents were handed back, so at most the last copy per stage can still be in flight:
+        // stages below the running index were last armed in this round of the ring, the others in the round before.
+        for (int i = 0; i < kStages; ++i)
+          if ((issued >> i) & 1u) mbar_wait_drain(smem_u32(&sm.full[i]), i < s ? sph ^ 1u : sph, limit);
+        for (int i = 0; i < kQBufs; ++i)
+          if ((q_issued >> i) & 1u) mbar_wait_drain(smem_u32(&sm.q_full[i]), i < qb ? qph ^ 1u : qph, limit);
       }
     } else if (warp == kWarpMma) {
       // =========================================================================== MMA issuer
-      if (lane == 0) {
-        int jg = 0, tg = 0, qn = 0;
-        bool ok = true;
-        // operand descriptors: the upper word is the same for every tile; the lower word is the address >> 4
-        const uint32_t desc_hi = (uint32_t)(smem_desc_sw128(0) >> 32);
-        const uint32_t k_lo = (k_smem & 0x3FFFFu) >> 4;
-        const uint32_t idesc = idesc_bf16(128, 128);
-        for (int u = cluster_id; ok && u - cluster_id < p.units; u += n_clusters) {
-          const UnitInfo ui = get_unit(u);
-          if (ui.T == 0) continue;
-          const int qb = qn % kQBufs;
-          ok = mbar_wait(smem_u32(&sm.q_full[qb]), (uint32_t)(qn / kQBufs) & 1u, abort_flag, p.status, 22, limit);
-          if (!ok) break;
-          const uint32_t q_lo = (smem_u32(sm.q[qb]) & 0x3FFFFu) >> 4;
-          // A tile's product is issued as MB jobs, one per block of 128 score rows, each into its own accumulator
-          // stage of 128 columns: S = Q_block * Ktile^T in pass 1, S^T = Ktile * Q_block^T in pass 2.
-          const int n_tiles = p.two_pass ? 2 * ui.T : ui.T;
-          for (int jt = 0; ok && jt < n_tiles; ++jt, ++tg) {
-            const int s = tg % kStages;
-            const bool stats = p.two_pass && jt < ui.T;
-            ok = mbar_wait(smem_u32(&sm.full[s]), (uint32_t)(tg / kStages) & 1u, abort_flag, p.status, 20, limit);
-            if (!ok) break;  // no product is issued on operands that are not ready
+      // The whole warp runs the loop and one elected lane issues: with the loop inside a single lane's branch the
+      // products of a job took 730 cycles instead of the 512 that the tensor pipe needs. The barriers of the next job
+      // are looked at in the middle of the current one, while products are still queued.
+      const bool leader = elect_one();
+      bool ok = true;
+      // operand descriptors: the upper word is the same for every tile; the lower word is the address >> 4
+      const uint32_t desc_hi = (uint32_t)(smem_desc_sw128(0) >> 32);
+      const uint32_t k_lo = (k_smem & 0x3FFFFu) >> 4;
+      const uint32_t q_lo0 = (smem_u32(sm.q[0]) & 0x3FFFFu) >> 4;
+      const uint32_t idesc = idesc_bf16(128, 128);
+      const uint32_t bar_full = smem_u32(&sm.full[0]), bar_empty = smem_u32(&sm.empty[0]);
+      const uint32_t bar_af = smem_u32(&sm.acc_full[0]), bar_ae = smem_u32(&sm.acc_empty[0]);
+      int qb = 0, s = 0, a = 0, us = 0;
+      uint32_t qph = 0, sph = 0, aph = 1, uph = 0;
+      bool k_ready = false, a_ready = false;  // the next job's key tile / accumulator stage is known to be ready
+      for (;;) {
+        ok = mbar_wait(smem_u32(&sm.ufull[us]), uph, abort_flag, p.status, 23, limit);
+        if (!ok) break;
+        const int T = __shfl_sync(0xffffffffu, sm.unit[us].T, 0), end = __shfl_sync(0xffffffffu, sm.unit[us].end, 0);
+        __syncwarp();
+        if (leader) mbar_arrive(smem_u32(&sm.ufree[us]));
+        if (++us == kUnitRing) us = 0, uph ^= 1;
+        if (end) break;
+        if (T == 0) continue;
+        ok = mbar_wait(smem_u32(&sm.q_full[qb]), qph, abort_flag, p.status, 22, limit);
+        if (!ok) break;
+        const uint32_t q_lo = q_lo0 + (uint32_t)((qb * (MB * 2 * kHalfBytes)) >> 4);
+        // A tile's product is issued as MB jobs, one per block of 128 score rows, each into its own accumulator
+        // stage of 128 columns: S = Q_block * Ktile^T in pass 1, S^T = Ktile * Q_block^T in pass 2. No product is issued
+        // on operands that are not ready, nor into an accumulator that was not handed back.
+        auto sweep = [&](auto stats_tag) {
+          constexpr bool stats = decltype(stats_tag)::value;
+#pragma unroll 1
+          for (int jt = 0; jt < T; ++jt) {
+            if (!k_ready && !mbar_wait(bar_full + s * 8, sph, abort_flag, p.status, 20, limit)) return false;
             const uint32_t dk_lo = k_lo + (uint32_t)((s * kKTileBytes) >> 4);
+            const uint32_t bar_es = bar_empty + s * 8;
+            if (++s == kStages) s = 0, sph ^= 1;
 #pragma unroll
-            for (int rb = 0; rb < MB; ++rb, ++jg) {
-              const int a = jg % kAcc;
-              ok = ok && mbar_wait(smem_u32(&sm.acc_empty[a]), ((uint32_t)(jg / kAcc) & 1u) ^ 1u, abort_flag, p.status,
-                                   21, limit);
-              if (ok) {  // (nor into an accumulator that was not handed back)
-                tc_fence_after();
-                const uint32_t acc = tmem_base + (uint32_t)(a * 128);
-#pragma unroll
-                for (int k = 0; k < 8; ++k) {
-                  const uint32_t dq = q_lo + (uint32_t)(((k >> 2) * (MB * kHalfBytes) + rb * kHalfBytes + (k & 3) * 32) >> 4);
-                  const uint32_t dk = dk_lo + (uint32_t)(((k >> 2) * kHalfBytes + (k & 3) * 32) >> 4);
-                  umma_bf16_lo(acc, stats ? dq : dk, stats ? dk : dq, desc_hi, idesc, k > 0);
-                }
-                if (rb == MB - 1) umma_commit(smem_u32(&sm.empty[s]));
-                umma_commit(smem_u32(&sm.acc_full[a]));
+            for (int rb = 0; rb < MB; ++rb) {
+              if (!a_ready && !mbar_wait(bar_ae + a * 8, aph, abort_flag, p.status, 21, limit)) return false;
+              tc_fence_after();
+              const uint32_t acc = tmem_base + (uint32_t)(a * 128);
+              const uint32_t bar_fa = bar_af + a * 8;
+              const uint32_t dq_lo = q_lo + (uint32_t)((rb * kHalfBytes) >> 4);
+              if (++a == kAcc) a = 0, aph ^= 1;
+              if (leader) issue_job<MB, stats, 0, 4>(acc, dq_lo, dk_lo, desc_hi, idesc);
+              a_ready = mbar_test(bar_ae + a * 8, aph);
+              if (rb == MB - 1) k_ready = mbar_test(bar_full + s * 8, sph);
+              if (leader) {
+                issue_job<MB, stats, 4, 8>(acc, dq_lo, dk_lo, desc_hi, idesc);
+                if (rb == MB - 1) umma_commit(bar_es);
+                umma_commit(bar_fa);
               }
             }
           }
-          if (!ok) break;
-          umma_commit(smem_u32(&sm.q_empty[qb]));  // the query tile may be overwritten once these MMAs are done
-          ++qn;
+          return true;
+        };
+        if (p.two_pass) ok = sweep(std::true_type{});
+        if (ok) ok = sweep(std::false_type{});
+        if (!ok) break;
+        if (leader) umma_commit(smem_u32(&sm.q_empty[qb]));  // the query tile may be overwritten once these MMAs are done
+        if (++qb == kQBufs) qb = 0, qph ^= 1;
+      }
+      if (!ok || *abort_flag) {  // make sure no MMA is still writing tensor memory before it is freed
+        if (leader) umma_commit(smem_u32(&sm.drain));
+        mbar_wait_drain(smem_u32(&sm.drain), 0, limit);
+      }
+    } else {
+      // =========================================================================== statistics warps
+      // Between the passes of a unit: merge the groups' row statistics, exchange them with the cluster's other CTAs and
+      // leave the rows' pass-2 constants in `tab`. Two warps of their own, so that no softmax warp waits for another
+      // before the constants are there.
+      const int r0 = (warp - kWarpStat) * 32 + lane;
+      int us = 0;
+      uint32_t uph = 0;
+      for (int it = 0;; ++it) {
+        if (!mbar_wait(smem_u32(&sm.ufull[us]), uph, abort_flag, p.status, 36, limit)) break;
+        const UnitInfo ui = sm.unit[us];
+        __syncwarp();
+        if (lane == 0) mbar_arrive(smem_u32(&sm.ufree[us]));
+        if (++us == kUnitRing) us = 0, uph ^= 1;
+        if (ui.end) break;
+        const int up = it & 1;
+        const uint32_t ph = (uint32_t)(it >> 1) & 1u;
+        mbar_wait(smem_u32(&sm.tab_free[up]), ph ^ 1u, abort_flag, p.status, 37, limit);
+        if (p.two_pass) mbar_wait(smem_u32(&sm.stat_full[up]), ph, abort_flag, p.status, 38, limit);
+        auto put = [&](int r, float lse2) {  // log2-domain log-sum-exp of row r (+inf: the row is mute)
+          const float beta = lse2 - sm.lv[r];
+          sm.tab[up][r] = poly_pair<MB>((r & 15) / 2) ? poly_bias(beta) : -beta;
+        };
+        if (p.two_pass) {
+#pragma unroll
+          for (int r = r0; r < kRowsPad; r += 32 * kStatWarps) {
+            float m = sm.part_m[up][0][r];
+#pragma unroll
+            for (int gq = 1; gq < kGroups; ++gq) m = fmaxf(m, sm.part_m[up][gq][r]);
+            float z = 0.0f;
+#pragma unroll
+            for (int gq = 0; gq < kGroups; ++gq) z += sm.part_z[up][gq][r] * ex2(sm.part_m[up][gq][r] - m);
+            if (p.cluster == 1) {  // nothing to exchange: the CTA's statistics are the unit's
+              put(r, z > 0.0f ? m + __log2f(z) : INFINITY);
+            } else {
+              sm.mine_m[up][r] = m;
+              sm.mine_z[up][r] = z;
+            }
+          }
+          if (p.cluster > 1) {
+            __syncwarp();
+            // one lane per peer tells that peer that this warp's rows of the CTA's statistics are in place
+            if (lane < p.cluster) {
+              fence_cluster();
+              mbar_arrive_remote(smem_u32(&sm.xchg_full[up]), (uint32_t)lane);
+            }
+            mbar_wait_cluster(smem_u32(&sm.xchg_full[up]), ph, abort_flag, p.status, 32, limit);
+#pragma unroll 1
+            for (int r = r0; r < kRowsPad; r += 32 * kStatWarps) {
+              float pm[kMaxCluster], pz[kMaxCluster];
+#pragma unroll
+              for (int q = 0; q < kMaxCluster; ++q) {
+                pm[q] = -1e30f;
+                pz[q] = 0.0f;
+                if (q < p.cluster) {
+                  pm[q] = ld_cluster_f32(smem_u32(&sm.mine_m[up][r]), (uint32_t)q);
+                  pz[q] = ld_cluster_f32(smem_u32(&sm.mine_z[up][r]), (uint32_t)q);
+                }
+              }
+              float m = pm[0], z = 0.0f;
+#pragma unroll
+              for (int q = 1; q < kMaxCluster; ++q) m = fmaxf(m, pm[q]);
+#pragma unroll
+              for (int q = 0; q < kMaxCluster; ++q) z += pz[q] * ex2(pm[q] - m);
+              put(r, z > 0.0f ? m + __log2f(z) : INFINITY);
+            }
+          }
+        } else {
+          for (int r = r0; r < kRowsPad; r += 32 * kStatWarps) {
+            float lse2 = INFINITY;
+            const int t = sm.row_t[r];
+            if (t >= 0 && ui.n - p.W + t >= 0) {
+              const int h = r / p.W;
+              const float lse = p.lse_obs[(((long long)ui.l * p.seq.batch + ui.b) * p.Hq + (ui.g * p.G + h)) * p.W + t];
+              lse2 = lse * 1.4426950408889634f;
+            }
+            put(r, lse2);
+          }
         }
-        if (!ok || *abort_flag) {  // make sure no MMA is still writing tensor memory before it is freed
-          umma_commit(smem_u32(&sm.drain));
-          mbar_wait_drain(smem_u32(&sm.drain), 0, limit);
-        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(smem_u32(&sm.tab_full[up]));
       }
     }
   } else {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsSoftmax));
     // =========================================================================== softmax warps
-    // A job is one block of 128 score rows of one key tile in one pass; jobs are dealt round-robin to the four
-    // groups. With two row blocks (MB 2) a tile is two consecutive jobs, every unit has an even number of jobs, and
-    // group g therefore always gets row block g & 1.
-    constexpr int kShare = kAcc;
-    const int st = tid;                     // 0..511
-    const int grp = st >> 7;
-    const int slot = grp;                   // serves jobs with (global job index % kShare) == slot
-    const int blk = MB == 1 ? 0 : grp & 1;  // the row block of every job this group gets
-    const int coff = blk * 128;              // first score row of that block
+    // A job is one block of 128 score rows of one key tile in one pass. Jobs are numbered through over passes and units
+    // and dealt round-robin: group grp takes jobs grp, grp + kGroups, ..; job J uses accumulator stage J mod kAcc.
+    const int grp = warp >> 2;
     const int quad = warp & 3;              // TMEM lane quadrant this warp may read
     const int row_in_tile = quad * 32 + lane;
     const uint32_t tlane = tmem_base + ((uint32_t)(quad * 32) << 16);
+    const uint32_t bar_af = smem_u32(&sm.acc_full[0]), bar_ae = smem_u32(&sm.acc_empty[0]);
     const float c = p.c;
     const float c252 = c * (1.0f / kPolyRange);
-    const int my_t = sm.row_t[coff + row_in_tile];  // pass 1: this thread's row is coff + row_in_tile
-    const int rows_mine = min(128, p.rows - coff);
-    const int n_chunks2 = (rows_mine + 31) >> 5;
 
-    auto acc_addr = [&](int jj) { return tlane + (uint32_t)((jj % kAcc) * 128); };
-    auto wait_full = [&](int jj, int where) {
-      mbar_wait(smem_u32(&sm.acc_full[jj % kAcc]), (uint32_t)(jj / kAcc) & 1u, abort_flag, p.status, where, limit);
+    auto acc_addr = [&](int J) { return tlane + (uint32_t)((J % kAcc) * 128); };
+    auto wait_full = [&](int J, int where) {
+      mbar_wait(bar_af + (J % kAcc) * 8, (uint32_t)(J / kAcc) & 1u, abort_flag, p.status, where, limit);
       tc_fence_after();
     };
-    auto release = [&](int jj) {  // the whole accumulator of the job is in registers: hand the stage back
+    auto release = [&](int J) {  // the whole accumulator of the job is in registers: hand the stage back
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(smem_u32(&sm.acc_empty[jj % kAcc]));
+      if (lane == 0) mbar_arrive(bar_ae + (J % kAcc) * 8);
     };
 
-    int jg = 0, it = 0;
-    int pc = 0;  // MB 2: tiles of pass 2 this group has handled (same count in both groups of a pair)
-    for (int u = cluster_id; u - cluster_id < p.units; u += n_clusters, ++it) {
-      const UnitInfo ui = get_unit(u);
-      const int n = ui.n, T = ui.T;
+    int J = grp;        // this group's next job
+    int jg = 0;         // first job of the current pass
+    int tg = 0;         // MB 2: pass-2 tiles of the units before this one
+    float ra[16], rb[16];
+    bool fetched = false;  // the first 16 columns of job J are in flight in `ra`
+    int us = 0;
+    uint32_t uph = 0;
+    for (int it = 0;; ++it) {
+      if (!mbar_wait(smem_u32(&sm.ufull[us]), uph, abort_flag, p.status, 35, limit)) break;
+      const UnitInfo ui = sm.unit[us];
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_u32(&sm.ufree[us]));
+      if (++us == kUnitRing) us = 0, uph ^= 1;
+      if (ui.end) break;
+      const int n = ui.n, n_jobs = MB * ui.T;
       const int up = it & 1;
-      const int Wp = min(p.W, n);
+      const uint32_t ph = (uint32_t)(it >> 1) & 1u;
+      const int j_last = jg + (p.two_pass ? 2 : 1) * n_jobs;  // end of the unit's jobs
+      auto fetch = [&](int Jn) {  // starts the load of job Jn's first 16 columns (waits for its products)
+        wait_full(Jn, 30);
+        tmem_ld16_issue(acc_addr(Jn), ra);
+      };
 
       if (p.two_pass) {
         // ---- pass 1: per row, sum of exp2(s*c - ref) against a reference `ref` that only has to keep the sum inside
         // the fp32 range (the result does not depend on it): the largest of the first 16 keys the row sees. After that
         // a key costs one multiply-add, one exponential and one add, and no maximum is tracked. A tile whose sum
-        // leaves the safe range (a score more than 2^60 above ref) is redone against its own maximum. That check must
-        // not wait for the tile's last exponentials (the accumulator stage is released right after it, and the next
-        // product into the stage waits for the release): it uses the sum without the last 16 keys and, for those,
-        // their largest score. The polynomial exponentials saturate at 2^126, which the same check catches.
-        float ref_c, z_run = 0.0f, pb;
-        const int pos = n - p.W + my_t;
-        const int lim = (my_t >= 0 && pos >= 0) ? (p.causal ? pos : n - 1) : -1;
-        // rows that see no key (padding) get a reference that turns every exponential into 0
-        ref_c = lim >= 0 ? -1e30f : 1e30f;
-        pb = poly_bias(ref_c);
+        // leaves the safe range (a score more than 2^60 above ref) is redone against its own maximum. The check runs
+        // before the accumulator stage is released and does not wait for the tile's last exponentials: it uses the sum
+        // without the last 16 keys and, for those, their largest score. The polynomial exponentials saturate at 2^126,
+        // which the same check catches; so does a row without a reference yet (ref -1e30).
+        float ref[MB], zsum[MB];
+        int lim[MB];
+#pragma unroll
+        for (int h = 0; h < MB; ++h) {
+          const int t = sm.row_t[h * 128 + row_in_tile];
+          const int pos = n - p.W + t;
+          lim[h] = (t >= 0 && pos >= 0) ? (p.causal ? pos : n - 1) : -1;
+          // rows that see no key (padding) get a reference that turns every exponential into 0
+          ref[h] = lim[h] >= 0 ? -1e30f : 1e30f;
+          zsum[h] = 0.0f;
+        }
         constexpr float kSumLimit = 1.0e18f;  // about 2^60
-        // 16 keys of one row: adds exp2(s*c - rc) to the four sums; `mix`: kPoly of them on the FMA pipe;
-        // `track`: also the largest s in `mx`. Masked tiles (cold) drop keys beyond `lim`.
-        auto half1 = [&](auto masked_tag, auto mix_tag, auto track_tag, const float(&cur)[16], float rc, float pbias,
-                         float(&s4)[4], float& mx, int kbase) {
+        // 16 keys of one row: adds exp2(s*c - rc) to the four sums; `mix`: some of them on the FMA pipe. Masked tiles
+        // drop keys beyond `lm`.
+        auto half1 = [&](auto masked_tag, auto mix_tag, const float(&cur)[16], float rc, float pbias, float(&s4)[4],
+                         int lm, int kbase) {
           constexpr bool masked = decltype(masked_tag)::value;
-          constexpr bool mix = decltype(mix_tag)::value && !masked;
-          constexpr bool track = decltype(track_tag)::value;
+          constexpr bool mix = decltype(mix_tag)::value;
           float v[16];
 #pragma unroll
-          for (int q = 0; q < 16; ++q) v[q] = cur[q];
-          if (masked) {
-#pragma unroll
-            for (int q = 0; q < 16; ++q)
-              if (kbase + q > lim) v[q] = -INFINITY;
-          }
+          for (int q = 0; q < 16; ++q) v[q] = (masked && kbase + q > lm) ? -INFINITY : cur[q];
 #pragma unroll
           for (int q = 0; q < 16; q += 2) {
-            if (mix && (poly_slot<MB>(q) || poly_slot<MB>(q + 1))) {
-#pragma unroll
-              for (int e2 = 0; e2 < 2; ++e2) {
-                const float e = poly_slot<MB>(q + e2) ? exp2_poly(v[q + e2], c252, pbias) : ex2(fmaf(v[q + e2], c, -rc));
-                s4[(q + e2) & 3] += e;
-              }
+            float e0, e1;
+            if (mix && !masked && poly_pair<MB>(q / 2)) {
+              exp2_poly2(e0, e1, v[q], v[q + 1], c252, pbias, pbias);
             } else {
-              float a0, a1;
-              fma2(a0, a1, v[q], v[q + 1], c, -rc, -rc);
-              add2(s4[q & 3], s4[(q & 3) + 1], ex2(a0), ex2(a1));
+              fma2(e0, e1, v[q], v[q + 1], c, -rc, -rc);
+              e0 = ex2(e0);
+              e1 = ex2(e1);
             }
-          }
-          if (track) {
-            float t4[4];
-#pragma unroll
-            for (int q = 0; q < 4; ++q) t4[q] = fmaxf(fmaxf(v[4 * q], v[4 * q + 1]), fmaxf(v[4 * q + 2], v[4 * q + 3]));
-            mx = fmaxf(mx, fmaxf(fmaxf(t4[0], t4[1]), fmaxf(t4[2], t4[3])));
+            add2(s4[q & 3], s4[(q & 3) + 1], e0, e1);
           }
         };
-        // largest of 16 keys of one row
-        auto max16 = [&](auto masked_tag, const float(&cur)[16], float& mx, int kbase) {
+        auto max16 = [&](auto masked_tag, const float(&cur)[16], int lm, int kbase) {  // largest of 16 keys of one row
           constexpr bool masked = decltype(masked_tag)::value;
           float t4[4];
 #pragma unroll
           for (int q = 0; q < 4; ++q) {
             float w[4];
 #pragma unroll
-            for (int e = 0; e < 4; ++e) w[e] = (masked && kbase + 4 * q + e > lim) ? -INFINITY : cur[4 * q + e];
+            for (int e = 0; e < 4; ++e) w[e] = (masked && kbase + 4 * q + e > lm) ? -INFINITY : cur[4 * q + e];
             t4[q] = fmaxf(fmaxf(w[0], w[1]), fmaxf(w[2], w[3]));
           }
-          mx = fmaxf(mx, fmaxf(fmaxf(t4[0], t4[1]), fmaxf(t4[2], t4[3])));
+          return fmaxf(fmaxf(t4[0], t4[1]), fmaxf(t4[2], t4[3]));
         };
-        float ra[16], rb[16];
-        int j = (slot - jg % kShare + kShare) % kShare;  // first job of this pass that belongs to the group
-        if (j < MB * T) {
-          wait_full(jg + j, 30);
-          tmem_ld16_issue(acc_addr(jg + j), ra);
-        }
         // One job: the 128 accumulator columns in 32-column chunks, each fetched as two 16-column loads (ra, rb) so
         // that one load is always in flight. On entry the load of the first 16 columns is in flight in `ra`.
-        auto job1 = [&](auto masked_tag, int j) {
-          const int jj = jg + j;
-          const int key0 = (ui.t_begin + j / MB) * kTileN;
-          const uint32_t abase = acc_addr(jj);
+        auto job1 = [&](auto masked_tag, float& ref_c, float& z_run, int lm, int key0) {
+          const uint32_t abase = acc_addr(J);
           float rc = ref_c;
-          const bool first = rc < -1e29f;
-          if (__any_sync(0xffffffffu, first)) {  // the row has no reference yet: take it from the 16 keys in flight
-            float mx = -INFINITY;
-            tmem_ld_wait(ra);
-            max16(masked_tag, ra, mx, key0);
-            if (first && mx > -INFINITY) {
-              rc = mx * c;
-              ref_c = rc;
-              pb = poly_bias(rc);
-            }
-          }
+          float pb = poly_bias(rc);
           float s4[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-          float sum_head = 0.0f, mx_tail = -INFINITY, unused = 0.0f;
 #pragma unroll 1
           for (int c4 = 0; c4 < 4; ++c4) {
             const uint32_t col = (uint32_t)(c4 * 32);
             tmem_ld_wait(ra);
             tmem_ld16_issue(abase + col + 16, rb);
-            half1(masked_tag, std::true_type{}, std::false_type{}, ra, rc, pb, s4, unused, key0 + c4 * 32);
+            half1(masked_tag, std::true_type{}, ra, rc, pb, s4, lm, key0 + c4 * 32);
             tmem_ld_wait(rb);
             if (c4 < 3) {
               tmem_ld16_issue(abase + col + 32, ra);
-              half1(masked_tag, std::true_type{}, std::false_type{}, rb, rc, pb, s4, unused, key0 + c4 * 32 + 16);
-            } else {
-              sum_head = (s4[0] + s4[1]) + (s4[2] + s4[3]);
-              half1(masked_tag, std::true_type{}, std::true_type{}, rb, rc, pb, s4, mx_tail, key0 + c4 * 32 + 16);
+              half1(masked_tag, std::true_type{}, rb, rc, pb, s4, lm, key0 + c4 * 32 + 16);
             }
           }
-          float sum = (s4[0] + s4[1]) + (s4[2] + s4[3]);
+          const float sum_head = (s4[0] + s4[1]) + (s4[2] + s4[3]);
+          const float mx_tail = max16(masked_tag, rb, lm, key0 + 112);
           // also true for inf and NaN sums
           const bool over = !(sum_head < kSumLimit) || fmaf(mx_tail, c, -rc) > 60.0f;
-          if (__any_sync(0xffffffffu, over)) {   // rare: a score far above the reference
+          if (__any_sync(0xffffffffu, over)) {  // rare: a score far above the reference
             float mx = -INFINITY;
 #pragma unroll 1
             for (int h = 0; h < 8; ++h) {
-              tmem_ld16_issue(abase + (uint32_t)(h * 16), rb);
-              tmem_ld_wait(rb);
-              max16(masked_tag, rb, mx, key0 + h * 16);
+              tmem_ld16_issue(abase + (uint32_t)(h * 16), ra);
+              tmem_ld_wait(ra);
+              mx = fmaxf(mx, max16(masked_tag, ra, lm, key0 + h * 16));
             }
             const float mx_c = mx * c;
             float r4[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll 1
-            for (int h = 0; h < 8; ++h) {
-              tmem_ld16_issue(abase + (uint32_t)(h * 16), rb);
-              tmem_ld_wait(rb);
-              half1(masked_tag, std::false_type{}, std::false_type{}, rb, over ? mx_c : rc, 0.0f, r4, unused,
-                    key0 + h * 16);
+            for (int h = 0; h < 7; ++h) {
+              tmem_ld16_issue(abase + (uint32_t)(h * 16), ra);
+              tmem_ld_wait(ra);
+              half1(masked_tag, std::false_type{}, ra, over ? mx_c : rc, 0.0f, r4, lm, key0 + h * 16);
             }
             if (over) {
               z_run *= ex2(rc - mx_c);
-              ref_c = mx_c;
+              rc = ref_c = mx_c;
               pb = poly_bias(mx_c);
-              sum = (r4[0] + r4[1]) + (r4[2] + r4[3]);
+#pragma unroll
+              for (int q = 0; q < 4; ++q) s4[q] = r4[q];
             }
           }
-          z_run += sum;
-          release(jj);
-          if (j + kShare < MB * T) {  // the next job of the group reuses this stage: fetch it once it is full again
-            wait_full(jj + kShare, 30);
-            tmem_ld16_issue(acc_addr(jj + kShare), ra);
-          }
+          release(J);
+          fetched = J + kGroups < j_last;
+          if (fetched) fetch(J + kGroups);
+          half1(masked_tag, std::true_type{}, rb, rc, pb, s4, lm, key0 + 112);
+          z_run += (s4[0] + s4[1]) + (s4[2] + s4[3]);
         };
-        for (; j < MB * T; j += kShare) {
+        const int j_end = jg + n_jobs;
+        bool first = true;
+        for (; J < j_end; J += kGroups) {
+          const int j = J - jg;
+          const int key0 = (ui.t_begin + j / MB) * kTileN;
+          if (!fetched) fetch(J);
+          // MB 2: the row block of a group's jobs alternates; its state is swapped into slot 0
+          const int h = MB == 2 ? j & 1 : 0;
+          float& rc = ref[0];
+          float& zr = zsum[0];
+          if (MB == 2 && h == 1) {
+            const float tr = ref[0], tz = zsum[0];
+            const int tl = lim[0];
+            ref[0] = ref[MB - 1], zsum[0] = zsum[MB - 1], lim[0] = lim[MB - 1];
+            ref[MB - 1] = tr, zsum[MB - 1] = tz, lim[MB - 1] = tl;
+          }
           // tiles that every row of the warp sees completely take the unmasked path (rows that see nothing at all,
           // i.e. padding, still run: their sums are never used)
-          const bool masked = lim >= 0 && (ui.t_begin + j / MB) * kTileN + kTileN - 1 > lim;
-          if (__any_sync(0xffffffffu, masked)) job1(std::true_type{}, j);
-          else job1(std::false_type{}, j);
-        }
-        // ---- exchange: group partials -> CTA partial -> every CTA of the cluster reads every other's
-        // rows that see no key at all (padding, window positions before the sequence start) stay mute
-        sm.part_m[grp][row_in_tile] = lim >= 0 ? ref_c : -1e30f;
-        sm.part_z[grp][row_in_tile] = lim >= 0 ? z_run : 0.0f;
-        softmax_bar<kGroups>();
-        float lse2_row = INFINITY;  // log2-domain log-sum-exp of row `st` (+inf: the row is mute)
-        if (st < kRowsPad) {
-          float m, z = 0.0f;
-          if (MB == 1) {
-            m = sm.part_m[0][st];
-#pragma unroll
-            for (int gq = 1; gq < kGroups; ++gq) m = fmaxf(m, sm.part_m[gq][st]);
-#pragma unroll
-            for (int gq = 0; gq < kGroups; ++gq) z += sm.part_z[gq][st] * ex2(sm.part_m[gq][st] - m);
-          } else {  // rows of block h were summed by groups h and h + 2
-            const int h = st >> 7, i = st & 127;
-            m = fmaxf(sm.part_m[h][i], sm.part_m[h + 2][i]);
-            z = sm.part_z[h][i] * ex2(sm.part_m[h][i] - m) + sm.part_z[h + 2][i] * ex2(sm.part_m[h + 2][i] - m);
+          const bool masked = __any_sync(0xffffffffu, lim[0] >= 0 && key0 + kTileN - 1 > lim[0]);
+          if (first) {  // the reference of the rows: from the 16 keys in flight
+            tmem_ld_wait(ra);
+            const float mx = masked ? max16(std::true_type{}, ra, lim[0], key0) : max16(std::false_type{}, ra, lim[0], key0);
+            if (rc < -1e29f && mx > -INFINITY) rc = mx * c;
+            first = MB == 2 && J < jg + kGroups;  // MB 2: the group's second job is the first of the other block
           }
-          if (p.cluster == 1) {  // nothing to exchange: the CTA's statistics are the unit's
-            lse2_row = (z > 0.0f) ? m + log2f(z) : INFINITY;
-          } else {
-            sm.mine_m[up][st] = m;
-            sm.mine_z[up][st] = z;
+          if (masked) job1(std::true_type{}, rc, zr, lim[0], key0);
+          else job1(std::false_type{}, rc, zr, lim[0], key0);
+          if (MB == 2 && h == 1) {
+            const float tr = ref[0], tz = zsum[0];
+            const int tl = lim[0];
+            ref[0] = ref[MB - 1], zsum[0] = zsum[MB - 1], lim[0] = lim[MB - 1];
+            ref[MB - 1] = tr, zsum[MB - 1] = tz, lim[MB - 1] = tl;
           }
         }
-        if (p.cluster > 1) {
-          softmax_bar<kGroups>();
-          // one thread per peer tells that peer that this CTA's statistics of the unit are in place
-          if (st < p.cluster) {
-            fence_cluster();
-            mbar_arrive_remote(smem_u32(&sm.xchg_full[up]), (uint32_t)st);
-          }
-          if (st < kRowsPad) {
-            mbar_wait_cluster(smem_u32(&sm.xchg_full[up]), (uint32_t)(it >> 1) & 1u, abort_flag, p.status, 32, limit);
-            float pm[kMaxCluster], pz[kMaxCluster];
+        // ---- the group's statistics of the unit; rows that see no key at all (padding, window positions before the
+        // sequence start) stay mute
 #pragma unroll
-            for (int r = 0; r < kMaxCluster; ++r) {
-              pm[r] = -1e30f;
-              pz[r] = 0.0f;
-              if (r < p.cluster) {
-                pm[r] = ld_cluster_f32(smem_u32(&sm.mine_m[up][st]), (uint32_t)r);
-                pz[r] = ld_cluster_f32(smem_u32(&sm.mine_z[up][st]), (uint32_t)r);
-              }
-            }
-            float m = pm[0];
-#pragma unroll
-            for (int r = 1; r < kMaxCluster; ++r) m = fmaxf(m, pm[r]);
-            float z = 0.0f;
-#pragma unroll
-            for (int r = 0; r < kMaxCluster; ++r) z += pz[r] * ex2(pm[r] - m);
-            lse2_row = (z > 0.0f) ? m + log2f(z) : INFINITY;
-          }
+        for (int h = 0; h < MB; ++h) {
+          sm.part_m[up][grp][h * 128 + row_in_tile] = lim[h] >= 0 ? ref[h] : -1e30f;
+          sm.part_z[up][grp][h * 128 + row_in_tile] = lim[h] >= 0 ? zsum[h] : 0.0f;
         }
-        if (st < kRowsPad) {
-          const float beta = lse2_row - sm.lv[st];
-          sm.nbeta[up][st] = -beta;
-          sm.tab[up][st] = poly_slot<MB>(st & 15) ? poly_bias(beta) : -beta;
-        }
-        softmax_bar<kGroups>();
-      } else {
-        if (st < kRowsPad) {
-          float lse2 = INFINITY;
-          const int t = sm.row_t[st];
-          if (t >= 0 && n - p.W + t >= 0) {
-            const int h = st / p.W;
-            const float lse = p.lse_obs[(((long long)ui.l * p.seq.batch + ui.b) * p.Hq + (ui.g * p.G + h)) * p.W + t];
-            lse2 = lse * 1.4426950408889634f;
-          }
-          const float beta = lse2 - sm.lv[st];
-          sm.nbeta[up][st] = -beta;
-          sm.tab[up][st] = poly_slot<MB>(st & 15) ? poly_bias(beta) : -beta;
-        }
-        softmax_bar<kGroups>();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(smem_u32(&sm.stat_full[up]));
+        jg = j_end;
       }
 
-      // ---- pass 2: for key row_in_tile of each tile, the sum over this group's rows of exp2(s*c - beta_row)
-      const int min_lim = p.causal ? n - Wp : n - 1;  // every valid row sees keys up to here
-      const int j0 = p.two_pass ? MB * T : 0;
-      const int n_jobs = j0 + MB * T;
-      const long long unit_off = ((long long)ui.l * p.Hkv + ui.g) * p.seq.total;
-      const float4* tab4 = reinterpret_cast<const float4*>(sm.tab[up] + coff);
-      const float4* nb4 = reinterpret_cast<const float4*>(sm.nbeta[up] + coff);
-      const float4* w4 = reinterpret_cast<const float4*>(sm.wrow + coff);
+      // ---- pass 2: for key row_in_tile of each tile, the sum over the job's rows of exp2(s*c - beta_row)
       {
-        float sA4[4], sP = 0.0f;
-        // 16 rows (half `hi` of the 32-row chunk cc) of this thread's key. Hot form: kPoly of the 16 exponentials on
-        // the FMA pipe, row constants from `tab`. Masked form (keys inside the observation window, cold tiles only):
-        // every exponential on the special-function unit against -beta, rows that do not see the key dropped.
-        auto chunk2 = [&](auto masked_tag, auto hi_tag, const float(&cur)[16], int cc, int key) {
+        mbar_wait(smem_u32(&sm.tab_full[up]), ph, abort_flag, p.status, 39, limit);
+        // every valid row sees keys up to here; key i beyond it is seen by the rows with t >= i - (n - W)
+        const int min_lim = p.causal ? n - min(p.W, n) : n - 1;
+        const long long out0 = ((long long)ui.l * p.Hkv + ui.g) * p.seq.total + ui.tok0;
+        float sA4[4], sP;
+        // 16 rows (half `hi` of the 32-row chunk cc) of this thread's key, a share of the exponentials on the FMA pipe.
+        // Masked form (keys inside the observation window): rows that do not see the key are dropped.
+        auto chunk2 = [&](auto masked_tag, auto hi_tag, const float(&cur)[16], int row0, int tau) {
           constexpr bool masked = decltype(masked_tag)::value;
-          constexpr int hi = decltype(hi_tag)::value;  // 0: rows 32cc..32cc+15, 1: rows 32cc+16..32cc+31
+          constexpr int hi = decltype(hi_tag)::value;  // 0: rows row0..row0+15, 1: rows row0+16..row0+31
+          const float4* tab4 = reinterpret_cast<const float4*>(&sm.tab[up][row0]) + hi * 4;
+          const float4* w4 = reinterpret_cast<const float4*>(&sm.wrow[row0]) + hi * 4;
+          const int4* t4 = reinterpret_cast<const int4*>(&sm.row_t[row0]) + hi * 4;
 #pragma unroll
           for (int q4 = 0; q4 < 4; ++q4) {
-            const float4 tb = masked ? nb4[cc * 8 + hi * 4 + q4] : tab4[cc * 8 + hi * 4 + q4];
+            const float4 tb = tab4[q4];
             const float tbv[4] = {tb.x, tb.y, tb.z, tb.w};
             float a[4];
 #pragma unroll
             for (int e = 0; e < 4; e += 2) {
-              if (!masked && (poly_slot<MB>(4 * q4 + e) || poly_slot<MB>(4 * q4 + e + 1))) {
-#pragma unroll
-                for (int e2 = e; e2 < e + 2; ++e2)
-                  a[e2] = poly_slot<MB>(4 * q4 + e2) ? exp2_poly(cur[4 * q4 + e2], c252, tbv[e2])
-                                                     : ex2(fmaf(cur[4 * q4 + e2], c, tbv[e2]));
+              if (poly_pair<MB>(2 * q4 + e / 2)) {
+                exp2_poly2(a[e], a[e + 1], cur[4 * q4 + e], cur[4 * q4 + e + 1], c252, tbv[e], tbv[e + 1]);
               } else {
-                float x0, x1;
-                fma2(x0, x1, cur[4 * q4 + e], cur[4 * q4 + e + 1], c, tbv[e], tbv[e + 1]);
-                a[e] = ex2(x0);
-                a[e + 1] = ex2(x1);
+                fma2(a[e], a[e + 1], cur[4 * q4 + e], cur[4 * q4 + e + 1], c, tbv[e], tbv[e + 1]);
+                a[e] = ex2(a[e]);
+                a[e + 1] = ex2(a[e + 1]);
               }
             }
-            if (masked) {  // row r sees key i only if i <= the row's own position
-#pragma unroll
-              for (int e = 0; e < 4; ++e) {
-                const int t = sm.row_t[coff + cc * 32 + hi * 16 + 4 * q4 + e];
-                const int pos = n - p.W + t;
-                const int lim = (t >= 0 && pos >= 0) ? (p.causal ? pos : n - 1) : -1;
-                if (key > lim) a[e] = 0.0f;
-              }
+            if (masked) {
+              const int4 tt = t4[q4];
+              if (tt.x < tau) a[0] = 0.0f;
+              if (tt.y < tau) a[1] = 0.0f;
+              if (tt.z < tau) a[2] = 0.0f;
+              if (tt.w < tau) a[3] = 0.0f;
             }
             add2(sA4[0], sA4[1], a[0], a[1]);
             add2(sA4[2], sA4[3], a[2], a[3]);
             if (PM == kOutAP) {
-              const float4 ws = w4[cc * 8 + hi * 4 + q4];
+              const float4 ws = w4[q4];
               sP = fmaf(ws.x, a[0], sP);
               sP = fmaf(ws.y, a[1], sP);
               sP = fmaf(ws.z, a[2], sP);
@@ -721,67 +800,60 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
             }
           }
         };
-        float ra[16], rb[16];
-        int j = j0 + (slot - (jg + j0) % kShare + kShare) % kShare;
-        if (j < n_jobs) {
-          wait_full(jg + j, 31);
-          tmem_ld16_issue(acc_addr(jg + j), ra);
-        }
         // one job: 32-row chunks, each as two 16-column loads (ra low half, rb high half)
-        auto job2 = [&](auto masked_tag, int j, int key) {
-          const int jj = jg + j;
-          const uint32_t abase = acc_addr(jj);
+        auto job2 = [&](auto masked_tag, int row0, int n_chunks, int tau) {
+          const uint32_t abase = acc_addr(J);
 #pragma unroll 1
-          for (int ci = 0; ci < n_chunks2; ++ci) {
+          for (int ci = 0; ci < n_chunks; ++ci) {
             const uint32_t col = (uint32_t)(ci * 32);
             tmem_ld_wait(ra);
             tmem_ld16_issue(abase + col + 16, rb);
-            chunk2(masked_tag, std::integral_constant<int, 0>{}, ra, ci, key);
+            chunk2(masked_tag, std::integral_constant<int, 0>{}, ra, row0 + ci * 32, tau);
             tmem_ld_wait(rb);
-            if (ci == n_chunks2 - 1) {
-              release(jj);
-              if (j + kShare < n_jobs) {
-                wait_full(jj + kShare, 31);
-                tmem_ld16_issue(acc_addr(jj + kShare), ra);
-              }
+            if (ci == n_chunks - 1) {
+              release(J);
+              fetched = J + kGroups < j_last;
+              if (fetched) fetch(J + kGroups);
             } else {
               tmem_ld16_issue(abase + col + 32, ra);
             }
-            chunk2(masked_tag, std::integral_constant<int, 1>{}, rb, ci, key);
+            chunk2(masked_tag, std::integral_constant<int, 1>{}, rb, row0 + ci * 32, tau);
           }
         };
-        for (; j < n_jobs; j += kShare) {
-          const int tl = (j - j0) / MB;  // the pass walks the CTA's tiles backwards after a first pass
-          const int key = (ui.t_begin + (p.two_pass ? T - 1 - tl : tl)) * kTileN + row_in_tile;
+        for (; J < j_last; J += kGroups) {
+          const int j = J - jg, h = MB == 2 ? j & 1 : 0;
+          const int tl = j / MB;  // the pass walks the CTA's tiles backwards after a first pass
+          const int key = (ui.t_begin + (p.two_pass ? ui.T - 1 - tl : tl)) * kTileN + row_in_tile;
+          const int n_chunks = (min(128, p.rows - h * 128) + 31) >> 5;
+          if (!fetched) fetch(J);
           sA4[0] = sA4[1] = sA4[2] = sA4[3] = 0.0f;
           sP = 0.0f;
           // only the last W-1 keys of a sequence are hidden from some rows: those tiles take the masked path
-          if (__all_sync(0xffffffffu, key <= min_lim || key >= n)) job2(std::false_type{}, j, key);
-          else job2(std::true_type{}, j, key);
+          if (__all_sync(0xffffffffu, key <= min_lim || key >= n)) job2(std::false_type{}, h * 128, n_chunks, 0);
+          else job2(std::true_type{}, h * 128, n_chunks, p.causal ? key - (n - p.W) : -1);
           float sA = (sA4[0] + sA4[1]) + (sA4[2] + sA4[3]);
           if (MB == 2) {
             // The two row blocks of a tile are consecutive jobs of two different groups. The group of block 0 leaves
             // its sums in a ring slot and goes on; the group of block 1, which gets its job later, picks them up, adds
             // its own and stores. Neither waits for the other unless the ring is full (block 0 four tiles ahead).
-            const int pr = grp >> 1, r = pc % Cfg::kRing;
-            const uint32_t ph = (uint32_t)(pc / Cfg::kRing) & 1u;
-            ++pc;
-            if (blk == 0) {
-              mbar_wait(smem_u32(&sm.pfree[pr][r]), ph ^ 1u, abort_flag, p.status, 33, limit);
-              sm.psum[pr][r][0][row_in_tile] = sA;
-              if (PM == kOutAP) sm.psum[pr][r][1][row_in_tile] = sP;
+            const int r = (tg + tl) % kRing;
+            const uint32_t rph = (uint32_t)((tg + tl) / kRing) & 1u;
+            if (h == 0) {
+              mbar_wait(smem_u32(&sm.pfree[r]), rph ^ 1u, abort_flag, p.status, 33, limit);
+              sm.psum[r][0][row_in_tile] = sA;
+              if (PM == kOutAP) sm.psum[r][1][row_in_tile] = sP;
               __syncwarp();
-              if (lane == 0) mbar_arrive(smem_u32(&sm.pfull[pr][r]));
+              if (lane == 0) mbar_arrive(smem_u32(&sm.pfull[r]));
             } else {
-              mbar_wait(smem_u32(&sm.pfull[pr][r]), ph, abort_flag, p.status, 34, limit);
-              sA += sm.psum[pr][r][0][row_in_tile];
-              if (PM == kOutAP) sP += sm.psum[pr][r][1][row_in_tile];
+              mbar_wait(smem_u32(&sm.pfull[r]), rph, abort_flag, p.status, 34, limit);
+              sA += sm.psum[r][0][row_in_tile];
+              if (PM == kOutAP) sP += sm.psum[r][1][row_in_tile];
               __syncwarp();
-              if (lane == 0) mbar_arrive(smem_u32(&sm.pfree[pr][r]));
+              if (lane == 0) mbar_arrive(smem_u32(&sm.pfree[r]));
             }
           }
-          if (blk == MB - 1 && key < n && !*abort_flag) {
-            const long long o = unit_off + ui.tok0 + key;
+          if (h == MB - 1 && key < n && !*abort_flag) {
+            const long long o = out0 + key;
             if (PM == kOutFused) {
               p.u[o] = sA;
             } else {
@@ -791,8 +863,11 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
             }
           }
         }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(smem_u32(&sm.tab_free[up]));
       }
-      if (T > 0) jg += n_jobs;
+      jg = j_last;
+      tg += ui.T;
     }
   }
 
@@ -888,6 +963,11 @@ cudaError_t launch_variant(ta_ctx* ctx, const CUtensorMap& mq, const CUtensorMap
     const long long rounds = (sp.units + avail - 1) / avail;
     const long long per_cta = (tiles_max + cl - 1) / cl;
     const long long cost = rounds * (per_cta + (cl > 1 ? 3 : 1));
+    if (sp.flat) {  // equal shares whatever the number of units: nothing to gain from more CTAs per unit
+      best_cl = cl;
+      best_cost = 0;
+      break;
+    }
     if (best_cost < 0 || cost < best_cost) {
       best_cost = cost;
       best_cl = cl;
@@ -898,7 +978,8 @@ cudaError_t launch_variant(ta_ctx* ctx, const CUtensorMap& mq, const CUtensorMap
   attr[0].val.clusterDim.x = (unsigned)best_cl;
   int n_clusters = max_clusters[best_cl] - (reserve_sms + best_cl - 1) / best_cl;
   if (n_clusters < 1) n_clusters = 1;
-  if (n_clusters > sp.units) n_clusters = sp.units;
+  const long long pieces = sp.flat ? (long long)sp.units * tiles_max : sp.units;
+  if (n_clusters > pieces) n_clusters = (int)pieces;
   ctx->score_cluster = sp.cluster;
   ctx->score_clusters = n_clusters;
   cfg.gridDim = dim3((unsigned)(n_clusters * sp.cluster), 1, 1);
@@ -973,6 +1054,7 @@ cudaError_t ta_launch_score(ta_ctx* ctx, const ta_score_args& a, ta_dev_status* 
   sp.rows = rows;
   sp.two_pass = a.lse_obs ? 0 : 1;
   sp.causal = a.causal;
+  sp.flat = a.lse_obs && !a.seq.cu && ctx->score_force_cluster <= 0;
   const float scale = a.scale > 0.0f ? a.scale : 1.0f / sqrtf((float)kD);
   sp.c = scale * 1.4426950408889634f;
   sp.alpha = a.alpha;

@@ -35,6 +35,26 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
       : "memory");
   return ok != 0;
 }
+// One look of a whole warp at a phase: true when it has completed. Never suspends.
+__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n"
+      ".reg .pred p;\n"
+      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+      "selp.u32 %0, 1, 0, p;\n"
+      "}\n"
+      : "=r"(ok)
+      : "r"(bar), "r"(parity)
+      : "memory");
+  return __all_sync(0xffffffffu, ok != 0);
+}
+// True on one lane of a converged warp.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n.reg .pred q;\nelect.sync _|q, 0xffffffff;\nselp.u32 %0, 1, 0, q;\n}" : "=r"(p));
+  return p != 0;
+}
 __device__ __forceinline__ unsigned long long globaltimer_ns() {
   unsigned long long t;
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
@@ -63,30 +83,25 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
-__device__ __forceinline__ void umma_bf16(uint32_t tmem_d, uint64_t desc_a, uint64_t desc_b, uint32_t idesc,
-                                          uint32_t accumulate) {
+// D (+)= A * B, bf16 inputs, one 128 x N x 16 product. The operand descriptors are given as their lower words (address
+// >> 4) with immediate offsets, and the common upper word; the sums are formed at the instruction and never kept in
+// registers across the caller's loop.
+template <uint32_t A_OFF, uint32_t B_OFF, bool ACC>
+__device__ __forceinline__ void umma_bf16_off(uint32_t tmem_d, uint32_t a_lo, uint32_t b_lo, uint32_t desc_hi,
+                                              uint32_t idesc) {
   asm volatile(
       "{\n"
       ".reg .pred p;\n"
-      "setp.ne.b32 p, %4, 0;\n"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n"
-      "}\n" ::"r"(tmem_d),
-      "l"(desc_a), "l"(desc_b), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-// The same with the descriptors given as their lower words (address >> 4) and the common upper word.
-__device__ __forceinline__ void umma_bf16_lo(uint32_t tmem_d, uint32_t a_lo, uint32_t b_lo, uint32_t desc_hi,
-                                             uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n"
-      ".reg .pred p;\n"
+      ".reg .b32 la, lb;\n"
       ".reg .b64 da, db;\n"
-      "mov.b64 da, {%1, %3};\n"
-      "mov.b64 db, {%2, %3};\n"
-      "setp.ne.b32 p, %5, 0;\n"
+      "add.u32 la, %1, %5;\n"
+      "add.u32 lb, %2, %6;\n"
+      "mov.b64 da, {la, %3};\n"
+      "mov.b64 db, {lb, %3};\n"
+      "setp.ne.b32 p, %7, 0;\n"
       "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p;\n"
       "}\n" ::"r"(tmem_d),
-      "r"(a_lo), "r"(b_lo), "r"(desc_hi), "r"(idesc), "r"(accumulate)
+      "r"(a_lo), "r"(b_lo), "r"(desc_hi), "r"(idesc), "n"(A_OFF), "n"(B_OFF), "n"(ACC ? 1 : 0)
       : "memory");
 }
 __device__ __forceinline__ void umma_commit(uint32_t bar) {
@@ -153,11 +168,6 @@ __device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t par
       : "memory");
   return ok != 0;
 }
-template <int NG>
-__device__ __forceinline__ void softmax_bar() {
-  asm volatile("bar.sync 1, %0;" ::"n"(NG * 128) : "memory");
-}
-
 // Shared-memory matrix descriptor for a K-major operand tile stored as rows of 128 bytes with the 128-byte swizzle
 // (what a TMA box of 64 bf16 x rows with CU_TENSOR_MAP_SWIZZLE_128B writes): 8-row groups are 1024 bytes apart.
 __device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t addr) {
@@ -175,9 +185,10 @@ __device__ __forceinline__ uint32_t idesc_bf16(int M, int N) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
-// Bounded wait on an mbarrier phase. Returns false (and raises the CTA's abort flag) when `limit_ns` of wall time
-// have passed or another thread of the CTA already gave up. The common case (the phase has completed) is one inlined
-// try_wait. CLUSTER: the barrier is arrived on by peers of the cluster (acquire at cluster scope).
+// Bounded wait of a whole (converged) warp on an mbarrier phase. Returns false on every lane (and raises the CTA's abort
+// flag) when `limit_ns` of wall time have passed or another warp of the CTA already gave up. The common case (the phase has
+// completed) is one inlined try_wait and a vote, which also tells the compiler that the branch is warp-uniform. CLUSTER:
+// the barrier is arrived on by peers of the cluster (acquire at cluster scope).
 template <bool CLUSTER>
 __device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
   if constexpr (CLUSTER) return mbar_try_wait_cluster(bar, parity);
@@ -212,8 +223,8 @@ __device__ __forceinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity, vo
 }
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag,
                                           ta_dev_status* status, int where, unsigned long long limit_ns) {
-  if (mbar_try_wait(bar, parity)) return true;
-  return mbar_wait_slow<false>(bar, parity, abort_flag, status, where, limit_ns);
+  if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+  return __all_sync(0xffffffffu, mbar_wait_slow<false>(bar, parity, abort_flag, status, where, limit_ns));
 }
 // Wait used while draining after a failed wait: bounded, reports nothing (the failure is already recorded).
 __device__ __forceinline__ void mbar_wait_drain(uint32_t bar, uint32_t parity, unsigned long long limit_ns) {
@@ -224,8 +235,8 @@ __device__ __forceinline__ void mbar_wait_drain(uint32_t bar, uint32_t parity, u
 // Bounded wait with cluster-scope acquire (for barriers that peers of the cluster arrive on).
 __device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity, volatile int* abort_flag,
                                                   ta_dev_status* status, int where, unsigned long long limit_ns) {
-  if (mbar_try_wait_cluster(bar, parity)) return true;
-  return mbar_wait_slow<true>(bar, parity, abort_flag, status, where, limit_ns);
+  if (__all_sync(0xffffffffu, mbar_try_wait_cluster(bar, parity))) return true;
+  return __all_sync(0xffffffffu, mbar_wait_slow<true>(bar, parity, abort_flag, status, where, limit_ns));
 }
 
 }  // namespace ta_sm100
