@@ -229,9 +229,6 @@ ta_status ta_ctx_create(int device, size_t scratch_bytes, ta_ctx** out) {
   if (e == cudaSuccess) e = cudaMemset(c->d_status, 0, sizeof(ta_dev_status));
   if (e == cudaSuccess && scratch_bytes) e = cudaMalloc(&c->scratch, scratch_bytes);
   for (int i = 0; e == cudaSuccess && i < 8; ++i) e = cudaEventCreate(&c->ev[i]);
-  if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking);
-  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming);
-  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming);
   if (e == cudaSuccess) {
     cudaDriverEntryPointQueryResult q;
     e = cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &c->encode_tiled, cudaEnableDefault, &q);
@@ -250,9 +247,6 @@ void ta_ctx_destroy(ta_ctx* c) {
   DeviceGuard guard(c->device);
   for (int i = 0; i < 8; ++i)
     if (c->ev[i]) cudaEventDestroy(c->ev[i]);
-  if (c->ev_fork) cudaEventDestroy(c->ev_fork);
-  if (c->ev_join) cudaEventDestroy(c->ev_join);
-  if (c->side) cudaStreamDestroy(c->side);
   if (c->scratch) cudaFree(c->scratch);
   if (c->d_status) cudaFree(c->d_status);
   delete c;
@@ -344,7 +338,7 @@ ta_status ta_ctx_read_timing(ta_ctx* ctx, float out_ms[5]) {
   if (!ctx->timing_valid) return TA_ERR_INVALID_ARG;
   DeviceGuard guard(ctx->device);
   cudaError_t e = cudaEventSynchronize(ctx->ev[4]);
-  if (e == cudaSuccess && ctx->ev_ran[0]) {  // per-sequence work runs on the side stream, beside the score kernel
+  if (e == cudaSuccess && ctx->ev_ran[0]) {
     e = cudaEventSynchronize(ctx->ev[6]);
     if (e == cudaSuccess) e = cudaEventElapsedTime(&out_ms[0], ctx->ev[5], ctx->ev[6]);
   }
@@ -760,40 +754,36 @@ ta_status compress_impl(ta_ctx* ctx, const ta_patterns* pats, const ta_policy* p
   ctx->last_select_gathered = select_gathers ? 1 : 0;
   int launches = 0;  // kernels of this library enqueued by this call
 
-  // Per-sequence work (anchor mask, vouchers, static utility, forced set) does not depend on Q/K: in scored mode it
-  // runs on the context's side stream beside the score kernel and joins before the per-unit selection.
+  // The chain runs on the caller's stream alone. Every kernel is launched as a programmatic dependent of the kernel before
+  // it (its launch overlaps that kernel's tail) and waits for it before it touches memory, with one exception: the
+  // per-sequence kernels let their dependents start at once, and the score kernel, which reads nothing that they write,
+  // runs beside them and waits for them at its own end.
   mark(0);
   ctx->ev_ran[0] = 0;
-  cudaStream_t seq_stream = stream;
-  // ...but only while the score kernel is short. It is persistent, so kernels beside it need SMs of their own (4 are
-  // left free); a long score kernel gains more from those SMs than the step gains from hiding the per-sequence work,
-  // which then simply runs first.
-  const long long score_jobs = (lse_obs ? 1LL : 2LL) * batch->n_layers * batch->batch * Hkv * ((batch->max_n + 127) / 128) *
-                               (((Hq / Hkv) * policy->obs_window + 127) / 128);
-  const bool fork = !reuse && !fast && !external && score_jobs <= 400LL * ctx->sm_count;
-  // Kernels of the chain that directly follow another kernel of the chain on their stream are launched as its
-  // programmatic dependents: their launch overlaps its tail, and they wait for it before they touch memory. The
-  // forced-set kernel follows the mask kernel; the selection follows the score kernel, the forced-set kernel or the
-  // head sum (not across the join with the side stream); the broadcast and the gather follow the selection.
   sel.pdl_forced = 1;
-  sel.pdl_units = fork ? 0 : 1;
-  if (fork) {
-    seq_stream = ctx->side;
-    e = cudaEventRecord(ctx->ev_fork, stream);
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(ctx->side, ctx->ev_fork, 0);
-  }
+  sel.pdl_units = 1;
+  bool beside = false;  // the kernel before the score kernel is one that lets it start at once
   if (!reuse) {
-    if (timing && e == cudaSuccess) e = cudaEventRecord(ctx->ev[5], seq_stream);
-    if (e == cudaSuccess)
-      e = ta_launch_mask(pats, *policy, seq, token_ids, flags, voucher, nullptr, hist, ctx->d_status, seq_stream);
-    if (e == cudaSuccess) e = ta_launch_forced(sel, ctx->d_status, seq_stream);
-    launches += 2;  // mask, forced set (which also writes the static utilities)
+    if (timing && e == cudaSuccess) e = cudaEventRecord(ctx->ev[5], stream);
+    if (!budgets && ta_front_fits(seq)) {
+      if (e == cudaSuccess) e = ta_launch_front(pats, *policy, sel, token_ids, hist, ctx->d_status, stream);
+      launches += 1;
+    } else {
+      if (e == cudaSuccess)
+        e = ta_launch_mask(pats, *policy, seq, token_ids, flags, voucher, nullptr, hist, ctx->d_status, stream);
+      if (e == cudaSuccess) e = ta_launch_forced(sel, ctx->d_status, stream);
+      launches += 2;  // mask, forced set (which also writes the static utilities)
+      if (e == cudaSuccess && fast) {
+        e = ta_launch_select_units(sel, stream);
+        launches += 1;
+      }
+    }
+    beside = true;
     if (timing && e == cudaSuccess) {
-      e = cudaEventRecord(ctx->ev[6], seq_stream);
+      e = cudaEventRecord(ctx->ev[6], stream);
       ctx->ev_ran[0] = 1;
     }
   }
-  if (fork && e == cudaSuccess) e = cudaEventRecord(ctx->ev_join, ctx->side);
   mark(1);
   if (e == cudaSuccess && !fast && !external) {
     ta_score_args a = {};
@@ -808,26 +798,22 @@ ta_status compress_impl(ta_ctx* ctx, const ta_patterns* pats, const ta_policy* p
     a.A = nullptr;
     a.P = nullptr;
     a.u = u;
-      a.alpha = policy->alpha;
+    a.alpha = policy->alpha;
     a.delta = policy->delta;
     a.rho = policy->pension_rho;
     a.scale = policy->softmax_scale;
     a.causal = policy->causal;
-    a.reserve_sms = fork ? 4 : 0;
+    a.pdl = beside && !timing ? 2 : 1;  // (timed: the event between the kernels orders them)
     a.order_scratch = batch->cu_seqlens ? reinterpret_cast<int32_t*>(sc + L.order) : nullptr;
-    e = ta_launch_score(ctx, a, ctx->d_status, stream);
-    launches += a.order_scratch && batch->batch > 1 ? 2 : 1;  // (unit order of a ragged batch,) score
+    e = ta_launch_score(ctx, a, ctx->d_status, stream, &launches);
   }
   mark(2);
-  if (fork && e == cudaSuccess) e = cudaStreamWaitEvent(stream, ctx->ev_join, 0);
   if (e == cudaSuccess && share_heads && !ext_u_all)
     e = ta_launch_headsum(batch->n_layers, Hkv, batch->total_tokens, u, u_all, stream);
-  if (e == cudaSuccess && !(fast && reuse)) e = ta_launch_select_units(sel, stream);
-  launches += (share_heads ? 2 : 0) + (fast && reuse ? 0 : 1) + (fast ? 1 : 0) + (select_gathers ? 0 : 1);
+  if (e == cudaSuccess && !fast) e = ta_launch_select_units(sel, stream);
+  launches += (share_heads ? 2 : 0) + (fast ? 0 : 1) + (select_gathers ? 0 : 1);
   if (e == cudaSuccess && share_heads)
     e = ta_launch_broadcast_heads(batch->n_layers, batch->batch, Hkv, K, idx_lb, count_lb, idx, count, stream);
-  if (e == cudaSuccess && fast)
-    e = ta_launch_broadcast_idx(batch->batch, Hkv, K, batch->n_layers, idx_seq, count_seq, idx, count, stream, true);
   mark(3);
   if (e == cudaSuccess && !select_gathers) {
     ta_compact_args a = {};
@@ -837,8 +823,10 @@ ta_status compress_impl(ta_ctx* ctx, const ta_patterns* pats, const ta_policy* p
     a.K = K;
     a.k = k;
     a.v = v;
-    a.idx = idx;
-    a.count = count;
+    a.idx = fast ? idx_seq : idx;  // fast mode: the per-sequence result is the same for all layers and heads
+    a.count = fast ? count_seq : count;
+    a.idx_out = fast ? idx : nullptr;
+    a.count_out = fast ? count : nullptr;
     a.k_out = k_out;
     a.v_out = v_out;
     a.pdl = 1;

@@ -30,6 +30,8 @@ __device__ __forceinline__ void st_stream(uint4* p, uint4 v) {
 __global__ void __launch_bounds__(kThreads) ta_compact_kernel(ta_seq_desc seq, int Hkv, int K, ta_bf16_view kv0,
                                                               ta_bf16_view kv1, const int32_t* __restrict__ idx,
                                                               const int32_t* __restrict__ count,
+                                                              int32_t* __restrict__ idx_out,
+                                                              int32_t* __restrict__ count_out,
                                                               uint4* __restrict__ out0, uint4* __restrict__ out1) {
   ta_wait_for_prior_grid();
   const int unit = blockIdx.x;
@@ -38,14 +40,21 @@ __global__ void __launch_bounds__(kThreads) ta_compact_kernel(ta_seq_desc seq, i
   const int l = unit / (Hkv * seq.batch);
   const ta_bf16_view src = blockIdx.z ? kv1 : kv0;
   uint4* out = (blockIdx.z ? out1 : out0) + (long long)unit * K * kLanesPerRow;
-  const int32_t* uidx = idx + (long long)unit * K;
-  const int cnt = count[unit];
+  const int res = idx_out ? b : unit;  // one result per sequence, or one per unit
+  const int32_t* uidx = idx + (long long)res * K;
+  const int cnt = count[res];
   const int n = seq.cu ? seq.cu[b + 1] - seq.cu[b] : seq.n_uniform;
   const long long base = (long long)l * src.stride_l + (long long)g * src.stride_h +
                          (seq.cu ? (long long)seq.cu[b] * src.stride_n : (long long)b * src.stride_b);
   const uint16_t* sp = reinterpret_cast<const uint16_t*>(src.ptr) + base;
   const int lane16 = threadIdx.x % kLanesPerRow;
   const int r0 = blockIdx.y * kRowsPerBlock + threadIdx.x / kLanesPerRow;
+
+  if (idx_out && blockIdx.z == 0) {  // the unit's copy of its sequence's result
+    const int r = blockIdx.y * kRowsPerBlock + threadIdx.x;
+    if (threadIdx.x < kRowsPerBlock && r < K) idx_out[(long long)unit * K + r] = uidx[r];
+    if (blockIdx.y == 0 && threadIdx.x == 0) count_out[unit] = cnt;
+  }
 
   uint4 v[kUnroll];
   int rows[kUnroll];
@@ -81,5 +90,5 @@ cudaError_t ta_launch_compact(const ta_compact_args& a, int sm_count, cudaStream
   cfg.attrs = attr;
   cfg.numAttrs = a.pdl ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, ta_compact_kernel, a.seq, a.Hkv, a.K, a.k, a.v, a.idx, a.count,
-                            reinterpret_cast<uint4*>(a.k_out), reinterpret_cast<uint4*>(a.v_out));
+                            a.idx_out, a.count_out, reinterpret_cast<uint4*>(a.k_out), reinterpret_cast<uint4*>(a.v_out));
 }

@@ -45,15 +45,12 @@ struct ta_ctx {
   int timing_valid;
   cudaEvent_t ev[8];
   int ev_ran[4];
-  // fork/join of the per-sequence work (mask, vouchers, forced set) beside the score kernel
-  cudaStream_t side;
-  cudaEvent_t ev_fork, ev_join;
   // launch shape of the most recent score kernel (diagnostics)
   int score_cluster, score_clusters;
   // score kernel launch state per instantiation (2 row-block counts x 3 output forms): attribute set, resident
   // clusters per cluster size (0: not queried yet, -1: does not fit)
   int score_attr_set[6];
-  int score_max_clusters[6][9];
+  int score_max_clusters[6][17];
   int last_select_gathered;           // the most recent ta_compress let the selection kernel gather the rows
   int last_kernel_launches;           // kernels enqueued by the most recent ta_compress
   int score_force_cluster;            // > 0: CTAs per unit fixed by ta_ctx_set_option (tuning, tests)
@@ -85,14 +82,26 @@ inline void ta_pdl_attribute(cudaLaunchAttribute* attr) {
 }
 #ifdef __CUDACC__
 __device__ __forceinline__ void ta_wait_for_prior_grid() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// Lets the programmatic dependent of this kernel be scheduled once every block has called this (or ended). Called after the
+// kernel's own wait: the dependent may then rely on everything before this kernel being complete.
+__device__ __forceinline__ void ta_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// x / n rounded to nearest for whole numbers 0 <= x <= 2^24 and 1 <= n <= 2^24, given r = 1/n rounded to nearest: one
+// product and one residual correction, which is correctly rounded because r is (Markstein's theorem; no over- or underflow
+// in this range). Many tokens share n: three instructions a quotient, where a division costs about twenty.
+__device__ __forceinline__ float ta_div_by(float x, float n, float r) {
+  const float q = __fmul_rn(x, r);
+  return __fmaf_rn(__fmaf_rn(-q, n, x), r, q);
+}
 
 // Static part of a token's utility (Eq. 3): u_static = ((beta*R + gamma*S) - lambda*F) + V with R = (i0+1)/n,
 // S = 1 on anchor tokens, F = count(id)/n; one rounding per operation. i0 is the 0-based position in the sequence.
 __device__ __forceinline__ float ta_static_utility(int i0, int n, int count, bool anchor_token, float V, float beta,
                                                    float gamma, float lambda) {
-  const float R = __fdiv_rn((float)(i0 + 1), (float)n);
+  const float r = __frcp_rn((float)n);  // (the same for all tokens of a sequence: hoisted out of their loop)
+  const float R = ta_div_by((float)(i0 + 1), (float)n, r);
   const float S = anchor_token ? 1.0f : 0.0f;
-  const float F = __fdiv_rn((float)count, (float)n);
+  const float F = ta_div_by((float)count, (float)n, r);
   const float t0 = __fadd_rn(__fmul_rn(beta, R), __fmul_rn(gamma, S));
   const float t1 = __fsub_rn(t0, __fmul_rn(lambda, F));
   return __fadd_rn(t1, V);
@@ -125,10 +134,16 @@ struct ta_score_args {
   float* u;              // nullable: fused attention part alpha*A + delta*P (u_static is added by the selection)
   float alpha, delta, rho, scale;
   int causal;
-  int reserve_sms;       // SMs left free for kernels running beside the (persistent) score kernel
-  int32_t* order_scratch; // nullable: n_layers*batch*Hkv ints; ragged batches then run longest sequences first
+  // launched as a programmatic dependent of the kernel before it on the stream. 1: it waits for that kernel before it
+  // touches memory. 2: that kernel let its dependents start after everything before it was complete, and the score kernel
+  // does not read what it writes: it runs beside it and waits for it only at its own end (so that what follows the score
+  // kernel follows both).
+  int pdl;
+  int32_t* order_scratch; // nullable: n_layers*batch*Hkv ints; large ragged batches then run longest sequences first
 };
-cudaError_t ta_launch_score(ta_ctx* ctx, const ta_score_args& a, ta_dev_status* status, cudaStream_t stream);
+// launches (nullable) is increased by the number of kernels enqueued
+cudaError_t ta_launch_score(ta_ctx* ctx, const ta_score_args& a, ta_dev_status* status, cudaStream_t stream,
+                            int* launches = nullptr);
 
 // diagnostic: one warp runs into the limit of a bounded wait (TA_ERR_TIMEOUT in `status`); *outcome gets bit 2 set when
 // the kernel ran to its end, bits 0/1 when a wait unexpectedly succeeded
@@ -182,6 +197,13 @@ struct ta_select_args {
   float beta, gamma, lambda;
 };
 bool ta_select_gathers(const ta_select_args& a);  // whether ta_launch_select_units will do the gather itself
+// Steps 1 and the per-sequence part of 3 in one kernel for sequences that fit one block (ta_front.cu): static utilities, forced
+// set and r_main as ta_launch_mask and ta_launch_forced leave them (without flags and vouchers); fast mode: idx and count
+// per sequence, and nothing else. hist is used only for vocabularies that do not fit in shared memory; needs no clearing.
+// The kernel lets its programmatic dependent start as soon as it runs itself.
+bool ta_front_fits(const ta_seq_desc& seq);
+cudaError_t ta_launch_front(const ta_patterns* pats, const ta_policy& pol, const ta_select_args& a, const int32_t* ids,
+                            int32_t* hist /*[B][vocab]*/, ta_dev_status* status, cudaStream_t stream);
 cudaError_t ta_launch_select(const ta_select_args& a, ta_dev_status* status, cudaStream_t stream);  // both below
 cudaError_t ta_launch_forced(const ta_select_args& a, ta_dev_status* status, cudaStream_t stream);
 cudaError_t ta_launch_select_units(const ta_select_args& a, cudaStream_t stream);
@@ -225,6 +247,10 @@ struct ta_compact_args {
   ta_bf16_view k, v;
   const int32_t* idx;
   const int32_t* count;
+  // optional: idx and count hold one result per sequence ([B][K], [B]); every unit gathers its sequence's rows and its
+  // copy of the result is written to idx_out and count_out ([L][B][Hkv][K], [L][B][Hkv])
+  int32_t* idx_out;
+  int32_t* count_out;
   void* k_out;
   void* v_out;
   int pdl;  // launch as a programmatic dependent of the kernel before it on the stream

@@ -86,6 +86,7 @@ __global__ void __launch_bounds__(kTile) ta_mask_kernel(ta_seq_desc seq, const i
   __shared__ float s_w[TA_MAX_SPAN + 1];
   __shared__ SegMax s_warp[kTile / 32];
 
+  ta_launch_dependents();  // (launched behind a memset: everything before this kernel is complete)
   const int tid = threadIdx.x;
   const long long T0 = (long long)blockIdx.x * kTile;  // first packed token of the tile
   const long long ext0 = T0 - kHaloL;                  // packed token of s_id[0]

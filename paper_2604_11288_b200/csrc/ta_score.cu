@@ -59,7 +59,8 @@ constexpr int kTileN = 128;                       // keys per tile
 constexpr int kD = TA_HEAD_DIM;                   // 128
 constexpr int kHalfBytes = kTileN * 128;          // one 64-column half of a 128-row operand tile: 16 KB
 constexpr int kKTileBytes = 2 * kHalfBytes;       // 32 KB
-constexpr int kMaxCluster = 8;
+constexpr int kMaxCluster = 16;                   // more than 8 CTAs is a non-portable cluster size; sm_100 allows 16
+constexpr int kRankedSeqs = 256;                  // sequences of a ragged batch that the kernel itself sorts by length
 constexpr int kGroups = 3;                        // softmax warpgroups
 constexpr int kSoftWarps = kGroups * 4;
 constexpr int kThreads = (kGroups + 1) * 128;     // 512
@@ -96,6 +97,8 @@ struct ScoreParams {
   float alpha, delta;
   const float* lse_obs;
   const int32_t* order;  // nullable: the clusters walk units order[0], order[1], .. (longest sequences first)
+  int by_length;         // the same walk from lengths ranked in the kernel (batches of up to kRankedSeqs sequences)
+  int late_wait;         // wait for the kernel before this one at the end instead of at the start (ta_score_args::pdl 2)
   float* A;
   float* P;
   float* u;
@@ -136,6 +139,7 @@ struct alignas(1024) ScoreSmem {
   unsigned long long pfull[kRing], pfree[kRing];
   uint32_t tmem_base;
   int abort_flag;
+  uint16_t by_rank[kRankedSeqs];           // by_length: sequence of every rank, longest first
 };
 
 // ---------------------------------------------------------------------------------------------- exponentials
@@ -240,13 +244,19 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
     } else {
       u = round * n_clusters + cluster_id;
       ui.end = round * n_clusters >= p.units;
-      if (p.order && (round & 1)) u = round * n_clusters + (n_clusters - 1 - cluster_id);
+      if ((p.order || p.by_length) && (round & 1)) u = round * n_clusters + (n_clusters - 1 - cluster_id);
     }
     if (ui.end || u >= p.units) return false;
     if (p.order) u = p.order[u];
     ui.g = u % p.Hkv;
-    ui.b = (u / p.Hkv) % p.seq.batch;
-    ui.l = u / (p.Hkv * p.seq.batch);
+    if (p.by_length) {  // every sequence's units together: rank, then layer, then head
+      const int per = p.n_layers * p.Hkv;
+      ui.b = sm.by_rank[u / per];
+      ui.l = (u % per) / p.Hkv;
+    } else {
+      ui.b = (u / p.Hkv) % p.seq.batch;
+      ui.l = u / (p.Hkv * p.seq.batch);
+    }
     ui.tok0 = ta_seq_begin(p.seq, ui.b);
     ui.n = (p.seq.cu ? p.seq.cu[ui.b + 1] : ui.tok0 + p.seq.n_uniform) - ui.tok0;
     // a sequence that does not lie inside the token arrays is skipped here and rejected by the selection step
@@ -301,6 +311,20 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
   if (warp == kWarpMma) {
     tmem_alloc(smem_u32(&sm.tmem_base), kTmemCols);
     tmem_relinquish();
+  }
+  if (!p.late_wait) ta_wait_for_prior_grid();  // nothing above reads what an earlier kernel wrote, but for the status word
+  if (p.by_length) {
+    // Longest first, equal lengths in sequence order. In unit order the lengths a cluster meets are random and the busiest
+    // cluster of a batch with lengths spread 8x carries about 30 % more than the average.
+    for (int b = tid; b < p.seq.batch; b += kThreads) {
+      const int nb = p.seq.cu[b + 1] - p.seq.cu[b];
+      int rank = 0;
+      for (int o = 0; o < p.seq.batch; ++o) {
+        const int no = p.seq.cu[o + 1] - p.seq.cu[o];
+        rank += (no > nb) || (no == nb && o < b);
+      }
+      sm.by_rank[rank] = (uint16_t)b;
+    }
   }
   // per-row tables: row r = h*W + t
   for (int r = tid; r < kRowsPad; r += kThreads) {
@@ -518,21 +542,15 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
             mbar_wait_cluster(smem_u32(&sm.xchg_full[up]), ph, abort_flag, p.status, 32, limit);
 #pragma unroll 1
             for (int r = r0; r < kRowsPad; r += 32 * kStatWarps) {
-              float pm[kMaxCluster], pz[kMaxCluster];
+              float pm[kMaxCluster], m = -1e30f, z = 0.0f;
 #pragma unroll
               for (int q = 0; q < kMaxCluster; ++q) {
-                pm[q] = -1e30f;
-                pz[q] = 0.0f;
-                if (q < p.cluster) {
-                  pm[q] = ld_cluster_f32(smem_u32(&sm.mine_m[up][r]), (uint32_t)q);
-                  pz[q] = ld_cluster_f32(smem_u32(&sm.mine_z[up][r]), (uint32_t)q);
-                }
+                pm[q] = q < p.cluster ? ld_cluster_f32(smem_u32(&sm.mine_m[up][r]), (uint32_t)q) : -1e30f;
+                m = fmaxf(m, pm[q]);
               }
-              float m = pm[0], z = 0.0f;
 #pragma unroll
-              for (int q = 1; q < kMaxCluster; ++q) m = fmaxf(m, pm[q]);
-#pragma unroll
-              for (int q = 0; q < kMaxCluster; ++q) z += pz[q] * ex2(pm[q] - m);
+              for (int q = 0; q < kMaxCluster; ++q)
+                if (q < p.cluster) z += ld_cluster_f32(smem_u32(&sm.mine_z[up][r]), (uint32_t)q) * ex2(pm[q] - m);
               put(r, z > 0.0f ? m + __log2f(z) : INFINITY);
             }
           }
@@ -881,6 +899,7 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
   // no CTA may leave while a peer can still store into its shared memory or arrive on its barriers
   cluster_arrive();
   cluster_wait();
+  if (p.late_wait && blockIdx.x == 0) ta_wait_for_prior_grid();  // this grid ends after the one it ran beside
 }
 
 template <int MB>
@@ -909,7 +928,7 @@ CUresult encode_5d(void* fn, CUtensorMap* map, const void* base, const uint64_t 
 
 template <int MB, int PM>
 cudaError_t launch_variant(ta_ctx* ctx, const CUtensorMap& mq, const CUtensorMap& mk, ScoreParams& sp,
-                           int tiles_max, int reserve_sms, cudaStream_t stream) {
+                           int tiles_max, int pdl, cudaStream_t stream) {
   auto kern = ta_score_kernel<MB, PM>;
   const size_t smem = score_smem_bytes<MB>();
   // per context (and so per device) and instantiation: the attribute is sticky, the occupancy does not change
@@ -917,6 +936,7 @@ cudaError_t launch_variant(ta_ctx* ctx, const CUtensorMap& mq, const CUtensorMap
   int* max_clusters = ctx->score_max_clusters[vi];
   if (!ctx->score_attr_set[vi]) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
     // the in-kernel register split must fit in what the launch provides, or the warps asking for more wait forever
     cudaFuncAttributes fa;
@@ -930,7 +950,7 @@ cudaError_t launch_variant(ta_ctx* ctx, const CUtensorMap& mq, const CUtensorMap
   cfg.blockDim = dim3(kThreads, 1, 1);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = (unsigned)sp.cluster;
   attr[0].val.clusterDim.y = 1;
@@ -946,6 +966,7 @@ cudaError_t launch_variant(ta_ctx* ctx, const CUtensorMap& mq, const CUtensorMap
   for (int cl = 1; cl <= kMaxCluster; cl *= 2) {
     if (ctx->score_force_cluster > 0 && cl != ctx->score_force_cluster) continue;
     if (cl > 1 && tiles_max < 2 * cl && ctx->score_force_cluster <= 0) break;
+    if (cl > 8 && sp.units > max_clusters[8]) break;  // only for a single round of few units
     if (max_clusters[cl] == 0) {
       attr[0].val.clusterDim.x = (unsigned)cl;
       cfg.gridDim = dim3((unsigned)(ctx->sm_count / cl * cl), 1, 1);
@@ -959,7 +980,7 @@ cudaError_t launch_variant(ta_ctx* ctx, const CUtensorMap& mq, const CUtensorMap
       continue;
     }
     if (ctx->score_force_cluster > 0) break;
-    const int avail = max_clusters[cl] - (reserve_sms + cl - 1) / cl > 0 ? max_clusters[cl] - (reserve_sms + cl - 1) / cl : 1;
+    const int avail = max_clusters[cl];
     const long long rounds = (sp.units + avail - 1) / avail;
     const long long per_cta = (tiles_max + cl - 1) / cl;
     const long long cost = rounds * (per_cta + (cl > 1 ? 3 : 1));
@@ -976,19 +997,17 @@ cudaError_t launch_variant(ta_ctx* ctx, const CUtensorMap& mq, const CUtensorMap
   if (best_cost < 0) return cudaErrorLaunchOutOfResources;
   sp.cluster = best_cl;
   attr[0].val.clusterDim.x = (unsigned)best_cl;
-  int n_clusters = max_clusters[best_cl] - (reserve_sms + best_cl - 1) / best_cl;
-  if (n_clusters < 1) n_clusters = 1;
+  int n_clusters = max_clusters[best_cl];
   const long long pieces = sp.flat ? (long long)sp.units * tiles_max : sp.units;
   if (n_clusters > pieces) n_clusters = (int)pieces;
   ctx->score_cluster = sp.cluster;
   ctx->score_clusters = n_clusters;
   cfg.gridDim = dim3((unsigned)(n_clusters * sp.cluster), 1, 1);
+  if (pdl) ta_pdl_attribute(&attr[cfg.numAttrs++]);
   return cudaLaunchKernelEx(&cfg, kern, mq, mk, sp);
 }
 
-// Ragged batches: units in descending order of sequence length (ties: lower sequence first). Walking this list
-// round-robin gives every cluster a similar number of key tiles; in unit order the lengths a cluster meets are
-// random and the busiest cluster of a batch with lengths spread 8x carries about 30 % more than the average.
+// Ragged batches of more than kRankedSeqs sequences: the order of the units, longest sequences first.
 __global__ void ta_unit_order_kernel(ta_seq_desc seq, int n_layers, int Hkv, int32_t* __restrict__ order) {
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b >= seq.batch) return;
@@ -1036,7 +1055,8 @@ cudaError_t ta_launch_wait_selftest(ta_dev_status* status, unsigned long long li
 // A stride that multiplies a coordinate which is always 0 still has to be a valid tensor-map stride.
 static uint64_t safe_stride(int64_t s, uint64_t dim) { return (dim <= 1 || s <= 0) ? 128 : (uint64_t)s; }
 
-cudaError_t ta_launch_score(ta_ctx* ctx, const ta_score_args& a, ta_dev_status* status, cudaStream_t stream) {
+cudaError_t ta_launch_score(ta_ctx* ctx, const ta_score_args& a, ta_dev_status* status, cudaStream_t stream,
+                            int* launches) {
   const int B = a.seq.batch, L = a.n_layers;
   const int units = L * B * a.Hkv;
   if (units == 0 || a.seq.total == 0) return cudaSuccess;
@@ -1068,12 +1088,17 @@ cudaError_t ta_launch_score(ta_ctx* ctx, const ta_score_args& a, ta_dev_status* 
   for (int t = 0; t < a.W; ++t) sp.wrow[t] = (float)((1.0 - (double)a.rho) * pow((double)a.rho, (double)(a.W - 1 - t)));
   sp.units = units;
   sp.order = nullptr;
-  if (a.seq.cu && a.order_scratch && B > 1) {
+  sp.late_wait = a.pdl == 2;
+  sp.by_length = a.seq.cu && B > 1 && B <= kRankedSeqs;
+  if (a.seq.cu && a.order_scratch && B > kRankedSeqs) {
     ta_unit_order_kernel<<<(B + 127) / 128, 128, 0, stream>>>(a.seq, L, a.Hkv, a.order_scratch);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     sp.order = a.order_scratch;
+    if (launches) ++*launches;
+    sp.late_wait = 0;  // the order comes from the kernel before this one (which itself follows all before it)
   }
+  if (launches) ++*launches;
   const int tiles_max = (a.seq.max_n + kTileN - 1) / kTileN;
   sp.cluster = 1;  // chosen at launch
 
@@ -1102,11 +1127,11 @@ cudaError_t ta_launch_score(ta_ctx* ctx, const ta_score_args& a, ta_dev_status* 
   for (int t = 0; fused && t < a.W; ++t) fused = a.alpha + a.delta * sp.wrow[t] > 0.0f;
   const bool need_p = a.P != nullptr || (a.u != nullptr && a.delta != 0.0f);
   if (MB == 1) {
-    if (fused) return launch_variant<1, kOutFused>(ctx, mq, mk, sp, tiles_max, a.reserve_sms, stream);
-    if (need_p) return launch_variant<1, kOutAP>(ctx, mq, mk, sp, tiles_max, a.reserve_sms, stream);
-    return launch_variant<1, kOutA>(ctx, mq, mk, sp, tiles_max, a.reserve_sms, stream);
+    if (fused) return launch_variant<1, kOutFused>(ctx, mq, mk, sp, tiles_max, a.pdl, stream);
+    if (need_p) return launch_variant<1, kOutAP>(ctx, mq, mk, sp, tiles_max, a.pdl, stream);
+    return launch_variant<1, kOutA>(ctx, mq, mk, sp, tiles_max, a.pdl, stream);
   }
-  if (fused) return launch_variant<2, kOutFused>(ctx, mq, mk, sp, tiles_max, a.reserve_sms, stream);
-  if (need_p) return launch_variant<2, kOutAP>(ctx, mq, mk, sp, tiles_max, a.reserve_sms, stream);
-  return launch_variant<2, kOutA>(ctx, mq, mk, sp, tiles_max, a.reserve_sms, stream);
+  if (fused) return launch_variant<2, kOutFused>(ctx, mq, mk, sp, tiles_max, a.pdl, stream);
+  if (need_p) return launch_variant<2, kOutAP>(ctx, mq, mk, sp, tiles_max, a.pdl, stream);
+  return launch_variant<2, kOutA>(ctx, mq, mk, sp, tiles_max, a.pdl, stream);
 }

@@ -20,9 +20,11 @@ struct SelectResult {
   int ties;         // how many elements equal to thresh are taken (lowest positions first)
   int all;          // 1: every eligible element is taken (fewer eligible than requested)
   int none;         // 1: nothing is taken
+  int all_ties;     // 1: every eligible element equal to thresh is taken (0: not known)
 };
 
 constexpr int kCandCap = 2048;  // candidates a split unit finishes locally
+constexpr int kCompareCap = 256;  // so few candidates are compared with one another instead of counted by digits
 
 struct SelectShared {
   uint32_t hist[256];
@@ -47,7 +49,9 @@ struct SelectShared {
   // a unit split over a cluster: once few candidates are left, their keys are collected (on rank 0, then copied by
   // every CTA) and the remaining passes run on that list inside each CTA, without cluster barriers
   uint32_t cand_n;
-  uint32_t cand_keys[kCandCap];
+  __align__(16) uint32_t cand_keys[kCandCap];
+  uint32_t cmp_n, cmp_thresh;  // the same inside one CTA, for at most kCompareCap candidates
+  int cmp_above, cmp_equal;
 };
 constexpr int kSelectCluster = 8;  // CTAs per unit when a sequence is longer than kItems * kThreads
 
@@ -115,6 +119,7 @@ __device__ SelectResult block_radix_select(int n, int want, KeyFn key_of, const 
   r.thresh = 0;
   r.ties = 0;
   r.all = 0;
+  r.all_ties = 0;
   r.none = (want <= 0);
   if (r.none) return r;
   const int tid = threadIdx.x, lane = tid & 31;
@@ -304,13 +309,42 @@ __device__ __forceinline__ void list_radix_finish(int m, int bits, int done, uin
   }
 }
 
+// The `remaining`-th largest of the m <= kCompareCap keys in sh.cand_keys, by comparing every key with every other: three
+// block barriers in place of three for every digit still to resolve (an 8-bit digit leaves about n / 256 candidates, and
+// two more digits would follow). Returns the key; above / equal: how many keys are larger than it / equal to it.
+__device__ __forceinline__ uint32_t compare_finish(int m, int remaining, int& above, int& equal, SelectShared& sh) {
+  const int tid = threadIdx.x;
+  if (tid < kCompareCap && tid >= m && tid < (m + 3) / 4 * 4) sh.cand_keys[tid] = 0u;  // below or equal to any key: see below
+  __syncthreads();
+  if (tid < m) {
+    const uint32_t mine = sh.cand_keys[tid];
+    int gt = 0, ge = 0;
+    const uint4* keys = reinterpret_cast<const uint4*>(sh.cand_keys);
+    for (int j = 0; j < (m + 3) / 4; ++j) {
+      const uint4 k = keys[j];
+      gt += (k.x > mine) + (k.y > mine) + (k.z > mine) + (k.w > mine);
+      ge += (k.x >= mine) + (k.y >= mine) + (k.z >= mine) + (k.w >= mine);
+    }
+    if (mine == 0u) ge = m;  // the padding keys are equal to a key of zero
+    if (gt < remaining && remaining <= ge) {  // every thread that holds the key writes the same
+      sh.cmp_thresh = mine;
+      sh.cmp_above = gt;
+      sh.cmp_equal = ge - gt;
+    }
+  }
+  __syncthreads();
+  above = sh.cmp_above;
+  equal = sh.cmp_equal;
+  return sh.cmp_thresh;
+}
+
 // Top-`want` of the eligible elements when the keys sit in registers. The eligible keys' range is taken first: the
 // bits above the highest bit in which two of them differ are common to all and need no pass, so the first 8-bit
 // digit already spreads the keys over the whole histogram (utilities of one unit span a few binades: the top byte of
 // a float alone would put most of them into two or three bins). The first pass counts every eligible element
 // (match.any merges equal digits of a warp into one shared-memory atomic); from then on each thread keeps a bit mask
 // of its elements that are still candidates, and the passes touch those only. The passes stop as soon as the
-// candidates left are exactly as many as are still to take. n_unit is the length of the whole unit (n is this CTA's
+// candidates left are exactly as many as are still to take, or so few that they are compared with one another. n_unit is the length of the whole unit (n is this CTA's
 // slice when CL > 1).
 template <int CL, int ITEMS>
 __device__ SelectResult cached_radix_select(int n, int n_unit, int want, const KeyCache<ITEMS>& kc, SelectShared& sh) {
@@ -318,6 +352,7 @@ __device__ SelectResult cached_radix_select(int n, int n_unit, int want, const K
   r.thresh = 0;
   r.ties = 0;
   r.all = 0;
+  r.all_ties = 0;
   r.none = (want <= 0);
   // the cluster barrier that split_unit_begin() arrived at before the keys were loaded: from here on every CTA of the
   // cluster is known to run (its shared memory may be written) and to have zeroed its ghist and cand_n
@@ -342,7 +377,10 @@ __device__ SelectResult cached_radix_select(int n, int n_unit, int want, const K
     sh.wmax[warp] = kmax;
     sh.wnum[warp] = num;
   }
-  if (tid == 0) sh.remaining = want;
+  if (tid == 0) {
+    sh.remaining = want;
+    sh.cmp_n = 0;
+  }
   __syncthreads();
   static_assert(kWarps <= 32, "one lane per warp in the second reduction step");
   kmin = __reduce_min_sync(0xffffffffu, lane < kWarps ? sh.wmin[lane] : 0xffffffffu);
@@ -378,6 +416,7 @@ __device__ SelectResult cached_radix_select(int n, int n_unit, int want, const K
   if (diff == 0u) {  // all eligible keys are equal
     r.thresh = kmin;
     r.ties = want;
+    r.all_ties = num == (uint32_t)want;
     return r;
   }
   const int bits = 32 - __clz(diff);  // low bits still to resolve
@@ -387,6 +426,26 @@ __device__ SelectResult cached_radix_select(int n, int n_unit, int want, const K
   int ncand = (int)num;
   int done = 0, pass = 0;
   while (done < bits) {
+    if (CL == 1 && ncand <= kCompareCap) {
+      uint32_t mine = 0;
+      if (cand != 0u) {
+#pragma unroll
+        for (int it = 0; it < ITEMS; ++it)
+          if (((cand >> it) & 1u) && (kc.key[it] & mask) == prefix) mine |= 1u << it;
+      }
+      if (mine != 0u) {
+        uint32_t slot = atomicAdd(&sh.cmp_n, (uint32_t)__popc(mine));
+#pragma unroll
+        for (int it = 0; it < ITEMS; ++it)
+          if ((mine >> it) & 1u) sh.cand_keys[slot++] = kc.key[it];
+      }
+      __syncthreads();
+      int above, equal;
+      r.thresh = compare_finish(ncand, remaining, above, equal, sh);
+      r.ties = remaining - above;
+      r.all_ties = r.ties == equal;
+      return r;
+    }
     if (CL > 1 && ncand <= kCandCap) {
       // Few candidates left (uniform over the cluster: ncand comes from the merged histogram, or is the number of
       // eligible elements before the first pass). Every CTA appends its own to the list on rank 0; after one cluster
@@ -477,7 +536,10 @@ __device__ SelectResult cached_radix_select(int n, int n_unit, int want, const K
     ncand = sh.ncand;
     done += width;
     ++pass;
-    if (ncand == remaining) break;  // every candidate left is taken: the low bits need no pass
+    if (ncand == remaining) {  // every candidate left is taken: the low bits need no pass
+      r.all_ties = 1;
+      break;
+    }
   }
   r.thresh = prefix;  // with the unresolved low bits zero: candidates above it are definite, equal ones are ties
   r.ties = remaining;
@@ -551,8 +613,8 @@ __device__ __forceinline__ uint32_t warp_transpose32(uint32_t x, int lane) {
 // them into what 32 ballots would give) and leaves two bitmaps in shared memory, definite and tie, in position
 // order: the bits of warp w in chunk it are word it*kWarps + w and cover positions 32 * word .. + 31.
 // From there on thread j owns word j: a block-wide exclusive scan over the words' populations gives it the number
-// of definite and of tie elements before its 32 positions, and it writes its taken positions itself (two per word on
-// average) -- no key is needed for that. Three block barriers (and one cluster barrier for the totals of the lower
+// of definite and of tie elements before its 32 positions, and the taken positions are written from the words alone
+// (no key is needed for that). Three block barriers (and one cluster barrier for the totals of the lower
 // ranks). emit may run on another thread than the one that holds the element's key.
 template <int CL, class EmitFn, int ITEMS>
 __device__ int cached_ordered_emit(int n, const SelectResult& r, const KeyCache<ITEMS>& kc, uint32_t always,
@@ -604,13 +666,9 @@ __device__ int cached_ordered_emit(int n, const SelectResult& r, const KeyCache<
   const uint32_t warp_total = __shfl_sync(0xffffffffu, run, 31);
   if (lane == 0) sh.wtot[warp] = warp_total;
   __syncthreads();
-  uint32_t before = 0, all = 0;
-#pragma unroll
-  for (int w = 0; w < kWarps; ++w) {
-    const uint32_t t = sh.wtot[w];
-    if (w < warp) before += t;
-    all += t;
-  }
+  const uint32_t wt_l = lane < kWarps ? sh.wtot[lane] : 0u;  // (no carry between the halves: at most 32768 elements)
+  const uint32_t before = __reduce_add_sync(0xffffffffu, lane < warp ? wt_l : 0u);
+  const uint32_t all = __reduce_add_sync(0xffffffffu, wt_l);
   const uint32_t ex = before + run - mine;
   int def_base = 0, tie_base = 0;
   int def_all = (int)(all & 0xffffu), tie_all = (int)(all >> 16);
@@ -638,16 +696,31 @@ __device__ int cached_ordered_emit(int n, const SelectResult& r, const KeyCache<
   int def_before = def_base + (int)(ex & 0xffffu);
   int ties_seen = tie_base + (int)(ex >> 16);
   uint32_t m = wd | wt;
-  while (m) {
-    const int bit = __ffs((int)m) - 1;
-    m &= m - 1u;
-    const int i = 32 * tid + bit;
-    if ((wd >> bit) & 1u) {
-      emit(i, def_before + min(ties_seen, ties_allowed));
-      ++def_before;
-    } else {
-      if (ties_seen < ties_allowed) emit(i, def_before + ties_seen);
-      ++ties_seen;
+  // Sparse words: every thread walks its own word. Dense ones (recency makes runs of neighbours win together, so that a few
+  // words hold most of what is taken): the warp takes its words one after the other, a lane per position.
+  const unsigned nonempty = __ballot_sync(0xffffffffu, m != 0u);
+  const int most = (int)__reduce_max_sync(0xffffffffu, (uint32_t)__popc(m));
+  if (2 * most > 3 * __popc(nonempty)) {
+    const unsigned lt = (1u << lane) - 1u;
+    for (unsigned left = nonempty; left != 0u; left &= left - 1u) {
+      const int src = __ffs((int)left) - 1;
+      const uint32_t d = __shfl_sync(0xffffffffu, wd, src), t = __shfl_sync(0xffffffffu, wt, src);
+      const int seen = __shfl_sync(0xffffffffu, ties_seen, src) + __popc(t & lt);
+      const int rank = __shfl_sync(0xffffffffu, def_before, src) + __popc(d & lt) + min(seen, ties_allowed);
+      if (((d >> lane) & 1u) || (((t >> lane) & 1u) && seen < ties_allowed)) emit(32 * (tid - lane + src) + lane, rank);
+    }
+  } else {
+    while (m) {
+      const int bit = __ffs((int)m) - 1;
+      m &= m - 1u;
+      const int i = 32 * tid + bit;
+      if ((wd >> bit) & 1u) {
+        emit(i, def_before + min(ties_seen, ties_allowed));
+        ++def_before;
+      } else {
+        if (ties_seen < ties_allowed) emit(i, def_before + ties_seen);
+        ++ties_seen;
+      }
     }
   }
   return def_all + min(tie_all, ties_allowed);
@@ -732,6 +805,7 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads) ta_forced_kernel(ta
                                                              int32_t* __restrict__ r_main, ta_dev_status* status,
                                                              const int32_t* __restrict__ class_K, ta_static_out so) {
   __shared__ SelectShared sh;
+  ta_launch_dependents();  // its dependent does not start before every block of the kernel before it runs
   ta_wait_for_prior_grid();
   // grid.x = classes * sequences * CL; without budget classes there is one class and K is the argument
   const int b = (blockIdx.x / CL) % seq.batch;
