@@ -136,3 +136,13 @@ def test_stream_budget_larger_than_a_block():
 def test_stream_no_patterns_tiny_budget():
     pol = oracle.preset("SEC33", 1, vocab_size=64)
     _run(K=1, L=1, B=3, Hkv=1, steps=12, pats=oracle.Patterns([]), pol=pol, seed=3)
+
+
+@pytest.mark.parametrize("K,preset,steps", [(31, "SEC33", 200), (64, "SEC33", 260), (63, "THEOREM", 260),
+                                            (1025, "SEC33", 1060), (2049, "SEC33", 2070)])
+def test_stream_more_sponsored_tokens_than_protected_slots(K, preset, steps):
+    # anchors every few tokens: most cached tokens are sponsored, many with equal vouchers; two, four and eight cached
+    # tokens per thread
+    pats = oracle.Patterns([[5], [6, 7]], budget=[15.0, 2.0], span=[3, 8])
+    pol = oracle.preset(preset, K, vocab_size=64, budget_decay=1.0 if K < 64 else 0.9)
+    _run(K=K, L=1, B=1, Hkv=2 if K < 100 else 1, steps=steps, pats=pats, pol=pol, seed=K, check_every=97)
