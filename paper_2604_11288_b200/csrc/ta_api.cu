@@ -772,7 +772,7 @@ ta_status compress_impl(ta_ctx* ctx, const ta_patterns* pats, const ta_policy* p
       if (e == cudaSuccess)
         e = ta_launch_mask(pats, *policy, seq, token_ids, flags, voucher, nullptr, hist, ctx->d_status, stream);
       if (e == cudaSuccess) e = ta_launch_forced(sel, ctx->d_status, stream);
-      launches += 2;  // mask, forced set (which also writes the static utilities)
+      launches += 3;  // cleared histogram, mask, forced set (which also writes the static utilities)
       if (e == cudaSuccess && fast) {
         e = ta_launch_select_units(sel, stream);
         launches += 1;

@@ -28,8 +28,7 @@ __device__ __forceinline__ void st_stream(uint4* p, uint4 v) {
 
 // grid.x = units (l, b, g), grid.y = ceil(K / 64) row blocks, grid.z = 2 (K cache, V cache)
 __global__ void __launch_bounds__(kThreads) ta_compact_kernel(ta_seq_desc seq, int Hkv, int K, ta_bf16_view kv0,
-                                                              ta_bf16_view kv1, const int32_t* __restrict__ idx,
-                                                              const int32_t* __restrict__ count,
+                                                              ta_bf16_view kv1, const int32_t* idx, const int32_t* count,
                                                               int32_t* __restrict__ idx_out,
                                                               int32_t* __restrict__ count_out,
                                                               uint4* __restrict__ out0, uint4* __restrict__ out1) {

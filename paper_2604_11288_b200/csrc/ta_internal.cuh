@@ -75,7 +75,9 @@ __host__ __device__ inline int ta_seq_begin(const ta_seq_desc& s, int b, const i
 
 // Programmatic dependent launch: a kernel launched with ta_pdl_attribute() may be scheduled while the kernel before it
 // on the stream is still draining (its launch latency overlaps that kernel's tail); it must call
-// ta_wait_for_prior_grid() before its first access to memory. The call returns at once in a kernel launched normally.
+// ta_wait_for_prior_grid() before its first access to memory. The call returns at once in a kernel launched normally. What
+// the kernel before it wrote must not be read through a const __restrict__ pointer: such loads count as invariant, and the
+// compiler may move them above the wait.
 inline void ta_pdl_attribute(cudaLaunchAttribute* attr) {
   attr->id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr->val.programmaticStreamSerializationAllowed = 1;
@@ -208,8 +210,7 @@ cudaError_t ta_launch_select(const ta_select_args& a, ta_dev_status* status, cud
 cudaError_t ta_launch_forced(const ta_select_args& a, ta_dev_status* status, cudaStream_t stream);
 cudaError_t ta_launch_select_units(const ta_select_args& a, cudaStream_t stream);
 cudaError_t ta_launch_broadcast_idx(int B, int Hkv, int K, int n_layers, const int32_t* idx_seq,
-                                    const int32_t* count_seq, int32_t* idx, int32_t* count, cudaStream_t stream,
-                                    bool pdl = false);
+                                    const int32_t* count_seq, int32_t* idx, int32_t* count, cudaStream_t stream);
 
 // selection shared by the KV heads of a layer: head sum of the utilities, copy of the result to every head
 cudaError_t ta_launch_headsum(int n_layers, int Hkv, long long total, const float* u, float* u_all,

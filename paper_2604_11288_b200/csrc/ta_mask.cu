@@ -27,7 +27,7 @@ __device__ __forceinline__ uint32_t bloom_hash(int32_t x) { return ((uint32_t)x 
 
 // sequence index of packed token `tok`
 __device__ __forceinline__ int seq_of(const ta_seq_desc& s, long long tok) {
-  if (!s.cu) return (int)(tok / s.n_uniform);
+  if (!s.cu) return (int)((uint32_t)tok / (uint32_t)s.n_uniform);  // (fewer than 2^31 tokens in all)
   int lo = 0, hi = s.batch;  // cu[lo] <= tok < cu[hi]
   while (hi - lo > 1) {
     const int mid = (lo + hi) >> 1;
@@ -42,6 +42,15 @@ __device__ __forceinline__ void report(ta_dev_status* st, int code, int where, i
     st->detail0 = d0;
     st->detail1 = d1;
   }
+}
+
+// hist = 0. A kernel and not a memset: it can be launched as a programmatic dependent and let its own dependent start.
+__global__ void __launch_bounds__(256) ta_clear_kernel(int32_t* __restrict__ hist, long long n) {
+  ta_wait_for_prior_grid();
+  ta_launch_dependents();
+  const long long step = (long long)gridDim.x * blockDim.x, i0 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  for (long long i = i0; i < n / 4; i += step) reinterpret_cast<int4*>(hist)[i] = make_int4(0, 0, 0, 0);
+  for (long long i = n / 4 * 4 + i0; i < n; i += step) hist[i] = 0;
 }
 
 struct ConfAnchors {   // anchors from a detector's confidences; conf == nullptr: token-id patterns are matched
@@ -86,7 +95,6 @@ __global__ void __launch_bounds__(kTile) ta_mask_kernel(ta_seq_desc seq, const i
   __shared__ float s_w[TA_MAX_SPAN + 1];
   __shared__ SegMax s_warp[kTile / 32];
 
-  ta_launch_dependents();  // (launched behind a memset: everything before this kernel is complete)
   const int tid = threadIdx.x;
   const long long T0 = (long long)blockIdx.x * kTile;  // first packed token of the tile
   const long long ext0 = T0 - kHaloL;                  // packed token of s_id[0]
@@ -127,6 +135,10 @@ __global__ void __launch_bounds__(kTile) ta_mask_kernel(ta_seq_desc seq, const i
     s_w[tid] = w;
   }
 
+  // Launched as a programmatic dependent of the kernel that clears the histogram, which lets this one start when everything
+  // before it is complete: only what follows needs the counters at zero.
+  ta_wait_for_prior_grid();
+  ta_launch_dependents();
   // phase a: ids + sequence starts for tile and halo; histogram for the tile proper
   for (int i = tid; i < kExt; i += kTile) {
     const long long tok = ext0 + i;
@@ -318,9 +330,8 @@ __global__ void __launch_bounds__(kTile) ta_mask_kernel(ta_seq_desc seq, const i
 
 // u_static = ((beta*R + gamma*S) - lambda*F) + V, R = (i0+1)/n, F = count(id)/n  (Eq. 3), one rounding per operation.
 __global__ void __launch_bounds__(256) ta_ustatic_kernel(ta_seq_desc seq, const int32_t* __restrict__ ids,
-                                                         const uint8_t* __restrict__ flags,
-                                                         const float* __restrict__ voucher,
-                                                         const int32_t* __restrict__ hist, int vocab, float beta,
+                                                         const uint8_t* flags, const float* voucher,
+                                                         const int32_t* hist, int vocab, float beta,
                                                          float gamma, float lambda, float* __restrict__ u_static) {
   ta_wait_for_prior_grid();  // launched as a programmatic dependent of the mask kernel
   const long long tok = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -337,51 +348,54 @@ __global__ void __launch_bounds__(256) ta_ustatic_kernel(ta_seq_desc seq, const 
 }  // namespace
 
 namespace {
-cudaError_t finish_static_utility(const ta_policy& pol, const ta_seq_desc& seq, const int32_t* ids, const uint8_t* flags,
-                                  const float* voucher, const int32_t* hist, float* u_static, cudaStream_t stream) {
-  if (!u_static) return cudaSuccess;  // left to the forced-set kernel
-  const int blocks = (int)((seq.total + 255) / 256);
+template <class Kern, class... Args>
+cudaError_t launch_dependent(Kern kern, long long blocks, int threads, cudaStream_t stream, Args... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)blocks, 1, 1);
-  cfg.blockDim = dim3(256, 1, 1);
+  cfg.blockDim = dim3((unsigned)threads, 1, 1);
   cfg.stream = stream;
   cudaLaunchAttribute attr[1];
-  ta_pdl_attribute(&attr[0]);  // always directly behind the mask kernel
+  ta_pdl_attribute(&attr[0]);
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, ta_ustatic_kernel, seq, ids, flags, voucher, hist, pol.vocab_size, pol.beta,
-                            pol.gamma, pol.lambda, u_static);
+  return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
+// clears the histogram, runs the mask kernel and (u_static given; otherwise it is left to the forced-set kernel) the
+// static-utility kernel
+cudaError_t launch_mask_chain(const ta_policy& pol, const ta_seq_desc& seq, const int32_t* ids, const ta_patterns& t,
+                              const ConfAnchors& ca, uint8_t* flags, float* voucher, float* u_static, int32_t* hist,
+                              ta_dev_status* status, cudaStream_t stream) {
+  if (seq.total == 0) return cudaSuccess;
+  const long long counters = (long long)seq.batch * pol.vocab_size;
+  const long long want = (counters / 4 + 255) / 256;
+  cudaError_t e = launch_dependent(ta_clear_kernel, want < 1 ? 1 : want > 1024 ? 1024 : want, 256, stream, hist, counters);
+  if (e != cudaSuccess) return e;
+  e = launch_dependent(ta_mask_kernel, (seq.total + kTile - 1) / kTile, kTile, stream, seq, ids, (const int32_t*)t.d_ids,
+                       (const int32_t*)t.d_len, (const float*)t.d_budget, (const int32_t*)t.d_span,
+                       (const uint32_t*)t.d_bloom, t.n_pat, t.max_len, t.max_span, pol.voucher_decay, pol.budget_decay,
+                       pol.age_steps, pol.vocab_size, flags, voucher, hist, status, ca);
+  if (e != cudaSuccess || !u_static) return e;
+  return launch_dependent(ta_ustatic_kernel, (seq.total + 255) / 256, 256, stream, seq, ids, (const uint8_t*)flags,
+                          (const float*)voucher, (const int32_t*)hist, pol.vocab_size, pol.beta, pol.gamma, pol.lambda,
+                          u_static);
 }
 }  // namespace
 
 cudaError_t ta_launch_mask_conf(const ta_policy& pol, const ta_seq_desc& seq, const int32_t* ids, const float* conf,
                                 float threshold, float budget, int span, int rank, uint8_t* flags, float* voucher,
                                 float* u_static, int32_t* hist, ta_dev_status* status, cudaStream_t stream) {
-  if (seq.total == 0) return cudaSuccess;
-  cudaError_t e = cudaMemsetAsync(hist, 0, (size_t)seq.batch * pol.vocab_size * sizeof(int32_t), stream);
-  if (e != cudaSuccess) return e;
-  const int tiles = (int)((seq.total + kTile - 1) / kTile);
-  ConfAnchors ca = {conf, threshold, budget, span, rank};
-  ta_mask_kernel<<<tiles, kTile, 0, stream>>>(seq, ids, nullptr, nullptr, nullptr, nullptr, nullptr, 1, 1, span,
-                                              pol.voucher_decay, pol.budget_decay, pol.age_steps, pol.vocab_size, flags,
-                                              voucher, hist, status, ca);
-  e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  return finish_static_utility(pol, seq, ids, flags, voucher, hist, u_static, stream);
+  ta_patterns one = {};  // one pseudo-pattern of length 1 stands for "the detector fired here"
+  one.n_pat = 1;
+  one.max_len = 1;
+  one.max_span = span;
+  return launch_mask_chain(pol, seq, ids, one, ConfAnchors{conf, threshold, budget, span, rank}, flags, voucher, u_static,
+                           hist, status, stream);
 }
 
 cudaError_t ta_launch_mask(const ta_patterns* pats, const ta_policy& pol, const ta_seq_desc& seq, const int32_t* ids,
                            uint8_t* flags, float* voucher, float* u_static, int32_t* hist, ta_dev_status* status,
                            cudaStream_t stream) {
-  if (seq.total == 0) return cudaSuccess;
-  cudaError_t e = cudaMemsetAsync(hist, 0, (size_t)seq.batch * pol.vocab_size * sizeof(int32_t), stream);
-  if (e != cudaSuccess) return e;
-  const int tiles = (int)((seq.total + kTile - 1) / kTile);
-  ta_mask_kernel<<<tiles, kTile, 0, stream>>>(seq, ids, pats->d_ids, pats->d_len, pats->d_budget, pats->d_span,
-                                              pats->d_bloom, pats->n_pat, pats->max_len, pats->max_span,
-                                              pol.voucher_decay, pol.budget_decay, pol.age_steps, pol.vocab_size, flags,
-                                              voucher, hist, status, ConfAnchors{nullptr, 0.0f, 0.0f, 0, 0});
-  e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  return finish_static_utility(pol, seq, ids, flags, voucher, hist, u_static, stream);
+  return launch_mask_chain(pol, seq, ids, *pats, ConfAnchors{nullptr, 0.0f, 0.0f, 0, 0}, flags, voucher, u_static, hist,
+                           status, stream);
 }

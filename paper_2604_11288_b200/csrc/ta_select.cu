@@ -40,7 +40,6 @@ using namespace sel512;  // the launchers below name the 512-thread kernels unle
 __global__ void ta_broadcast_idx_kernel(int B, int Hkv, int K, int n_layers, const int32_t* __restrict__ idx_seq,
                                         const int32_t* __restrict__ count_seq, int32_t* __restrict__ idx,
                                         int32_t* __restrict__ count) {
-  ta_wait_for_prior_grid();
   const long long total = (long long)n_layers * B * Hkv * K;
   for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < total;
        t += (long long)gridDim.x * blockDim.x) {
@@ -176,13 +175,19 @@ cudaError_t ta_launch_forced(const ta_select_args& a, ta_dev_status* status, cud
                           a.n_recent, a.k_protected, a.voucher, a.forced, a.r_main, status, ck, so);
 }
 
+// Few short units (at most one block per SM): a launch is then all latency, and blocks of 1024 threads with a quarter of the
+// keys per thread take less time than 512 (8 units of 4096 keys with the gather of 16 rows: 9.5 -> 7.1 us).
+bool few_short_units(const ta_select_args& a) {
+  return !a.fast && a.seq.max_n <= 8 * sel1024::kThreads && a.n_layers * a.seq.batch * a.Hkv <= sm_count_of(a);
+}
+
 bool ta_select_gathers(const ta_select_args& a) {
-  if (!a.gather_k_out || a.fast || a.K > kGatherMaxK) return false;
-  // The gather adds one dependent load chain (index -> row -> store, about 2 us) to every block, the separate kernel
-  // costs one launch (about 8 us for so few rows): fusing pays only while the blocks run in a few waves. Short units
-  // (keys in 16 registers: two blocks per SM) only.
-  const int units = a.n_layers * a.seq.batch * a.Hkv;
-  return a.seq.max_n <= kItems * kThreads && units <= 4 * sm_count_of(a);
+  if (!a.gather_k_out || a.fast || a.seq.max_n > kItems * kThreads) return false;
+  // The gather adds a dependent load chain (index -> row -> store, about 2 us) to every block, the separate kernel costs a
+  // launch and its tail (about 5 us for so few rows): fusing pays while the blocks run in a few waves and a block's rows
+  // are few rounds of its threads. Short units (keys in registers, more than one block per SM) only.
+  if (few_short_units(a)) return a.K <= 256;  // at most 8 pieces of 16 bytes per thread
+  return a.K <= 16 && a.n_layers * a.seq.batch * a.Hkv <= 4 * sm_count_of(a);
 }
 
 cudaError_t ta_launch_select_units(const ta_select_args& a, cudaStream_t stream_) {
@@ -199,20 +204,13 @@ cudaError_t ta_launch_select_units(const ta_select_args& a, cudaStream_t stream_
   const int32_t* co = a.n_classes > 0 ? a.class_of : nullptr;
   const int sms = sm_count_of(a);
   GatherDst gd = {};
-  if (ta_select_gathers(a)) {  // implies the first variant below
+  const bool gathers = ta_select_gathers(a);
+  if (gathers) {
     gd.k = a.gather_k;
     gd.v = a.gather_v;
     gd.k_out = reinterpret_cast<uint4*>(a.gather_k_out);
     gd.v_out = reinterpret_cast<uint4*>(a.gather_v_out);
-    return launch_clustered(ta_select_kernel<true, 1, kItems, true>, units, 1, stream, a.seq, a.n_layers, a.Hkv, a.K,
-                            a.fast, src, a.forced, a.r_main, a.idx, a.count, gd, co);
   }
-  if (a.seq.max_n <= kItems * kThreads)
-    return launch_clustered(ta_select_kernel<true, 1>, units, 1, stream, a.seq, a.n_layers, a.Hkv, a.K, a.fast, src,
-                            a.forced, a.r_main, a.idx, a.count, gd, co);
-  if (!split_units(units, a.seq.max_n, sms) && a.seq.max_n <= kItemsLong * kThreads)
-    return launch_clustered(ta_select_kernel<true, 1, kItemsLong>, units, 1, stream, a.seq, a.n_layers, a.Hkv, a.K, a.fast,
-                            src, a.forced, a.r_main, a.idx, a.count, gd, co);
   sel1024::UnitSrc src2;  // the same fields for the kernels built for 1024 threads
   src2.u = src.u;
   src2.A = src.A;
@@ -220,7 +218,23 @@ cudaError_t ta_launch_select_units(const ta_select_args& a, cudaStream_t stream_
   src2.u_static = src.u_static;
   src2.alpha = src.alpha;
   src2.delta = src.delta;
-  sel1024::GatherDst gd2 = {};
+  const sel1024::GatherDst gd2 = {gd.k, gd.v, gd.k_out, gd.v_out};
+  if (few_short_units(a)) {
+    auto kern = a.seq.max_n <= 4 * sel1024::kThreads
+                    ? (gathers ? sel1024::ta_select_kernel<true, 1, 4, true> : sel1024::ta_select_kernel<true, 1, 4, false>)
+                    : (gathers ? sel1024::ta_select_kernel<true, 1, 8, true> : sel1024::ta_select_kernel<true, 1, 8, false>);
+    return launch_threads(sel1024::kThreads, kern, units, 1, stream, a.seq, a.n_layers, a.Hkv, a.K, a.fast, src2, a.forced,
+                          a.r_main, a.idx, a.count, gd2, co);
+  }
+  if (gathers)  // implies the first variant below
+    return launch_clustered(ta_select_kernel<true, 1, kItems, true>, units, 1, stream, a.seq, a.n_layers, a.Hkv, a.K,
+                            a.fast, src, a.forced, a.r_main, a.idx, a.count, gd, co);
+  if (a.seq.max_n <= kItems * kThreads)
+    return launch_clustered(ta_select_kernel<true, 1>, units, 1, stream, a.seq, a.n_layers, a.Hkv, a.K, a.fast, src,
+                            a.forced, a.r_main, a.idx, a.count, gd, co);
+  if (!split_units(units, a.seq.max_n, sms) && a.seq.max_n <= kItemsLong * kThreads)
+    return launch_clustered(ta_select_kernel<true, 1, kItemsLong>, units, 1, stream, a.seq, a.n_layers, a.Hkv, a.K, a.fast,
+                            src, a.forced, a.r_main, a.idx, a.count, gd, co);
   if (!split_units(units, a.seq.max_n, sms) && a.seq.max_n <= sel1024::kItemsLong * sel1024::kThreads) {
     // many long units: blocks of 1024 threads hold a unit of up to 32768 keys in registers (read once instead of
     // once per radix pass and once more for the ordered write)
@@ -252,20 +266,12 @@ cudaError_t ta_launch_select(const ta_select_args& a, ta_dev_status* status, cud
 }
 
 cudaError_t ta_launch_broadcast_idx(int B, int Hkv, int K, int n_layers, const int32_t* idx_seq,
-                                    const int32_t* count_seq, int32_t* idx, int32_t* count, cudaStream_t stream,
-                                    bool pdl) {
+                                    const int32_t* count_seq, int32_t* idx, int32_t* count, cudaStream_t stream) {
   const long long total = (long long)n_layers * B * Hkv * K;
   if (total == 0) return cudaSuccess;
   const int blocks = (int)((total + 255) / 256 < 4096 ? (total + 255) / 256 : 4096);
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)blocks, 1, 1);
-  cfg.blockDim = dim3(256, 1, 1);
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  if (pdl) ta_pdl_attribute(&attr[0]);
-  cfg.attrs = attr;
-  cfg.numAttrs = pdl ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, ta_broadcast_idx_kernel, B, Hkv, K, n_layers, idx_seq, count_seq, idx, count);
+  ta_broadcast_idx_kernel<<<blocks, 256, 0, stream>>>(B, Hkv, K, n_layers, idx_seq, count_seq, idx, count);
+  return cudaGetLastError();
 }
 
 cudaError_t ta_launch_headsum(int n_layers, int Hkv, long long total, const float* u, float* u_all,

@@ -800,7 +800,7 @@ __device__ __forceinline__ SeqInfo seq_info(const ta_seq_desc& seq, int b, int K
 
 template <bool CACHED, int CL, int ITEMS = kItems>
 __global__ void __launch_bounds__(kThreads, 1024 / kThreads) ta_forced_kernel(ta_seq_desc seq, int K, int n_sink, int n_recent,
-                                                             int k_protected, const float* __restrict__ voucher,
+                                                             int k_protected, const float* voucher,
                                                              uint8_t* __restrict__ forced,
                                                              int32_t* __restrict__ r_main, ta_dev_status* status,
                                                              const int32_t* __restrict__ class_K, ta_static_out so) {
@@ -925,12 +925,12 @@ struct GatherDst {
   uint4* k_out;
   uint4* v_out;
 };
-constexpr int kGatherMaxK = 16;  // one 16-byte piece per thread
 
 __device__ __forceinline__ void gather_unit(const GatherDst& gd, const ta_seq_desc& seq, int unit, int l, int b, int g,
                                             int n, int K, const int32_t* out, int taken) {
   constexpr int kLanesPerRow = TA_HEAD_DIM * 2 / 16;
   __syncthreads();  // the unit's indices were written by other threads of this block
+#pragma unroll 4
   for (int t = threadIdx.x; t < K * 2 * kLanesPerRow; t += kThreads) {
     const int r = t / (2 * kLanesPerRow), which = (t / kLanesPerRow) & 1, lane16 = t % kLanesPerRow;
     const ta_bf16_view& src = which ? gd.v : gd.k;
@@ -951,12 +951,13 @@ __device__ __forceinline__ void gather_unit(const GatherDst& gd, const ta_seq_de
 // grid.x = units. scored: unit = (l*B + b)*Hkv + g; fast: unit = b.
 template <bool CACHED, int CL, int ITEMS = kItems, bool GATHER = false>
 __global__ void __launch_bounds__(kThreads, 1024 / kThreads) ta_select_kernel(ta_seq_desc seq, int n_layers, int Hkv, int K, int fast,
-                                                             UnitSrc src, const uint8_t* __restrict__ forced,
-                                                             const int32_t* __restrict__ r_main,
+                                                             UnitSrc src, const uint8_t* forced,
+                                                             const int32_t* r_main,
                                                              int32_t* __restrict__ idx, int32_t* __restrict__ count,
                                                              GatherDst gd, const int32_t* __restrict__ class_of) {
   __shared__ SelectShared sh;
   ta_wait_for_prior_grid();
+  ta_launch_dependents();
   const int unit = blockIdx.x / CL;
   const bool lead = blockIdx.x % CL == 0;
   int b, l = 0, g = 0;
@@ -1019,18 +1020,19 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads) ta_select_kernel(ta
         uu[it] = i < nl ? up[i] : 0.0f;
       }
       // the per-token values in groups of 8 (registers: a group's loads are in flight together, no more)
+      constexpr int kGroup = ITEMS < 8 ? ITEMS : 8;
 #pragma unroll
-      for (int g0 = 0; g0 < ITEMS; g0 += 8) {
-        float us[8];
-        uint8_t ff[8];
+      for (int g0 = 0; g0 < ITEMS; g0 += kGroup) {
+        float us[kGroup];
+        uint8_t ff[kGroup];
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {
+        for (int q = 0; q < kGroup; ++q) {
           const int i = tid + (g0 + q) * kThreads;
           us[q] = i < nl ? sp[i] : 0.0f;
           ff[q] = i < nl ? f[i] : (uint8_t)1;
         }
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {
+        for (int q = 0; q < kGroup; ++q) {
           const int it = g0 + q;
           const bool in = tid + it * kThreads < nl;
           kc.key[it] = in ? sortable_key(__fadd_rn(uu[it], us[q])) : 0u;
