@@ -229,6 +229,10 @@ ta_status ta_ctx_create(int device, size_t scratch_bytes, ta_ctx** out) {
   if (e == cudaSuccess) e = cudaMemset(c->d_status, 0, sizeof(ta_dev_status));
   if (e == cudaSuccess && scratch_bytes) e = cudaMalloc(&c->scratch, scratch_bytes);
   for (int i = 0; e == cudaSuccess && i < 8; ++i) e = cudaEventCreate(&c->ev[i]);
+  if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&c->copy_in, cudaStreamNonBlocking);
+  if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&c->copy_out, cudaStreamNonBlocking);
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_in, cudaEventDisableTiming);
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_out, cudaEventDisableTiming);
   if (e == cudaSuccess) {
     cudaDriverEntryPointQueryResult q;
     e = cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &c->encode_tiled, cudaEnableDefault, &q);
@@ -247,6 +251,10 @@ void ta_ctx_destroy(ta_ctx* c) {
   DeviceGuard guard(c->device);
   for (int i = 0; i < 8; ++i)
     if (c->ev[i]) cudaEventDestroy(c->ev[i]);
+  if (c->ev_in) cudaEventDestroy(c->ev_in);
+  if (c->ev_out) cudaEventDestroy(c->ev_out);
+  if (c->copy_in) cudaStreamDestroy(c->copy_in);
+  if (c->copy_out) cudaStreamDestroy(c->copy_out);
   if (c->scratch) cudaFree(c->scratch);
   if (c->d_status) cudaFree(c->d_status);
   delete c;
@@ -1096,14 +1104,6 @@ ta_status ta_compress_host(ta_ctx* ctx, const ta_patterns* pats, const ta_policy
   cudaStream_t stream = (cudaStream_t)stream_v;
   uint8_t* ws = reinterpret_cast<uint8_t*>(workspace);
   const size_t total = (size_t)batch->total_tokens;
-  cudaError_t e = cudaMemcpyAsync(ws + H.ids, token_ids, total * 4, cudaMemcpyHostToDevice, stream);
-  ta_batch db = *batch;
-  if (batch->cu_seqlens) {
-    if (e == cudaSuccess)
-      e = cudaMemcpyAsync(ws + H.cu, batch->cu_seqlens, ((size_t)batch->batch + 1) * 4, cudaMemcpyHostToDevice, stream);
-    db.cu_seqlens = reinterpret_cast<const int32_t*>(ws + H.cu);
-  }
-  if (e == cudaSuccess && !fast) e = cudaMemcpyAsync(ws + H.q, q_obs, H.q_bytes, cudaMemcpyHostToDevice, stream);
   // Only the retained rows of V are ever read (and, in fast mode, of K): when such a cache sits in pinned or
   // registered host memory the gather kernel reads those rows straight over the bus and the full copy is skipped.
   auto device_visible_host = [&](const void* ptr, const void** dev_alias) {
@@ -1119,29 +1119,92 @@ ta_status ta_compress_host(ta_ctx* ctx, const ta_patterns* pats, const ta_policy
   const void* k_src = ws + H.k;
   const void* v_src = ws + H.v;
   const void* alias = nullptr;
-  if (fast && device_visible_host(k, &alias)) k_src = alias;
-  else if (e == cudaSuccess) e = cudaMemcpyAsync(ws + H.k, k, H.kv_bytes, cudaMemcpyHostToDevice, stream);
-  if (device_visible_host(v, &alias)) v_src = alias;
-  else if (e == cudaSuccess) e = cudaMemcpyAsync(ws + H.v, v, H.kv_bytes, cudaMemcpyHostToDevice, stream);
-  if (e != cudaSuccess) return cuda_fail(ctx, e);
-  const int64_t n = batch->n_uniform, W = policy->obs_window;
-  ta_bf16_view vq = {ws + H.q, (int64_t)batch->batch * Hq * W * d, (int64_t)Hq * W * d, W * d, d};
-  ta_bf16_view vk, vv;
+  const bool copy_k = !(fast && device_visible_host(k, &alias));
+  if (!copy_k) k_src = alias;
+  const bool copy_v = !device_visible_host(v, &alias);
+  if (!copy_v) v_src = alias;
+
+  // The layers are independent of one another: their caches are copied, compressed and copied back in a few groups, so that
+  // the copies of one group run beside the kernels of another and both directions of the bus are busy (8 layers of 2 x 3000
+  // tokens: 2.20 -> 2.06 ms, 107 MB to the device at 55 GB/s being 1.95 ms). A group's cache is at least kGroupBytes, below which its copy is no longer worth the launches.
+  constexpr size_t kGroupBytes = 8u << 20;
+  constexpr int kMaxGroups = 16;
+  const int n_layers = batch->n_layers;
+  const size_t q_layer = H.q_bytes / n_layers, kv_layer = H.kv_bytes / n_layers, out_layer = H.out_bytes / n_layers;
+  const size_t idx_layer = H.idx_bytes / n_layers, count_layer = H.count_bytes / n_layers;
+  int group = (n_layers + kMaxGroups - 1) / kMaxGroups;
+  if (kv_layer * group < kGroupBytes) group = kv_layer ? (int)((kGroupBytes + kv_layer - 1) / kv_layer) : n_layers;
+  if ((!copy_k && !copy_v) || ctx->timing_enabled) group = n_layers;  // nothing large to copy in; timed as one call
+  if (group > n_layers) group = n_layers;
+  const bool several = group < n_layers;
+  cudaStream_t in = several ? ctx->copy_in : stream, out = several ? ctx->copy_out : stream;
+
+  cudaError_t e = cudaSuccess;
+  auto then = [&](cudaStream_t from, cudaStream_t to, cudaEvent_t ev) {  // what is enqueued on `to` next follows `from`
+    if (from == to) return;
+    if (e == cudaSuccess) e = cudaEventRecord(ev, from);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(to, ev, 0);
+  };
+  auto copy = [&](void* dst, const void* src, size_t bytes, cudaMemcpyKind kind, cudaStream_t on) {
+    if (e == cudaSuccess && bytes) e = cudaMemcpyAsync(dst, src, bytes, kind, on);
+  };
+  then(stream, in, ctx->ev_in);
+  copy(ws + H.ids, token_ids, total * 4, cudaMemcpyHostToDevice, in);
+  ta_batch db = *batch;
   if (batch->cu_seqlens) {
-    vk = {k_src, (int64_t)Hkv * (int64_t)total * d, 0, (int64_t)total * d, d};
-  } else {
-    vk = {k_src, (int64_t)batch->batch * Hkv * n * d, (int64_t)Hkv * n * d, n * d, d};
+    copy(ws + H.cu, batch->cu_seqlens, ((size_t)batch->batch + 1) * 4, cudaMemcpyHostToDevice, in);
+    db.cu_seqlens = reinterpret_cast<const int32_t*>(ws + H.cu);
   }
-  vv = vk;
-  vv.ptr = v_src;
-  s = ta_compress(ctx, pats, policy, &db, Hq, Hkv, d, K, reinterpret_cast<const int32_t*>(ws + H.ids), vq, vk, vv, 0,
-                  ws + H.k_out, ws + H.v_out, reinterpret_cast<int32_t*>(ws + H.idx),
-                  reinterpret_cast<int32_t*>(ws + H.count), stream);
+  copy(ws + H.q, q_obs, H.q_bytes, cudaMemcpyHostToDevice, in);  // small, and few copies: all layers at once
+  const int64_t n = batch->n_uniform, W = policy->obs_window;
+  ta_bf16_view vq = {nullptr, (int64_t)batch->batch * Hq * W * d, (int64_t)Hq * W * d, W * d, d};
+  ta_bf16_view vk;
+  if (batch->cu_seqlens) {
+    vk = {nullptr, (int64_t)Hkv * (int64_t)total * d, 0, (int64_t)total * d, d};
+  } else {
+    vk = {nullptr, (int64_t)batch->batch * Hkv * n * d, (int64_t)Hkv * n * d, n * d, d};
+  }
+  ta_bf16_view vv = vk;
+  // the groups share the per-sequence work under an epoch of this call's own
+  const uint64_t epoch = several ? (1ull << 63) | ++ctx->host_calls : 0;
+  ctx->cached_epoch = 0;
+  auto at = [](const void* base, size_t bytes) { return static_cast<const uint8_t*>(base) + bytes; };
+  auto to = [](void* base, size_t bytes) { return static_cast<uint8_t*>(base) + bytes; };
+  int launches = 0;
+  s = TA_OK;
+  for (int l = 0; s == TA_OK && e == cudaSuccess && l < n_layers; l += group) {
+    const int g = l + group < n_layers ? group : n_layers - l;
+    if (copy_k) copy(ws + H.k + kv_layer * l, at(k, kv_layer * l), kv_layer * g, cudaMemcpyHostToDevice, in);
+    if (copy_v) copy(ws + H.v + kv_layer * l, at(v, kv_layer * l), kv_layer * g, cudaMemcpyHostToDevice, in);
+    then(in, stream, ctx->ev_in);
+    if (e != cudaSuccess) break;
+    db.n_layers = g;
+    vq.ptr = ws + H.q + q_layer * l;
+    vk.ptr = at(k_src, kv_layer * l);
+    vv.ptr = at(v_src, kv_layer * l);
+    s = ta_compress(ctx, pats, policy, &db, Hq, Hkv, d, K, reinterpret_cast<const int32_t*>(ws + H.ids), vq, vk, vv, epoch,
+                    ws + H.k_out + out_layer * l, ws + H.v_out + out_layer * l,
+                    reinterpret_cast<int32_t*>(ws + H.idx + idx_layer * l),
+                    reinterpret_cast<int32_t*>(ws + H.count + count_layer * l), stream);
+    if (s != TA_OK) break;
+    then(stream, out, ctx->ev_out);
+    copy(to(k_out, out_layer * l), ws + H.k_out + out_layer * l, out_layer * g, cudaMemcpyDeviceToHost, out);
+    copy(to(v_out, out_layer * l), ws + H.v_out + out_layer * l, out_layer * g, cudaMemcpyDeviceToHost, out);
+    launches += ctx->last_kernel_launches;
+  }
+  if (s == TA_OK) {
+    copy(idx, ws + H.idx, H.idx_bytes, cudaMemcpyDeviceToHost, out);
+    copy(count, ws + H.count, H.count_bytes, cudaMemcpyDeviceToHost, out);
+  }
+  ctx->last_kernel_launches = launches;
+  ctx->cached_epoch = 0;
+  // the caller's stream follows everything that was enqueued, also after an error in between
+  const cudaError_t first = e;
+  e = cudaSuccess;
+  then(in, stream, ctx->ev_in);
+  then(out, stream, ctx->ev_out);
+  if (first != cudaSuccess) e = first;
   if (s != TA_OK) return s;
-  e = cudaMemcpyAsync(k_out, ws + H.k_out, H.out_bytes, cudaMemcpyDeviceToHost, stream);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(v_out, ws + H.v_out, H.out_bytes, cudaMemcpyDeviceToHost, stream);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(idx, ws + H.idx, H.idx_bytes, cudaMemcpyDeviceToHost, stream);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(count, ws + H.count, H.count_bytes, cudaMemcpyDeviceToHost, stream);
   return e == cudaSuccess ? TA_OK : cuda_fail(ctx, e);
 }
 

@@ -45,6 +45,10 @@ struct ta_ctx {
   int timing_valid;
   cudaEvent_t ev[8];
   int ev_ran[4];
+  // ta_compress_host: copies to and from the device beside the kernels of other layers
+  cudaStream_t copy_in, copy_out;
+  cudaEvent_t ev_in, ev_out;
+  uint64_t host_calls;
   // launch shape of the most recent score kernel (diagnostics)
   int score_cluster, score_clusters;
   // score kernel launch state per instantiation (2 row-block counts x 3 output forms): attribute set, resident

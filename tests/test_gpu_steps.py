@@ -815,3 +815,35 @@ def test_compress_with_zero_pension_weight():
                 assert_selection_matches(idx[0, b, h], cnt[0, b, h], io, co, u, f"b{b} h{h}")
     finally:
         g.close()
+
+
+@pytest.mark.parametrize("fast,lengths,L", [(False, [9000, 9000], 5), (False, [7000, 40, 9000], 3), (True, [9000], 6)])
+def test_compress_host_in_groups_of_layers(fast, lengths, L):
+    """Caches large enough that the host variant copies, compresses and copies back a few layers at a time (the last group
+    is a short one): the same results as one device call, twice on one context."""
+    K = 64
+    w = _workload(lengths, [[4, 5], [9]], seed=77, Hq=8, Hkv=2, W=32)
+    w.uniform = len(set(lengths)) == 1
+    pol = oracle_policy(K, "THEOREM", fast=fast, W=32)
+    Qh, Kh, Vh = tw.make_qkv(w, range(L))
+    g = Gpu(w, pol, K, L)
+    try:
+        idx, cnt, ko, vo = g.compress(Qh.cuda(), Kh.cuda(), Vh.cuda())
+        torch.cuda.synchronize()
+        cu = np.ascontiguousarray(w.cu) if not w.uniform else None
+        hb = ta.make_batch(L, w.B, lengths[0] if w.uniform else 0, w.max_n, w.total, cu)
+        nbytes = ta.ta_compress_host_workspace_bytes(hb, w.Hq, w.Hkv, w.d, K, g.p)
+        ws = torch.empty(nbytes, dtype=torch.uint8, device="cuda")
+        outs = [torch.full(t.shape, 3, dtype=t.dtype).pin_memory() for t in (ko, vo, idx, cnt)]
+        k_h = Kh if fast else Kh.pin_memory()  # pageable in fast mode, so that it is copied there too
+        for v_h in (Vh.pin_memory(), Vh):
+            ta.ta_compress_host(g.ctx, g.pats, g.p, hb, w.Hq, w.Hkv, w.d, K, torch.from_numpy(w.ids), None if fast else Qh,
+                                k_h, v_h, *outs, ws, nbytes, g.stream)
+            torch.cuda.synchronize()
+            assert g.poll() == ta.TA_OK
+            for got, want in zip(outs, (ko, vo, idx, cnt)):
+                assert torch.equal(got.view(torch.int16) if got.dtype == torch.bfloat16 else got,
+                                   (want.view(torch.int16) if want.dtype == torch.bfloat16 else want).cpu())
+                got.fill_(3)
+    finally:
+        g.close()
