@@ -14,18 +14,6 @@ constexpr int kRowsPerIter = kThreads / kLanesPerRow;        // 16
 constexpr int kUnroll = 4;
 constexpr int kRowsPerBlock = kRowsPerIter * kUnroll;        // 64
 
-__device__ __forceinline__ uint4 ld_stream(const uint4* p) {
-  uint4 v;
-  asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
-               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
-               : "l"(p));
-  return v;
-}
-__device__ __forceinline__ void st_stream(uint4* p, uint4 v) {
-  asm volatile("st.global.cs.v4.u32 [%0], {%1,%2,%3,%4};" ::"l"(p), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w)
-               : "memory");
-}
-
 // grid.x = units (l, b, g), grid.y = ceil(K / 64) row blocks, grid.z = 2 (K cache, V cache)
 __global__ void __launch_bounds__(kThreads) ta_compact_kernel(ta_seq_desc seq, int Hkv, int K, ta_bf16_view kv0,
                                                               ta_bf16_view kv1, const int32_t* idx, const int32_t* count,
@@ -61,16 +49,14 @@ __global__ void __launch_bounds__(kThreads) ta_compact_kernel(ta_seq_desc seq, i
   for (int j = 0; j < kUnroll; ++j) {
     const int r = r0 + j * kRowsPerIter;
     rows[j] = r;
-    v[j] = make_uint4(0u, 0u, 0u, 0u);
-    if (r < K && r < cnt) {
-      const int i = uidx[r];
-      if (i >= 0 && i < n)  // an index outside the sequence is skipped, never dereferenced
-        v[j] = ld_stream(reinterpret_cast<const uint4*>(sp + (long long)i * src.stride_n) + lane16);
-    }
+    const bool kept = r < K && r < cnt;
+    const int i = kept ? uidx[r] : -1;
+    // an index outside the sequence is skipped, never dereferenced
+    v[j] = ta_ld_stream_if(reinterpret_cast<const uint4*>(sp + (long long)i * src.stride_n) + lane16, i >= 0 && i < n);
   }
 #pragma unroll
   for (int j = 0; j < kUnroll; ++j)
-    if (rows[j] < K) st_stream(out + (long long)rows[j] * kLanesPerRow + lane16, v[j]);
+    if (rows[j] < K) ta_st_stream(out + (long long)rows[j] * kLanesPerRow + lane16, v[j]);
 }
 
 }  // namespace

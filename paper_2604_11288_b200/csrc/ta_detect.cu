@@ -34,14 +34,6 @@ __device__ __forceinline__ float sq2(uint32_t w) {  // sum of squares of a bf16 
   return fmaf(lo, lo, hi * hi);
 }
 
-__device__ __forceinline__ uint4 ld_stream(const uint4* p) {
-  uint4 v;
-  asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
-               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
-               : "l"(p));
-  return v;
-}
-
 __global__ void __launch_bounds__(kWarps * 32, 3)
 ta_embed_conf_kernel(long long total, const __nv_bfloat16* __restrict__ emb, long long stride, int D,
                      const __nv_bfloat16* __restrict__ concepts, int C, float* __restrict__ conf) {
@@ -103,13 +95,13 @@ ta_embed_conf_kernel(long long total, const __nv_bfloat16* __restrict__ emb, lon
       uint4 v0[kAhead], v1[kAhead];
 #pragma unroll
       for (int j = 0; j < kAhead; ++j) {
-        v0[j] = ld_stream(e0 + (k >> 3) + 4 * j);
-        v1[j] = ld_stream(e1 + (k >> 3) + 4 * j);
+        v0[j] = ta_ld_stream(e0 + (k >> 3) + 4 * j);
+        v1[j] = ta_ld_stream(e1 + (k >> 3) + 4 * j);
       }
 #pragma unroll
       for (int j = 0; j < kAhead; ++j) step(v0[j], v1[j], k + 32 * j);
     }
-    for (; k < k_hi; k += 32) step(ld_stream(e0 + (k >> 3)), ld_stream(e1 + (k >> 3)), k);
+    for (; k < k_hi; k += 32) step(ta_ld_stream(e0 + (k >> 3)), ta_ld_stream(e1 + (k >> 3)), k);
     // the four lanes of a row hold its norm in parts, and its dot products with concepts 2q and 2q + 1
     n0 += __shfl_xor_sync(0xffffffffu, n0, 1);
     n0 += __shfl_xor_sync(0xffffffffu, n0, 2);

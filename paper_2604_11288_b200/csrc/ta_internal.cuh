@@ -92,6 +92,28 @@ __device__ __forceinline__ void ta_wait_for_prior_grid() { asm volatile("griddep
 // kernel's own wait: the dependent may then rely on everything before this kernel being complete.
 __device__ __forceinline__ void ta_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// 16-byte loads and stores of rows that are touched once
+__device__ __forceinline__ uint4 ta_ld_stream(const uint4* p) {
+  uint4 v;
+  asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
+               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+               : "l"(p));
+  return v;
+}
+// the same under a predicate, zero without it. Not a load under a branch: several of those in a row waited for one another.
+__device__ __forceinline__ uint4 ta_ld_stream_if(const uint4* p, bool wanted) {
+  uint4 v;
+  asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %5, 0;\n\tmov.u32 %0, 0;\n\tmov.u32 %1, 0;\n\tmov.u32 %2, 0;\n\tmov.u32 %3, 0;\n\t"
+               "@q ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];\n\t}"
+               : "=&r"(v.x), "=&r"(v.y), "=&r"(v.z), "=&r"(v.w)
+               : "l"(p), "r"((uint32_t)wanted));
+  return v;
+}
+__device__ __forceinline__ void ta_st_stream(uint4* p, uint4 v) {
+  asm volatile("st.global.cs.v4.u32 [%0], {%1,%2,%3,%4};" ::"l"(p), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w)
+               : "memory");
+}
+
 // x / n rounded to nearest for whole numbers 0 <= x <= 2^24 and 1 <= n <= 2^24, given r = 1/n rounded to nearest: one
 // product and one residual correction, which is correctly rounded because r is (Markstein's theorem; no over- or underflow
 // in this range). Many tokens share n: three instructions a quotient, where a division costs about twenty.

@@ -181,13 +181,11 @@ bool few_short_units(const ta_select_args& a) {
   return !a.fast && a.seq.max_n <= 8 * sel1024::kThreads && a.n_layers * a.seq.batch * a.Hkv <= sm_count_of(a);
 }
 
+// Whether the selecting blocks move the rows: keys in registers, one block per unit (see gather_unit).
 bool ta_select_gathers(const ta_select_args& a) {
-  if (!a.gather_k_out || a.fast || a.seq.max_n > kItems * kThreads) return false;
-  // The gather adds a dependent load chain (index -> row -> store, about 2 us) to every block, the separate kernel costs a
-  // launch and its tail (about 5 us for so few rows): fusing pays while the blocks run in a few waves and a block's rows
-  // are few rounds of its threads. Short units (keys in registers, more than one block per SM) only.
-  if (few_short_units(a)) return a.K <= 256;  // at most 8 pieces of 16 bytes per thread
-  return a.K <= 16 && a.n_layers * a.seq.batch * a.Hkv <= 4 * sm_count_of(a);
+  const int units = a.n_layers * a.seq.batch * a.Hkv;
+  return a.gather_k_out && !a.fast && a.seq.max_n <= sel1024::kItemsLong * sel1024::kThreads &&
+         !split_units(units, a.seq.max_n, sm_count_of(a));
 }
 
 cudaError_t ta_launch_select_units(const ta_select_args& a, cudaStream_t stream_) {
@@ -226,20 +224,20 @@ cudaError_t ta_launch_select_units(const ta_select_args& a, cudaStream_t stream_
     return launch_threads(sel1024::kThreads, kern, units, 1, stream, a.seq, a.n_layers, a.Hkv, a.K, a.fast, src2, a.forced,
                           a.r_main, a.idx, a.count, gd2, co);
   }
-  if (gathers)  // implies the first variant below
-    return launch_clustered(ta_select_kernel<true, 1, kItems, true>, units, 1, stream, a.seq, a.n_layers, a.Hkv, a.K,
-                            a.fast, src, a.forced, a.r_main, a.idx, a.count, gd, co);
-  if (a.seq.max_n <= kItems * kThreads)
-    return launch_clustered(ta_select_kernel<true, 1>, units, 1, stream, a.seq, a.n_layers, a.Hkv, a.K, a.fast, src,
-                            a.forced, a.r_main, a.idx, a.count, gd, co);
-  if (!split_units(units, a.seq.max_n, sms) && a.seq.max_n <= kItemsLong * kThreads)
-    return launch_clustered(ta_select_kernel<true, 1, kItemsLong>, units, 1, stream, a.seq, a.n_layers, a.Hkv, a.K, a.fast,
-                            src, a.forced, a.r_main, a.idx, a.count, gd, co);
+  if (!split_units(units, a.seq.max_n, sms) && a.seq.max_n <= kItemsLong * kThreads) {
+    auto kern = a.seq.max_n <= kItems * kThreads
+                    ? (gathers ? ta_select_kernel<true, 1, kItems, true> : ta_select_kernel<true, 1, kItems, false>)
+                    : (gathers ? ta_select_kernel<true, 1, kItemsLong, true> : ta_select_kernel<true, 1, kItemsLong, false>);
+    return launch_clustered(kern, units, 1, stream, a.seq, a.n_layers, a.Hkv, a.K, a.fast, src, a.forced, a.r_main, a.idx,
+                            a.count, gd, co);
+  }
   if (!split_units(units, a.seq.max_n, sms) && a.seq.max_n <= sel1024::kItemsLong * sel1024::kThreads) {
     // many long units: blocks of 1024 threads hold a unit of up to 32768 keys in registers (read once instead of
     // once per radix pass and once more for the ordered write)
-    return launch_threads(sel1024::kThreads, sel1024::ta_select_kernel<true, 1, sel1024::kItemsLong>, units, 1, stream,
-                          a.seq, a.n_layers, a.Hkv, a.K, a.fast, src2, a.forced, a.r_main, a.idx, a.count, gd2, co);
+    auto kern = gathers ? sel1024::ta_select_kernel<true, 1, sel1024::kItemsLong, true>
+                        : sel1024::ta_select_kernel<true, 1, sel1024::kItemsLong, false>;
+    return launch_threads(sel1024::kThreads, kern, units, 1, stream, a.seq, a.n_layers, a.Hkv, a.K, a.fast, src2, a.forced,
+                          a.r_main, a.idx, a.count, gd2, co);
   }
   if (!split_units(units, a.seq.max_n, sms))
     return launch_clustered(ta_select_kernel<false, 1>, units, 1, stream, a.seq, a.n_layers, a.Hkv, a.K, a.fast, src,

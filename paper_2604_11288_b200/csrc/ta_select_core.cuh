@@ -917,34 +917,45 @@ __device__ __forceinline__ float unit_utility(const UnitSrc& src, long long unit
   return __fadd_rn(__fadd_rn(aA, dP), u0);
 }
 
-// Small budgets and few units: the block that selected a unit also moves its retained K and V rows (Algorithm 1
-// step 9), which saves the launch of the gather kernel where that launch costs more than the copy. Same result as ta_compact_kernel:
-// rows at and beyond the retained count, and rows whose index lies outside the sequence, are zero.
+// The block that selected a unit also moves its retained K and V rows (Algorithm 1 step 9): same result as
+// ta_compact_kernel (rows at and beyond the retained count, and rows whose index lies outside the sequence, are zero).
+// Selection is bound by latency and instruction issue, the copy by HBM: with many units the blocks of one kernel are in
+// different phases and the two overlap in part (2048 units of up to 8000 tokens, K = 512: 105 + 175 us as two kernels,
+// 232 us as one; starting half of the blocks half a period late changed nothing); with few, a launch is saved.
 struct GatherDst {
   ta_bf16_view k, v;
   uint4* k_out;
   uint4* v_out;
 };
 
+// Rows are listed in sh.cand_keys (the first kCandCap of them) and in `out`; all: row r is position r.
 __device__ __forceinline__ void gather_unit(const GatherDst& gd, const ta_seq_desc& seq, int unit, int l, int b, int g,
-                                            int n, int K, const int32_t* out, int taken) {
-  constexpr int kLanesPerRow = TA_HEAD_DIM * 2 / 16;
+                                            int n, int K, const int32_t* out, int taken, bool all, const SelectShared& sh) {
+  constexpr int kLanesPerRow = TA_HEAD_DIM * 2 / 16;  // a warp moves the K and the V row of one position at a time
+  constexpr int kUnroll = 8;
+  static_assert(2 * kLanesPerRow == 32, "one lane per 16-byte piece of a K row and a V row");
   __syncthreads();  // the unit's indices were written by other threads of this block
-#pragma unroll 4
-  for (int t = threadIdx.x; t < K * 2 * kLanesPerRow; t += kThreads) {
-    const int r = t / (2 * kLanesPerRow), which = (t / kLanesPerRow) & 1, lane16 = t % kLanesPerRow;
-    const ta_bf16_view& src = which ? gd.v : gd.k;
-    uint4 val = make_uint4(0u, 0u, 0u, 0u);
-    if (r < taken) {
-      const int i = out[r];
-      if (i >= 0 && i < n) {
-        const long long base = (long long)l * src.stride_l + (long long)g * src.stride_h +
-                               (seq.cu ? (long long)seq.cu[b] * src.stride_n : (long long)b * src.stride_b);
-        val = __ldg(reinterpret_cast<const uint4*>(reinterpret_cast<const uint16_t*>(src.ptr) + base +
-                                                   (long long)i * src.stride_n) + lane16);
-      }
+  const int lane = threadIdx.x & 31, which = lane / kLanesPerRow, piece = lane % kLanesPerRow;
+  const ta_bf16_view& src = which ? gd.v : gd.k;
+  const long long base = (long long)l * src.stride_l + (long long)g * src.stride_h +
+                         (seq.cu ? (long long)seq.cu[b] * src.stride_n : (long long)b * src.stride_b);
+  const uint4* from = reinterpret_cast<const uint4*>(reinterpret_cast<const uint16_t*>(src.ptr) + base) + piece;
+  uint4* to = (which ? gd.v_out : gd.k_out) + (long long)unit * K * kLanesPerRow + piece;
+  const long long row_pieces = src.stride_n / 8;
+  for (int r0 = threadIdx.x / 32; r0 < K; r0 += kUnroll * kWarps) {
+    uint4 val[kUnroll];
+#pragma unroll
+    for (int j = 0; j < kUnroll; ++j) {
+      const int r = r0 + j * kWarps;
+      int i = all ? r : (int)sh.cand_keys[min(r, kCandCap - 1)];
+      if (r >= kCandCap && r < taken && !all) i = out[r];
+      val[j] = ta_ld_stream_if(from + i * row_pieces, r < taken && i >= 0 && i < n);
     }
-    (which ? gd.v_out : gd.k_out)[((long long)unit * K + r) * kLanesPerRow + lane16] = val;
+#pragma unroll
+    for (int j = 0; j < kUnroll; ++j) {
+      const int r = r0 + j * kWarps;
+      if (r < K) ta_st_stream(to + (long long)r * kLanesPerRow, val[j]);
+    }
   }
 }
 
@@ -983,7 +994,7 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads) ta_select_kernel(ta
       for (int r = tid; r < K; r += kThreads) out[r] = -1;
       if (tid == 0) count[unit] = 0;
     }
-    if constexpr (GATHER) gather_unit(gd, seq, unit, l, b, g, n, K, out, 0);
+    if constexpr (GATHER) gather_unit(gd, seq, unit, l, b, g, n, K, out, 0, true, sh);
     return;
   }
   if (want == -1) {  // K >= n: keep everything
@@ -991,7 +1002,7 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads) ta_select_kernel(ta
       for (int r = tid; r < K; r += kThreads) out[r] = r < n ? r : -1;
       if (tid == 0) count[unit] = n;
     }
-    if constexpr (GATHER) gather_unit(gd, seq, unit, l, b, g, n, K, out, n);
+    if constexpr (GATHER) gather_unit(gd, seq, unit, l, b, g, n, K, out, n, true, sh);
     return;
   }
   const long long unit_off = fast ? 0 : ((long long)l * Hkv + g) * seq.total;
@@ -1053,6 +1064,7 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads) ta_select_kernel(ta
   };
   auto emit = [&](int il, int rank) {
     if (rank < K) out[rank] = lo + il;
+    if (GATHER && rank < min(K, kCandCap)) sh.cand_keys[rank] = (uint32_t)il;  // (the selection is done with the list)
   };
   int taken;
   if constexpr (CACHED)  // forced tokens (not eligible, inside the unit) are taken whatever their key
@@ -1062,7 +1074,7 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads) ta_select_kernel(ta
   if (!lead) return;
   for (int q = taken + tid; q < K; q += kThreads) out[q] = -1;
   if (tid == 0) count[unit] = taken;
-  if constexpr (GATHER) gather_unit(gd, seq, unit, l, b, g, n, K, out, min(taken, K));
+  if constexpr (GATHER) gather_unit(gd, seq, unit, l, b, g, n, K, out, min(taken, K), false, sh);
 }
 
 }  // namespace TA_SEL_NS

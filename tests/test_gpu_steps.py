@@ -847,3 +847,31 @@ def test_compress_host_in_groups_of_layers(fast, lengths, L):
                 got.fill_(3)
     finally:
         g.close()
+
+
+@pytest.mark.parametrize("K,lengths,L", [(2049, [4000], 1), (4096, [5000, 100], 2), (3000, [8192] * 5, 32),
+                                         (2600, [12000] * 3, 30), (2600, [30000] * 3, 30), (70, [500, 60, 8000], 60)])
+def test_selecting_blocks_gather_like_the_separate_kernel(K, lengths, L):
+    """Selection and gather in one kernel (all block sizes; budgets beyond the index list in shared memory, sequences
+    shorter than the budget) against ta_select_topk and ta_compact_kv on the same scores."""
+    w = _workload(lengths, [[5, 6], [9]], seed=K, Hq=4, Hkv=2)
+    pol = oracle_policy(K, "THEOREM")
+    g = Gpu(w, pol, K, L)
+    try:
+        gen = torch.Generator(device="cuda")
+        gen.manual_seed(K)
+        kv = [torch.randn((L, w.Hkv, w.total, w.d), generator=gen, dtype=torch.bfloat16, device="cuda") for _ in range(2)]
+        A = torch.randn((L, w.Hkv, w.total), generator=gen, dtype=torch.float32, device="cuda")
+        w.uniform = False
+        g.cu = torch.from_numpy(w.cu).cuda()
+        g.batch = ta.make_batch(L, w.B, 0, w.max_n, w.total, g.cu)
+        idx, cnt, ko, vo = g.compress_scores(A, None, *kv)
+        idx2, cnt2 = g.select(*g.sponsor_mask(), A)
+        ko2, vo2 = g.compact(*kv, idx2, cnt2)
+        torch.cuda.synchronize()
+        assert g.poll() == ta.TA_OK
+        assert torch.equal(idx, idx2) and torch.equal(cnt, cnt2)
+        assert torch.equal(ko.view(torch.int16), ko2.view(torch.int16))
+        assert torch.equal(vo.view(torch.int16), vo2.view(torch.int16))
+    finally:
+        g.close()
