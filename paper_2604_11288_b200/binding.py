@@ -1,16 +1,20 @@
 """ctypes binding of libta.so: the same names and arguments as include/ta.h, marshalling only.
 
 Every step of the method runs in the CUDA kernels behind these calls. There is no CPU path: if the shared library is
-missing, loading raises. Tensors are passed as raw device (or, for ta_compress_host, host) addresses; torch is used
+missing, loading raises. The calls that a program makes once per layer or per token go through the native module _ta_call
+(one layer of a 4096-token prompt: 22 -> 17 us on the host, 32 layers one by one 890 -> 535 us), the others through ctypes. Tensors are passed as raw device (or, for ta_compress_host, host) addresses; torch is used
 by callers only to own memory and streams.
 """
 from __future__ import annotations
 
 import ctypes as C
+import importlib.machinery
+import importlib.util
 import os
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libta.so")
+CALL_PATH = os.path.join(_HERE, "_ta_call.so")
 
 TA_OK = 0
 TA_ERR_INVALID_ARG, TA_ERR_UNSUPPORTED, TA_ERR_ALIGNMENT, TA_ERR_SCRATCH_TOO_SMALL = 1, 2, 3, 4
@@ -53,11 +57,30 @@ class TAError(RuntimeError):
 
 
 _lib = None
+_call = None  # the native module, once lib() has run
+
+
+def _load_call(L):
+    if not os.path.exists(CALL_PATH):
+        raise FileNotFoundError(f"{CALL_PATH} is missing: run `python -m paper_2604_11288_b200.build`")
+    loader = importlib.machinery.ExtensionFileLoader("_ta_call", CALL_PATH)
+    m = importlib.util.module_from_spec(importlib.util.spec_from_loader("_ta_call", loader))
+    loader.exec_module(m)
+    m.set_types(C.c_void_p, ta_bf16_view, ta_policy, ta_batch, ta_stream)
+    for name in ("ta_compress", "ta_compress_lse", "ta_compress_scores", "ta_stream_step", "ta_detect_embedding",
+                 "ta_sponsor_mask_conf"):
+        m.set_function(name, C.cast(getattr(L, name), C.c_void_p).value)
+    return m
+
+
+def _native():
+    lib()
+    return _call
 
 
 def lib():
     """Loads libta.so (built in-tree by paper_2604_11288_b200.build). Raises if it is not there."""
-    global _lib
+    global _lib, _call
     if _lib is None:
         if not os.path.exists(LIB_PATH):
             raise FileNotFoundError(f"{LIB_PATH} is missing: run `python -m paper_2604_11288_b200.build` (there is no "
@@ -114,6 +137,7 @@ def lib():
             fn = getattr(L, name)
             fn.restype = res
             fn.argtypes = args
+        _call = _load_call(L)
         _lib = L
     return _lib
 
@@ -140,15 +164,7 @@ def _ptr(t):
 
 def view(t, ragged=False) -> ta_bf16_view:
     """ta_bf16_view of a bf16 tensor [L, B, H, n, d] (uniform) or [L, H, total, d] (ragged); strides in elements."""
-    if t is None:
-        return ta_bf16_view(None, 0, 0, 0, 0)
-    s = t.stride()
-    assert s[-1] == 1, "head_dim must be contiguous"
-    if ragged:
-        assert t.dim() == 4
-        return ta_bf16_view(t.data_ptr(), s[0], 0, s[1], s[2])
-    assert t.dim() == 5
-    return ta_bf16_view(t.data_ptr(), s[0], s[1], s[2], s[3])
+    return (_call or _native()).view(t, ragged)
 
 
 def ta_policy_default(preset: int, K: int) -> ta_policy:
@@ -215,15 +231,15 @@ def ta_patterns_destroy(pats):
 
 
 def ta_detect_embedding(ctx, total_tokens, emb, stride_tok, D, concepts, n_concepts, conf, stream=None):
-    _check(lib().ta_detect_embedding(ctx, int(total_tokens), _ptr(emb), int(stride_tok), int(D), _ptr(concepts),
-                                     int(n_concepts), _ptr(conf), stream), "ta_detect_embedding")
+    _check((_call or _native()).ta_detect_embedding(ctx, total_tokens, emb, stride_tok, D, concepts, n_concepts, conf, stream),
+           "ta_detect_embedding")
 
 
 def ta_sponsor_mask_conf(ctx, policy, batch, token_ids, conf, threshold, budget, span, rank_by_confidence, flags,
                          voucher, u_static, stream=None):
-    _check(lib().ta_sponsor_mask_conf(ctx, C.byref(policy), C.byref(batch), _ptr(token_ids), _ptr(conf),
-                                      C.c_float(threshold), C.c_float(budget), int(span), int(rank_by_confidence),
-                                      _ptr(flags), _ptr(voucher), _ptr(u_static), stream), "ta_sponsor_mask_conf")
+    _check((_call or _native()).ta_sponsor_mask_conf(ctx, policy, batch, token_ids, conf, threshold, budget, span,
+                                                     rank_by_confidence, flags, voucher, u_static, stream),
+           "ta_sponsor_mask_conf")
 
 
 def ta_sponsor_mask(ctx, pats, policy, batch, token_ids, flags, voucher, u_static, stream=None):
@@ -247,9 +263,8 @@ def ta_ctx_set_wait_limit(ctx, nanoseconds: int):
 
 def ta_compress_lse(ctx, pats, policy, batch, Hq, Hkv, d, K, token_ids, q_obs: ta_bf16_view, k: ta_bf16_view,
                     v: ta_bf16_view, lse_obs, seq_epoch, k_out, v_out, idx, count, stream=None):
-    _check(lib().ta_compress_lse(ctx, pats, C.byref(policy), C.byref(batch), Hq, Hkv, d, K, _ptr(token_ids), q_obs, k, v,
-                                 _ptr(lse_obs), seq_epoch, _ptr(k_out), _ptr(v_out), _ptr(idx), _ptr(count), stream),
-           "ta_compress_lse")
+    _check((_call or _native()).ta_compress_lse(ctx, pats, policy, batch, Hq, Hkv, d, K, token_ids, q_obs, k, v, lse_obs,
+                                                seq_epoch, k_out, v_out, idx, count, stream), "ta_compress_lse")
 
 
 def ta_score_headsum(ctx, policy, batch, Hq, Hkv, d, q_obs: ta_bf16_view, k: ta_bf16_view, u_heads, stream=None):
@@ -299,8 +314,8 @@ def ta_compact_kv(ctx, batch, Hkv, d, K, k: ta_bf16_view, v: ta_bf16_view, idx, 
 
 def ta_compress(ctx, pats, policy, batch, Hq, Hkv, d, K, token_ids, q_obs: ta_bf16_view, k: ta_bf16_view,
                 v: ta_bf16_view, seq_epoch, k_out, v_out, idx, count, stream=None):
-    _check(lib().ta_compress(ctx, pats, C.byref(policy), C.byref(batch), Hq, Hkv, d, K, _ptr(token_ids), q_obs, k, v,
-                             int(seq_epoch), _ptr(k_out), _ptr(v_out), _ptr(idx), _ptr(count), stream), "ta_compress")
+    _check((_call or _native()).ta_compress(ctx, pats, policy, batch, Hq, Hkv, d, K, token_ids, q_obs, k, v, seq_epoch, k_out,
+                                            v_out, idx, count, stream), "ta_compress")
 
 
 def ta_compress_allheads(ctx, pats, policy, batch, Hq, Hkv, d, K, token_ids, q_obs: ta_bf16_view, k: ta_bf16_view,
@@ -312,9 +327,8 @@ def ta_compress_allheads(ctx, pats, policy, batch, Hq, Hkv, d, K, token_ids, q_o
 
 def ta_compress_scores(ctx, pats, policy, batch, Hkv, d, K, token_ids, score, score2, k: ta_bf16_view,
                        v: ta_bf16_view, seq_epoch, k_out, v_out, idx, count, stream=None):
-    _check(lib().ta_compress_scores(ctx, pats, C.byref(policy), C.byref(batch), Hkv, d, K, _ptr(token_ids),
-                                    _ptr(score), _ptr(score2), k, v, int(seq_epoch), _ptr(k_out), _ptr(v_out),
-                                    _ptr(idx), _ptr(count), stream), "ta_compress_scores")
+    _check((_call or _native()).ta_compress_scores(ctx, pats, policy, batch, Hkv, d, K, token_ids, score, score2, k, v,
+                                                   seq_epoch, k_out, v_out, idx, count, stream), "ta_compress_scores")
 
 
 def ta_scratch_bytes_budgets(batch: ta_batch, Hkv, K_max, policy: ta_policy, n_budget_classes) -> int:
@@ -347,8 +361,7 @@ def ta_stream_scratch_bytes(st: ta_stream) -> int:
 
 
 def ta_stream_step(ctx, pats, policy, st: ta_stream, new_ids, attn, evicted_pos, stream=None):
-    _check(lib().ta_stream_step(ctx, pats, C.byref(policy), C.byref(st), _ptr(new_ids), _ptr(attn), _ptr(evicted_pos),
-                                stream), "ta_stream_step")
+    _check((_call or _native()).ta_stream_step(ctx, pats, policy, st, new_ids, attn, evicted_pos, stream), "ta_stream_step")
 
 
 def ta_compress_host_workspace_bytes(batch, Hq, Hkv, d, K, policy) -> int:

@@ -1,14 +1,18 @@
-"""Builds paper_2604_11288_b200/libta.so from csrc/*.cu with nvcc for sm_100a (cross-compiles without a GPU)."""
+"""Builds paper_2604_11288_b200/libta.so from csrc/*.cu with nvcc for sm_100a (cross-compiles without a GPU), and the CPython
+module _ta_call.so (argument marshalling of the most frequent calls) from csrc/py_call.cpp with g++."""
 from __future__ import annotations
 
 import glob
 import os
 import subprocess
 import sys
+import sysconfig
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 _ROOT = os.path.dirname(_HERE)
 LIB_PATH = os.path.join(_HERE, "libta.so")
+CALL_PATH = os.path.join(_HERE, "_ta_call.so")
+CALL_SOURCE = os.path.join(_HERE, "csrc", "py_call.cpp")
 
 
 def sources():
@@ -24,7 +28,13 @@ def _stale():
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
-    """Compile every CUDA source into one shared library. Returns its path."""
+    """Compile every CUDA source into one shared library, and the marshalling module. Returns the library's path."""
+    header = os.path.join(_ROOT, "include", "ta.h")
+    if force or not os.path.exists(CALL_PATH) or any(os.path.getmtime(f) > os.path.getmtime(CALL_PATH)
+                                                     for f in (CALL_SOURCE, header)):
+        subprocess.run([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-I",
+                        os.path.join(_ROOT, "include"), "-I", sysconfig.get_paths()["include"], CALL_SOURCE, "-o",
+                        CALL_PATH], check=True)
     if not force and not _stale():
         return LIB_PATH
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")

@@ -58,6 +58,9 @@ struct ta_ctx {
   int last_select_gathered;           // the most recent ta_compress let the selection kernel gather the rows
   int last_kernel_launches;           // kernels enqueued by the most recent ta_compress
   int score_force_cluster;            // > 0: CTAs per unit fixed by ta_ctx_set_option (tuning, tests)
+  // pension weights of the window rows for the (rho, W) they were last formed for
+  float wrow_rho, wrow[TA_MAX_WINDOW];
+  int wrow_W;
   unsigned long long wait_limit_ns;   // 0: default limit of device-side waits
   // driver entry point for tensor-map encoding (resolved at create time)
   void* encode_tiled;

@@ -10,9 +10,9 @@
 // Both passes use the same shared-memory operand tiles (both K-major, 128-byte swizzle); only the roles in the
 // instruction descriptor swap, which puts the reduction axis of each pass along a thread's own registers.
 // A unit is handled by a cluster of 1, 2, 4 or 8 CTAs (chosen per launch: one CTA when there are many units, more when
-// there are few); each CTA owns a contiguous range of 128-key tiles. Between the passes every CTA publishes its
-// per-row (reference, sum) pairs in its own shared memory, signals its peers with a remote mbarrier arrive, and reads
-// the peers' pairs with distributed-shared-memory loads. Pass 2 walks the CTA's tiles backwards so that the tiles read
+// there are few, up to 16 for a handful of units); each CTA owns a contiguous range of 128-key tiles. Between the passes
+// every CTA stores its per-row (reference, sum) pairs into the shared memory of all its peers and signals them with a remote
+// mbarrier arrive (posted stores: reading the peers' pairs over the cluster took 1.9 us of a 15 us kernel). Pass 2 walks the CTA's tiles backwards so that the tiles read
 // last are re-read first from L2. When the caller supplies the rows' log-sum-exp (lse_obs), pass 1 is skipped; the keys
 // of a unit are then independent, and a uniform batch is cut into equal shares of tiles, one per CTA (32 layers x 8111
 // tokens: 256 units on 148 CTAs are 2 rounds of whole units but 1.73 rounds of shares; 118 -> 105 us with the rest).
@@ -45,6 +45,7 @@
 // and MMA warps stop issuing work, the copies and MMAs in flight are drained, and the other warps leave their loops
 // without storing. The only unbounded waits are hardware barriers that every thread reaches on every path.
 #include <cuda.h>
+#include <string.h>
 
 #include <type_traits>
 
@@ -123,10 +124,11 @@ struct alignas(1024) ScoreSmem {
   static constexpr int kRowsPad = MB * 128;
   uint8_t q[kQBufs][MB * 2 * kHalfBytes];  // [buffer][half][MB*128 rows][128 B]
   uint8_t k[kStages][kKTileBytes];         // [stage][half][128 rows][128 B]
-  float part_m[2][kGroups][kRowsPad];      // [unit parity][softmax group][row]: reference and sum of the group's keys
-  float part_z[2][kGroups][kRowsPad];
-  float mine_m[2][kRowsPad];               // [unit parity][row]: this CTA's row statistics, read by its peers
-  float mine_z[2][kRowsPad];
+  // [softmax group][row]: reference and sum of the group's keys (one unit's at a time: a softmax warp waits for the row
+  // constants that are formed from them before it goes on to the next unit)
+  float part_m[kGroups][kRowsPad], part_z[kGroups][kRowsPad];
+  static constexpr int kPeers = MB == 1 ? kMaxCluster : 8;  // largest cluster the exchange has room for
+  float2 peer[kPeers][kRowsPad];           // row statistics (reference, sum) as the CTAs of the cluster sent them
   float tab[2][kRowsPad];                  // [unit parity][row] pass-2 constant of the row
   float wrow[kRowsPad];                    // pension weight per row
   float lv[kRowsPad];                      // log2 of the row's output weight (kOutFused), else 0
@@ -135,7 +137,7 @@ struct alignas(1024) ScoreSmem {
   UnitInfo unit[kUnitRing];
   unsigned long long full[kStages], empty[kStages], acc_full[kAcc], acc_empty[kAcc];
   unsigned long long q_full[kQBufs], q_empty[kQBufs], ufull[kUnitRing], ufree[kUnitRing];
-  unsigned long long stat_full[2], tab_full[2], tab_free[2], xchg_full[2], drain;
+  unsigned long long stat_full[2], tab_full[2], tab_free[2], xchg_full, xchg_free, drain;
   unsigned long long pfull[kRing], pfree[kRing];
   uint32_t tmem_base;
   int abort_flag;
@@ -230,6 +232,7 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
   // order the rounds are taken in alternating direction (the cluster that got the longest unit of one round gets the
   // shortest of the next), which evens out the clusters' totals. False: there is nothing to do in this round (ui.end: nor in
   // any later one).
+  // (Runs ahead of everything else in the CTA: 32-bit arithmetic, a 64-bit division costs some 0.2 us.)
   auto get_unit = [&](int round, UnitInfo& ui) {
     ui = UnitInfo{};
     int u, t_lo = 0, t_hi = 0;
@@ -248,15 +251,12 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
     }
     if (ui.end || u >= p.units) return false;
     if (p.order) u = p.order[u];
-    ui.g = u % p.Hkv;
-    if (p.by_length) {  // every sequence's units together: rank, then layer, then head
-      const int per = p.n_layers * p.Hkv;
-      ui.b = sm.by_rank[u / per];
-      ui.l = (u % per) / p.Hkv;
-    } else {
-      ui.b = (u / p.Hkv) % p.seq.batch;
-      ui.l = u / (p.Hkv * p.seq.batch);
-    }
+    // by_length: every sequence's units together (rank, then layer, then head); otherwise layer, sequence, head
+    const uint32_t heads = (uint32_t)u / (uint32_t)p.Hkv, inner = (uint32_t)(p.by_length ? p.n_layers : p.seq.batch);
+    const int major = (int)(heads / inner), minor = (int)(heads - (uint32_t)major * inner);
+    ui.g = (int)((uint32_t)u - heads * (uint32_t)p.Hkv);
+    ui.b = p.by_length ? sm.by_rank[major] : minor;
+    ui.l = p.by_length ? minor : major;
     ui.tok0 = ta_seq_begin(p.seq, ui.b);
     ui.n = (p.seq.cu ? p.seq.cu[ui.b + 1] : ui.tok0 + p.seq.n_uniform) - ui.tok0;
     // a sequence that does not lie inside the token arrays is skipped here and rejected by the selection step
@@ -269,62 +269,44 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
       return false;
     }
     const int tiles_total = (ui.n + kTileN - 1) / kTileN;
-    ui.t_begin = p.flat ? t_lo : (int)((long long)tiles_total * rank / p.cluster);
-    ui.T = (p.flat ? t_hi : (int)((long long)tiles_total * (rank + 1) / p.cluster)) - ui.t_begin;
+    const uint32_t cl = (uint32_t)p.cluster;  // (at most 16, and at most 2^13 tiles)
+    ui.t_begin = p.flat ? t_lo : (int)((uint32_t)tiles_total * rank / cl);
+    ui.T = (p.flat ? t_hi : (int)((uint32_t)tiles_total * (rank + 1) / cl)) - ui.t_begin;
     // a CTA without tiles still takes part in its cluster's exchange of statistics
     return ui.T > 0 || (ui.n > 0 && p.two_pass && p.cluster > 1);
   };
 
-  // ---- set-up (once per CTA)
-  if (tid == 0) {
-    for (int s = 0; s < kStages; ++s) {
-      mbar_init(smem_u32(&sm.full[s]), 1);
-      mbar_init(smem_u32(&sm.empty[s]), 1);
-    }
-    for (int a = 0; a < kAcc; ++a) {
-      mbar_init(smem_u32(&sm.acc_full[a]), 1);
-      mbar_init(smem_u32(&sm.acc_empty[a]), 4);
-    }
-    for (int i = 0; i < 2; ++i) {
-      mbar_init(smem_u32(&sm.stat_full[i]), kSoftWarps);
-      mbar_init(smem_u32(&sm.tab_full[i]), kStatWarps);
-      mbar_init(smem_u32(&sm.tab_free[i]), kSoftWarps);
-      mbar_init(smem_u32(&sm.xchg_full[i]), (uint32_t)p.cluster * kStatWarps);
-    }
-    for (int i = 0; i < kQBufs; ++i) {
-      mbar_init(smem_u32(&sm.q_full[i]), 1);
-      mbar_init(smem_u32(&sm.q_empty[i]), 1);
-    }
-    for (int r = 0; r < kUnitRing; ++r) {
-      mbar_init(smem_u32(&sm.ufull[r]), 1);
-      mbar_init(smem_u32(&sm.ufree[r]), kSoftWarps + 1 + kStatWarps);  // softmax warps, MMA issuer, statistics warps
-    }
-    for (int r = 0; r < kRing; ++r) {
-      mbar_init(smem_u32(&sm.pfull[r]), 4);
-      mbar_init(smem_u32(&sm.pfree[r]), 4);
-    }
-    mbar_init(smem_u32(&sm.drain), 1);
-    // a wait that ran out in an earlier CTA or call (not yet polled) makes the remaining CTAs skip their waits
-    sm.abort_flag = (*reinterpret_cast<volatile int*>(&p.status->code) == (int)TA_ERR_TIMEOUT) ? 1 : 0;
+  // ---- set-up (once per CTA); a lane per barrier
+  if (warp == 0) {
+    auto init = [&](unsigned long long* bar, int n, uint32_t count) {
+      if (lane < n) mbar_init(smem_u32(bar + lane), count);
+    };
+    init(sm.full, kStages, 1);
+    init(sm.empty, kStages, 1);
+    init(sm.acc_full, kAcc, 1);
+    init(sm.acc_empty, kAcc, 4);
+    init(sm.stat_full, 2, kSoftWarps);
+    init(sm.tab_full, 2, kStatWarps);
+    init(sm.tab_free, 2, kSoftWarps);
+    init(&sm.xchg_full, 1, (uint32_t)p.cluster * kStatWarps);
+    init(&sm.xchg_free, 1, (uint32_t)p.cluster * kStatWarps);
+    init(sm.q_full, kQBufs, 1);
+    init(sm.q_empty, kQBufs, 1);
+    init(sm.ufull, kUnitRing, 1);
+    init(sm.ufree, kUnitRing, kSoftWarps + 1 + kStatWarps);  // softmax warps, MMA issuer, statistics warps
+    init(sm.pfull, kRing, 4);
+    init(sm.pfree, kRing, 4);
+    init(&sm.drain, 1, 1);
+    if (lane == 0) sm.abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == kWarpTma && lane == 0) {
+    tma_prefetch_map(&map_q);
+    tma_prefetch_map(&map_k);
   }
   if (warp == kWarpMma) {
     tmem_alloc(smem_u32(&sm.tmem_base), kTmemCols);
     tmem_relinquish();
-  }
-  if (!p.late_wait) ta_wait_for_prior_grid();  // nothing above reads what an earlier kernel wrote, but for the status word
-  if (p.by_length) {
-    // Longest first, equal lengths in sequence order. In unit order the lengths a cluster meets are random and the busiest
-    // cluster of a batch with lengths spread 8x carries about 30 % more than the average.
-    for (int b = tid; b < p.seq.batch; b += kThreads) {
-      const int nb = p.seq.cu[b + 1] - p.seq.cu[b];
-      int rank = 0;
-      for (int o = 0; o < p.seq.batch; ++o) {
-        const int no = p.seq.cu[o + 1] - p.seq.cu[o];
-        rank += (no > nb) || (no == nb && o < b);
-      }
-      sm.by_rank[rank] = (uint16_t)b;
-    }
   }
   // per-row tables: row r = h*W + t
   for (int r = tid; r < kRowsPad; r += kThreads) {
@@ -347,13 +329,27 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
+  if (!p.late_wait) ta_wait_for_prior_grid();  // nothing above reads memory
+  if (p.by_length) {
+    // Longest first, equal lengths in sequence order. In unit order the lengths a cluster meets are random and the busiest
+    // cluster of a batch with lengths spread 8x carries about 30 % more than the average.
+    for (int b = tid; b < p.seq.batch; b += kThreads) {
+      const int nb = p.seq.cu[b + 1] - p.seq.cu[b];
+      int rank = 0;
+      for (int o = 0; o < p.seq.batch; ++o) {
+        const int no = p.seq.cu[o + 1] - p.seq.cu[o];
+        rank += (no > nb) || (no == nb && o < b);
+      }
+      sm.by_rank[rank] = (uint16_t)b;
+    }
+  }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = sm.tmem_base;
-  // every CTA of the cluster must be running (barriers initialised) before any peer writes into its shared memory
+  // Every CTA of the cluster must be running (barriers initialised) before a peer arrives on its barriers or reads its shared
+  // memory: the statistics warps wait for that before their first exchange, the others only when they leave.
   cluster_arrive();
-  cluster_wait();
 
   const uint32_t k_smem = smem_u32(sm.k);
 
@@ -500,7 +496,10 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
       // before the constants are there.
       const int r0 = (warp - kWarpStat) * 32 + lane;
       int us = 0;
-      uint32_t uph = 0;
+      uint32_t uph = 0, xph = 0;
+      cluster_wait();
+      // a wait that ran out in an earlier CTA or call (not yet polled) makes the remaining CTAs give up their waits at once
+      if (*reinterpret_cast<volatile int*>(&p.status->code) == (int)TA_ERR_TIMEOUT) *abort_flag = 1;
       for (int it = 0;; ++it) {
         if (!mbar_wait(smem_u32(&sm.ufull[us]), uph, abort_flag, p.status, 36, limit)) break;
         const UnitInfo ui = sm.unit[us];
@@ -517,19 +516,20 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
           sm.tab[up][r] = poly_pair<MB>((r & 15) / 2) ? poly_bias(beta) : -beta;
         };
         if (p.two_pass) {
+          if (p.cluster > 1) mbar_wait_cluster(smem_u32(&sm.xchg_free), xph ^ 1u, abort_flag, p.status, 31, limit);
 #pragma unroll
           for (int r = r0; r < kRowsPad; r += 32 * kStatWarps) {
-            float m = sm.part_m[up][0][r];
+            float m = sm.part_m[0][r];
 #pragma unroll
-            for (int gq = 1; gq < kGroups; ++gq) m = fmaxf(m, sm.part_m[up][gq][r]);
+            for (int gq = 1; gq < kGroups; ++gq) m = fmaxf(m, sm.part_m[gq][r]);
             float z = 0.0f;
 #pragma unroll
-            for (int gq = 0; gq < kGroups; ++gq) z += sm.part_z[up][gq][r] * ex2(sm.part_m[up][gq][r] - m);
+            for (int gq = 0; gq < kGroups; ++gq) z += sm.part_z[gq][r] * ex2(sm.part_m[gq][r] - m);
             if (p.cluster == 1) {  // nothing to exchange: the CTA's statistics are the unit's
               put(r, z > 0.0f ? m + __log2f(z) : INFINITY);
             } else {
-              sm.mine_m[up][r] = m;
-              sm.mine_z[up][r] = z;
+#pragma unroll 4
+              for (int q = 0; q < p.cluster; ++q) st_cluster_f32x2(smem_u32(&sm.peer[rank][r]), (uint32_t)q, m, z);
             }
           }
           if (p.cluster > 1) {
@@ -537,22 +537,30 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
             // one lane per peer tells that peer that this warp's rows of the CTA's statistics are in place
             if (lane < p.cluster) {
               fence_cluster();
-              mbar_arrive_remote(smem_u32(&sm.xchg_full[up]), (uint32_t)lane);
+              mbar_arrive_remote(smem_u32(&sm.xchg_full), (uint32_t)lane);
             }
-            mbar_wait_cluster(smem_u32(&sm.xchg_full[up]), ph, abort_flag, p.status, 32, limit);
+            mbar_wait_cluster(smem_u32(&sm.xchg_full), xph, abort_flag, p.status, 32, limit);
+            auto merge = [&](auto most) {  // all pairs requested before the first is used
+              constexpr int kMost = decltype(most)::value;
 #pragma unroll 1
-            for (int r = r0; r < kRowsPad; r += 32 * kStatWarps) {
-              float pm[kMaxCluster], m = -1e30f, z = 0.0f;
+              for (int r = r0; r < kRowsPad; r += 32 * kStatWarps) {
+                float2 v[kMost];
+                float m = -1e30f, z = 0.0f;
 #pragma unroll
-              for (int q = 0; q < kMaxCluster; ++q) {
-                pm[q] = q < p.cluster ? ld_cluster_f32(smem_u32(&sm.mine_m[up][r]), (uint32_t)q) : -1e30f;
-                m = fmaxf(m, pm[q]);
+                for (int q = 0; q < kMost; ++q) v[q] = sm.peer[min(q, p.cluster - 1)][r];
+#pragma unroll
+                for (int q = 0; q < kMost; ++q) m = fmaxf(m, v[q].x);
+#pragma unroll
+                for (int q = 0; q < kMost; ++q) z += q < p.cluster ? v[q].y * ex2(v[q].x - m) : 0.0f;
+                put(r, z > 0.0f ? m + __log2f(z) : INFINITY);
               }
-#pragma unroll
-              for (int q = 0; q < kMaxCluster; ++q)
-                if (q < p.cluster) z += ld_cluster_f32(smem_u32(&sm.mine_z[up][r]), (uint32_t)q) * ex2(pm[q] - m);
-              put(r, z > 0.0f ? m + __log2f(z) : INFINITY);
-            }
+            };
+            if (p.cluster <= 4) merge(std::integral_constant<int, 4>{});
+            else if (p.cluster <= 8) merge(std::integral_constant<int, 8>{});
+            else merge(std::integral_constant<int, Smem::kPeers>{});
+            __syncwarp();
+            if (lane < p.cluster) mbar_arrive_remote(smem_u32(&sm.xchg_free), (uint32_t)lane);  // the slots may be written again
+            xph ^= 1u;
           }
         } else {
           for (int r = r0; r < kRowsPad; r += 32 * kStatWarps) {
@@ -762,8 +770,8 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
         // sequence start) stay mute
 #pragma unroll
         for (int h = 0; h < MB; ++h) {
-          sm.part_m[up][grp][h * 128 + row_in_tile] = lim[h] >= 0 ? ref[h] : -1e30f;
-          sm.part_z[up][grp][h * 128 + row_in_tile] = lim[h] >= 0 ? zsum[h] : 0.0f;
+          sm.part_m[grp][h * 128 + row_in_tile] = lim[h] >= 0 ? ref[h] : -1e30f;
+          sm.part_z[grp][h * 128 + row_in_tile] = lim[h] >= 0 ? zsum[h] : 0.0f;
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(smem_u32(&sm.stat_full[up]));
@@ -896,7 +904,8 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
     tc_fence_after();
     tmem_dealloc(tmem_base, kTmemCols);
   }
-  // no CTA may leave while a peer can still store into its shared memory or arrive on its barriers
+  // no CTA may leave while a peer can still read its shared memory or arrive on its barriers
+  if (warp < kWarpStat || warp >= kWarpStat + kStatWarps) cluster_wait();  // the set-up's arrival
   cluster_arrive();
   cluster_wait();
   if (p.late_wait && blockIdx.x == 0) ta_wait_for_prior_grid();  // this grid ends after the one it ran beside
@@ -904,6 +913,7 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
 
 template <int MB>
 size_t score_smem_bytes() {
+  static_assert(sizeof(ScoreSmem<MB>) + 1024 <= 227 * 1024, "shared memory of a block");
   return sizeof(ScoreSmem<MB>) + 1024;
 }
 
@@ -963,7 +973,7 @@ cudaError_t launch_variant(ta_ctx* ctx, const CUtensorMap& mq, const CUtensorMap
   // all units in flight fit in L2 was measured and lost: 16 x 32768 tokens, 8 CTAs per unit 2.02 ms against 1.63 ms.)
   int best_cl = ctx->score_force_cluster;
   long long best_cost = best_cl > 0 ? 0 : -1;
-  for (int cl = 1; cl <= kMaxCluster; cl *= 2) {
+  for (int cl = 1; cl <= ScoreSmem<MB>::kPeers; cl = cl < 8 ? 2 * cl : cl + 1) {
     if (ctx->score_force_cluster > 0 && cl != ctx->score_force_cluster) continue;
     if (cl > 1 && tiles_max < 2 * cl && ctx->score_force_cluster <= 0) break;
     if (cl > 8 && sp.units > max_clusters[8]) break;  // only for a single round of few units
@@ -982,8 +992,9 @@ cudaError_t launch_variant(ta_ctx* ctx, const CUtensorMap& mq, const CUtensorMap
     if (ctx->score_force_cluster > 0) break;
     const int avail = max_clusters[cl];
     const long long rounds = (sp.units + avail - 1) / avail;
-    const long long per_cta = (tiles_max + cl - 1) / cl;
-    const long long cost = rounds * (per_cta + (cl > 1 ? 3 : 1));
+    // a pass takes whole rounds of the softmax groups
+    const long long per_cta = (((tiles_max + cl - 1) / cl) * MB + kGroups - 1) / kGroups * kGroups;
+    const long long cost = rounds * (per_cta + MB * (cl > 1 ? 3 : 1));
     if (sp.flat) {  // equal shares whatever the number of units: nothing to gain from more CTAs per unit
       best_cl = cl;
       best_cost = 0;
@@ -1085,7 +1096,13 @@ cudaError_t ta_launch_score(ta_ctx* ctx, const ta_score_args& a, ta_dev_status* 
   sp.u = a.u;
   sp.status = status;
   sp.wait_limit_ns = ctx->wait_limit_ns ? ctx->wait_limit_ns : kWaitLimitNs;
-  for (int t = 0; t < a.W; ++t) sp.wrow[t] = (float)((1.0 - (double)a.rho) * pow((double)a.rho, (double)(a.W - 1 - t)));
+  if (ctx->wrow_W != a.W || ctx->wrow_rho != a.rho) {  // 32 calls of pow() are a microsecond of host time
+    for (int t = 0; t < a.W; ++t)
+      ctx->wrow[t] = (float)((1.0 - (double)a.rho) * pow((double)a.rho, (double)(a.W - 1 - t)));
+    ctx->wrow_W = a.W;
+    ctx->wrow_rho = a.rho;
+  }
+  memcpy(sp.wrow, ctx->wrow, sizeof(float) * a.W);
   sp.units = units;
   sp.order = nullptr;
   sp.late_wait = a.pdl == 2;
