@@ -66,17 +66,6 @@ struct KeyCache {
   uint32_t elig;  // bit `it`: element tid + it*kThreads exists and is eligible
 };
 
-template <class KeyFn, int ITEMS>
-__device__ __forceinline__ void fill_cache(int n, KeyFn key_of, KeyCache<ITEMS>& kc) {
-  kc.elig = 0;
-#pragma unroll
-  for (int it = 0; it < ITEMS; ++it) {
-    const int i = (int)threadIdx.x + it * kThreads;
-    kc.key[it] = 0;
-    if (i < n && key_of(i, kc.key[it])) kc.elig |= 1u << it;
-  }
-}
-
 // Calls body(i, exists, eligible, key) for every element slot in ascending chunks of kThreads; every thread of the
 // block makes the same number of calls (the body may hold block-wide barriers).
 template <bool CACHED, class KeyFn, class Body, int ITEMS>
@@ -869,7 +858,21 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads) ta_forced_kernel(ta
   };
   KeyCache<ITEMS> kc;
   if constexpr (CACHED) split_unit_begin<CL>(sh);
-  if (CACHED) fill_cache(hi - lo, key_of, kc);
+  if constexpr (CACHED) {  // loads as selects, never under a branch: nothing keeps them from being in flight together
+    float v[ITEMS];
+#pragma unroll
+    for (int it = 0; it < ITEMS; ++it) {
+      const int il = (int)threadIdx.x + it * kThreads;
+      v[it] = il < hi - lo ? V[il] : 0.0f;
+    }
+    kc.elig = 0;
+#pragma unroll
+    for (int it = 0; it < ITEMS; ++it) {
+      const int il = (int)threadIdx.x + it * kThreads;
+      kc.key[it] = sortable_key(v[it]);
+      if (il < hi - lo && v[it] > 0.0f && !mandatory(lo + il)) kc.elig |= 1u << it;
+    }
+  }
   SelectResult r;
   if constexpr (CACHED) r = cached_radix_select<CL>(hi - lo, s.n, s.p, kc, sh);
   else r = block_radix_select<CACHED, CL>(hi - lo, s.p, key_of, kc, sh);
@@ -921,7 +924,7 @@ __device__ __forceinline__ float unit_utility(const UnitSrc& src, long long unit
 // ta_compact_kernel (rows at and beyond the retained count, and rows whose index lies outside the sequence, are zero).
 // Selection is bound by latency and instruction issue, the copy by HBM: with many units the blocks of one kernel are in
 // different phases and the two overlap in part (2048 units of up to 8000 tokens, K = 512: 105 + 175 us as two kernels,
-// 232 us as one; starting half of the blocks half a period late changed nothing); with few, a launch is saved.
+// 210 us as one; starting half of the blocks half a period late changed nothing); with few, a launch is saved.
 struct GatherDst {
   ta_bf16_view k, v;
   uint4* k_out;
@@ -987,8 +990,26 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads) ta_select_kernel(ta
   const int start = ta_seq_begin(seq, b);
   const int n = (seq.cu ? seq.cu[b + 1] : start + seq.n_uniform) - start;
   int32_t* out = idx + (long long)unit * K;
-  const int want = r_main[b];
   const int tid = threadIdx.x;
+  const long long unit_off = fast ? 0 : ((long long)l * Hkv + g) * seq.total;
+  // a sequence that does not lie inside the token arrays (want -2 below) is not read
+  const bool inside = n >= 0 && n <= seq.max_n && start >= 0 && (long long)start + n <= seq.total;
+  int lo, hi;
+  unit_slice<CL>(inside ? n : 0, lo, hi);
+  const int nl = hi - lo;
+  const float* ap = src.u ? src.u : src.A;
+  KeyCache<ITEMS> kc;
+  float uu[CACHED ? ITEMS : 1];  // the attention part: from L2 or HBM, requested first (before it is known to be needed)
+  if constexpr (CACHED) {
+    // loads as selects, never under a branch: nothing then keeps them from being in flight together
+    const float* up = ap + unit_off + start + lo;
+#pragma unroll
+    for (int it = 0; it < ITEMS; ++it) {
+      const int i = tid + it * kThreads;
+      uu[it] = ap && i < nl ? up[i] : 0.0f;
+    }
+  }
+  const int want = r_main[b];
   if (want == -2) {  // sequence rejected by ta_forced_kernel
     if (lead) {
       for (int r = tid; r < K; r += kThreads) out[r] = -1;
@@ -1005,54 +1026,41 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads) ta_select_kernel(ta
     if constexpr (GATHER) gather_unit(gd, seq, unit, l, b, g, n, K, out, n, true, sh);
     return;
   }
-  const long long unit_off = fast ? 0 : ((long long)l * Hkv + g) * seq.total;
-  int lo, hi;
-  unit_slice<CL>(n, lo, hi);
   const uint8_t* f = forced + start + lo;
   auto key_of = [&](int il, uint32_t& key) {
     key = sortable_key(unit_utility(src, unit_off, (long long)start + lo + il));
     return f[il] == 0;
   };
-  KeyCache<ITEMS> kc;
   if constexpr (CACHED) {
     split_unit_begin<CL>(sh);
-    if (src.u) {
-      // the attention part comes from HBM, the per-token arrays mostly from L2: issue all loads of the former first
-      // (they land in the registers that hold the keys afterwards), so one memory latency covers the whole unit
-      const int nl = hi - lo;
-      const float* up = src.u + unit_off + start + lo;
-      const float* sp = src.u_static + start + lo;
-      kc.elig = 0;
-      // loads as selects, never under a branch: nothing then keeps them from being in flight together
-      float uu[ITEMS];
+    const float* sp = src.u_static + start + lo;
+    const float* pp = !src.u && src.A && src.P ? src.P + unit_off + start + lo : nullptr;
+    kc.elig = 0;
+    // the per-token values, mostly from L2, in groups (registers: a group's loads are in flight together, no more)
+    constexpr int kGroup = ITEMS < 8 ? ITEMS : ITEMS > 16 ? 4 : 8;
 #pragma unroll
-      for (int it = 0; it < ITEMS; ++it) {
-        const int i = tid + it * kThreads;
-        uu[it] = i < nl ? up[i] : 0.0f;
+    for (int g0 = 0; g0 < ITEMS; g0 += kGroup) {
+      float us[kGroup], ps[kGroup];
+      uint8_t ff[kGroup];
+#pragma unroll
+      for (int q = 0; q < kGroup; ++q) {
+        const int i = tid + (g0 + q) * kThreads;
+        us[q] = i < nl ? sp[i] : 0.0f;
+        ff[q] = i < nl ? f[i] : (uint8_t)1;
+        ps[q] = pp && i < nl ? pp[i] : 0.0f;
       }
-      // the per-token values in groups of 8 (registers: a group's loads are in flight together, no more)
-      constexpr int kGroup = ITEMS < 8 ? ITEMS : 8;
 #pragma unroll
-      for (int g0 = 0; g0 < ITEMS; g0 += kGroup) {
-        float us[kGroup];
-        uint8_t ff[kGroup];
-#pragma unroll
-        for (int q = 0; q < kGroup; ++q) {
-          const int i = tid + (g0 + q) * kThreads;
-          us[q] = i < nl ? sp[i] : 0.0f;
-          ff[q] = i < nl ? f[i] : (uint8_t)1;
-        }
-#pragma unroll
-        for (int q = 0; q < kGroup; ++q) {
-          const int it = g0 + q;
-          const bool in = tid + it * kThreads < nl;
-          kc.key[it] = in ? sortable_key(__fadd_rn(uu[it], us[q])) : 0u;
-          kc.elig |= (in && ff[q] == 0) ? (1u << it) : 0u;
-        }
-        asm volatile("" ::: "memory");  // keeps the next group's loads behind this group's use
+      for (int q = 0; q < kGroup; ++q) {
+        const int it = g0 + q;
+        const bool in = tid + it * kThreads < nl;
+        // the same roundings as unit_utility()
+        float v = us[q];
+        if (src.u) v = __fadd_rn(uu[it], v);
+        else if (src.A) v = __fadd_rn(__fadd_rn(__fmul_rn(src.alpha, uu[it]), __fmul_rn(src.delta, ps[q])), v);
+        kc.key[it] = in ? sortable_key(v) : 0u;
+        kc.elig |= (in && ff[q] == 0) ? (1u << it) : 0u;
       }
-    } else {
-      fill_cache(hi - lo, key_of, kc);
+      asm volatile("" ::: "memory");  // keeps the next group's loads behind this group's use
     }
   }
   SelectResult r;
