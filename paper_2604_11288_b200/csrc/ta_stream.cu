@@ -14,9 +14,9 @@
 //                           voucher by budget_decay (Algorithm 1 step 10)
 // The second kernel runs beside the first: it reads the unit's state and waits for the first only where the new token comes
 // in. What bounds it: latency at few units, the state's bytes (25 read, 12 to 25 written per cached token, 4 of attention
-// mass read) at many. 4096 units of 257 tokens, three states in turn (180 MB: more than L2): 52 -> 22 us a step,
-// 2.6 TB/s (serial scans by one thread in the pool selection, one lane per sequence for the voucher, all entries through
-// shared memory before).
+// mass read) at many. 4096 units of 257 tokens, three states in turn (180 MB: more than L2): 52 -> 18.4 us a step,
+// 3.1 TB/s (serial scans by one thread in the pool selection, one lane per sequence for the voucher, all entries through
+// shared memory before; then 22 us with two entries in 64 registers, of which an SM held 6 blocks).
 // All arithmetic that decides the selection is fp32 with one rounding per operation, in the order the CPU oracle uses.
 #include "ta_internal.cuh"
 
@@ -133,13 +133,25 @@ __device__ __forceinline__ uint32_t sortable_key(float f) {
   return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
 }
 
+// The largest block per number of entries in a thread, which at two blocks an SM sets the registers: 56 with three
+// entries, 64 with four. The step is bound by how many blocks' loads are in flight, so registers are traded for blocks
+// until values spill in the common path (time of 4096 units in us, entries/registers):
+//   tokens   2/64   2/40   3/77   3/64   3/56   3/48   4/76   4/64   5/64
+//      257   22.0   20.7   21.2   18.3   18.6   20.1   21.8   19.9   21.6
+//      513   44.5   37.6   41.5   38.3   35.7   38.9   44.2   37.2   40.8
+//     1001   71.6   65.5   80.8   82.8   68.1   74.2   71.9   62.5   77.0
+//     1501      -      -      -   94.4   97.8  106.8  101.5  106.9  107.2
+//     2041      -      -      -      -      -      -  183.4  123.5  156.1
+constexpr int step_threads(int e) { return e == 3 ? 576 : e == 4 ? 512 : 544; }
+constexpr int step_regs(int e) { return e == 3 ? 56 : 64; }
+
 // One block per unit; thread tid holds the entries tid, tid + nt, .. (E of them) in registers for the whole step.
 // Selection (Section 3.3 on the K+1 cached tokens): mandatory sinks and recents; the protected pool = the sponsored,
 // non-mandatory tokens with the largest vouchers (lower position first among equals); exactly one token is then not
 // forced and loses: the one with the smallest utility, the latest position among equals. When the sponsored tokens fit the
 // protected slots, or are one too many, block-wide minima decide; otherwise a radix select on the voucher keys.
 template <int E>
-__global__ void __launch_bounds__(E == 8 ? 544 : 512)
+__global__ void __launch_bounds__(step_threads(E), E == 8 ? 1 : 2)
 ta_stream_step_kernel(ta_stream_dev st, const ta_stream_seq_info* info, const float* __restrict__ attn,
                       int vocab, float alpha, float beta, float gamma, float delta, float lambda, float rho,
                       float budget_decay, int n_sink, int n_recent, int k_protected, int32_t* __restrict__ evicted_pos,
@@ -156,8 +168,9 @@ ta_stream_step_kernel(ta_stream_dev st, const ta_stream_seq_info* info, const fl
   __shared__ int tie_cnt[E * 17];
   __shared__ int sel_bin, sel_above, sel_pop;
 
-  // ---- the unit's state (from L2: other blocks wrote it) and its attention masses, all requested before the first is used. Launched as a programmatic
-  // dependent of the per-sequence kernel, which lets this one start when everything before it is complete.
+  // ---- the unit's state (from L2: other blocks wrote it) and its attention masses, all requested before the first is used.
+  // Launched as a programmatic dependent of the per-sequence kernel, which lets this one start when everything before it
+  // is complete.
   int pos[E], row[E], id[E], S[E];
   float A[E], P[E], V[E];
 #pragma unroll
@@ -403,12 +416,14 @@ cudaError_t ta_launch_stream_step(const ta_stream_dev& st, const ta_policy& pol,
                                   const float* attn, int32_t* evicted_pos, ta_dev_status* status,
                                   cudaStream_t stream) {
   const int U = st.n_layers * st.B * st.Hkv, C = st.K + 1;
-  // entries per thread: few threads with several entries each keep more loads in flight per block; a block stays at 544
-  // threads up to the largest budget
-  const int items = C <= 1024 ? 2 : C <= 2048 ? 4 : 8;
-  const int threads = ((C + items - 1) / items + 31) / 32 * 32;
+  // entries per thread: three or four, whichever lets an SM hold more blocks (three when equal: fewer spills); eight where
+  // a block would have to be larger than those kernels allow
+  auto block = [&](int e) { return ((C + e - 1) / e + 31) / 32 * 32; };
+  auto resident = [&](int e) { return block(e) <= step_threads(e) ? 65536 / (block(e) * step_regs(e)) : 0; };
+  const int items = resident(3) == 0 && resident(4) == 0 ? 8 : resident(3) >= resident(4) ? 3 : 4;
+  const int threads = block(items);
   const size_t smem = (size_t)C * 4;  // at most 16 KB
-  auto kern = items == 2 ? ta_stream_step_kernel<2> : items == 4 ? ta_stream_step_kernel<4> : ta_stream_step_kernel<8>;
+  auto kern = items == 3 ? ta_stream_step_kernel<3> : items == 4 ? ta_stream_step_kernel<4> : ta_stream_step_kernel<8>;
   // runs beside the kernel before it on the stream (ta_stream_seq_kernel in ta_stream_step)
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)U, 1, 1);

@@ -139,10 +139,11 @@ def test_stream_no_patterns_tiny_budget():
 
 
 @pytest.mark.parametrize("K,preset,steps", [(31, "SEC33", 200), (64, "SEC33", 260), (63, "THEOREM", 260),
-                                            (1025, "SEC33", 1060), (2049, "SEC33", 2070)])
+                                            (254, "SEC33", 280), (255, "SEC33", 280), (1727, "SEC33", 1740),
+                                            (2047, "SEC33", 2060), (2048, "SEC33", 2070)])
 def test_stream_more_sponsored_tokens_than_protected_slots(K, preset, steps):
-    # anchors every few tokens: most cached tokens are sponsored, many with equal vouchers; two, four and eight cached
-    # tokens per thread
+    # anchors every few tokens: most cached tokens are sponsored, many with equal vouchers; three, four and eight cached
+    # tokens per thread at the edges of their ranges
     pats = oracle.Patterns([[5], [6, 7]], budget=[15.0, 2.0], span=[3, 8])
     pol = oracle.preset(preset, K, vocab_size=64, budget_decay=1.0 if K < 64 else 0.9)
     _run(K=K, L=1, B=1, Hkv=2 if K < 100 else 1, steps=steps, pats=pats, pol=pol, seed=K, check_every=97)
