@@ -13,7 +13,7 @@
 //   e  fast mode: main pool by utility and the ordered write
 // What bounds it: latency (a few barriers, one trip to memory). The same results took a memset and three to five kernels
 // (ta_mask.cu, ta_select.cu: still the path for longer sequences, where one block per sequence would be too few), each
-// with its own launch, trip to memory and tail: one sequence of 4096 tokens 25 -> 10 us, fast mode 37 -> 16 us.
+// with its own launch, trip to memory and tail: one sequence of 4096 tokens 25 -> 10 us, fast mode 37 -> 14 us.
 #include <cooperative_groups.h>
 
 #include <atomic>
@@ -34,7 +34,7 @@ using namespace front1024;
 
 constexpr int kPad = TA_MAX_PATTERN_LEN;  // ids before the sequence (never part of a match)
 constexpr int kMaxItems = 16;             // tokens per thread
-constexpr int kMaxDynamicSmem = 190 * 1024;  // beside about 32 KB of static shared memory (a block may use 227 KB)
+constexpr int kMaxDynamicSmem = 187 * 1024;  // beside 40 KB of static shared memory (a block may use 227 KB)
 
 struct FrontParams {
   ta_seq_desc seq;

@@ -401,6 +401,19 @@ def test_select_three_distinct_utilities_keep_every_pass_crowded(lengths, L):
     _select_case(w, oracle_policy(K, "THEOREM", beta=0.0, gamma=0.0, lam=0.0), K, L, (A, P))
 
 
+@pytest.mark.parametrize("m", [31, 32, 33, 129, 256, 257])
+def test_select_threshold_among_m_close_neighbours(m):
+    # m consecutive tokens whose utilities share all but their last bits, with equal ones among them, and the threshold in
+    # their middle: the search ends by comparing them with one another, and what is taken is a dense run of positions
+    w = _workload([4000, 2 * m], [[5, 6, 7], [9]], seed=m, Hq=4, Hkv=2)
+    gen = torch.Generator().manual_seed(m)
+    A = torch.rand((1, w.Hkv, w.total), generator=gen) / 2
+    A[:, :, 100:140] += 2.0
+    A[:, :, 1000:1000 + m] = 1.0 + (torch.arange(m) * 7 % 11) * 2.0**-22
+    P = torch.zeros_like(A).cuda()
+    _select_case(w, oracle_policy(45 + m // 2, "THEOREM", beta=0.0, gamma=0.0, lam=0.0), 45 + m // 2, 1, (A.cuda(), P))
+
+
 def test_select_sponsored_overflow_and_precedence():
     # far more sponsored tokens than protected slots: nearest-to-anchor first, earlier anchors win ties
     w = _workload([5000], [[1]], [12], alphabet=40, seed=4)
