@@ -166,8 +166,8 @@ ta_status ta_ctx_selftest_wait(ta_ctx* ctx, uint64_t limit_ns, int32_t* outcome,
 ta_status ta_ctx_set_score_cluster(ta_ctx* ctx, int ctas_per_unit);
 
 /* What the most recent ta_compress (or variant) call on this context launched: out[0] = CTAs per unit of the score
- * kernel, out[1] = its clusters, out[2] = 1 when the selection kernel gathered the retained rows itself (small
- * budgets; no separate gather kernel), out[3] = kernels of this library the call enqueued. */
+ * kernel, out[1] = its clusters, out[2] = 1 when the selection kernel gathered the retained rows itself (no
+ * separate gather kernel), out[3] = kernels of this library the call enqueued. */
 ta_status ta_ctx_last_launch_info(const ta_ctx* ctx, int32_t out[4] /*HOST*/);
 
 /* Every entry point that enqueues work opens an NVTX range of its own name around its host side (visible in timeline
