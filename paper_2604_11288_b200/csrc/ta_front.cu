@@ -13,7 +13,7 @@
 //   e  fast mode: main pool by utility and the ordered write
 // What bounds it: latency (a few barriers, one trip to memory). The same results took a memset and three to five kernels
 // (ta_mask.cu, ta_select.cu: still the path for longer sequences, where one block per sequence would be too few), each
-// with its own launch, trip to memory and tail: one sequence of 4096 tokens 25 -> 10 us, fast mode 37 -> 14 us.
+// with its own launch, trip to memory and tail: one sequence of 4096 tokens 25 -> 9 us, fast mode 37 -> 13 us.
 #include <cooperative_groups.h>
 
 #include <atomic>
@@ -173,6 +173,7 @@ __global__ void __launch_bounds__(kThreads, 1) ta_front_kernel(const __grid_cons
     const int i = tid + it * kThreads;
     const int x = s_id[i];
     int best = -1;
+    bool may_end = false;
     if (i < n) {
       if (x >= 0 && x < p.vocab) {
         if (SMEM_HIST) atomicAdd(&s_hist[x >> 1], (x & 1) ? 0x10000u : 1u);
@@ -183,24 +184,28 @@ __global__ void __launch_bounds__(kThreads, 1) ta_front_kernel(const __grid_cons
         p.status->detail1 = x;
       }
       const uint32_t h = ((uint32_t)x * 2654435761u) >> 22;
-      if (x >= 0 && ((s_bloom[h >> 5] >> (h & 31)) & 1u)) {
-        int best_len = 0;
-        const int avail = min(TA_MAX_PATTERN_LEN, i + 1);  // matches never cross the start of the sequence
+      may_end = x >= 0 && ((s_bloom[h >> 5] >> (h & 31)) & 1u);
+    }
+    // a position behind the filter is matched by its whole warp, a lane per pattern (one lane with all patterns in turn held
+    // the block up: 3.8 K cycles for this phase at 4096 tokens and 8 patterns)
 #pragma unroll 1
-        for (int q = 0; q < p.n_pat; ++q) {
-          const int len = s_plen[q];
-          if (len <= best_len || len > avail) continue;
-          const int32_t* pid = &s_pid[q * TA_MAX_PATTERN_LEN];
-          if (pid[len - 1] != x) continue;
-          bool ok = true;
+    for (unsigned left = __ballot_sync(0xffffffffu, may_end); left != 0u; left &= left - 1u) {
+      const int src = __ffs((int)left) - 1, end = i - lane + src;
+      const int y = __shfl_sync(0xffffffffu, x, src);
+      const int avail = min(TA_MAX_PATTERN_LEN, end + 1);  // matches never cross the start of the sequence
+      uint32_t mine = 0;                                   // length, then the complement of the index: the largest wins
 #pragma unroll 1
-          for (int k = 0; k < len - 1; ++k) ok = ok && s_id[i - len + 1 + k] == pid[k];
-          if (ok) {
-            best = q;
-            best_len = len;
-          }
-        }
+      for (int q = lane; q < p.n_pat; q += 32) {
+        const int len = s_plen[q];
+        const int32_t* pid = &s_pid[q * TA_MAX_PATTERN_LEN];
+        if (len > avail || pid[len - 1] != y) continue;
+        bool ok = true;
+#pragma unroll 1
+        for (int k = 0; k < len - 1; ++k) ok = ok && s_id[end - len + 1 + k] == pid[k];
+        if (ok) mine = max(mine, ((uint32_t)len << 16) | (uint32_t)(0xffff - q));
       }
+      mine = __reduce_max_sync(0xffffffffu, mine);
+      if (lane == src && mine != 0u) best = 0xffff - (int)(mine & 0xffffu);
     }
     const unsigned word = __ballot_sync(0xffffffffu, best >= 0);
     if (word) s_apat[i] = (int16_t)best;  // read only where a bit of `word` is set
