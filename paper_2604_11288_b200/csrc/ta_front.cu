@@ -34,6 +34,7 @@ using namespace front1024;
 
 constexpr int kPad = TA_MAX_PATTERN_LEN;  // ids before the sequence (never part of a match)
 constexpr int kMaxItems = 16;             // tokens per thread
+constexpr int kListCap = 256;             // so few sponsored tokens are ranked by comparing them with one another
 constexpr int kMaxDynamicSmem = 187 * 1024;  // beside 40 KB of static shared memory (a block may use 227 KB)
 
 struct FrontParams {
@@ -84,7 +85,7 @@ __global__ void __launch_bounds__(kThreads, 1) ta_front_kernel(const __grid_cons
   __shared__ float s_w[TA_MAX_SPAN + 1];
   __shared__ uint32_t s_fbits[kMaxItems * kWarps];  // bit of every token: forced
   __shared__ int s_count;
-  __shared__ __align__(8) uint2 s_list[kCompareCap];  // key and position of sponsored, not mandatory tokens
+  __shared__ __align__(8) uint2 s_list[kListCap];  // key and position of sponsored, not mandatory tokens
   __shared__ int s_listed;                            // how many there are (also beyond the capacity of the list)
   const FrontSmem L = front_smem(ITEMS, p.vocab, SMEM_HIST);
   int32_t* s_id = reinterpret_cast<int32_t*>(dyn + L.ids) + kPad;       // s_id[-kPad .. n)
@@ -263,7 +264,7 @@ __global__ void __launch_bounds__(kThreads, 1) ta_front_kernel(const __grid_cons
       else p.u_static[(long long)s.start + i] = u;
       if (V > 0.0f && !mandatory(i)) {
         const int slot = atomicAdd(&s_listed, 1);
-        if (slot < kCompareCap) s_list[slot] = make_uint2(sortable_key(V), (uint32_t)i);
+        if (slot < kListCap) s_list[slot] = make_uint2(sortable_key(V), (uint32_t)i);
       }
     }
   }
@@ -283,7 +284,7 @@ __global__ void __launch_bounds__(kThreads, 1) ta_front_kernel(const __grid_cons
   KeyCache<ITEMS> kc;
   const int m = s_listed;
   int taken = s.s_take + s.r_take;
-  if (m <= kCompareCap) {
+  if (m <= kListCap) {
     if (tid < m) {
       const uint2 mine = s_list[tid];
       int before = 0;  // listed tokens that come first

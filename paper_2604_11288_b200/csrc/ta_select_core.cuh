@@ -24,7 +24,7 @@ struct SelectResult {
 };
 
 constexpr int kCandCap = 2048;  // candidates a split unit finishes locally
-constexpr int kCompareCap = 256;  // so few candidates are compared with one another instead of counted by digits
+constexpr int kCompareCap = 32;  // so few candidates are compared with one another instead of counted by digits
 
 struct SelectShared {
   uint32_t hist[256];
@@ -299,74 +299,38 @@ __device__ __forceinline__ void list_radix_finish(int m, int bits, int done, uin
   }
 }
 
-// The `remaining`-th largest of the m <= kCompareCap keys in sh.cand_keys, by comparing every key with every other: two to
-// four block barriers in place of three for every digit still to resolve (an 8-bit digit leaves about n / 256 candidates, and
-// two more digits would follow). Returns the key; above / equal: how many keys are larger than it / equal to it. Every warp
-// of the block compares a share of the list with 32 of the keys, the counts are added in shared memory (129 keys among 4096,
-// one thread per key against the whole list: 3.3 K cycles, half of the search). What bounds it are
-// the integer compares (half rate), so only the larger keys are counted: the key looked for is the one with the most keys
-// above it among those with fewer than `remaining`, and equal keys have equal counts.
+// The `remaining`-th largest of the m <= kCompareCap keys in sh.cand_keys, by comparing every key with every other: two block
+// barriers in place of three for every digit still to resolve. Returns the key; above / equal: how many keys are larger than
+// it / equal to it. One warp, a key per lane: beyond 32 keys another digit is cheaper, integer compares run at half rate (256
+// keys among 4096: 3.6 K cycles shared out over 32 warps, 1.7 K for a digit and the comparison of what it leaves).
 // compare_begin() runs before the barrier that publishes the keys.
 __device__ __forceinline__ void compare_begin(int m, SelectShared& sh) {
   const int tid = threadIdx.x;
-  if (tid < kCompareCap) {
-    sh.hist[tid] = 0u;
-    if (tid >= m && tid < (m + 3) / 4 * 4) sh.cand_keys[tid] = 0u;  // above no key
-  }
-  if (tid == 0) {
-    sh.cmp_above = 0;
-    sh.cmp_equal = 0;
-  }
+  if (tid >= m && tid < (m + 3) / 4 * 4) sh.cand_keys[tid] = 0u;  // above no key
 }
 __device__ __forceinline__ uint32_t compare_finish(int m, int remaining, int& above, int& equal, SelectShared& sh) {
-  const int tid = threadIdx.x, warp = tid >> 5;
-  const uint4* keys = reinterpret_cast<const uint4*>(sh.cand_keys);
-  if (m <= 32) {  // one warp, a key per lane
-    if (warp == 0) {
-      const uint32_t mine = tid < m ? sh.cand_keys[tid] : 0u;
-      int gt = 0;
+  const int tid = threadIdx.x;
+  static_assert(kCompareCap == 32, "a key per lane");
+  if (tid < 32) {
+    const uint32_t mine = tid < m ? sh.cand_keys[tid] : 0u;
+    const uint4* keys = reinterpret_cast<const uint4*>(sh.cand_keys);
+    int gt = 0;
 #pragma unroll 2
-      for (int j = 0; j < (m + 3) / 4; ++j) {
-        const uint4 k = keys[j];
-        gt += (k.x > mine) + (k.y > mine) + (k.z > mine) + (k.w > mine);
-      }
-      const int best = __reduce_max_sync(0xffffffffu, tid < m && gt < remaining ? gt : -1);
-      const unsigned same = __ballot_sync(0xffffffffu, tid < m && gt == best);
-      if (tid == __ffs((int)same) - 1) {
-        sh.cmp_thresh = mine;
-        sh.cmp_above = best;
-        sh.cmp_equal = __popc(same);
-      }
-    }
-    __syncthreads();
-    above = sh.cmp_above;
-    equal = sh.cmp_equal;
-    return sh.cmp_thresh;
-  }
-  const int columns = (m + 31) / 32, shares = kWarps / columns;  // columns <= kCompareCap / 32 <= kWarps
-  static_assert(kCompareCap / 32 <= kWarps, "at least one share of the list");
-  const int share = warp / columns, c = tid - share * columns * 32;
-  if (share < shares && c < m) {
-    const uint32_t mine = sh.cand_keys[c];
-    uint32_t gt = 0;
-    const int quads = (m + 3) / 4, per = (quads + shares - 1) / shares, end = min(quads, (share + 1) * per);
-#pragma unroll 1
-    for (int j = share * per; j < end; ++j) {
+    for (int j = 0; j < (m + 3) / 4; ++j) {
       const uint4 k = keys[j];
       gt += (k.x > mine) + (k.y > mine) + (k.z > mine) + (k.w > mine);
     }
-    if (gt != 0u) atomicAdd(&sh.hist[c], gt);
+    // the key with the most keys above it among those with fewer than `remaining`; equal keys have equal counts
+    const int best = __reduce_max_sync(0xffffffffu, tid < m && gt < remaining ? gt : -1);
+    const unsigned same = __ballot_sync(0xffffffffu, tid < m && gt == best);
+    if (tid == __ffs((int)same) - 1) {
+      sh.cmp_thresh = mine;
+      sh.cmp_above = best;
+      sh.cmp_equal = __popc(same);
+    }
   }
-  __syncthreads();
-  const int gt = tid < m ? (int)sh.hist[tid] : 0;
-  if (tid < m && gt < remaining) atomicMax(&sh.cmp_above, gt);
   __syncthreads();
   above = sh.cmp_above;
-  if (tid < m && gt == above) {
-    sh.cmp_thresh = sh.cand_keys[tid];  // every thread that holds the key writes the same
-    atomicAdd(&sh.cmp_equal, 1);
-  }
-  __syncthreads();
   equal = sh.cmp_equal;
   return sh.cmp_thresh;
 }
