@@ -142,8 +142,30 @@ __device__ __forceinline__ uint32_t sortable_key(float f) {
 //     1001   71.6   65.5   80.8   82.8   68.1   74.2   71.9   62.5   77.0
 //     1501      -      -      -   94.4   97.8  106.8  101.5  106.9  107.2
 //     2041      -      -      -      -      -      -  183.4  123.5  156.1
-constexpr int step_threads(int e) { return e == 3 ? 576 : e == 4 ? 512 : 544; }
+__host__ __device__ constexpr int step_threads(int e) { return e == 3 ? 576 : e == 4 ? 512 : 544; }
 constexpr int step_regs(int e) { return e == 3 ? 56 : 64; }
+// warps of the largest block: what the shared arrays are sized for
+__host__ __device__ constexpr int step_warps(int e) { return step_threads(e) / 32; }
+
+// Entries per thread for units of C cached tokens: three or four, whichever lets an SM hold more blocks (three when equal:
+// fewer spills); eight where a block would have to be larger than those kernels allow.
+constexpr int step_block(int C, int e) { return ((C + e - 1) / e + 31) / 32 * 32; }
+constexpr int step_resident(int C, int e) {
+  return step_block(C, e) <= step_threads(e) ? 65536 / (step_block(C, e) * step_regs(e)) : 0;
+}
+constexpr int step_items(int C) {
+  const int r3 = step_resident(C, 3), r4 = step_resident(C, 4);
+  return r3 == 0 && r4 == 0 ? 8 : r3 >= r4 ? 3 : 4;
+}
+// every block that the rule can choose holds its unit and is no larger than its kernel's arrays and launch bounds
+constexpr bool step_shapes_fit() {
+  for (int C = 2; C <= TA_MAX_BUDGET + 1; ++C) {
+    const int e = step_items(C), nt = step_block(C, e);
+    if (nt * e < C || nt > step_threads(e) || nt / 32 > step_warps(e) || nt > 1024) return false;
+  }
+  return true;
+}
+static_assert(step_shapes_fit(), "a budget for which the step's block does not fit its kernel");
 
 // One block per unit; thread tid holds the entries tid, tid + nt, .. (E of them) in registers for the whole step.
 // Selection (Section 3.3 on the K+1 cached tokens): mandatory sinks and recents; the protected pool = the sponsored,
@@ -165,7 +187,7 @@ ta_stream_step_kernel(ta_stream_dev st, const ta_stream_seq_info* info, const fl
   __shared__ unsigned long long wfree[32], wmin[32];
   __shared__ int wcand[32];
   __shared__ uint32_t hist[256];
-  __shared__ int tie_cnt[E * 17];
+  __shared__ int tie_cnt[E * step_warps(E)];  // [entry][warp]
   __shared__ int sel_bin, sel_above, sel_pop;
 
   // ---- the unit's state (from L2: other blocks wrote it) and its attention masses, all requested before the first is used.
@@ -416,12 +438,7 @@ cudaError_t ta_launch_stream_step(const ta_stream_dev& st, const ta_policy& pol,
                                   const float* attn, int32_t* evicted_pos, ta_dev_status* status,
                                   cudaStream_t stream) {
   const int U = st.n_layers * st.B * st.Hkv, C = st.K + 1;
-  // entries per thread: three or four, whichever lets an SM hold more blocks (three when equal: fewer spills); eight where
-  // a block would have to be larger than those kernels allow
-  auto block = [&](int e) { return ((C + e - 1) / e + 31) / 32 * 32; };
-  auto resident = [&](int e) { return block(e) <= step_threads(e) ? 65536 / (block(e) * step_regs(e)) : 0; };
-  const int items = resident(3) == 0 && resident(4) == 0 ? 8 : resident(3) >= resident(4) ? 3 : 4;
-  const int threads = block(items);
+  const int items = step_items(C), threads = step_block(C, items);
   const size_t smem = (size_t)C * 4;  // at most 16 KB
   auto kern = items == 3 ? ta_stream_step_kernel<3> : items == 4 ? ta_stream_step_kernel<4> : ta_stream_step_kernel<8>;
   // runs beside the kernel before it on the stream (ta_stream_seq_kernel in ta_stream_step)

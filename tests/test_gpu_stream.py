@@ -115,6 +115,7 @@ def _run(K, L, B, Hkv, steps, pats, pol, seed, check_every=1):
                             np.testing.assert_array_equal(S["tok"][u, :n],
                                                           np.array([ora[b].ids[p] for p in un.pos], np.int32))
         assert ta.ta_ctx_poll(g.ctx) == ta.TA_OK
+        return ora
     finally:
         g.close()
 
@@ -147,3 +148,16 @@ def test_stream_more_sponsored_tokens_than_protected_slots(K, preset, steps):
     pats = oracle.Patterns([[5], [6, 7]], budget=[15.0, 2.0], span=[3, 8])
     pol = oracle.preset(preset, K, vocab_size=64, budget_decay=1.0 if K < 64 else 0.9)
     _run(K=K, L=1, B=1, Hkv=2 if K < 100 else 1, steps=steps, pats=pats, pol=pol, seed=K, check_every=97)
+
+
+@pytest.mark.parametrize("K", [1632, 1700, 1727])
+def test_stream_equal_vouchers_at_the_threshold_in_the_largest_block(K):
+    # vouchers that never decay: a few distinct values shared by hundreds of tokens, so that the last protected slots go to
+    # the earliest of equal ones; K + 1 entries in the largest blocks of the three-entry kernel (18 warps)
+    pats = oracle.Patterns([[5], [6, 7]], budget=[15.0, 2.0], span=[3, 8])
+    pol = oracle.preset("SEC33", K, vocab_size=64, budget_decay=1.0)
+    ora = _run(K=K, L=1, B=1, Hkv=1, steps=K + 12, pats=pats, pol=pol, seed=K, check_every=97)
+    V = np.array(ora[0].units[0].V, np.float32)[pol.n_sink:K - pol.n_recent]
+    V = np.sort(V[V > 0])[::-1]
+    p = pol.k_protected
+    assert V.size > p + 1 and V[p - 1] == V[p], "the threshold must fall between equal vouchers"
