@@ -540,18 +540,24 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
               mbar_arrive_remote(smem_u32(&sm.xchg_full), (uint32_t)lane);
             }
             mbar_wait_cluster(smem_u32(&sm.xchg_full), xph, abort_flag, p.status, 32, limit);
-            auto merge = [&](auto most) {  // all pairs requested before the first is used
+            // The first slots of all rows, however many CTAs the cluster has: addresses that differ by constants, two sweeps
+            // over shared memory. (One sweep that holds 16 pairs, and an address per slot, does not fit the 56 registers
+            // these warps have left: 132 bytes spilled per thread.)
+            auto merge = [&](auto most) {
               constexpr int kMost = decltype(most)::value;
 #pragma unroll 1
               for (int r = r0; r < kRowsPad; r += 32 * kStatWarps) {
-                float2 v[kMost];
                 float m = -1e30f, z = 0.0f;
 #pragma unroll
-                for (int q = 0; q < kMost; ++q) v[q] = sm.peer[min(q, p.cluster - 1)][r];
+                for (int q = 0; q < kMost; ++q) {
+                  const float x = sm.peer[q][r].x;
+                  m = q < p.cluster ? fmaxf(m, x) : m;
+                }
 #pragma unroll
-                for (int q = 0; q < kMost; ++q) m = fmaxf(m, v[q].x);
-#pragma unroll
-                for (int q = 0; q < kMost; ++q) z += q < p.cluster ? v[q].y * ex2(v[q].x - m) : 0.0f;
+                for (int q = 0; q < kMost; ++q) {
+                  const float2 v = sm.peer[q][r];
+                  z += q < p.cluster ? v.y * ex2(v.x - m) : 0.0f;
+                }
                 put(r, z > 0.0f ? m + __log2f(z) : INFINITY);
               }
             };

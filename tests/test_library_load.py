@@ -3,6 +3,7 @@ include/ta.h declares, and its pure-host helpers behave. No kernel is launched h
 import ctypes as C
 import os
 import re
+import subprocess
 
 import pytest
 
@@ -73,3 +74,16 @@ def test_missing_library_fails_loudly(monkeypatch, tmp_path):
     monkeypatch.setattr(ta.binding, "LIB_PATH", str(tmp_path / "libta.so"))
     with pytest.raises(FileNotFoundError):
         ta.binding.lib()
+
+
+def test_score_kernel_keeps_its_values_in_registers(tmp_path):
+    # setmaxnreg leaves the statistics warps 56 registers; what does not fit goes to local memory on the path between the
+    # two passes. A spilled scalar or two outside the loops is tolerated, an array is not.
+    csrc = os.path.join(ROOT, "paper_2604_11288_b200", "csrc")
+    out = subprocess.run([os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc"), "-gencode", "arch=compute_100a,code=sm_100a",
+                          "-O3", "-lineinfo", "-std=c++17", "-I", os.path.join(ROOT, "include"), "-I", csrc, "-Xptxas", "-v",
+                          "-c", os.path.join(csrc, "ta_score.cu"), "-o", str(tmp_path / "score.o")],
+                         check=True, capture_output=True, text=True).stderr
+    spills = dict(re.findall(r"Compiling entry function '(\S*ta_score_kernel\S*)'.*?(\d+) bytes spill stores", out, re.S))
+    assert len(spills) == 6
+    assert max(int(n) for n in spills.values()) <= 8, spills
