@@ -72,12 +72,24 @@ constexpr int kRegsOther = 56;
 constexpr int kRegsNeeded = (kSoftWarps * kRegsSoftmax + 4 * kRegsOther) * 32;
 
 // Of every 16 exponentials, this many (an even number: they are taken in pairs) run on the FMA pipe with 129 to 256 score
-// rows. Back to back the kernel runs into the board's 1000 W limit, and a polynomial costs more energy than ex2 while it
-// relieves the special-function unit: 8 layers of 16 x 32768 tokens with 256 rows 0: 6.22 ms, 2: 6.02 ms, more: the same.
+// rows, in tiles that are not masked. Back to back the kernel runs into the board's 1000 W limit, and a polynomial costs more
+// energy than ex2 while it relieves the special-function unit: 8 layers of 16 x 32768 tokens with 256 rows 0: 6.22 ms,
+// 2: 6.02 ms, more: the same.
 // With up to 128 rows no share pays (one pass over 32 x 8111 tokens: 0: 122 us, 4: 125 us) and none is taken.
 #ifndef TA_SCORE_POLY_MB2
 #define TA_SCORE_POLY_MB2 2
 #endif
+
+// Of the eight pairs of a 16-element group, this many run on the FMA pipe; pair q2 (elements 2*q2, 2*q2 + 1) does when
+// poly_pair is true (spread evenly).
+template <int MB>
+__host__ __device__ constexpr int poly_pairs() {
+  return MB == 1 ? 0 : TA_SCORE_POLY_MB2 / 2;
+}
+template <int MB>
+__host__ __device__ constexpr bool poly_pair(int q2) {
+  return ((q2 * poly_pairs<MB>()) / 8) != (((q2 + 1) * poly_pairs<MB>()) / 8);
+}
 
 // how pass 2 turns the exponentials of a key into outputs
 constexpr int kOutA = 0;      // A only
@@ -129,7 +141,8 @@ struct alignas(1024) ScoreSmem {
   float part_m[kGroups][kRowsPad], part_z[kGroups][kRowsPad];
   static constexpr int kPeers = MB == 1 ? kMaxCluster : 8;  // largest cluster the exchange has room for
   float2 peer[kPeers][kRowsPad];           // row statistics (reference, sum) as the CTAs of the cluster sent them
-  float tab[2][kRowsPad];                  // [unit parity][row] pass-2 constant of the row
+  // [unit parity][row] pass-2 constant of the row; behind them the form that ex2 takes, for rows whose own is the polynomial's
+  float tab[2][poly_pairs<MB>() ? 2 * kRowsPad : kRowsPad];
   float wrow[kRowsPad];                    // pension weight per row
   float lv[kRowsPad];                      // log2 of the row's output weight (kOutFused), else 0
   int row_t[kRowsPad];                     // window index t of the row, -1 for padding rows
@@ -145,12 +158,6 @@ struct alignas(1024) ScoreSmem {
 };
 
 // ---------------------------------------------------------------------------------------------- exponentials
-// Pair q2 (elements 2*q2, 2*q2 + 1) of a 16-element group runs on the FMA pipe when this is true (spread evenly).
-template <int MB>
-__host__ __device__ constexpr bool poly_pair(int q2) {
-  constexpr int kPairs = MB == 1 ? 0 : TA_SCORE_POLY_MB2 / 2;
-  return ((q2 * kPairs) / 8) != (((q2 + 1) * kPairs) / 8);
-}
 constexpr float kPolyRange = 252.0f;                // width of the clamped argument range [-126, 126]
 constexpr float kPolyMagic = 12582912.0f - 126.0f;  // 1.5 * 2^23 - 126: adding it leaves the integer part in the low bits
 // minimax cubic for 2^f on [0, 1) in relative error (7.5e-5)
@@ -513,7 +520,11 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
         if (p.two_pass) mbar_wait(smem_u32(&sm.stat_full[up]), ph, abort_flag, p.status, 38, limit);
         auto put = [&](int r, float lse2) {  // log2-domain log-sum-exp of row r (+inf: the row is mute)
           const float beta = lse2 - sm.lv[r];
-          sm.tab[up][r] = poly_pair<MB>((r & 15) / 2) ? poly_bias(beta) : -beta;
+          const bool poly = poly_pair<MB>((r & 15) / 2);
+          sm.tab[up][r] = poly ? poly_bias(beta) : -beta;
+          if constexpr (poly_pairs<MB>() > 0) {
+            if (poly) sm.tab[up][kRowsPad + r] = -beta;
+          }
         };
         if (p.two_pass) {
           if (p.cluster > 1) mbar_wait_cluster(smem_u32(&sm.xchg_free), xph ^ 1u, abort_flag, p.status, 31, limit);
@@ -792,7 +803,9 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
         const long long out0 = ((long long)ui.l * p.Hkv + ui.g) * p.seq.total + ui.tok0;
         float sA4[4], sP;
         // 16 rows (half `hi` of the 32-row chunk cc) of this thread's key, a share of the exponentials on the FMA pipe.
-        // Masked form (keys inside the observation window): rows that do not see the key are dropped.
+        // Masked form (keys inside the observation window): rows that do not see the key are dropped, and every exponential
+        // is ex2's. The last keys are seen by few rows (the last one by one row per head), so that a share of cubics, 2 of
+        // 16 over many rows, would be all of such a key's sum there (7.5e-5 instead of 1e-6); a few tiles per unit.
         auto chunk2 = [&](auto masked_tag, auto hi_tag, const float(&cur)[16], int row0, int tau) {
           constexpr bool masked = decltype(masked_tag)::value;
           constexpr int hi = decltype(hi_tag)::value;  // 0: rows row0..row0+15, 1: rows row0+16..row0+31
@@ -802,13 +815,18 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
 #pragma unroll
           for (int q4 = 0; q4 < 4; ++q4) {
             const float4 tb = tab4[q4];
-            const float tbv[4] = {tb.x, tb.y, tb.z, tb.w};
+            float tbv[4] = {tb.x, tb.y, tb.z, tb.w};
             float a[4];
 #pragma unroll
             for (int e = 0; e < 4; e += 2) {
-              if (poly_pair<MB>(2 * q4 + e / 2)) {
+              if (poly_pair<MB>(2 * q4 + e / 2) && !masked) {
                 exp2_poly2(a[e], a[e + 1], cur[4 * q4 + e], cur[4 * q4 + e + 1], c252, tbv[e], tbv[e + 1]);
               } else {
+                if (poly_pair<MB>(2 * q4 + e / 2)) {
+                  const float2 nb = *reinterpret_cast<const float2*>(&sm.tab[up][kRowsPad + row0 + hi * 16 + 4 * q4 + e]);
+                  tbv[e] = nb.x;
+                  tbv[e + 1] = nb.y;
+                }
                 fma2(a[e], a[e + 1], cur[4 * q4 + e], cur[4 * q4 + e + 1], c, tbv[e], tbv[e + 1]);
                 a[e] = ex2(a[e]);
                 a[e + 1] = ex2(a[e + 1]);

@@ -332,3 +332,37 @@ def test_compress_with_supplied_normalisers_reads_the_keys_once(W):
                                ta.view(Vd, True), None, 0, ko, vo, idx, cnt, g.stream)
     finally:
         g.close()
+
+
+@pytest.mark.parametrize("W,n,causal", [(64, 1000, 1), (64, 640, 1), (48, 777, 1), (64, 30, 1), (64, 1000, 0)])
+def test_window_keys_with_two_row_blocks_take_no_cubic(W, n, causal):
+    # The last keys are seen by few rows: were the cubic's share of the exponentials used for them, the last key of a head
+    # would carry its whole error, 7.5e-5. What remains: the normalisers (2 of 16 of a row's terms are cubics: 9.4e-6 at
+    # most), ex2.approx (2^-22) and fp32 rounding of the scores and sums (about 2e-6).
+    L, Hq, Hkv, d = 2, 8, 2, 128
+    g = torch.Generator(device="cuda")
+    g.manual_seed(n + W)
+    q = torch.randn((L, 1, Hq, W, d), generator=g, dtype=torch.bfloat16, device="cuda")
+    k = torch.randn((L, 1, Hkv, n, d), generator=g, dtype=torch.bfloat16, device="cuda")
+    pol = ta.ta_policy_default(ta.TA_PRESET_THEOREM, 4)
+    pol.obs_window, pol.causal = W, causal
+    batch = ta.make_batch(L, 1, n, n, n)
+    ctx = ta.ta_ctx_create(0, ta.ta_scratch_bytes(batch, Hq, Hkv, d, 4, pol))
+    try:
+        u = torch.empty((L, Hkv, n), device="cuda")
+        ta.ta_score_weighted(ctx, pol, batch, Hq, Hkv, d, ta.view(q), ta.view(k), None, u,
+                             torch.cuda.current_stream().cuda_stream)
+        assert ta.ta_ctx_poll(ctx) == ta.TA_OK
+    finally:
+        ta.ta_ctx_destroy(ctx)
+    Wv = min(W, n)  # the window rows that exist; a row's weight counts from the newest
+    s = torch.matmul(q[:, 0, :, W - Wv:].double().view(L, Hkv, Hq // Hkv * Wv, d), k[:, 0].double().transpose(2, 3)) / d ** 0.5
+    s = s.view(L, Hkv, Hq // Hkv, Wv, n)
+    if causal:
+        last = torch.arange(n - Wv, n, device="cuda").view(-1, 1)
+        s = s.masked_fill(torch.arange(n, device="cuda").view(1, -1) > last, float("-inf"))
+    age = torch.arange(Wv - 1, -1, -1, device="cuda").double()
+    w = pol.alpha + pol.delta * (1 - pol.pension_rho) * pol.pension_rho ** age
+    want = (torch.softmax(s, -1) * w.view(-1, 1)).sum((2, 3))
+    err = ((u.double() - want).abs() / want)[:, :, n - Wv if causal else 0:].max().item()
+    assert err <= (2e-5 if causal else 7.5e-5), err
