@@ -537,7 +537,7 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
 #pragma unroll
             for (int gq = 0; gq < kGroups; ++gq) z += sm.part_z[gq][r] * ex2(sm.part_m[gq][r] - m);
             if (p.cluster == 1) {  // nothing to exchange: the CTA's statistics are the unit's
-              put(r, z > 0.0f ? m + __log2f(z) : INFINITY);
+              put(r, z > 0.0f ? m + log2f(z) : INFINITY);
             } else {
 #pragma unroll 4
               for (int q = 0; q < p.cluster; ++q) st_cluster_f32x2(smem_u32(&sm.peer[rank][r]), (uint32_t)q, m, z);
@@ -569,7 +569,7 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
                   const float2 v = sm.peer[q][r];
                   z += q < p.cluster ? v.y * ex2(v.x - m) : 0.0f;
                 }
-                put(r, z > 0.0f ? m + __log2f(z) : INFINITY);
+                put(r, z > 0.0f ? m + log2f(z) : INFINITY);
               }
             };
             if (p.cluster <= 4) merge(std::integral_constant<int, 4>{});

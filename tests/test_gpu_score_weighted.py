@@ -334,14 +334,11 @@ def test_compress_with_supplied_normalisers_reads_the_keys_once(W):
         g.close()
 
 
-@pytest.mark.parametrize("W,n,causal", [(64, 1000, 1), (64, 640, 1), (48, 777, 1), (64, 30, 1), (64, 1000, 0)])
-def test_window_keys_with_two_row_blocks_take_no_cubic(W, n, causal):
-    # The last keys are seen by few rows: were the cubic's share of the exponentials used for them, the last key of a head
-    # would carry its whole error, 7.5e-5. What remains: the normalisers (2 of 16 of a row's terms are cubics: 9.4e-6 at
-    # most), ex2.approx (2^-22) and fp32 rounding of the scores and sums (about 2e-6).
+def _weighted_against_64_bits(W, n, causal=1, cluster=0, seed=0):
+    """ta_score_weighted of random inputs, and the same in 64 bits."""
     L, Hq, Hkv, d = 2, 8, 2, 128
     g = torch.Generator(device="cuda")
-    g.manual_seed(n + W)
+    g.manual_seed(n + W + seed)
     q = torch.randn((L, 1, Hq, W, d), generator=g, dtype=torch.bfloat16, device="cuda")
     k = torch.randn((L, 1, Hkv, n, d), generator=g, dtype=torch.bfloat16, device="cuda")
     pol = ta.ta_policy_default(ta.TA_PRESET_THEOREM, 4)
@@ -349,6 +346,7 @@ def test_window_keys_with_two_row_blocks_take_no_cubic(W, n, causal):
     batch = ta.make_batch(L, 1, n, n, n)
     ctx = ta.ta_ctx_create(0, ta.ta_scratch_bytes(batch, Hq, Hkv, d, 4, pol))
     try:
+        ta.ta_ctx_set_score_cluster(ctx, cluster)
         u = torch.empty((L, Hkv, n), device="cuda")
         ta.ta_score_weighted(ctx, pol, batch, Hq, Hkv, d, ta.view(q), ta.view(k), None, u,
                              torch.cuda.current_stream().cuda_stream)
@@ -363,6 +361,26 @@ def test_window_keys_with_two_row_blocks_take_no_cubic(W, n, causal):
         s = s.masked_fill(torch.arange(n, device="cuda").view(1, -1) > last, float("-inf"))
     age = torch.arange(Wv - 1, -1, -1, device="cuda").double()
     w = pol.alpha + pol.delta * (1 - pol.pension_rho) * pol.pension_rho ** age
-    want = (torch.softmax(s, -1) * w.view(-1, 1)).sum((2, 3))
-    err = ((u.double() - want).abs() / want)[:, :, n - Wv if causal else 0:].max().item()
+    return u.double(), (torch.softmax(s, -1) * w.view(-1, 1)).sum((2, 3))
+
+
+@pytest.mark.parametrize("W,n,causal", [(64, 1000, 1), (64, 640, 1), (48, 777, 1), (64, 30, 1), (64, 1000, 0)])
+def test_window_keys_with_two_row_blocks_take_no_cubic(W, n, causal):
+    # The last keys are seen by few rows: were the cubic's share of the exponentials used for them, the last key of a head
+    # would carry its whole error, 7.5e-5. What remains: the normalisers (2 of 16 of a row's terms are cubics: 9.4e-6 at
+    # most), ex2.approx (2^-22) and fp32 rounding of the scores and sums (about 2e-6).
+    u, want = _weighted_against_64_bits(W, n, causal)
+    err = ((u - want).abs() / want)[:, :, n - min(W, n) if causal else 0:].max().item()
     assert err <= (2e-5 if causal else 7.5e-5), err
+
+
+@pytest.mark.parametrize("n", [2000, 4096, 8229])
+@pytest.mark.parametrize("cluster", [1, 2, 8])
+def test_row_normalisers_are_rounded_once(n, cluster):
+    # A row's log-sum-exp of about 12 binary digits before the point has half a unit in the last place of 2^-22 * 2; its
+    # rounding moves all of the row's terms alike, by 0.69 * 2^-21 at most, of random sign from row to row: over the 128
+    # rows of a key 3.3e-7 / sqrt(3) / sqrt(128) = 1.7e-8. ex2.approx (2^-22 a term) and the fp32 sums of some thousand
+    # terms bring about 1e-7. A logarithm that is off by more, and to one side, shows at once (3e-7).
+    u, want = _weighted_against_64_bits(32, n, cluster=cluster, seed=cluster)
+    err = ((u - want).norm() / want.norm()).item()
+    assert err <= 2e-7, err
