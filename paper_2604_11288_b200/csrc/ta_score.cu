@@ -998,10 +998,16 @@ cudaError_t launch_variant(ta_ctx* ctx, const CUtensorMap& mq, const CUtensorMap
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  // Persistent grid: as many clusters as can be resident at once (queried once per cluster size). CTAs per unit:
-  // the size with the fewest tile-times on the busiest CTA, counting ~1 tile-time of overhead per unit and ~2 more
-  // for the statistics exchange when a unit spans several CTAs. (Choosing more CTAs per unit so that the keys of
-  // all units in flight fit in L2 was measured and lost: 16 x 32768 tokens, 8 CTAs per unit 2.02 ms against 1.63 ms.)
+  // Persistent grid: as many clusters as can be resident at once (queried once per cluster size). CTAs per unit: the size
+  // with the shortest busiest CTA, counted in half jobs: two per job, a tile-time of overhead per unit, and for the
+  // statistics exchange of a unit that spans several CTAs another tile-time with 256 rows, 1.5 with 128. Where every cluster
+  // has one unit a pass takes whole rounds of the softmax groups; with more, the next unit's jobs fill the last round.
+  // Measured on 32 to 640 units of 1000 to 16384 tokens, 100 sizes per row count, every size forced in turn: what this takes
+  // is 0.1 % slower on average than the best (1.3 % with every pass rounded up and two tile-times for the exchange, up to
+  // 17 %: 152 units of 2048 tokens with 256 rows 100.6 us with 1 CTA, 87 us with 2; 0.5 % and up to 9 % with 128 rows: 320
+  // units of 4096 tokens 152 us with 1, 139 us with 2).
+  // (Choosing more CTAs per unit so that the keys of all units in flight fit in L2 was measured and lost: 16 x 32768
+  // tokens, 8 CTAs per unit 2.02 ms against 1.63 ms.)
   int best_cl = ctx->score_force_cluster;
   long long best_cost = best_cl > 0 ? 0 : -1;
   for (int cl = 1; cl <= ScoreSmem<MB>::kPeers; cl = cl < 8 ? 2 * cl : cl + 1) {
@@ -1023,9 +1029,9 @@ cudaError_t launch_variant(ta_ctx* ctx, const CUtensorMap& mq, const CUtensorMap
     if (ctx->score_force_cluster > 0) break;
     const int avail = max_clusters[cl];
     const long long rounds = (sp.units + avail - 1) / avail;
-    // a pass takes whole rounds of the softmax groups
-    const long long per_cta = (((tiles_max + cl - 1) / cl) * MB + kGroups - 1) / kGroups * kGroups;
-    const long long cost = rounds * (per_cta + MB * (cl > 1 ? 3 : 1));
+    long long jobs = (long long)((tiles_max + cl - 1) / cl) * MB;
+    if (rounds == 1) jobs = (jobs + kGroups - 1) / kGroups * kGroups;
+    const long long cost = rounds * (2 * jobs + (cl == 1 ? 2 * MB : MB == 1 ? 5 : 8));
     if (sp.flat) {  // equal shares whatever the number of units: nothing to gain from more CTAs per unit
       best_cl = cl;
       best_cost = 0;

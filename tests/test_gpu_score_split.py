@@ -1,0 +1,58 @@
+"""CTAs per unit of the score kernel: where the rule has to choose between whole units and units spread over a cluster, it
+takes the size that was measured to be the fastest on 148 SMs, and the scores are those of one CTA per unit."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2604_11288_b200 as ta
+from ta_testlib import SCORE_ATOL, SCORE_RTOL
+
+pytestmark = pytest.mark.gpu
+GUARD = 1
+
+
+def _score(L, B, Hkv, n, W, force):
+    Hq, d = 4 * Hkv, 128
+    g = torch.Generator(device="cuda")
+    g.manual_seed(n + W)
+    q = torch.randn((L, B, Hq, W, d), generator=g, dtype=torch.bfloat16, device="cuda")
+    k = torch.randn((L, B, Hkv, n, d), generator=g, dtype=torch.bfloat16, device="cuda")
+    pol = ta.ta_policy_default(ta.TA_PRESET_THEOREM, 4)
+    pol.obs_window = W
+    batch = ta.make_batch(L, B, n, n, B * n)
+    ctx = ta.ta_ctx_create(0, ta.ta_scratch_bytes(batch, Hq, Hkv, d, 4, pol))
+    try:
+        ta.ta_ctx_set_score_cluster(ctx, force)
+        u = torch.full((L + GUARD, Hkv, B * n), float("nan"), device="cuda")
+        ta.ta_score_weighted(ctx, pol, batch, Hq, Hkv, d, ta.view(q), ta.view(k), None, u,
+                             torch.cuda.current_stream().cuda_stream)
+        assert ta.ta_ctx_poll(ctx) == ta.TA_OK
+        assert torch.isnan(u[L:]).all(), "wrote behind its output"
+        return u[:L].cpu().numpy(), ta.ta_ctx_last_launch_info(ctx)[0]
+    finally:
+        ta.ta_ctx_destroy(ctx)
+
+
+@pytest.mark.parametrize("L,B,Hkv,n,W,want", [
+    # 256 score rows
+    (19, 1, 8, 2048, 64, 2), (24, 1, 8, 2048, 64, 2), (19, 1, 8, 4096, 64, 4), (10, 1, 8, 4096, 64, 4),
+    (40, 1, 8, 3000, 64, 2), (8, 1, 8, 1024, 64, 2), (32, 1, 8, 4096, 64, 1),
+    # 128 score rows
+    (40, 1, 8, 4096, 32, 2), (10, 1, 8, 5000, 32, 4), (19, 1, 8, 5000, 32, 4), (16, 1, 8, 4096, 32, 1)])
+def test_fastest_size_is_taken(L, B, Hkv, n, W, want):
+    got, size = _score(L, B, Hkv, n, W, 0)
+    assert size == want
+    ref, one = _score(L, B, Hkv, n, W, 1)
+    assert one == 1
+    np.testing.assert_allclose(got, ref, rtol=SCORE_RTOL, atol=SCORE_ATOL)
+
+
+@pytest.mark.parametrize("L,Hkv,n", [(1, 1, 16384), (1, 2, 9001), (1, 7, 6000), (1, 4, 4096), (2, 2, 3700),
+                                     (1, 3, 3200)])
+def test_more_than_eight_ctas_for_a_handful_of_units(L, Hkv, n):
+    # sizes that cannot be asked for: the rule takes them when all units fit at once and a round of jobs is saved (9 CTAs for
+    # 25 tiles, 10 for 29, 11 for 32, 12 for 71, 16 for 47 and 128)
+    got, size = _score(L, 1, Hkv, n, 32, 0)
+    assert 8 < size <= 16
+    ref, _ = _score(L, 1, Hkv, n, 32, 1)
+    np.testing.assert_allclose(got, ref, rtol=SCORE_RTOL, atol=SCORE_ATOL)
