@@ -2,8 +2,9 @@
 
 Every step of the method runs in the CUDA kernels behind these calls. There is no CPU path: if the shared library is
 missing, loading raises. The calls that a program makes once per layer or per token go through the native module _ta_call
-(one layer of a 4096-token prompt: 22 -> 17 us on the host, 32 layers one by one 890 -> 535 us), the others through ctypes. Tensors are passed as raw device (or, for ta_compress_host, host) addresses; torch is used
-by callers only to own memory and streams.
+where it was built for this Python (one layer of a 4096-token prompt: 22 -> 17 us on the host, 32 layers one by one
+890 -> 535 us), otherwise, and all others, through ctypes: same arguments, same results. Tensors are passed as raw device (or,
+for ta_compress_host, host) addresses; torch is used by callers only to own memory and streams.
 """
 from __future__ import annotations
 
@@ -11,10 +12,11 @@ import ctypes as C
 import importlib.machinery
 import importlib.util
 import os
+import sysconfig
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libta.so")
-CALL_PATH = os.path.join(_HERE, "_ta_call.so")
+CALL_PATH = os.path.join(_HERE, "_ta_call" + (sysconfig.get_config_var("EXT_SUFFIX") or ".so"))  # of this Python's ABI
 
 TA_OK = 0
 TA_ERR_INVALID_ARG, TA_ERR_UNSUPPORTED, TA_ERR_ALIGNMENT, TA_ERR_SCRATCH_TOO_SMALL = 1, 2, 3, 4
@@ -57,15 +59,64 @@ class TAError(RuntimeError):
 
 
 _lib = None
-_call = None  # the native module, once lib() has run
+_call = None  # marshalling of the frequent calls, once lib() has run: the native module or _CtypesCalls
+
+
+class _CtypesCalls:
+    """The calls of the native module _ta_call through ctypes, for a Python that it was not built for."""
+
+    def __init__(self, L):
+        self._lib = L
+
+    def view(self, t, ragged):
+        if t is None:
+            return ta_bf16_view(None, 0, 0, 0, 0)
+        s = t.stride()
+        assert len(s) == (4 if ragged else 5), f"a tensor of {4 if ragged else 5} dimensions is needed"
+        assert s[-1] == 1, "head_dim must be contiguous"
+        return ta_bf16_view(t.data_ptr(), s[0], 0 if ragged else s[1], s[1 if ragged else 2], s[2 if ragged else 3])
+
+    def ta_compress(self, ctx, pats, policy, batch, Hq, Hkv, d, K, token_ids, q_obs, k, v, seq_epoch, k_out, v_out, idx, count,
+                    stream):
+        return self._lib.ta_compress(ctx, pats, C.byref(policy), C.byref(batch), Hq, Hkv, d, K, _ptr(token_ids), q_obs, k, v,
+                                     int(seq_epoch), _ptr(k_out), _ptr(v_out), _ptr(idx), _ptr(count), stream)
+
+    def ta_compress_lse(self, ctx, pats, policy, batch, Hq, Hkv, d, K, token_ids, q_obs, k, v, lse_obs, seq_epoch, k_out,
+                        v_out, idx, count, stream):
+        return self._lib.ta_compress_lse(ctx, pats, C.byref(policy), C.byref(batch), Hq, Hkv, d, K, _ptr(token_ids), q_obs, k,
+                                         v, _ptr(lse_obs), int(seq_epoch), _ptr(k_out), _ptr(v_out), _ptr(idx), _ptr(count),
+                                         stream)
+
+    def ta_compress_scores(self, ctx, pats, policy, batch, Hkv, d, K, token_ids, score, score2, k, v, seq_epoch, k_out, v_out,
+                           idx, count, stream):
+        return self._lib.ta_compress_scores(ctx, pats, C.byref(policy), C.byref(batch), Hkv, d, K, _ptr(token_ids),
+                                            _ptr(score), _ptr(score2), k, v, int(seq_epoch), _ptr(k_out), _ptr(v_out),
+                                            _ptr(idx), _ptr(count), stream)
+
+    def ta_stream_step(self, ctx, pats, policy, st, new_ids, attn, evicted_pos, stream):
+        return self._lib.ta_stream_step(ctx, pats, C.byref(policy), C.byref(st), _ptr(new_ids), _ptr(attn),
+                                        _ptr(evicted_pos), stream)
+
+    def ta_detect_embedding(self, ctx, total_tokens, emb, stride_tok, D, concepts, n_concepts, conf, stream):
+        return self._lib.ta_detect_embedding(ctx, int(total_tokens), _ptr(emb), int(stride_tok), int(D), _ptr(concepts),
+                                             int(n_concepts), _ptr(conf), stream)
+
+    def ta_sponsor_mask_conf(self, ctx, policy, batch, token_ids, conf, threshold, budget, span, rank_by_confidence, flags,
+                             voucher, u_static, stream):
+        return self._lib.ta_sponsor_mask_conf(ctx, C.byref(policy), C.byref(batch), _ptr(token_ids), _ptr(conf),
+                                              C.c_float(threshold), C.c_float(budget), int(span), int(rank_by_confidence),
+                                              _ptr(flags), _ptr(voucher), _ptr(u_static), stream)
 
 
 def _load_call(L):
-    if not os.path.exists(CALL_PATH):
-        raise FileNotFoundError(f"{CALL_PATH} is missing: run `python -m paper_2604_11288_b200.build`")
+    if not os.path.exists(CALL_PATH):  # not built, or built for another Python
+        return _CtypesCalls(L)
     loader = importlib.machinery.ExtensionFileLoader("_ta_call", CALL_PATH)
-    m = importlib.util.module_from_spec(importlib.util.spec_from_loader("_ta_call", loader))
-    loader.exec_module(m)
+    try:
+        m = importlib.util.module_from_spec(importlib.util.spec_from_loader("_ta_call", loader))
+        loader.exec_module(m)
+    except ImportError:  # built against other system libraries
+        return _CtypesCalls(L)
     m.set_types(C.c_void_p, ta_bf16_view, ta_policy, ta_batch, ta_stream)
     for name in ("ta_compress", "ta_compress_lse", "ta_compress_scores", "ta_stream_step", "ta_detect_embedding",
                  "ta_sponsor_mask_conf"):

@@ -1,5 +1,7 @@
 """Builds paper_2604_11288_b200/libta.so from csrc/*.cu with nvcc for sm_100a (cross-compiles without a GPU), and the CPython
-module _ta_call.so (argument marshalling of the most frequent calls) from csrc/py_call.cpp with g++."""
+module _ta_call (argument marshalling of the most frequent calls, for the Python that runs this) from csrc/py_call.cpp with g++.
+The module saves host time and nothing depends on it: where it cannot be built (no Python headers, no C++ compiler) those calls
+go through ctypes like the others."""
 from __future__ import annotations
 
 import glob
@@ -11,7 +13,7 @@ import sysconfig
 _HERE = os.path.dirname(os.path.abspath(__file__))
 _ROOT = os.path.dirname(_HERE)
 LIB_PATH = os.path.join(_HERE, "libta.so")
-CALL_PATH = os.path.join(_HERE, "_ta_call.so")
+CALL_PATH = os.path.join(_HERE, "_ta_call" + (sysconfig.get_config_var("EXT_SUFFIX") or ".so"))
 CALL_SOURCE = os.path.join(_HERE, "csrc", "py_call.cpp")
 
 
@@ -27,14 +29,24 @@ def _stale():
     return any(os.path.getmtime(d) > t for d in deps)
 
 
-def build(force: bool = False, verbose: bool = False) -> str:
-    """Compile every CUDA source into one shared library, and the marshalling module. Returns the library's path."""
+def _build_call(force: bool) -> None:
     header = os.path.join(_ROOT, "include", "ta.h")
-    if force or not os.path.exists(CALL_PATH) or any(os.path.getmtime(f) > os.path.getmtime(CALL_PATH)
-                                                     for f in (CALL_SOURCE, header)):
+    if not force and os.path.exists(CALL_PATH) and all(os.path.getmtime(f) <= os.path.getmtime(CALL_PATH)
+                                                       for f in (CALL_SOURCE, header)):
+        return
+    try:
         subprocess.run([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-I",
                         os.path.join(_ROOT, "include"), "-I", sysconfig.get_paths()["include"], CALL_SOURCE, "-o",
-                        CALL_PATH], check=True)
+                        CALL_PATH], check=True, capture_output=True, text=True)
+    except (OSError, subprocess.CalledProcessError) as e:
+        if os.path.exists(CALL_PATH):  # older than the source or the header
+            os.remove(CALL_PATH)
+        print(f"_ta_call was not built, its calls go through ctypes: {e}\n{getattr(e, 'stderr', None) or ''}", file=sys.stderr)
+
+
+def build(force: bool = False, verbose: bool = False) -> str:
+    """Compile every CUDA source into one shared library, and the marshalling module. Returns the library's path."""
+    _build_call(force)
     if not force and not _stale():
         return LIB_PATH
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")

@@ -87,3 +87,56 @@ def test_score_kernel_keeps_its_values_in_registers(tmp_path):
     spills = dict(re.findall(r"Compiling entry function '(\S*ta_score_kernel\S*)'.*?(\d+) bytes spill stores", out, re.S))
     assert len(spills) == 6
     assert max(int(n) for n in spills.values()) <= 8, spills
+
+
+@pytest.fixture
+def ctypes_calls(lib, monkeypatch, tmp_path):
+    """The binding as it loads where the native module is missing."""
+    monkeypatch.setattr(ta.binding, "_lib", None)
+    monkeypatch.setattr(ta.binding, "_call", None)
+    monkeypatch.setattr(ta.binding, "CALL_PATH", str(tmp_path / "_ta_call.so"))
+    ta.binding.lib()
+    return ta.binding._call
+
+
+def _refused(calls):
+    """Status of every call of the native module without a context (nothing reaches a device)."""
+    p, b, v, st = ta.ta_policy_default(0, 16), ta.make_batch(1, 1, 64, 64, 64), ta.ta_bf16_view(), ta.ta_stream()
+    return [calls.ta_compress(None, None, p, b, 8, 2, 128, 16, None, v, v, v, 0, None, None, None, None, None),
+            calls.ta_compress_lse(None, None, p, b, 8, 2, 128, 16, None, v, v, v, None, 0, None, None, None, None, None),
+            calls.ta_compress_scores(None, None, p, b, 2, 128, 16, None, None, None, v, v, 0, None, None, None, None, None),
+            calls.ta_stream_step(None, None, p, st, None, None, None, None),
+            calls.ta_detect_embedding(None, 64, None, 2048, 2048, None, 8, None, None),
+            calls.ta_sponsor_mask_conf(None, p, b, None, None, 0.5, 15.0, 6, 0, None, None, None, None)]
+
+
+def test_library_loads_without_the_native_module(lib, ctypes_calls, monkeypatch):
+    import torch
+    assert type(ctypes_calls).__name__ == "_CtypesCalls"
+    with pytest.raises(ta.TAError):
+        ta.ta_stream_step(None, None, ta.ta_policy_default(0, 16), ta.ta_stream(), None, None, None)
+    monkeypatch.undo()
+    native = ta.binding._native()
+    assert type(native).__name__ == "module"
+    assert _refused(ctypes_calls) == _refused(native) == [ta.TA_ERR_INVALID_ARG] * 6
+    for t, ragged in ((torch.zeros(2, 3, 4, 8, 128, dtype=torch.bfloat16)[:, :, 1:], False),
+                      (torch.zeros(2, 4, 9, 128, dtype=torch.bfloat16), True), (None, False)):
+        assert bytes(ctypes_calls.view(t, ragged)) == bytes(native.view(t, ragged))
+    for bad, ragged in ((torch.zeros(2, 3, 8, 128), False), (torch.zeros(1, 2, 3, 128, 8).transpose(3, 4), False),
+                        (torch.zeros(2, 3, 4, 8, 128), True)):
+        for c in (ctypes_calls, native):
+            with pytest.raises(AssertionError):
+                c.view(bad, ragged)
+
+
+def test_native_module_is_of_this_python(lib):
+    import sysconfig
+    assert ta.binding.CALL_PATH == ta_build.CALL_PATH
+    assert ta.binding.CALL_PATH.endswith(sysconfig.get_config_var("EXT_SUFFIX"))
+
+
+def test_build_without_a_compiler_for_the_module(lib, monkeypatch, tmp_path, capfd):
+    monkeypatch.setattr(ta_build, "CALL_PATH", str(tmp_path / "_ta_call.so"))
+    monkeypatch.setenv("CXX", str(tmp_path / "no_such_compiler"))
+    assert ta_build.build() == ta_build.LIB_PATH
+    assert not os.path.exists(ta_build.CALL_PATH) and "ctypes" in capfd.readouterr().err
