@@ -741,7 +741,7 @@ ta_status compress_impl(ta_ctx* ctx, const ta_patterns* pats, const ta_policy* p
     sel.u = ext_u_all ? ext_u_all : u_all;
     sel.idx = idx_lb;
     sel.count = count_lb;
-  } else if (!fast) {  // small budgets: the selecting block gathers the unit's rows itself
+  } else if (!fast) {  // the selecting block gathers the unit's rows itself where ta_select_gathers says so
     sel.gather_k = k;
     sel.gather_v = v;
     sel.gather_k_out = k_out;

@@ -214,7 +214,7 @@ struct ta_select_args {
   int n_classes;            // 0: one budget K for all units
   const int32_t* class_K;   // DEVICE [n_classes]
   const int32_t* class_of;  // DEVICE [n_layers][Hkv]
-  // optional: the select kernel also gathers the retained rows (small K, one block per unit; see ta_select_gathers)
+  // optional: the select kernel also gathers the retained rows (any K; units whose keys one block holds: ta_select_gathers)
   ta_bf16_view gather_k, gather_v;
   void* gather_k_out;  // null: no gather
   void* gather_v_out;

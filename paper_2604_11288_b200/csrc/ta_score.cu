@@ -9,13 +9,14 @@
 //   pass 2  S^T = Ktile * Q^T (TMEM lane = key)        -> sum over rows of exp2(s*c - beta_row) per key
 // Both passes use the same shared-memory operand tiles (both K-major, 128-byte swizzle); only the roles in the
 // instruction descriptor swap, which puts the reduction axis of each pass along a thread's own registers.
-// A unit is handled by a cluster of 1, 2, 4 or 8 CTAs (chosen per launch: one CTA when there are many units, more when
-// there are few, up to 16 for a handful of units); each CTA owns a contiguous range of 128-key tiles. Between the passes
-// every CTA stores its per-row (reference, sum) pairs into the shared memory of all its peers and signals them with a remote
-// mbarrier arrive (posted stores: reading the peers' pairs over the cluster took 1.9 us of a 15 us kernel). Pass 2 walks the CTA's tiles backwards so that the tiles read
-// last are re-read first from L2. When the caller supplies the rows' log-sum-exp (lse_obs), pass 1 is skipped; the keys
-// of a unit are then independent, and a uniform batch is cut into equal shares of tiles, one per CTA (32 layers x 8111
-// tokens: 256 units on 148 CTAs are 2 rounds of whole units but 1.73 rounds of shares; 118 -> 105 us with the rest).
+// A unit is handled by a cluster of 1, 2, 4 or 8 CTAs (chosen per launch: one CTA when there are many units, more when there
+// are few, 9 to 16 for the 7 or fewer units of up to 128 rows that so many CTAs hold at once); each CTA owns a contiguous
+// range of 128-key tiles. Between the passes every CTA stores its per-row (reference, sum) pairs into the shared memory of all
+// its peers and signals them with a remote mbarrier arrive (posted stores: reading the peers' pairs over the cluster took
+// 1.9 us of a 15 us kernel). Pass 2 walks the CTA's tiles backwards so that the tiles read last are re-read first from L2.
+// When the caller supplies the rows' log-sum-exp (lse_obs), pass 1 is skipped; the keys of a unit are then independent, and
+// a uniform batch is cut into equal shares of tiles, one per CTA (32 layers x 8111 tokens: 256 units on 148 CTAs are 2 rounds
+// of whole units but 1.73 rounds of shares; 118 -> 105 us with the rest).
 //
 // The grid is persistent: as many clusters as the device can hold at once, each walking over its units. Roles, all of them
 // whole warps that meet only at mbarriers (no barrier among the softmax warps: each runs on as soon as its own data is
@@ -31,15 +32,17 @@
 //                       shared-memory ring.
 // After set-up the producer's warpgroup gives registers back (setmaxnreg) and the softmax warps take them.
 //
-// What bounds it. Back to back, the board's power limit (1000 W): a call takes its energy over 1000 W, whatever the clock.
-// On 32 layers x 4096 tokens (118 mJ, 120 us; 122 mJ with the earlier four groups, single-lane issuer and barriers at
-// every unit border) the copies alone take 71 mJ, the products 55 mJ, the softmax arithmetic 34 mJ, each with its share of the
-// idle power. Copies dominate, from L2 as well as from HBM (keeping the keys of all units in flight inside L2 with 4 CTAs
-// per unit costs as much energy), so what helps is fewer bytes and fewer stalls, not more arithmetic throughput.
-// In single calls, at full clock: the softmax warps (two exponentials per score element, 16 per clock and SM on the
-// special-function unit) and the memory system, at about the same time each: the parts alone take 85 us (softmax), 73 us
-// (products) and 72 us (copies), together 107 us (112 us before). The scale-and-shift and the running sums are taken two at
-// a time (fma.rn.f32x2, add.rn.f32x2: the same roundings as the scalar forms, a third fewer issue slots per element).
+// What bounds it. With up to 128 rows at full clock (32 layers x 4096 tokens): the softmax warps (two exponentials per score
+// element, 16 per clock and SM on the special-function unit) and the memory system, at about the same time each: the parts
+// alone take 85 us (softmax), 73 us (products: 64 KB of operand reads and 32 KB of copies through shared memory per job) and
+// 72 us (copies), together 107 us; 256 units on 148 CTAs are two rounds where 1.73 would do. With 256 rows (16 x 32768
+// tokens): the special-function unit, 74 % of the active cycles. Back to back the board's power limit (1000 W) adds to that by
+// lowering the clock from 1965 MHz: to 1807 on the first call (8 %), 1455 on 64 ragged sequences of up to 16384 tokens with 128
+// rows (3.82 -> 4.47 ms a call), 1582 with 256 rows (11.2 -> 13.0 ms). Of the first call's 118 mJ (122 mJ with the earlier
+// four groups, single-lane issuer and barriers at every unit border) the copies alone take 71 mJ, the products 55 mJ, the
+// softmax arithmetic 34 mJ, each with its share of the idle power: copies dominate, from L2 as well as from HBM (keeping the
+// keys of all units in flight inside L2 with 4 CTAs per unit costs as much energy). The scale-and-shift and the running sums
+// are taken two at a time (fma.rn.f32x2, add.rn.f32x2: the same roundings as the scalar forms, a third fewer issue slots).
 //
 // Every wait on an mbarrier is bounded by wall time; when one runs out the CTA records TA_ERR_TIMEOUT, its producer
 // and MMA warps stop issuing work, the copies and MMAs in flight are drained, and the other warps leave their loops

@@ -715,8 +715,8 @@ __device__ int cached_ordered_emit(int n, const SelectResult& r, const KeyCache<
   uint32_t m = wd | wt;
   // Sparse words: every thread walks its own word. Dense ones (recency makes runs of neighbours win together, so that a few
   // words hold most of what is taken): the warps of the block share the words, a lane per position (TA-Fast, 1024 of 4096
-// tokens, with the search above: 58.2 -> 55.8 us a call). A warp meets at most
-  // `chunks` words that are not empty that way, a thread up to `most` positions the other way.
+  // tokens, with the search above: 58.2 -> 55.8 us a call). A warp meets at most `chunks` words that are not empty that
+  // way, a thread up to `most` positions the other way.
   if (most > min(chunks, (def_mine + tie_mine) / kWarps + 1) + 2) {
     sh.before[tid] = ex;
     __syncthreads();
