@@ -14,9 +14,10 @@
 //                           voucher by budget_decay (Algorithm 1 step 10)
 // The second kernel runs beside the first: it reads the unit's state and waits for the first only where the new token comes
 // in. What bounds it: latency at few units, the state's bytes (25 read, 12 to 25 written per cached token, 4 of attention
-// mass read) at many. 4096 units of 257 tokens, three states in turn (180 MB: more than L2): 52 -> 18.4 us a step,
-// 3.1 TB/s (serial scans by one thread in the pool selection, one lane per sequence for the voucher, all entries through
-// shared memory before; then 22 us with two entries in 64 registers, of which an SM held 6 blocks).
+// mass read) at many. 4096 units of 257 tokens, three states in turn (180 MB: more than L2), a step of both kernels: where the
+// tokens with a voucher fit the protected slots 31 -> 18.5 us, where all compete for a quarter of the slots 70 -> 25.6 us, the
+// extremes of what a generation meets (serial scans by one thread in the pool selection, one lane per sequence for the voucher,
+// all entries through shared memory before; then 22 us with two entries in 64 registers, of which an SM held 6 blocks).
 // All arithmetic that decides the selection is fp32 with one rounding per operation, in the order the CPU oracle uses.
 #include "ta_internal.cuh"
 
