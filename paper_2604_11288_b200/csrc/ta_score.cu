@@ -10,10 +10,11 @@
 // Both passes use the same shared-memory operand tiles (both K-major, 128-byte swizzle); only the roles in the
 // instruction descriptor swap, which puts the reduction axis of each pass along a thread's own registers.
 // A unit is handled by a cluster of 1, 2, 4 or 8 CTAs (chosen per launch: one CTA when there are many units, more when there
-// are few, 9 to 16 for the 7 or fewer units of up to 128 rows that so many CTAs hold at once); each CTA owns a contiguous
-// range of 128-key tiles. Between the passes every CTA stores its per-row (reference, sum) pairs into the shared memory of all
-// its peers and signals them with a remote mbarrier arrive (posted stores: reading the peers' pairs over the cluster took
-// 1.9 us of a 15 us kernel). Pass 2 walks the CTA's tiles backwards so that the tiles read last are re-read first from L2.
+// are few, 9 to 16 for a handful of units of up to 128 rows, where all of them fit at once: a cluster stays inside a group of
+// SMs, 148 SMs hold 8 clusters of 9 or 10 CTAs and 7 of 11 to 16); each CTA owns a contiguous range of 128-key tiles. Between
+// the passes every CTA stores its per-row (reference, sum) pairs into the shared memory of all its peers and signals them
+// with a remote mbarrier arrive (posted stores: reading the peers' pairs over the cluster took 1.9 us of a 15 us kernel).
+// Pass 2 walks the CTA's tiles backwards so that the tiles read last are re-read first from L2.
 // When the caller supplies the rows' log-sum-exp (lse_obs), pass 1 is skipped; the keys of a unit are then independent, and
 // a uniform batch is cut into equal shares of tiles, one per CTA (32 layers x 8111 tokens: 256 units on 148 CTAs are 2 rounds
 // of whole units but 1.73 rounds of shares; 118 -> 105 us with the rest).

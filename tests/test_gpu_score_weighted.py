@@ -377,8 +377,8 @@ def test_window_keys_with_two_row_blocks_take_no_cubic(W, n, causal):
 @pytest.mark.parametrize("n", [2000, 4096, 8229])
 @pytest.mark.parametrize("cluster", [1, 2, 8])
 def test_row_normalisers_are_rounded_once(n, cluster):
-    # A row's log-sum-exp of about 12 binary digits before the point has half a unit in the last place of 2^-22 * 2; its
-    # rounding moves all of the row's terms alike, by 0.69 * 2^-21 at most, of random sign from row to row: over the 128
+    # A row's log-sum-exp lies between 8 and 16 binary units here, where half a unit in the last place is 2^-21; its rounding
+    # moves all of the row's terms alike, by 0.69 * 2^-21 = 3.3e-7 at most, of random sign from row to row: over the 128
     # rows of a key 3.3e-7 / sqrt(3) / sqrt(128) = 1.7e-8. ex2.approx (2^-22 a term) and the fp32 sums of some thousand
     # terms bring about 1e-7. A logarithm that is off by more, and to one side, shows at once (3e-7).
     u, want = _weighted_against_64_bits(32, n, cluster=cluster, seed=cluster)
