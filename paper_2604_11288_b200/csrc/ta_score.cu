@@ -12,8 +12,9 @@
 // A unit is handled by a cluster of 1, 2, 4 or 8 CTAs (chosen per launch: one CTA when there are many units, more when there
 // are few, 9 to 16 for a handful of units of up to 128 rows, where all of them fit at once: a cluster stays inside a group of
 // SMs, 148 SMs hold 8 clusters of 9 or 10 CTAs and 7 of 11 to 16); each CTA owns a contiguous range of 128-key tiles. Between
-// the passes every CTA stores its per-row (reference, sum) pairs into the shared memory of all its peers and signals them
-// with a remote mbarrier arrive (posted stores: reading the peers' pairs over the cluster took 1.9 us of a 15 us kernel).
+// the passes every CTA stores its per-row (reference, sum) pairs into the shared memory of all its peers with stores that count
+// on the receiver's mbarrier when they land (reading the peers' pairs over the cluster took 1.9 us of a 15 us kernel, plain
+// remote stores with a fence and a signal behind them 0.4 us more than these).
 // Pass 2 walks the CTA's tiles backwards so that the tiles read last are re-read first from L2.
 // When the caller supplies the rows' log-sum-exp (lse_obs), pass 1 is skipped; the keys of a unit are then independent, and
 // a uniform batch is cut into equal shares of tiles, one per CTA (32 layers x 8111 tokens: 256 units on 148 CTAs are 2 rounds
@@ -24,14 +25,20 @@
 // there):
 //   TMA producer        walks the units, publishes each one's description in a small ring, streams query and key tiles
 //   MMA issuer          TMEM owner; one elected lane issues, the warp around it is uniform
-//   2 statistics warps  merge the row statistics between the passes, exchange them over the cluster, form the row constants
+//   2 statistics warps  one pass only: form the row constants from the log-sum-exps that the caller supplies, a unit ahead
 //   12 softmax warps    three groups of four. A "job" is one block of up to 128 score rows of one key tile in one pass; jobs
 //                       are dealt round-robin to the three groups and to the four accumulator stages, so that the products
 //                       of a group's next job are ready when it hands back the current one (four groups on four stages
 //                       waited 30 % of their time for their own stage to be refilled). With 129..256 score rows (MB 2) a
 //                       tile is two consecutive jobs, one per block of 128 rows; in pass 2 their partial sums meet in a
-//                       shared-memory ring.
-// After set-up the producer's warpgroup gives registers back (setmaxnreg) and the softmax warps take them.
+//                       shared-memory ring. Between the passes the group that ends the first one first merges the row
+//                       statistics, exchanges them over the cluster and forms the row constants for pass 2.
+// The producer's warpgroup gives registers back (setmaxnreg) at its start and the softmax warps take them.
+//
+// A call of few units is a chain of latencies (one layer of 4096 tokens: 8 units, 8 CTAs each, four tiles and 26 K cycles per
+// CTA, of which the exponentials need 9 K). What the chain waits for is started as early as it can be: the producer requests its
+// first tiles before the CTA's set-up is complete (first scores after 4.8 K cycles instead of 7 K), and nothing but the
+// barriers that it needs itself precedes them. 21.9 -> 20.5 us a call, 32 calls of 8 shorter units 905 -> 865 us.
 //
 // What bounds it. With up to 128 rows at full clock (32 layers x 4096 tokens): the softmax warps (two exponentials per score
 // element, 16 per clock and SM on the special-function unit) and the memory system, at about the same time each: the parts
@@ -65,7 +72,7 @@ constexpr int kD = TA_HEAD_DIM;                   // 128
 constexpr int kHalfBytes = kTileN * 128;          // one 64-column half of a 128-row operand tile: 16 KB
 constexpr int kKTileBytes = 2 * kHalfBytes;       // 32 KB
 constexpr int kMaxCluster = 16;                   // more than 8 CTAs is a non-portable cluster size; sm_100 allows 16
-constexpr int kRankedSeqs = 256;                  // sequences of a ragged batch that the kernel itself sorts by length
+constexpr int kRankedSeqs = 256;                  // (an index is a byte) sequences of a ragged batch that the kernel itself sorts by length
 constexpr int kGroups = 3;                        // softmax warpgroups
 constexpr int kSoftWarps = kGroups * 4;
 constexpr int kThreads = (kGroups + 1) * 128;     // 512
@@ -148,17 +155,16 @@ struct alignas(1024) ScoreSmem {
   // [unit parity][row] pass-2 constant of the row; behind them the form that ex2 takes, for rows whose own is the polynomial's
   float tab[2][poly_pairs<MB>() ? 2 * kRowsPad : kRowsPad];
   float wrow[kRowsPad];                    // pension weight per row
-  float lv[kRowsPad];                      // log2 of the row's output weight (kOutFused), else 0
-  int row_t[kRowsPad];                     // window index t of the row, -1 for padding rows
+  int8_t row_t[kRowsPad];                  // window index t of the row, -1 for padding rows
   float psum[kRing][2][128];               // MB 2: [ring slot][A|P][key] partial sums of row block 0
   UnitInfo unit[kUnitRing];
   unsigned long long full[kStages], empty[kStages], acc_full[kAcc], acc_empty[kAcc];
   unsigned long long q_full[kQBufs], q_empty[kQBufs], ufull[kUnitRing], ufree[kUnitRing];
-  unsigned long long stat_full[2], tab_full[2], tab_free[2], xchg_full, xchg_free, drain;
+  unsigned long long stat_full, tab_full[2], tab_free[2], xchg_full, xchg_free, drain;
   unsigned long long pfull[kRing], pfree[kRing];
   uint32_t tmem_base;
   int abort_flag;
-  uint16_t by_rank[kRankedSeqs];           // by_length: sequence of every rank, longest first
+  uint8_t by_rank[kRankedSeqs];            // by_length: sequence of every rank, longest first
 };
 
 // ---------------------------------------------------------------------------------------------- exponentials
@@ -247,6 +253,7 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
   const uint32_t rank = cluster_ctarank();
   const int cluster_id = blockIdx.x / p.cluster;
   const int n_clusters = gridDim.x / p.cluster;
+  const bool one_round = p.units <= n_clusters;  // every cluster has at most one unit
   volatile int* abort_flag = &sm.abort_flag;
   const unsigned long long limit = p.wait_limit_ns;
 
@@ -298,138 +305,141 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
     return ui.T > 0 || (ui.n > 0 && p.two_pass && p.cluster > 1);
   };
 
-  // ---- set-up (once per CTA); a lane per barrier
-  if (warp == 0) {
-    auto init = [&](unsigned long long* bar, int n, uint32_t count) {
-      if (lane < n) mbar_init(smem_u32(bar + lane), count);
-    };
-    init(sm.full, kStages, 1);
-    init(sm.empty, kStages, 1);
-    init(sm.acc_full, kAcc, 1);
-    init(sm.acc_empty, kAcc, 4);
-    init(sm.stat_full, 2, kSoftWarps);
-    init(sm.tab_full, 2, kStatWarps);
-    init(sm.tab_free, 2, kSoftWarps);
-    init(&sm.xchg_full, 1, (uint32_t)p.cluster * kStatWarps);
-    init(&sm.xchg_free, 1, (uint32_t)p.cluster * kStatWarps);
-    init(sm.q_full, kQBufs, 1);
-    init(sm.q_empty, kQBufs, 1);
-    init(sm.ufull, kUnitRing, 1);
-    init(sm.ufree, kUnitRing, kSoftWarps + 1 + kStatWarps);  // softmax warps, MMA issuer, statistics warps
-    init(sm.pfull, kRing, 4);
-    init(sm.pfree, kRing, 4);
-    init(&sm.drain, 1, 1);
-    if (lane == 0) sm.abort_flag = 0;
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  if (warp == kWarpTma && lane == 0) {
-    tma_prefetch_map(&map_q);
-    tma_prefetch_map(&map_k);
-  }
-  if (warp == kWarpMma) {
-    tmem_alloc(smem_u32(&sm.tmem_base), kTmemCols);
-    tmem_relinquish();
-  }
-  // per-row tables: row r = h*W + t
-  for (int r = tid; r < kRowsPad; r += kThreads) {
-    const int t = r < p.rows ? r % p.W : -1;
-    sm.row_t[r] = t;
-    const float w = t >= 0 ? p.wrow[t] : 0.0f;  // (1-rho) rho^(W-1-t); also right for W' < W (same exponent)
-    sm.wrow[r] = w;
-    // kOutFused: the row's contribution alpha + delta*w (positive, checked by the host) goes into the exponent
-    sm.lv[r] = (PM == kOutFused && t >= 0) ? log2f(fmaf(p.delta, w, p.alpha)) : 0.0f;
-  }
-  // Rows of the query tile that the TMA box does not cover are multiplied like any other row: make them zeros so
-  // that the padded score columns are finite.
-  if (p.rows < kRowsPad) {
-    const int pad_rows = kRowsPad - p.rows;
-    for (int i = tid; i < kQBufs * 2 * pad_rows * 8; i += kThreads) {
-      const int qb = i / (2 * pad_rows * 8), i2 = i % (2 * pad_rows * 8);
-      const int half = i2 / (pad_rows * 8), rem = i2 % (pad_rows * 8);
-      const int row = p.rows + rem / 8, chunk = rem % 8;
-      *reinterpret_cast<uint4*>(&sm.q[qb][half * (MB * kHalfBytes) + row * 128 + chunk * 16]) = make_uint4(0, 0, 0, 0);
-    }
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-  }
-  if (!p.late_wait) ta_wait_for_prior_grid();  // nothing above reads memory
-  if (p.by_length) {
-    // Longest first, equal lengths in sequence order. In unit order the lengths a cluster meets are random and the busiest
-    // cluster of a batch with lengths spread 8x carries about 30 % more than the average.
-    for (int b = tid; b < p.seq.batch; b += kThreads) {
-      const int nb = p.seq.cu[b + 1] - p.seq.cu[b];
-      int rank = 0;
-      for (int o = 0; o < p.seq.batch; ++o) {
-        const int no = p.seq.cu[o + 1] - p.seq.cu[o];
-        rank += (no > nb) || (no == nb && o < b);
-      }
-      sm.by_rank[rank] = (uint16_t)b;
-    }
-  }
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem_base = sm.tmem_base;
-  // Every CTA of the cluster must be running (barriers initialised) before a peer arrives on its barriers or reads its shared
-  // memory: the statistics warps wait for that before their first exchange, the others only when they leave.
-  cluster_arrive();
+  // the query tile of a unit into buffer qb; key tile j of a unit's walk (both passes) into stage s
+  auto load_q = [&](const UnitInfo& ui, int qb) {
+    const uint32_t bar = smem_u32(&sm.q_full[qb]);
+    const uint32_t dst = smem_u32(sm.q[qb]);
+    mbar_expect_tx(bar, (uint32_t)(2 * p.rows * 128));
+    tma_load_5d(dst, &map_q, bar, 0, 0, ui.g * p.G, ui.b, ui.l);
+    tma_load_5d(dst + MB * kHalfBytes, &map_q, bar, 64, 0, ui.g * p.G, ui.b, ui.l);
+  };
+  auto load_k = [&](const UnitInfo& ui, int j, int s) {
+    // the second sweep walks the CTA's tiles backwards: the tiles read last are the ones still in L2
+    const int tile = ui.t_begin + (j >= ui.T ? 2 * ui.T - 1 - j : j);
+    const int row = (p.seq.cu ? ui.tok0 : 0) + tile * kTileN;  // ragged: tokens are packed along the row axis
+    const int bc = p.seq.cu ? 0 : ui.b;
+    const uint32_t bar = smem_u32(&sm.full[s]);
+    const uint32_t dst = smem_u32(sm.k[s]);
+    mbar_expect_tx(bar, kKTileBytes);
+    tma_load_5d(dst, &map_k, bar, 0, row, ui.g, bc, ui.l);
+    tma_load_5d(dst + kHalfBytes, &map_k, bar, 64, row, ui.g, bc, ui.l);
+  };
 
-  const uint32_t k_smem = smem_u32(sm.k);
+  // ---- set-up (once per CTA). The warps share it, each its own barriers, a lane per barrier (all of them in one warp kept the
+  // others waiting for 0.5 us). Every role gives or takes its registers first: later the softmax warps would wait for the
+  // producer to come by.
+  auto init = [&](unsigned long long* bar, int n, uint32_t count) {
+    if (lane < n) mbar_init(smem_u32(bar + lane), count);
+  };
+  auto init_done = [&] {
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    __syncwarp();
+  };
+  bool cluster_known = false, cluster_left = false;  // this warp knows its peers to run / will touch no peer any more
+  // The end of the set-up. Every CTA of the cluster must be running (barriers initialised) before a peer writes to its shared
+  // memory or arrives on its barriers: warps that do wait for that before the first time, the others only when they leave.
+  auto set_up = [&] {
+    tc_fence_before();
+    asm volatile("bar.sync 1, %0;" ::"n"(kThreads) : "memory");
+    tc_fence_after();
+    cluster_arrive_relaxed();
+  };
+  // pass-2 constant of row r from its log2-domain log-sum-exp (+inf: the row is mute)
+  // window index t of score row r = h*W + t, -1 for padding rows
+  auto row_index = [&](int r) { return r < p.rows ? (int)((uint32_t)r % (uint32_t)p.W) : -1; };
+  // the tables that pass 2 reads; written before the first row constants are published
+  auto put_tables = [&](int r, int t) {
+    sm.row_t[r] = (int8_t)t;
+    sm.wrow[r] = t >= 0 ? p.wrow[t] : 0.0f;  // (1-rho) rho^(W-1-t); also right for W' < W (same exponent)
+  };
+  // kOutFused: log2 of the row's contribution alpha + delta*w (positive, checked by the host), which goes into the exponent
+  auto row_weight = [&](int t) { return PM == kOutFused && t >= 0 ? log2f(fmaf(p.delta, p.wrow[t], p.alpha)) : 0.0f; };
+  auto put_row = [&](int up, int r, float lse2, float lv) {
+    const float beta = lse2 - lv;
+    const bool poly = poly_pair<MB>((r & 15) / 2);
+    sm.tab[up][r] = poly ? poly_bias(beta) : -beta;
+    if constexpr (poly_pairs<MB>() > 0) {
+      if (poly) sm.tab[up][kRowsPad + r] = -beta;
+    }
+  };
 
   if (warp >= kSoftWarps) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsOther));
     if (warp == kWarpTma) {
       // =========================================================================== TMA producer
-      // Walks the units of this cluster, publishes each one's description in the unit ring and streams its tiles.
+      // Walks the units of this cluster, publishes each one's description in the unit ring and streams its tiles. It does not
+      // wait for the others' set-up: it publishes its first unit and requests that unit's query tile and first key tiles at
+      // once, unless the walk needs the lengths ranked first.
       const bool leader = elect_one();
-      uint32_t issued = 0, q_issued = 0;  // stages that were armed at least once
-      int s = 0, qb = 0, us = 0;
-      uint32_t sph = 1, qph = 1, uph = 1;
+      init(sm.full, kStages, 1);
+      init(sm.empty, kStages, 1);
+      init(sm.q_full, kQBufs, 1);
+      init(sm.q_empty, kQBufs, 1);
+      init(sm.ufull, kUnitRing, 1);
+      init(sm.ufree, kUnitRing, kSoftWarps + 1 + (p.two_pass ? 0 : kStatWarps));  // softmax warps, MMA issuer, statistics warps
+      if (lane == 0) sm.abort_flag = 0;
+      init_done();
+      UnitInfo first = {};
+      bool first_work = false;
+      int pre = 0;  // tiles of the first unit that are requested here
+      if (p.by_length) {
+        set_up();
+        ta_wait_for_prior_grid();
+      } else {
+        asm volatile("bar.arrive 1, %0;" ::"n"(kThreads) : "memory");
+        cluster_arrive_relaxed();
+        if (!p.late_wait) ta_wait_for_prior_grid();  // nothing above reads memory
+        first_work = get_unit(0, first);
+        if (first_work) {
+          pre = __shfl_sync(0xffffffffu, min(kStages, p.two_pass ? 2 * first.T : first.T), 0);
+          if (leader) {
+            if (pre > 0) load_q(first, 0);
+            for (int j = 0; j < pre; ++j) load_k(first, j, j);
+            sm.unit[0] = first;
+            mbar_arrive(smem_u32(&sm.ufull[0]));
+          }
+          __syncwarp();
+        }
+      }
+      uint32_t issued = (1u << pre) - 1u, q_issued = 0;  // stages that were armed at least once
+      int s = pre % kStages, qb = 0, us = 0;
+      uint32_t sph = pre == kStages ? 0 : 1, qph = 1, uph = 1;
       bool ok = true;
       for (int round = 0;; ++round) {
-        UnitInfo ui;
-        const bool work = get_unit(round, ui);
-        const bool end = ui.end != 0;
+        UnitInfo ui = first;
+        const bool begun = round == 0 && first_work;  // during set-up
+        const bool work = begun || get_unit(round, ui);
+        const bool end = !begun && ui.end != 0;
         if (!work && !end) continue;
         const int T = __shfl_sync(0xffffffffu, ui.T, 0);
-        ok = mbar_wait(smem_u32(&sm.ufree[us]), uph, abort_flag, p.status, 12, limit);
-        if (!ok) break;
-        if (leader) {
-          sm.unit[us] = ui;
-          mbar_arrive(smem_u32(&sm.ufull[us]));
+        if (!begun) {
+          ok = mbar_wait(smem_u32(&sm.ufree[us]), uph, abort_flag, p.status, 12, limit);
+          if (!ok) break;
+          if (leader) {
+            sm.unit[us] = ui;
+            mbar_arrive(smem_u32(&sm.ufull[us]));
+          }
         }
         if (++us == kUnitRing) us = 0, uph ^= 1;
         if (end) break;
         if (T == 0) continue;
-        ok = mbar_wait(smem_u32(&sm.q_empty[qb]), qph, abort_flag, p.status, 11, limit);
-        if (!ok) break;  // nothing may be copied into a buffer that was not handed back
-        if (leader) {
-          const uint32_t bar = smem_u32(&sm.q_full[qb]);
-          const uint32_t dst = smem_u32(sm.q[qb]);
-          mbar_expect_tx(bar, (uint32_t)(2 * p.rows * 128));
-          tma_load_5d(dst, &map_q, bar, 0, 0, ui.g * p.G, ui.b, ui.l);
-          tma_load_5d(dst + MB * kHalfBytes, &map_q, bar, 64, 0, ui.g * p.G, ui.b, ui.l);
+        if (!begun) {
+          ok = mbar_wait(smem_u32(&sm.q_empty[qb]), qph, abort_flag, p.status, 11, limit);
+          if (!ok) break;  // nothing may be copied into a buffer that was not handed back
+          if (leader) load_q(ui, qb);
         }
         q_issued |= 1u << qb;
         if (++qb == kQBufs) qb = 0, qph ^= 1;
-        const int row0 = p.seq.cu ? ui.tok0 : 0;  // ragged: tokens are packed along the row axis
-        const int bc = p.seq.cu ? 0 : ui.b;
         const int n_tiles = p.two_pass ? 2 * T : T;
 #pragma unroll 1
-        for (int j = 0; j < n_tiles; ++j) {
+        for (int j = pre; j < n_tiles; ++j) {
           ok = mbar_wait(smem_u32(&sm.empty[s]), sph, abort_flag, p.status, 10, limit);
           if (!ok) break;
-          if (leader) {
-            // the second sweep walks the CTA's tiles backwards: the tiles read last are the ones still in L2
-            const int row = row0 + (ui.t_begin + (j >= T ? 2 * T - 1 - j : j)) * kTileN;
-            const uint32_t bar = smem_u32(&sm.full[s]);
-            mbar_expect_tx(bar, kKTileBytes);
-            const uint32_t dst = k_smem + s * kKTileBytes;
-            tma_load_5d(dst, &map_k, bar, 0, row, ui.g, bc, ui.l);
-            tma_load_5d(dst + kHalfBytes, &map_k, bar, 64, row, ui.g, bc, ui.l);
-          }
+          if (leader) load_k(ui, j, s);
           issued |= 1u << s;
           if (++s == kStages) s = 0, sph ^= 1;
         }
+        pre = 0;  // (requested during set-up: the first unit's only)
         if (!ok) break;
       }
       if (!ok || *abort_flag) {
@@ -447,10 +457,18 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
       // products of a job took 730 cycles instead of the 512 that the tensor pipe needs. The barriers of the next job
       // are looked at in the middle of the current one, while products are still queued.
       const bool leader = elect_one();
+      init(sm.acc_full, kAcc, 1);
+      init(sm.acc_empty, kAcc, 4);
+      init(&sm.drain, 1, 1);
+      init_done();
+      tmem_alloc(smem_u32(&sm.tmem_base), kTmemCols);
+      tmem_relinquish();
+      set_up();
+      const uint32_t tmem_base = sm.tmem_base;
       bool ok = true;
       // operand descriptors: the upper word is the same for every tile; the lower word is the address >> 4
       const uint32_t desc_hi = (uint32_t)(smem_desc_sw128(0) >> 32);
-      const uint32_t k_lo = (k_smem & 0x3FFFFu) >> 4;
+      const uint32_t k_lo = (smem_u32(sm.k) & 0x3FFFFu) >> 4;
       const uint32_t q_lo0 = (smem_u32(sm.q[0]) & 0x3FFFFu) >> 4;
       const uint32_t idesc = idesc_bf16(128, 128);
       const uint32_t bar_full = smem_u32(&sm.full[0]), bar_empty = smem_u32(&sm.empty[0]);
@@ -513,16 +531,38 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
       }
     } else {
       // =========================================================================== statistics warps
-      // Between the passes of a unit: merge the groups' row statistics, exchange them with the cluster's other CTAs and
-      // leave the rows' pass-2 constants in `tab`. Two warps of their own, so that no softmax warp waits for another
-      // before the constants are there.
+      // One pass: the row constants of the units, ahead of the softmax warps, from the log-sum-exps that the caller supplied.
+      // (Between two passes the softmax warps have nothing else to do and form them themselves.)
+      if (warp == kWarpStat) {
+        init(&sm.stat_full, 1, kSoftWarps);
+        init(sm.tab_full, 2, p.two_pass ? 4 : kStatWarps);
+        init(sm.tab_free, 2, kSoftWarps);
+        init(&sm.xchg_full, 1, 1);
+        init(&sm.xchg_free, 1, (uint32_t)p.cluster * 4);
+      } else {
+        init(sm.pfull, kRing, 4);
+        init(sm.pfree, kRing, 4);
+      }
+      init_done();
+      set_up();
+      if (!p.late_wait) ta_wait_for_prior_grid();
       const int r0 = (warp - kWarpStat) * 32 + lane;
       int us = 0;
-      uint32_t uph = 0, xph = 0;
-      cluster_wait();
+      uint32_t uph = 0;
       // a wait that ran out in an earlier CTA or call (not yet polled) makes the remaining CTAs give up their waits at once
       if (*reinterpret_cast<volatile int*>(&p.status->code) == (int)TA_ERR_TIMEOUT) *abort_flag = 1;
-      for (int it = 0;; ++it) {
+      constexpr int kRows = kRowsPad / (32 * kStatWarps);
+      int tr[kRows];
+      float lv[kRows];
+      if (!p.two_pass) {
+#pragma unroll
+        for (int i = 0; i < kRows; ++i) {
+          tr[i] = row_index(r0 + 32 * kStatWarps * i);
+          lv[i] = row_weight(tr[i]);
+          put_tables(r0 + 32 * kStatWarps * i, tr[i]);
+        }
+      }
+      for (int it = 0; !p.two_pass; ++it) {
         if (!mbar_wait(smem_u32(&sm.ufull[us]), uph, abort_flag, p.status, 36, limit)) break;
         const UnitInfo ui = sm.unit[us];
         __syncwarp();
@@ -532,85 +572,54 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
         const int up = it & 1;
         const uint32_t ph = (uint32_t)(it >> 1) & 1u;
         mbar_wait(smem_u32(&sm.tab_free[up]), ph ^ 1u, abort_flag, p.status, 37, limit);
-        if (p.two_pass) mbar_wait(smem_u32(&sm.stat_full[up]), ph, abort_flag, p.status, 38, limit);
-        auto put = [&](int r, float lse2) {  // log2-domain log-sum-exp of row r (+inf: the row is mute)
-          const float beta = lse2 - sm.lv[r];
-          const bool poly = poly_pair<MB>((r & 15) / 2);
-          sm.tab[up][r] = poly ? poly_bias(beta) : -beta;
-          if constexpr (poly_pairs<MB>() > 0) {
-            if (poly) sm.tab[up][kRowsPad + r] = -beta;
+#pragma unroll
+        for (int i = 0; i < kRows; ++i) {
+          const int r = r0 + 32 * kStatWarps * i, t = tr[i];
+          float lse2 = INFINITY;
+          if (t >= 0 && ui.n - p.W + t >= 0) {
+            const int h = r / p.W;
+            const float lse = p.lse_obs[(((long long)ui.l * p.seq.batch + ui.b) * p.Hq + (ui.g * p.G + h)) * p.W + t];
+            lse2 = lse * 1.4426950408889634f;
           }
-        };
-        if (p.two_pass) {
-          if (p.cluster > 1) mbar_wait_cluster(smem_u32(&sm.xchg_free), xph ^ 1u, abort_flag, p.status, 31, limit);
-          constexpr int kRows = kRowsPad / (32 * kStatWarps);
-          float m[kRows], z[kRows];
-#pragma unroll
-          for (int i = 0; i < kRows; ++i) {
-            const int r = r0 + 32 * kStatWarps * i;
-            m[i] = sm.part_m[0][r];
-#pragma unroll
-            for (int gq = 1; gq < kGroups; ++gq) m[i] = fmaxf(m[i], sm.part_m[gq][r]);
-            z[i] = 0.0f;
-#pragma unroll
-            for (int gq = 0; gq < kGroups; ++gq) z[i] += sm.part_z[gq][r] * ex2(sm.part_m[gq][r] - m[i]);
-          }
-          if (p.cluster > 1) {  // (alone, the CTA's statistics are the unit's)
-#pragma unroll 2
-            for (int q = 0; q < p.cluster; ++q)
-#pragma unroll
-              for (int i = 0; i < kRows; ++i)
-                st_cluster_f32x2(smem_u32(&sm.peer[rank][r0 + 32 * kStatWarps * i]), (uint32_t)q, m[i], z[i]);
-            __syncwarp();
-            // one lane per peer tells that peer that this warp's rows of the CTA's statistics are in place
-            if (lane < p.cluster) {
-              fence_cluster();
-              mbar_arrive_remote(smem_u32(&sm.xchg_full), (uint32_t)lane);
-            }
-            mbar_wait_cluster(smem_u32(&sm.xchg_full), xph, abort_flag, p.status, 32, limit);
-            // All of the lane's rows at once, two sweeps over the CTAs' pairs in shared memory. (A row at a time with 16
-            // pairs held, and an address per slot, did not fit the 56 registers these warps have left: 132 bytes spilled
-            // per thread.)
-#pragma unroll
-            for (int i = 0; i < kRows; ++i) m[i] = -1e30f, z[i] = 0.0f;
-#pragma unroll 2
-            for (int q = 0; q < p.cluster; ++q)
-#pragma unroll
-              for (int i = 0; i < kRows; ++i) m[i] = fmaxf(m[i], sm.peer[q][r0 + 32 * kStatWarps * i].x);
-#pragma unroll 2
-            for (int q = 0; q < p.cluster; ++q)
-#pragma unroll
-              for (int i = 0; i < kRows; ++i) {
-                const float2 v = sm.peer[q][r0 + 32 * kStatWarps * i];
-                z[i] += v.y * ex2(v.x - m[i]);
-              }
-            __syncwarp();
-            if (lane < p.cluster) mbar_arrive_remote(smem_u32(&sm.xchg_free), (uint32_t)lane);  // the slots may be written again
-            xph ^= 1u;
-          }
-#pragma unroll
-          for (int i = 0; i < kRows; ++i) put(r0 + 32 * kStatWarps * i, log2_sum(m[i], z[i]));
-        } else {
-          for (int r = r0; r < kRowsPad; r += 32 * kStatWarps) {
-            float lse2 = INFINITY;
-            const int t = sm.row_t[r];
-            if (t >= 0 && ui.n - p.W + t >= 0) {
-              const int h = r / p.W;
-              const float lse = p.lse_obs[(((long long)ui.l * p.seq.batch + ui.b) * p.Hq + (ui.g * p.G + h)) * p.W + t];
-              lse2 = lse * 1.4426950408889634f;
-            }
-            put(r, lse2);
-          }
+          put_row(up, r, lse2, lv[i]);
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(smem_u32(&sm.tab_full[up]));
       }
     }
   } else {
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsSoftmax));
     // =========================================================================== softmax warps
     // A job is one block of 128 score rows of one key tile in one pass. Jobs are numbered through over passes and units
     // and dealt round-robin: group grp takes jobs grp, grp + kGroups, ..; job J uses accumulator stage J mod kAcc.
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsSoftmax));
+    // Rows of the query tile that the TMA box does not cover are multiplied like any other row: make them zeros so
+    // that the padded score columns are finite.
+    if (p.rows < kRowsPad) {
+      const int pad_rows = kRowsPad - p.rows;
+      for (int i = tid; i < kQBufs * 2 * pad_rows * 8; i += kSoftWarps * 32) {
+        const int qb = i / (2 * pad_rows * 8), i2 = i % (2 * pad_rows * 8);
+        const int half = i2 / (pad_rows * 8), rem = i2 % (pad_rows * 8);
+        const int row = p.rows + rem / 8, chunk = rem % 8;
+        *reinterpret_cast<uint4*>(&sm.q[qb][half * (MB * kHalfBytes) + row * 128 + chunk * 16]) = make_uint4(0, 0, 0, 0);
+      }
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    if (!p.late_wait) ta_wait_for_prior_grid();
+    if (p.by_length) {
+      // Longest first, equal lengths in sequence order. In unit order the lengths a cluster meets are random and the busiest
+      // cluster of a batch with lengths spread 8x carries about 30 % more than the average.
+      for (int b = tid; b < p.seq.batch; b += kSoftWarps * 32) {
+        const int nb = p.seq.cu[b + 1] - p.seq.cu[b];
+        int rank = 0;
+        for (int o = 0; o < p.seq.batch; ++o) {
+          const int no = p.seq.cu[o + 1] - p.seq.cu[o];
+          rank += (no > nb) || (no == nb && o < b);
+        }
+        sm.by_rank[rank] = (uint8_t)b;
+      }
+    }
+    set_up();
+    const uint32_t tmem_base = sm.tmem_base;
     const int grp = warp >> 2;
     const int quad = warp & 3;              // TMEM lane quadrant this warp may read
     const int row_in_tile = quad * 32 + lane;
@@ -630,6 +639,17 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
       if (lane == 0) mbar_arrive(bar_ae + (J % kAcc) * 8);
     };
 
+    int tr[MB];  // of this thread's rows in pass 1
+    float lv[MB];
+    if (p.two_pass) {
+#pragma unroll
+      for (int h = 0; h < MB; ++h) {
+        const int r = h * 128 + row_in_tile;
+        tr[h] = row_index(r);
+        lv[h] = row_weight(tr[h]);
+        if (grp == 0) put_tables(r, tr[h]);
+      }
+    }
     int J = grp;        // this group's next job
     int jg = 0;         // first job of the current pass
     int tg = 0;         // MB 2: pass-2 tiles of the units before this one
@@ -652,6 +672,13 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
         wait_full(Jn, 30);
         tmem_ld16_issue(acc_addr(Jn), ra);
       };
+      // the same if job Jn is one of the unit's and its products are there
+      auto try_fetch = [&](int Jn) {
+        if (Jn >= j_last || !mbar_test(bar_af + (Jn % kAcc) * 8, (uint32_t)(Jn / kAcc) & 1u)) return false;
+        tc_fence_after();
+        tmem_ld16_issue(acc_addr(Jn), ra);
+        return true;
+      };
 
       if (p.two_pass) {
         // ---- pass 1: per row, sum of exp2(s*c - ref) against a reference `ref` that only has to keep the sum inside
@@ -665,9 +692,8 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
         int lim[MB];
 #pragma unroll
         for (int h = 0; h < MB; ++h) {
-          const int t = sm.row_t[h * 128 + row_in_tile];
-          const int pos = n - p.W + t;
-          lim[h] = (t >= 0 && pos >= 0) ? (p.causal ? pos : n - 1) : -1;
+          const int pos = n - p.W + tr[h];
+          lim[h] = (tr[h] >= 0 && pos >= 0) ? (p.causal ? pos : n - 1) : -1;
           // rows that see no key (padding) get a reference that turns every exponential into 0
           ref[h] = lim[h] >= 0 ? -1e30f : 1e30f;
           zsum[h] = 0.0f;
@@ -755,8 +781,7 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
             }
           }
           release(J);
-          fetched = J + kGroups < j_last;
-          if (fetched) fetch(J + kGroups);
+          fetched = try_fetch(J + kGroups);
           half1(masked_tag, std::true_type{}, rb, rc, pb, s4, lm, key0 + 112);
           z_run += (s4[0] + s4[1]) + (s4[2] + s4[3]);
         };
@@ -802,13 +827,71 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
           sm.part_z[grp][h * 128 + row_in_tile] = lim[h] >= 0 ? zsum[h] : 0.0f;
         }
         __syncwarp();
-        if (lane == 0) mbar_arrive(smem_u32(&sm.stat_full[up]));
+        if (lane == 0) mbar_arrive(smem_u32(&sm.stat_full));
+        // ---- The group that was done first (the next job would be its) merges the groups' statistics, exchanges them with the
+        // cluster's other CTAs and leaves the rows' constants for pass 2: a thread per row (MB 2: two).
+        if (J == j_end) {
+          mbar_wait(smem_u32(&sm.stat_full), (uint32_t)it & 1u, abort_flag, p.status, 38, limit);
+          float m[MB], z[MB];
+#pragma unroll
+          for (int h = 0; h < MB; ++h) {
+            const int r = h * 128 + row_in_tile;
+            m[h] = sm.part_m[0][r];
+#pragma unroll
+            for (int gq = 1; gq < kGroups; ++gq) m[h] = fmaxf(m[h], sm.part_m[gq][r]);
+            z[h] = 0.0f;
+#pragma unroll
+            for (int gq = 0; gq < kGroups; ++gq) z[h] += sm.part_z[gq][r] * ex2(sm.part_m[gq][r] - m[h]);
+          }
+          if (p.cluster > 1) {  // (alone, the CTA's statistics are the unit's)
+            if (!cluster_known) cluster_wait();
+            cluster_known = true;
+            // the peers have read what was sent to them for the unit before
+            if (it > 0) mbar_wait_cluster(smem_u32(&sm.xchg_free), (uint32_t)(it - 1) & 1u, abort_flag, p.status, 31, limit);
+            if (quad == 0 && lane == 0) mbar_expect_tx(smem_u32(&sm.xchg_full), (uint32_t)(p.cluster * kRowsPad * 8));
+            // stores that count on the receiver's barrier when they land: no fence, no separate signal
+#pragma unroll 2
+            for (int q = 0; q < p.cluster; ++q) {
+              const uint32_t bar = map_peer(smem_u32(&sm.xchg_full), (uint32_t)q);
+#pragma unroll
+              for (int h = 0; h < MB; ++h)
+                st_async_f32x2(map_peer(smem_u32(&sm.peer[rank][h * 128 + row_in_tile]), (uint32_t)q), m[h], z[h], bar);
+            }
+            mbar_wait_cluster(smem_u32(&sm.xchg_full), (uint32_t)it & 1u, abort_flag, p.status, 32, limit);
+#pragma unroll
+            for (int h = 0; h < MB; ++h) m[h] = -1e30f, z[h] = 0.0f;
+#pragma unroll 4
+            for (int q = 0; q < p.cluster; ++q)
+#pragma unroll
+              for (int h = 0; h < MB; ++h) m[h] = fmaxf(m[h], sm.peer[q][h * 128 + row_in_tile].x);
+#pragma unroll 4
+            for (int q = 0; q < p.cluster; ++q)
+#pragma unroll
+              for (int h = 0; h < MB; ++h) {
+                const float2 v = sm.peer[q][h * 128 + row_in_tile];
+                z[h] += v.y * ex2(v.x - m[h]);
+              }
+            if (!one_round) {  // the slots may be written again
+              __syncwarp();
+              if (lane < p.cluster) mbar_arrive_remote(smem_u32(&sm.xchg_free), (uint32_t)lane);
+            }
+          }
+#pragma unroll
+          for (int h = 0; h < MB; ++h) put_row(up, h * 128 + row_in_tile, log2_sum(m[h], z[h]), lv[h]);
+          __syncwarp();
+          if (lane == 0) mbar_arrive(smem_u32(&sm.tab_full[up]));
+        }
         jg = j_end;
       }
 
       // ---- pass 2: for key row_in_tile of each tile, the sum over the job's rows of exp2(s*c - beta_row)
       {
         mbar_wait(smem_u32(&sm.tab_full[up]), ph, abort_flag, p.status, 39, limit);
+        if (one_round && p.cluster > 1) {  // nothing will be sent to a peer any more: said early, so that no CTA waits for it at its end
+          if (!cluster_known) cluster_wait();
+          cluster_arrive_relaxed();
+          cluster_known = cluster_left = true;
+        }
         // every valid row sees keys up to here; key i beyond it is seen by the rows with t >= i - (n - W)
         const int min_lim = p.causal ? n - min(p.W, n) : n - 1;
         const long long out0 = ((long long)ui.l * p.Hkv + ui.g) * p.seq.total + ui.tok0;
@@ -822,7 +905,7 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
           constexpr int hi = decltype(hi_tag)::value;  // 0: rows row0..row0+15, 1: rows row0+16..row0+31
           const float4* tab4 = reinterpret_cast<const float4*>(&sm.tab[up][row0]) + hi * 4;
           const float4* w4 = reinterpret_cast<const float4*>(&sm.wrow[row0]) + hi * 4;
-          const int4* t4 = reinterpret_cast<const int4*>(&sm.row_t[row0]) + hi * 4;
+          const char4* t4 = reinterpret_cast<const char4*>(&sm.row_t[row0]) + hi * 4;
 #pragma unroll
           for (int q4 = 0; q4 < 4; ++q4) {
             const float4 tb = tab4[q4];
@@ -844,7 +927,7 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
               }
             }
             if (masked) {
-              const int4 tt = t4[q4];
+              const char4 tt = t4[q4];
               if (tt.x < tau) a[0] = 0.0f;
               if (tt.y < tau) a[1] = 0.0f;
               if (tt.z < tau) a[2] = 0.0f;
@@ -873,8 +956,7 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
             tmem_ld_wait(rb);
             if (ci == n_chunks - 1) {
               release(J);
-              fetched = J + kGroups < j_last;
-              if (fetched) fetch(J + kGroups);
+              fetched = try_fetch(J + kGroups);
             } else {
               tmem_ld16_issue(abase + col + 32, ra);
             }
@@ -924,8 +1006,10 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
             }
           }
         }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(smem_u32(&sm.tab_free[up]));
+        if (!p.two_pass) {
+          __syncwarp();
+          if (lane == 0) mbar_arrive(smem_u32(&sm.tab_free[up]));
+        }
       }
       jg = j_last;
       tg += ui.T;
@@ -937,12 +1021,14 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
   __syncthreads();
   if (warp == kWarpMma) {
     tc_fence_after();
-    tmem_dealloc(tmem_base, kTmemCols);
+    tmem_dealloc(sm.tmem_base, kTmemCols);
   }
-  // no CTA may leave while a peer can still read its shared memory or arrive on its barriers
-  if (warp < kWarpStat || warp >= kWarpStat + kStatWarps) cluster_wait();  // the set-up's arrival
-  cluster_arrive();
+  // no CTA may leave while a peer can still write to its shared memory or arrive on its barriers
+  if (!cluster_known) cluster_wait();  // the set-up's arrival
+  if (!cluster_left) cluster_arrive();
   cluster_wait();
+  // (after a wait that ran out, statistics that this CTA did not wait for may still be on their way to it)
+  if (*abort_flag) __nanosleep(50000);
   if (p.late_wait && blockIdx.x == 0) ta_wait_for_prior_grid();  // this grid ends after the one it ran beside
 }
 
