@@ -26,10 +26,12 @@
 //   TMA producer        walks the units, publishes each one's description in a small ring, streams query and key tiles
 //   MMA issuer          TMEM owner; one elected lane issues, the warp around it is uniform
 //   2 statistics warps  one pass only: form the row constants from the log-sum-exps that the caller supplies, a unit ahead
-//   12 softmax warps    three groups of four. A "job" is one block of up to 128 score rows of one key tile in one pass; jobs
-//                       are dealt round-robin to the three groups and to the four accumulator stages, so that the products
-//                       of a group's next job are ready when it hands back the current one (four groups on four stages
-//                       waited 30 % of their time for their own stage to be refilled). With 129..256 score rows (MB 2) a
+//   16 softmax warps    four groups of four. A "job" is one block of up to 128 score rows of one key tile in one pass; jobs
+//                       are dealt round-robin to the four groups and to the four accumulator stages. Two groups at work
+//                       keep the special-function unit as busy as it can be (1105 cycles a job against 1095 with three);
+//                       the others hide a group's way from one job to the next: its stage's products (some 800 cycles)
+//                       and the signals around them. Three groups with a stage to spare took 2 to 5 % longer. With
+//                       129..256 score rows (MB 2) a
 //                       tile is two consecutive jobs, one per block of 128 rows; in pass 2 their partial sums meet in a
 //                       shared-memory ring. Between the passes the group that ends the first one first merges the row
 //                       statistics, exchanges them over the cluster and forms the row constants for pass 2.
@@ -73,13 +75,13 @@ constexpr int kHalfBytes = kTileN * 128;          // one 64-column half of a 128
 constexpr int kKTileBytes = 2 * kHalfBytes;       // 32 KB
 constexpr int kMaxCluster = 16;                   // more than 8 CTAs is a non-portable cluster size; sm_100 allows 16
 constexpr int kRankedSeqs = 256;                  // (an index is a byte) sequences of a ragged batch that the kernel itself sorts by length
-constexpr int kGroups = 3;                        // softmax warpgroups
+constexpr int kGroups = 4;                        // softmax warpgroups
 constexpr int kSoftWarps = kGroups * 4;
-constexpr int kThreads = (kGroups + 1) * 128;     // 512
+constexpr int kThreads = (kGroups + 1) * 128;     // 640
 // Register split after set-up (setmaxnreg); the shares must fit in threads x registers at launch:
-// 512 threads x 128 = 65536 = 12*32*152 + 4*32*56
-constexpr int kRegsSoftmax = 152;
-constexpr int kRegsOther = 56;
+// 640 threads x 96 = 61440 = 16*32*104 + 4*32*64
+constexpr int kRegsSoftmax = 104;
+constexpr int kRegsOther = 64;
 constexpr int kRegsNeeded = (kSoftWarps * kRegsSoftmax + 4 * kRegsOther) * 32;
 
 // Of every 16 exponentials, this many (an even number: they are taken in pairs) run on the FMA pipe with 129 to 256 score
@@ -147,9 +149,9 @@ struct alignas(1024) ScoreSmem {
   static constexpr int kRowsPad = MB * 128;
   uint8_t q[kQBufs][MB * 2 * kHalfBytes];  // [buffer][half][MB*128 rows][128 B]
   uint8_t k[kStages][kKTileBytes];         // [stage][half][128 rows][128 B]
-  // [softmax group][row]: reference and sum of the group's keys (one unit's at a time: a softmax warp waits for the row
-  // constants that are formed from them before it goes on to the next unit)
-  float part_m[kGroups][kRowsPad], part_z[kGroups][kRowsPad];
+  // [softmax group][row of its block]: reference and sum of the group's keys (one unit's at a time: a softmax warp waits for
+  // the row constants that are formed from them before it goes on to the next unit)
+  float part_m[kGroups][128], part_z[kGroups][128];
   static constexpr int kPeers = MB == 1 ? kMaxCluster : 8;  // largest cluster the exchange has room for
   float2 peer[kPeers][kRowsPad];           // row statistics (reference, sum) as the CTAs of the cluster sent them
   // [unit parity][row] pass-2 constant of the row; behind them the form that ex2 takes, for rows whose own is the polynomial's
@@ -623,6 +625,8 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
     const int grp = warp >> 2;
     const int quad = warp & 3;              // TMEM lane quadrant this warp may read
     const int row_in_tile = quad * 32 + lane;
+    static_assert(kGroups % MB == 0, "a group's jobs are all of one row block");
+    const int block = MB == 2 ? grp & 1 : 0;  // row block of this group's jobs (a unit has an even number of jobs)
     const uint32_t tlane = tmem_base + ((uint32_t)(quad * 32) << 16);
     const uint32_t bar_af = smem_u32(&sm.acc_full[0]), bar_ae = smem_u32(&sm.acc_empty[0]);
     const float c = p.c;
@@ -688,16 +692,10 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
         // before the accumulator stage is released and does not wait for the tile's last exponentials: it uses the sum
         // without the last 16 keys and, for those, their largest score. The polynomial exponentials saturate at 2^126,
         // which the same check catches; so does a row without a reference yet (ref -1e30).
-        float ref[MB], zsum[MB];
-        int lim[MB];
-#pragma unroll
-        for (int h = 0; h < MB; ++h) {
-          const int pos = n - p.W + tr[h];
-          lim[h] = (tr[h] >= 0 && pos >= 0) ? (p.causal ? pos : n - 1) : -1;
-          // rows that see no key (padding) get a reference that turns every exponential into 0
-          ref[h] = lim[h] >= 0 ? -1e30f : 1e30f;
-          zsum[h] = 0.0f;
-        }
+        const int pos = n - p.W + tr[block];
+        const int lim = (tr[block] >= 0 && pos >= 0) ? (p.causal ? pos : n - 1) : -1;  // last key that the thread's row sees
+        // rows that see no key (padding) get a reference that turns every exponential into 0
+        float ref = lim >= 0 ? -1e30f : 1e30f, zsum = 0.0f;
         constexpr float kSumLimit = 1.0e18f;  // about 2^60
         // 16 keys of one row: adds exp2(s*c - rc) to the four sums; `mix`: some of them on the FMA pipe. Masked tiles
         // drop keys beyond `lm`.
@@ -788,44 +786,24 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
         const int j_end = jg + n_jobs;
         bool first = true;
         for (; J < j_end; J += kGroups) {
-          const int j = J - jg;
-          const int key0 = (ui.t_begin + j / MB) * kTileN;
+          const int key0 = (ui.t_begin + (J - jg) / MB) * kTileN;
           if (!fetched) fetch(J);
-          // MB 2: the row block of a group's jobs alternates; its state is swapped into slot 0
-          const int h = MB == 2 ? j & 1 : 0;
-          float& rc = ref[0];
-          float& zr = zsum[0];
-          if (MB == 2 && h == 1) {
-            const float tr = ref[0], tz = zsum[0];
-            const int tl = lim[0];
-            ref[0] = ref[MB - 1], zsum[0] = zsum[MB - 1], lim[0] = lim[MB - 1];
-            ref[MB - 1] = tr, zsum[MB - 1] = tz, lim[MB - 1] = tl;
-          }
           // tiles that every row of the warp sees completely take the unmasked path (rows that see nothing at all,
           // i.e. padding, still run: their sums are never used)
-          const bool masked = __any_sync(0xffffffffu, lim[0] >= 0 && key0 + kTileN - 1 > lim[0]);
+          const bool masked = __any_sync(0xffffffffu, lim >= 0 && key0 + kTileN - 1 > lim);
           if (first) {  // the reference of the rows: from the 16 keys in flight
             tmem_ld_wait(ra);
-            const float mx = masked ? max16(std::true_type{}, ra, lim[0], key0) : max16(std::false_type{}, ra, lim[0], key0);
-            if (rc < -1e29f && mx > -INFINITY) rc = mx * c;
-            first = MB == 2 && J < jg + kGroups;  // MB 2: the group's second job is the first of the other block
+            const float mx = masked ? max16(std::true_type{}, ra, lim, key0) : max16(std::false_type{}, ra, lim, key0);
+            if (ref < -1e29f && mx > -INFINITY) ref = mx * c;
+            first = false;
           }
-          if (masked) job1(std::true_type{}, rc, zr, lim[0], key0);
-          else job1(std::false_type{}, rc, zr, lim[0], key0);
-          if (MB == 2 && h == 1) {
-            const float tr = ref[0], tz = zsum[0];
-            const int tl = lim[0];
-            ref[0] = ref[MB - 1], zsum[0] = zsum[MB - 1], lim[0] = lim[MB - 1];
-            ref[MB - 1] = tr, zsum[MB - 1] = tz, lim[MB - 1] = tl;
-          }
+          if (masked) job1(std::true_type{}, ref, zsum, lim, key0);
+          else job1(std::false_type{}, ref, zsum, lim, key0);
         }
         // ---- the group's statistics of the unit; rows that see no key at all (padding, window positions before the
         // sequence start) stay mute
-#pragma unroll
-        for (int h = 0; h < MB; ++h) {
-          sm.part_m[grp][h * 128 + row_in_tile] = lim[h] >= 0 ? ref[h] : -1e30f;
-          sm.part_z[grp][h * 128 + row_in_tile] = lim[h] >= 0 ? zsum[h] : 0.0f;
-        }
+        sm.part_m[grp][row_in_tile] = lim >= 0 ? ref : -1e30f;
+        sm.part_z[grp][row_in_tile] = lim >= 0 ? zsum : 0.0f;
         __syncwarp();
         if (lane == 0) mbar_arrive(smem_u32(&sm.stat_full));
         // ---- The group that was done first (the next job would be its) merges the groups' statistics, exchanges them with the
@@ -835,13 +813,12 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
           float m[MB], z[MB];
 #pragma unroll
           for (int h = 0; h < MB; ++h) {
-            const int r = h * 128 + row_in_tile;
-            m[h] = sm.part_m[0][r];
+            m[h] = sm.part_m[h][row_in_tile];
 #pragma unroll
-            for (int gq = 1; gq < kGroups; ++gq) m[h] = fmaxf(m[h], sm.part_m[gq][r]);
+            for (int gq = h + MB; gq < kGroups; gq += MB) m[h] = fmaxf(m[h], sm.part_m[gq][row_in_tile]);
             z[h] = 0.0f;
 #pragma unroll
-            for (int gq = 0; gq < kGroups; ++gq) z[h] += sm.part_z[gq][r] * ex2(sm.part_m[gq][r] - m[h]);
+            for (int gq = h; gq < kGroups; gq += MB) z[h] += sm.part_z[gq][row_in_tile] * ex2(sm.part_m[gq][row_in_tile] - m[h]);
           }
           if (p.cluster > 1) {  // (alone, the CTA's statistics are the unit's)
             if (!cluster_known) cluster_wait();
@@ -964,16 +941,15 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
           }
         };
         for (; J < j_last; J += kGroups) {
-          const int j = J - jg, h = MB == 2 ? j & 1 : 0;
-          const int tl = j / MB;  // the pass walks the CTA's tiles backwards after a first pass
+          const int tl = (J - jg) / MB;  // the pass walks the CTA's tiles backwards after a first pass
           const int key = (ui.t_begin + (p.two_pass ? ui.T - 1 - tl : tl)) * kTileN + row_in_tile;
-          const int n_chunks = (min(128, p.rows - h * 128) + 31) >> 5;
+          const int n_chunks = (min(128, p.rows - block * 128) + 31) >> 5;
           if (!fetched) fetch(J);
           sA4[0] = sA4[1] = sA4[2] = sA4[3] = 0.0f;
           sP = 0.0f;
           // only the last W-1 keys of a sequence are hidden from some rows: those tiles take the masked path
-          if (__all_sync(0xffffffffu, key <= min_lim || key >= n)) job2(std::false_type{}, h * 128, n_chunks, 0);
-          else job2(std::true_type{}, h * 128, n_chunks, p.causal ? key - (n - p.W) : -1);
+          if (__all_sync(0xffffffffu, key <= min_lim || key >= n)) job2(std::false_type{}, block * 128, n_chunks, 0);
+          else job2(std::true_type{}, block * 128, n_chunks, p.causal ? key - (n - p.W) : -1);
           float sA = (sA4[0] + sA4[1]) + (sA4[2] + sA4[3]);
           if (MB == 2) {
             // The two row blocks of a tile are consecutive jobs of two different groups. The group of block 0 leaves
@@ -981,7 +957,7 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
             // its own and stores. Neither waits for the other unless the ring is full (block 0 four tiles ahead).
             const int r = (tg + tl) % kRing;
             const uint32_t rph = (uint32_t)((tg + tl) / kRing) & 1u;
-            if (h == 0) {
+            if (block == 0) {
               mbar_wait(smem_u32(&sm.pfree[r]), rph ^ 1u, abort_flag, p.status, 33, limit);
               sm.psum[r][0][row_in_tile] = sA;
               if (PM == kOutAP) sm.psum[r][1][row_in_tile] = sP;
@@ -995,7 +971,7 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
               if (lane == 0) mbar_arrive(smem_u32(&sm.pfree[r]));
             }
           }
-          if (h == MB - 1 && key < n && !*abort_flag) {
+          if (block == MB - 1 && key < n && !*abort_flag) {
             const long long o = out0 + key;
             if (PM == kOutFused) {
               p.u[o] = sA;
@@ -1089,13 +1065,12 @@ cudaError_t launch_variant(ta_ctx* ctx, const CUtensorMap& mq, const CUtensorMap
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   // Persistent grid: as many clusters as can be resident at once (queried once per cluster size). CTAs per unit: the size
-  // with the shortest busiest CTA, counted in half jobs: two per job, a tile-time of overhead per unit, and for the
-  // statistics exchange of a unit that spans several CTAs another tile-time with 256 rows, 1.5 with 128. Where every cluster
-  // has one unit a pass takes whole rounds of the softmax groups; with more, the next unit's jobs fill the last round.
-  // Measured on 32 to 640 units of 1000 to 16384 tokens, 100 sizes per row count, every size forced in turn: what this takes
-  // is 0.1 % slower on average than the best (1.3 % with every pass rounded up and two tile-times for the exchange, up to
-  // 17 %: 152 units of 2048 tokens with 256 rows 100.6 us with 1 CTA, 87 us with 2; 0.5 % and up to 9 % with 128 rows: 320
-  // units of 4096 tokens 152 us with 1, 139 us with 2).
+  // with the shortest busiest CTA, counted in half jobs: two per job, and per unit what its start and the statistics between the
+  // passes take, four per row block with one CTA per unit, 5 (128 rows) or 8 (256) with several. Measured on 32 to 512 units of
+  // 1000 to 12000 tokens, 80 sizes per row count, every size forced in turn: what this takes is 0.2 % (256 rows) and 0.00 %
+  // (128) slower on average than the best, at most 4.1 % and 0.2 % (152 units of 2048 tokens with 256 rows: 98 us with 1 CTA,
+  // 83 us with 2; 320 units of 4096 tokens with 128 rows: 149 us with 1, 134 us with 2). Jobs are not rounded up to whole
+  // rounds of the softmax groups: fewer than four at work take little longer per job.
   // (Choosing more CTAs per unit so that the keys of all units in flight fit in L2 was measured and lost: 16 x 32768
   // tokens, 8 CTAs per unit 2.02 ms against 1.63 ms.)
   int best_cl = ctx->score_force_cluster;
@@ -1119,9 +1094,8 @@ cudaError_t launch_variant(ta_ctx* ctx, const CUtensorMap& mq, const CUtensorMap
     if (ctx->score_force_cluster > 0) break;
     const int avail = max_clusters[cl];
     const long long rounds = (sp.units + avail - 1) / avail;
-    long long jobs = (long long)((tiles_max + cl - 1) / cl) * MB;
-    if (rounds == 1) jobs = (jobs + kGroups - 1) / kGroups * kGroups;
-    const long long cost = rounds * (2 * jobs + (cl == 1 ? 2 * MB : MB == 1 ? 5 : 8));
+    const long long jobs = (long long)((tiles_max + cl - 1) / cl) * MB;
+    const long long cost = rounds * (2 * jobs + (cl == 1 ? 4 * MB : MB == 1 ? 5 : 8));
     if (sp.flat) {  // equal shares whatever the number of units: nothing to gain from more CTAs per unit
       best_cl = cl;
       best_cost = 0;
