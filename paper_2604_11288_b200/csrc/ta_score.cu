@@ -84,11 +84,13 @@ constexpr int kRegsSoftmax = 104;
 constexpr int kRegsOther = 64;
 constexpr int kRegsNeeded = (kSoftWarps * kRegsSoftmax + 4 * kRegsOther) * 32;
 
-// Of every 16 exponentials, this many (an even number: they are taken in pairs) run on the FMA pipe with 129 to 256 score
-// rows, in tiles that are not masked. Back to back the kernel runs into the board's 1000 W limit, and a polynomial costs more
-// energy than ex2 while it relieves the special-function unit: 8 layers of 16 x 32768 tokens with 256 rows 0: 6.22 ms,
-// 2: 6.02 ms, more: the same.
-// With up to 128 rows no share pays (one pass over 32 x 8111 tokens: 0: 122 us, 4: 125 us) and none is taken.
+// Of every 16 exponentials, two (they are taken in pairs) run on the FMA pipe in tiles that are not masked, which relieves the
+// special-function unit. Back to back the kernel runs into the board's 1000 W limit, and a polynomial costs more energy than
+// ex2, so that a larger share does not pay.
+// 129 to 256 score rows: a cubic. 8 layers of 16 x 32768 tokens, share 0: 6.22 ms, 2: 6.02 ms, more: the same.
+// Up to 128 rows: a polynomial of degree 5, so that a score is as precise as ex2 alone gives it (2-norm error of 4096 tokens
+// 8.7e-8 with either). 32 layers of 4096 tokens alone, share 0: 139 us, 2: 134 us, 4: 136 us, 6: 137 us; back to back 120.5,
+// 119, 121, 125 us; 2 layers of 16384 tokens 73.0, 70.5, 70.1, 71.9 us.
 #ifndef TA_SCORE_POLY_MB2
 #define TA_SCORE_POLY_MB2 2
 #endif
@@ -97,7 +99,7 @@ constexpr int kRegsNeeded = (kSoftWarps * kRegsSoftmax + 4 * kRegsOther) * 32;
 // poly_pair is true (spread evenly).
 template <int MB>
 __host__ __device__ constexpr int poly_pairs() {
-  return MB == 1 ? 0 : TA_SCORE_POLY_MB2 / 2;
+  return MB == 1 ? 1 : TA_SCORE_POLY_MB2 / 2;
 }
 template <int MB>
 __host__ __device__ constexpr bool poly_pair(int q2) {
@@ -155,7 +157,7 @@ struct alignas(1024) ScoreSmem {
   static constexpr int kPeers = MB == 1 ? kMaxCluster : 8;  // largest cluster the exchange has room for
   float2 peer[kPeers][kRowsPad];           // row statistics (reference, sum) as the CTAs of the cluster sent them
   // [unit parity][row] pass-2 constant of the row; behind them the form that ex2 takes, for rows whose own is the polynomial's
-  float tab[2][poly_pairs<MB>() ? 2 * kRowsPad : kRowsPad];
+  float tab[2][MB == 2 && poly_pairs<MB>() ? 2 * kRowsPad : kRowsPad];
   float wrow[kRowsPad];                    // pension weight per row
   int8_t row_t[kRowsPad];                  // window index t of the row, -1 for padding rows
   float psum[kRing][2][128];               // MB 2: [ring slot][A|P][key] partial sums of row block 0
@@ -198,6 +200,33 @@ __device__ __forceinline__ void exp2_poly2(float& e0, float& e1, float s0, float
       "mov.b64 {%0, %1}, p;\n\tmov.b64 {%2, %3}, y;\n\t}"
       : "=f"(p0), "=f"(p1), "=r"(y0), "=r"(y1)
       : "f"(t0), "f"(t1), "f"(kPolyRange), "f"(kPolyMagic), "f"(-1.0f), "f"(kC3), "f"(kC2), "f"(kC1), "f"(kC0));
+  e0 = __uint_as_float((y0 << 23) + __float_as_uint(p0));
+  e1 = __uint_as_float((y1 << 23) + __float_as_uint(p1));
+}
+// Two values of exp2(x) as precise as ex2's: a polynomial of degree 5 for 2^f on [0, 1) (minimax in relative error, 7.5e-8) of
+// the same argument that ex2 would take. Arguments are clamped below at -126; CLAMP: also above at 126.
+// Not a number becomes the largest finite number, which mutes the row in pass 1 as a sum that is none does.
+constexpr float kQ0 = 0.9999999404f, kQ1 = 0.6931530833f, kQ2 = 0.2401536107f, kQ3 = 0.05582631752f, kQ4 = 0.008989339694f, kQ5 = 0.001877576695f;
+template <bool CLAMP>
+__device__ __forceinline__ void exp2_poly5(float& e0, float& e1, float x0, float x1) {
+  asm("max.NaN.f32 %0, %0, %2;\n\tmax.NaN.f32 %1, %1, %2;" : "+f"(x0), "+f"(x1) : "f"(-126.0f));
+  if (CLAMP) asm("min.NaN.f32 %0, %0, %2;\n\tmin.NaN.f32 %1, %1, %2;" : "+f"(x0), "+f"(x1) : "f"(126.0f));
+  float p0, p1;
+  uint32_t y0, y1;
+  asm("{\n\t.reg .b64 x, m, y, w, f, p, k;\n\t"
+      "mov.b64 x, {%4, %5};\n\tmov.b64 m, {%6, %6};\n\tmov.b64 k, {%7, %7};\n\t"
+      "fma.rm.f32x2 y, x, k, m;\n\t"        // 1.5*2^23 + floor(x)
+      "mov.b64 k, {%8, %8};\n\t"
+      "fma.rn.f32x2 w, y, k, m;\n\t"        // -floor(x), exact
+      "add.rn.f32x2 f, x, w;\n\t"           // x - floor(x), exact
+      "mov.b64 p, {%9, %9};\n\tmov.b64 k, {%10, %10};\n\tfma.rn.f32x2 p, p, f, k;\n\t"
+      "mov.b64 k, {%11, %11};\n\tfma.rn.f32x2 p, p, f, k;\n\t"
+      "mov.b64 k, {%12, %12};\n\tfma.rn.f32x2 p, p, f, k;\n\t"
+      "mov.b64 k, {%13, %13};\n\tfma.rn.f32x2 p, p, f, k;\n\t"
+      "mov.b64 k, {%14, %14};\n\tfma.rn.f32x2 p, p, f, k;\n\t"
+      "mov.b64 {%0, %1}, p;\n\tmov.b64 {%2, %3}, y;\n\t}"
+      : "=f"(p0), "=f"(p1), "=r"(y0), "=r"(y1)
+      : "f"(x0), "f"(x1), "f"(12582912.0f), "f"(1.0f), "f"(-1.0f), "f"(kQ5), "f"(kQ4), "f"(kQ3), "f"(kQ2), "f"(kQ1), "f"(kQ0));
   e0 = __uint_as_float((y0 << 23) + __float_as_uint(p0));
   e1 = __uint_as_float((y1 << 23) + __float_as_uint(p1));
 }
@@ -358,9 +387,9 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
   auto row_weight = [&](int t) { return PM == kOutFused && t >= 0 ? log2f(fmaf(p.delta, p.wrow[t], p.alpha)) : 0.0f; };
   auto put_row = [&](int up, int r, float lse2, float lv) {
     const float beta = lse2 - lv;
-    const bool poly = poly_pair<MB>((r & 15) / 2);
+    const bool poly = MB == 2 && poly_pair<MB>((r & 15) / 2);
     sm.tab[up][r] = poly ? poly_bias(beta) : -beta;
-    if constexpr (poly_pairs<MB>() > 0) {
+    if constexpr (MB == 2 && poly_pairs<MB>() > 0) {
       if (poly) sm.tab[up][kRowsPad + r] = -beta;
     }
   };
@@ -710,7 +739,12 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
           for (int q = 0; q < 16; q += 2) {
             float e0, e1;
             if (mix && !masked && poly_pair<MB>(q / 2)) {
-              exp2_poly2(e0, e1, v[q], v[q + 1], c252, pbias, pbias);
+              if constexpr (MB == 2) {
+                exp2_poly2(e0, e1, v[q], v[q + 1], c252, pbias, pbias);
+              } else {
+                fma2(e0, e1, v[q], v[q + 1], c, -rc, -rc);
+                exp2_poly5<true>(e0, e1, e0, e1);
+              }
             } else {
               fma2(e0, e1, v[q], v[q + 1], c, -rc, -rc);
               e0 = ex2(e0);
@@ -891,9 +925,14 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
 #pragma unroll
             for (int e = 0; e < 4; e += 2) {
               if (poly_pair<MB>(2 * q4 + e / 2) && !masked) {
-                exp2_poly2(a[e], a[e + 1], cur[4 * q4 + e], cur[4 * q4 + e + 1], c252, tbv[e], tbv[e + 1]);
+                if constexpr (MB == 2) {
+                  exp2_poly2(a[e], a[e + 1], cur[4 * q4 + e], cur[4 * q4 + e + 1], c252, tbv[e], tbv[e + 1]);
+                } else {
+                  fma2(a[e], a[e + 1], cur[4 * q4 + e], cur[4 * q4 + e + 1], c, tbv[e], tbv[e + 1]);
+                  exp2_poly5<false>(a[e], a[e + 1], a[e], a[e + 1]);
+                }
               } else {
-                if (poly_pair<MB>(2 * q4 + e / 2)) {
+                if (MB == 2 && poly_pair<MB>(2 * q4 + e / 2)) {
                   const float2 nb = *reinterpret_cast<const float2*>(&sm.tab[up][kRowsPad + row0 + hi * 16 + 4 * q4 + e]);
                   tbv[e] = nb.x;
                   tbv[e + 1] = nb.y;

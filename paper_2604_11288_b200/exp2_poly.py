@@ -1,5 +1,5 @@
-"""Coefficients of the cubic that the score kernel uses for 2^f on [0, 1) (csrc/ta_score.cu, kC0..kC3), and a
-bit-level model of the kernel's polynomial exp2 in numpy.
+"""Coefficients of the polynomials that the score kernel uses for 2^f on [0, 1) (csrc/ta_score.cu: the cubic kC0..kC3 and the
+one of degree 5, kQ0..kQ5), and bit-level models of the kernel's polynomial exp2 in numpy.
 
 Run as a script to print the coefficients; tests/test_exp2_poly.py checks that the constants in the CUDA source are
 the ones this derivation gives and that the model stays inside the stated error.
@@ -66,6 +66,24 @@ def exp2_poly_model(s, c, beta, coef):
     return (bits & 0xFFFFFFFF).astype(np.uint32).view(f32)
 
 
+def exp2_poly5_model(x, coef, clamp=False):
+    """What exp2_poly5(x) computes, step by step in fp32 (numpy): clamp, round-down add onto 1.5 * 2^23, exact fraction, Horner
+    polynomial, exponent splice."""
+    f32 = np.float32
+    x = np.maximum(np.asarray(x, f32), f32(-126.0))
+    if clamp:
+        x = np.minimum(x, f32(126.0))
+    y = np.floor(x.astype(np.float64) + 12582912.0)                       # an integer below 2^24: exact in fp32
+    f = (x.astype(np.float64) + (12582912.0 - y)).astype(f32)             # exact
+    p = f32(coef[5])
+    for ci in coef[4::-1]:
+        p = (np.asarray(p, np.float64) * f.astype(np.float64) + np.float64(ci)).astype(f32)
+    j = (y - 12582912.0).astype(np.int64)
+    bits = p.view(np.int32).astype(np.int64) + (j << 23)
+    return (bits & 0xFFFFFFFF).astype(np.uint32).view(f32)
+
+
 if __name__ == "__main__":
-    coef, err = remez_exp2()
-    print("coefficients", [float(v) for v in coef], "max relative error", err)
+    for degree in (3, 5):
+        coef, err = remez_exp2(degree)
+        print("degree", degree, "coefficients", [float(v) for v in coef], "max relative error", err)

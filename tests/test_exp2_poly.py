@@ -45,3 +45,23 @@ def test_model_error_and_clamps():
     # exact powers of two come out within the polynomial's error at f = 0
     p2 = ep.exp2_poly_model((np.arange(-100, 100) / c).astype(np.float32), c, 0.0, coef).astype(np.float64)
     assert np.max(np.abs(p2 / np.exp2((np.arange(-100, 100) / c).astype(np.float32).astype(np.float64) * c) - 1)) < 1e-4
+
+
+def test_degree_5_is_the_remez_solution_and_as_precise_as_ex2():
+    m = re.search(r"kQ0 = ([0-9.eE+-]+)f, kQ1 = ([0-9.eE+-]+)f, kQ2 = ([0-9.eE+-]+)f, kQ3 = ([0-9.eE+-]+)f, "
+                  r"kQ4 = ([0-9.eE+-]+)f, kQ5 = ([0-9.eE+-]+)f", open(SRC).read())
+    assert m, "coefficients not found in ta_score.cu"
+    src = np.array([float(g) for g in m.groups()], np.float32)
+    coef, err = ep.remez_exp2(5)
+    assert err < 7.6e-8
+    np.testing.assert_allclose(src, coef, rtol=0, atol=2e-7)
+    rng = np.random.default_rng(1)
+    x = rng.uniform(-126.0, 60.0, size=400000).astype(np.float32)
+    got = ep.exp2_poly5_model(x, src).astype(np.float64)
+    # the polynomial's error, its fp32 coefficients' and Horner steps' roundings: below 2^-22, the bound of ex2.approx
+    assert np.max(np.abs(got / np.exp2(x.astype(np.float64)) - 1.0)) < 2.0 ** -22
+    # masked rows and far below: a tiny positive number; far above, clamped: 2^126, which pass 1 notices
+    lo = ep.exp2_poly5_model(np.array([-np.inf, -1e30, -500.0], np.float32), src)
+    assert (lo >= 0).all() and (lo < 2e-38).all()
+    hi = ep.exp2_poly5_model(np.array([np.inf, 1e30, 127.0], np.float32), src, clamp=True)
+    assert np.isfinite(hi).all() and (hi > 8e37).all()

@@ -56,3 +56,31 @@ def test_more_than_eight_ctas_for_a_handful_of_units(L, Hkv, n):
     assert 8 < size <= 16
     ref, _ = _score(L, 1, Hkv, n, 32, 1)
     np.testing.assert_allclose(got, ref, rtol=SCORE_RTOL, atol=SCORE_ATOL)
+
+
+@pytest.mark.parametrize("n", [1000, 4096])
+def test_128_rows_are_as_precise_as_fp32_sums(n):
+    # Every term carries the rounding of its exponent (|x| < 32: 2^-20 absolute, 0.7 of it relative) and of its exponential
+    # (2^-22), each term's own; the row's normaliser moves all of a row's terms by its own error (2^-22). Over 128 rows the
+    # terms' errors average out: 2-norm error at most 2^-20 * 0.7 / sqrt(128) + 2^-22 < 3e-7. (A cubic in 2 of 16: 1.9e-6.)
+    L, Hkv, W, d = 2, 4, 32, 128
+    g = torch.Generator(device="cuda")
+    g.manual_seed(n)
+    q = torch.randn((L, 1, 4 * Hkv, W, d), generator=g, dtype=torch.bfloat16, device="cuda")
+    k = torch.randn((L, 1, Hkv, n, d), generator=g, dtype=torch.bfloat16, device="cuda")
+    pol = ta.ta_policy_default(ta.TA_PRESET_THEOREM, 4)
+    batch = ta.make_batch(L, 1, n, n, n)
+    ctx = ta.ta_ctx_create(0, ta.ta_scratch_bytes(batch, 4 * Hkv, Hkv, d, 4, pol))
+    try:
+        u = torch.empty((L, Hkv, n), device="cuda")
+        ta.ta_score_weighted(ctx, pol, batch, 4 * Hkv, Hkv, d, ta.view(q), ta.view(k), None, u,
+                             torch.cuda.current_stream().cuda_stream)
+        assert ta.ta_ctx_poll(ctx) == ta.TA_OK
+    finally:
+        ta.ta_ctx_destroy(ctx)
+    t = torch.arange(W - 1, -1, -1, device="cuda", dtype=torch.double)
+    w = (pol.alpha + pol.delta * (1 - pol.pension_rho) * pol.pension_rho ** t).view(-1, 1)
+    s = torch.einsum("lghd,lgnd->lghn", q.double().view(L, Hkv, 4 * W, d), k[:, 0].double()) / d ** 0.5
+    hidden = torch.arange(n, device="cuda").view(1, -1) > torch.arange(n - W, n, device="cuda").view(-1, 1)
+    want = (torch.softmax(s.view(L, Hkv, 4, W, n).masked_fill(hidden, float("-inf")), -1) * w).sum((2, 3))
+    assert (u.double() - want).norm() / want.norm() < 3e-7
