@@ -225,8 +225,11 @@ ta_status ta_ctx_create(int device, size_t scratch_bytes, ta_ctx** out) {
   c->device = device;
   c->sm_count = prop.multiProcessorCount;
   c->scratch_bytes = scratch_bytes;
-  cudaError_t e = cudaMalloc(&c->d_status, sizeof(ta_dev_status));
-  if (e == cudaSuccess) e = cudaMemset(c->d_status, 0, sizeof(ta_dev_status));
+  // the status block and, behind it, the decode step's words
+  constexpr size_t kWords = 256, kSyncBytes = kWords + kStreamWords * sizeof(ulonglong2);
+  cudaError_t e = cudaMalloc(&c->d_status, kSyncBytes);
+  if (e == cudaSuccess) e = cudaMemset(c->d_status, 0, kSyncBytes);
+  c->stream_sync.words = reinterpret_cast<ulonglong2*>(reinterpret_cast<uint8_t*>(c->d_status) + kWords);
   if (e == cudaSuccess && scratch_bytes) e = cudaMalloc(&c->scratch, scratch_bytes);
   for (int i = 0; e == cudaSuccess && i < 8; ++i) e = cudaEventCreate(&c->ev[i]);
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&c->copy_in, cudaStreamNonBlocking);
@@ -295,6 +298,8 @@ ta_status ta_ctx_poll(ta_ctx* ctx) {
   if (e != cudaSuccess) return cuda_fail(ctx, e);
   if (st.code != 0) {
     cudaMemset(ctx->d_status, 0, sizeof st);
+    if (st.code == TA_ERR_TIMEOUT)  // a block that gave up waiting for its word may have left it to come
+      cudaMemset(ctx->stream_sync.words, 0, kStreamWords * sizeof(ulonglong2));
     ctx->cached_epoch = 0;
     return (ta_status)st.code;
   }
@@ -966,15 +971,8 @@ ta_status ta_compress_budgets(ta_ctx* ctx, const ta_patterns* pats, const ta_pol
 
 // ---------------------------------------------------------------------------------------------- decode loop
 namespace {
-struct StreamLayout {
-  size_t info, end;
-};
-StreamLayout stream_layout(const ta_stream& st) {
-  StreamLayout L;
-  L.info = 0;
-  L.end = align_up((size_t)st.batch * sizeof(ta_stream_seq_info));
-  return L;
-}
+// The step needs no scratch any more; what callers must provide is unchanged (16 bytes per sequence).
+size_t stream_scratch(const ta_stream& st) { return align_up((size_t)st.batch * 16); }
 ta_status check_stream(const ta_stream* st) {
   if (!st) return TA_ERR_INVALID_ARG;
   if (st->n_layers < 1 || st->batch < 1 || st->Hkv < 1 || st->K < 1) return TA_ERR_INVALID_ARG;
@@ -991,7 +989,7 @@ ta_status check_stream(const ta_stream* st) {
 ta_status ta_stream_scratch_bytes(const ta_stream* st, size_t* out_bytes) {
   if (!out_bytes || !st) return TA_ERR_INVALID_ARG;
   if (st->n_layers < 1 || st->batch < 1 || st->Hkv < 1 || st->K < 1) return TA_ERR_INVALID_ARG;
-  *out_bytes = stream_layout(*st).end + kAlign;
+  *out_bytes = stream_scratch(*st) + kAlign;
   return TA_OK;
 }
 
@@ -1003,12 +1001,10 @@ ta_status ta_stream_step(ta_ctx* ctx, const ta_patterns* pats, const ta_policy* 
   if (s == TA_OK) s = check_stream(st);
   if (s != TA_OK) return s;
   if (pats->device != ctx->device) return TA_ERR_INVALID_ARG;
-  const StreamLayout L = stream_layout(*st);
-  if (L.end > ctx->scratch_bytes) return TA_ERR_SCRATCH_TOO_SMALL;
+  if (stream_scratch(*st) > ctx->scratch_bytes) return TA_ERR_SCRATCH_TOO_SMALL;
   DeviceGuard guard(ctx->device);
   ctx->cached_epoch = 0;  // the scratch is shared with ta_compress's per-sequence cache
   cudaStream_t stream = (cudaStream_t)stream_v;
-  uint8_t* sc = ctx->scratch;
   ta_stream_dev d = {};
   d.n_layers = st->n_layers;
   d.B = st->batch;
@@ -1028,11 +1024,11 @@ ta_status ta_stream_step(ta_ctx* ctx, const ta_patterns* pats, const ta_policy* 
   d.tok_ring = st->tok_ring;
   d.anc_B = st->anc_B;
   d.anc_L = st->anc_L;
-  auto* info = reinterpret_cast<ta_stream_seq_info*>(sc + L.info);
   const bool evict = st->cache_len + 1 > st->K;
+  ta_stream_sync sync = ctx->stream_sync;
+  sync.wait_limit_ns = ctx->wait_limit_ns ? ctx->wait_limit_ns : 2000000000ull;
 
-  cudaError_t e = ta_launch_stream_seq(d, pats, *policy, new_ids, info, ctx->d_status, stream);
-  if (e == cudaSuccess) e = ta_launch_stream_step(d, *policy, info, attn, evicted_pos, ctx->d_status, stream);
+  cudaError_t e = ta_launch_stream_step(d, pats, *policy, new_ids, attn, sync, evicted_pos, ctx->d_status, stream);
   if (e != cudaSuccess) return cuda_fail(ctx, e);
   st->cache_len = evict ? st->K : st->cache_len + 1;
   return TA_OK;

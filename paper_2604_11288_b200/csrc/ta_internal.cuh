@@ -27,6 +27,12 @@ struct ta_patterns {
   uint32_t* d_bloom;  // [32] 1024-bit filter over the last id of every pattern
 };
 
+constexpr int kStreamWords = 65536;  // blocks of one launch of the decode step
+struct ta_stream_sync {
+  ulonglong2* words;  // device [kStreamWords], 0 between launches: what a sequence's first block tells its others
+  unsigned long long wait_limit_ns;
+};
+
 struct ta_ctx {
   int device;
   int sm_count;
@@ -34,6 +40,7 @@ struct ta_ctx {
   size_t scratch_bytes;
   uint8_t* scratch;         // device
   ta_dev_status* d_status;  // device
+  ta_stream_sync stream_sync;  // of the decode step
   // cache of per-sequence results inside scratch (ta_compress)
   uint64_t cached_epoch;
   uint64_t cached_key;  // policy fields and pattern set the cached results were computed with
@@ -257,17 +264,8 @@ struct ta_stream_dev {  // the caller's ta_stream with the cached length of this
   float* anc_B;
   int32_t* anc_L;
 };
-struct ta_stream_seq_info {  // per sequence, written by the sequence kernel of a step
-  int t;          // position of the new token
-  int match_len;  // tokens t - match_len + 1 .. t belong to a pattern completed by the new token (0: none)
-  float v_new;    // voucher of the new token
-  int id;         // its token id
-};
-cudaError_t ta_launch_stream_seq(const ta_stream_dev& st, const ta_patterns* pats, const ta_policy& pol,
-                                 const int32_t* new_ids, ta_stream_seq_info* info, ta_dev_status* status,
-                                 cudaStream_t stream);
-cudaError_t ta_launch_stream_step(const ta_stream_dev& st, const ta_policy& pol, const ta_stream_seq_info* info,
-                                  const float* attn, int32_t* evicted_pos, ta_dev_status* status,
+cudaError_t ta_launch_stream_step(const ta_stream_dev& st, const ta_patterns* pats, const ta_policy& pol, const int32_t* new_ids,
+                                  const float* attn, const ta_stream_sync& sync, int32_t* evicted_pos, ta_dev_status* status,
                                   cudaStream_t stream);
 
 // ---- step 4 ------------------------------------------------------------------------------------------------

@@ -1,23 +1,22 @@
 // Algorithm 1 in the decode loop: one new token per sequence and step, at most K cached tokens per unit afterwards.
 // (Section 3.1: a retention policy selects S, |S| <= K, "after each generation step"; Algorithm 1 steps 1-10.)
 //
-// Per step two kernels run:
-//   ta_stream_seq_kernel    one warp per sequence: token histogram, pattern match ending at the new token (longest
-//                           pattern wins, then the lowest index), the new token's voucher from the anchors of the last
-//                           TA_MAX_SPAN positions (Eq. 2 with budgets that decayed once per step since detection; a lane
-//                           per distance)
-//   ta_stream_step_kernel   one block per unit, its K+1 entries in registers: appends the new token to the position-ordered
-//                           state, adds this step's attention mass to A, updates the pension average P, forms the
-//                           utility of Eq. 1, applies the budget partition of Section 3.3 to the K+1 cached tokens
-//                           (exactly one token loses), removes it from the ordered state (4-byte entries move;
-//                           key/value rows never do: the freed cache row is handed to the next token) and decays every
-//                           voucher by budget_decay (Algorithm 1 step 10)
-// The second kernel runs beside the first: it reads the unit's state and waits for the first only where the new token comes
-// in. What bounds it: latency at few units, the state's bytes (25 read, 12 to 25 written per cached token, 4 of attention
-// mass read) at many. 4096 units of 257 tokens, three states in turn (180 MB: more than L2), a step of both kernels: where the
-// tokens with a voucher fit the protected slots 31 -> 18.5 us, where all compete for a quarter of the slots 70 -> 25.6 us, the
-// extremes of what a generation meets (serial scans by one thread in the pool selection, one lane per sequence for the voucher,
-// all entries through shared memory before; then 22 us with two entries in 64 registers, of which an SM held 6 blocks).
+// Per step one kernel runs, ta_stream_step_kernel, a block per unit with its K+1 entries in registers. The block of a sequence's
+// first unit works out what the step means for the sequence (pattern match ending at the new token: longest pattern wins, then
+// the lowest index; the new token's voucher from the anchors of the last TA_MAX_SPAN positions, Eq. 2 with budgets that decayed
+// once per step since detection: a lane per anchor), tells the blocks of the sequence's other units, in two words that each of
+// them clears again (a counter of those that have read took 0.8 ns a block), and brings the state that they share (histogram,
+// last ids, anchors, tokens seen) up to date: they read none of it but counts of other ids than the new one. Every block appends the new token to its unit's position-ordered state, adds this step's attention mass to A,
+// updates the pension average P, forms the utility of Eq. 1, applies the budget partition of Section 3.3 to the K+1 cached
+// tokens (exactly one token loses), removes it from the ordered state (4-byte entries move; key/value rows never do: the freed
+// cache row is handed to the next token) and decays every voucher by budget_decay (Algorithm 1 step 10).
+// (A kernel of its own for the sequences, in front of this one, cost its launch and tail: 256 units of 257 tokens 11.7 us a step,
+// now 9.5; 4096 units 18.5, now 17.9, alone 38 and 35.5; 2048 units of 1001 tokens 35.4, now 33.7.)
+// What bounds it: latency at few units, the state's bytes (25 read, 12 to 25 written per cached token, 4 of attention
+// mass read) at many. 4096 units of 257 tokens, three states in turn (180 MB: more than L2), where the tokens with a voucher fit
+// the protected slots, and where all compete for a quarter of the slots (the extremes of what a generation meets): 31 and 70 us
+// with serial scans by one thread in the pool selection, one lane per sequence for the voucher and all entries through shared
+// memory; 22 with two entries in 64 registers, of which an SM held 6 blocks; 18.5 and 25.6 with three in 56.
 // All arithmetic that decides the selection is fp32 with one rounding per operation, in the order the CPU oracle uses.
 #include "ta_internal.cuh"
 
@@ -31,101 +30,132 @@ __device__ __forceinline__ void report(ta_dev_status* st, int code, int where, i
   }
 }
 
-__global__ void __launch_bounds__(32) ta_stream_seq_kernel(ta_stream_dev st, const int32_t* __restrict__ new_ids,
-                                                           const int32_t* __restrict__ p_ids,
-                                                           const int32_t* __restrict__ p_len,
-                                                           const float* __restrict__ p_budget,
-                                                           const int32_t* __restrict__ p_span, int n_pat,
-                                                           float voucher_decay, float budget_decay, int vocab,
-                                                           ta_stream_seq_info* __restrict__ info,
-                                                           ta_dev_status* status) {
+constexpr unsigned long long kPublished = 1ull << 63;
+
+struct PatternTable {
+  const int32_t* ids;
+  const int32_t* len;
+  const float* budget;
+  const int32_t* span;
+  int n;
+};
+
+// What the new token means for its sequence; one warp, the same on every lane.
+struct SeqStep {
+  int t;          // position of the new token
+  int match_len;  // tokens t - match_len + 1 .. t belong to a pattern completed by the new token (0: none)
+  float v_new;    // voucher of the new token
+  int count;      // earlier occurrences of its id
+  int best;       // the pattern that it completes (-1: none)
+};
+// Everything is requested before the first value is used, by place in the rings and not by distance from the new token: one trip
+// to memory (two for the count and for patterns beyond the first 32).
+__device__ __forceinline__ SeqStep sequence_step(const ta_stream_dev& st, const PatternTable& pt, int b, int x, int vocab,
+                                                 float voucher_decay, float budget_decay) {
   constexpr int kHalves = TA_MAX_SPAN / 32;
-  static_assert(TA_MAX_SPAN % 32 == 0 && TA_MAX_PATTERN_LEN == 8, "a lane per distance, eight ids in registers");
-  const int b = blockIdx.x, lane = threadIdx.x;
-  // decay^k by repeated multiplication (one rounding per step) for the distances k = lane + 1, lane + 33, ..
-  float w[kHalves];
-  {
-    float x = 1.0f;
-    int done = 0;
-#pragma unroll
-    for (int h = 0; h < kHalves; ++h) {
-      for (; done < 32 * h + lane + 1; ++done) x = __fmul_rn(x, voucher_decay);
-      w[h] = x;
-    }
-  }
-  ta_wait_for_prior_grid();
-  ta_launch_dependents();
-  const int x = new_ids[b];
-  const int t = st.n_seen[b];
-  int32_t* ring = st.tok_ring + (size_t)b * TA_MAX_PATTERN_LEN;
-  float* aB = st.anc_B + (size_t)b * TA_MAX_SPAN;
-  int32_t* aL = st.anc_L + (size_t)b * TA_MAX_SPAN;
-  // the anchors of the last positions and the last ids, requested together
+  static_assert(TA_MAX_SPAN == 64 && TA_MAX_PATTERN_LEN == 8, "two anchors per lane, eight ids in registers");
+  const unsigned all = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  SeqStep r;
+  r.t = __ldcg(&st.n_seen[b]);
   int L[kHalves];
   float Bk[kHalves];
 #pragma unroll
   for (int h = 0; h < kHalves; ++h) {
-    const int k = 32 * h + lane + 1;
-    L[h] = k <= t ? aL[(t - k) % TA_MAX_SPAN] : 0;
-    Bk[h] = k <= t ? aB[(t - k) % TA_MAX_SPAN] : 0.0f;
+    L[h] = __ldcg(&st.anc_L[(size_t)b * TA_MAX_SPAN + 32 * h + lane]);
+    Bk[h] = __ldcg(&st.anc_B[(size_t)b * TA_MAX_SPAN + 32 * h + lane]);
   }
-  const int last = lane < TA_MAX_PATTERN_LEN - 1 && t - 1 - lane >= 0 ? ring[(t - 1 - lane) % TA_MAX_PATTERN_LEN] : -1;
+  const int last = __ldcg(&st.tok_ring[(size_t)b * TA_MAX_PATTERN_LEN + (lane & 7)]);
+  int len = lane < pt.n ? pt.len[lane] : 0;
+  const int4 none = make_int4(0, 0, 0, 0);
+  int4 p0 = lane < pt.n ? reinterpret_cast<const int4*>(pt.ids)[2 * lane] : none;
+  int4 p1 = lane < pt.n ? reinterpret_cast<const int4*>(pt.ids)[2 * lane + 1] : none;
+  r.count = x >= 0 && x < vocab ? __ldcg(&st.hist[(size_t)b * vocab + x]) : 0;
+  const int t = r.t;
   int ids[TA_MAX_PATTERN_LEN];  // ids[k]: the token k positions before the new one
   ids[0] = x;
 #pragma unroll
-  for (int k = 1; k < TA_MAX_PATTERN_LEN; ++k) ids[k] = __shfl_sync(0xffffffffu, last, k - 1);
-  if (lane == 0) {
-    ring[t % TA_MAX_PATTERN_LEN] = x;
-    if (x >= 0 && x < vocab) atomicAdd(&st.hist[(size_t)b * vocab + x], 1);
-    else report(status, TA_ERR_DEVICE_BOUNDS, 5, b, x);
+  for (int k = 1; k < TA_MAX_PATTERN_LEN; ++k) {
+    const int id = __shfl_sync(all, last, (t - k) & 7);
+    ids[k] = k <= t ? id : -1;
   }
-  // patterns ending at t
-  int best = -1, best_len = 0;
-  for (int p = lane; p < n_pat; p += 32) {
-    const int len = p_len[p];
-    if (len > t + 1 || len <= best_len) continue;  // within a lane p ascends: a later pattern wins only if longer
-    const int32_t* pid = p_ids + p * TA_MAX_PATTERN_LEN;
-    bool ok = true;
+  // patterns ending at t: the longest, of equal lengths the lowest index
+  uint32_t mine = 0;
+#pragma unroll 1
+  for (int p = lane;;) {
+    const int pid[TA_MAX_PATTERN_LEN] = {p0.x, p0.y, p0.z, p0.w, p1.x, p1.y, p1.z, p1.w};
+    bool ok = len > 0 && len <= t + 1;
 #pragma unroll
-    for (int k = 0; k < TA_MAX_PATTERN_LEN; ++k) ok = ok && (k >= len || ids[k] == pid[max(len - 1 - k, 0)]);
-    if (ok) {
-      best = p;
-      best_len = len;
-    }
-  }
+    for (int m = 0; m < TA_MAX_PATTERN_LEN; ++m) {  // id m of the pattern against the token len - 1 - m positions back
+      int id = ids[0];
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const int ol = __shfl_xor_sync(0xffffffffu, best_len, o), ob = __shfl_xor_sync(0xffffffffu, best, o);
-    if (ol > best_len || (ol == best_len && ob >= 0 && (best < 0 || ob < best))) {
-      best_len = ol;
-      best = ob;
+      for (int k = 1; k < TA_MAX_PATTERN_LEN; ++k) id = len - 1 - m == k ? ids[k] : id;
+      ok = ok && (m >= len || pid[m] == id);
     }
+    if (ok) mine = max(mine, ((uint32_t)len << 16) | (uint32_t)(0xffff - p));
+    p += 32;
+    if (p - lane >= pt.n) break;
+    len = p < pt.n ? pt.len[p] : 0;
+    p0 = p < pt.n ? reinterpret_cast<const int4*>(pt.ids)[2 * p] : none;
+    p1 = p < pt.n ? reinterpret_cast<const int4*>(pt.ids)[2 * p + 1] : none;
   }
-  // voucher of the new token from the anchors at t-1, t-2, ..: every lane its own term, summed nearest first
-  float v = 0.0f;
+  static_assert(TA_MAX_PATTERNS <= 0xffff, "an index in 16 bits");
+  mine = __reduce_max_sync(all, mine);
+  r.match_len = (int)(mine >> 16);  // the longest matching pattern covers the tokens of every pattern that ends here
+  r.best = mine ? 0xffff - (int)(mine & 0xffffu) : -1;
+  // voucher of the new token from the anchors at t-1, t-2, ..: every lane its own terms, summed nearest first
+  r.v_new = 0.0f;
+  int k[kHalves];  // distance of the lane's anchors; one that does not reach the new token: farther than any
+  float term[kHalves];
 #pragma unroll
   for (int h = 0; h < kHalves; ++h) {
-    const int k = 32 * h + lane + 1;
-    const bool reaches = L[h] > 0 && k <= L[h];
-    float term = 0.0f;
-    if (reaches) {
-      for (int s = 0; s < k; ++s) Bk[h] = __fmul_rn(Bk[h], budget_decay);
-      term = __fmul_rn(Bk[h], w[h]);
+    k[h] = ((t - (32 * h + lane) - 1) & (TA_MAX_SPAN - 1)) + 1;
+    if (!(k[h] <= t && L[h] > 0 && k[h] <= L[h])) k[h] = TA_MAX_SPAN + 1;
+    term[h] = 0.0f;
+    if (k[h] <= TA_MAX_SPAN) {
+      float w = 1.0f;  // decay^k by repeated multiplication (one rounding per step), like the budget's
+#pragma unroll 1
+      for (int s = 0; s < k[h]; ++s) {
+        Bk[h] = __fmul_rn(Bk[h], budget_decay);
+        w = __fmul_rn(w, voucher_decay);
+      }
+      term[h] = __fmul_rn(Bk[h], w);
     }
-    for (unsigned left = __ballot_sync(0xffffffffu, reaches); left != 0u; left &= left - 1u)
-      v = __fadd_rn(v, __shfl_sync(0xffffffffu, term, __ffs((int)left) - 1));
   }
-  if (lane == 0) {
-    aB[t % TA_MAX_SPAN] = best >= 0 ? p_budget[best] : 0.0f;
-    aL[t % TA_MAX_SPAN] = best >= 0 ? p_span[best] : 0;
-    st.n_seen[b] = t + 1;
-    ta_stream_seq_info si;
-    si.t = t;
-    si.match_len = best_len;  // the longest matching pattern covers the tokens of every pattern that ends here
-    si.v_new = v;
-    si.id = x;
-    info[b] = si;
+#pragma unroll 1
+  for (;;) {
+    const int near = __reduce_min_sync(all, min(k[0], k[1]));
+    if (near > TA_MAX_SPAN) break;
+    const unsigned in0 = __ballot_sync(all, k[0] == near), in1 = __ballot_sync(all, k[1] == near);
+    const float add = in0 ? __shfl_sync(all, term[0], __ffs((int)in0) - 1) : __shfl_sync(all, term[1], __ffs((int)in1) - 1);
+    r.v_new = __fadd_rn(r.v_new, add);
+#pragma unroll
+    for (int h = 0; h < kHalves; ++h)
+      if (k[h] == near) k[h] = TA_MAX_SPAN + 1;
   }
+  return r;
+}
+// the two words of a sequence: voucher and match length; position and earlier occurrences
+__device__ __forceinline__ ulonglong2 seq_words(const SeqStep& r) {
+  return make_ulonglong2(kPublished | ((unsigned long long)r.match_len << 32) | __float_as_uint(r.v_new),
+                         kPublished | ((unsigned long long)r.t << 32) | (uint32_t)r.count);
+}
+// One word, once it is there. (The block that writes it has a lower index than every block that waits for it.)
+__device__ __forceinline__ unsigned long long wait_word(const unsigned long long* word, unsigned long long limit_ns,
+                                                        ta_dev_status* status, int u) {
+  unsigned long long w, t0 = 0;
+  for (int it = 0; ((w = *(volatile const unsigned long long*)word) & kPublished) == 0; ++it) {
+    if ((it & 63) != 63) continue;
+    unsigned long long now;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
+    if (t0 == 0) t0 = now;
+    // (the step's results are then not to be used; the waits of other blocks end with this one)
+    if (now - t0 > limit_ns || *(volatile int*)&status->code == (int)TA_ERR_TIMEOUT) {
+      report(status, TA_ERR_TIMEOUT, 7, u, 0);
+      break;
+    }
+  }
+  return w;
 }
 
 __device__ __forceinline__ uint32_t sortable_key(float f) {
@@ -173,15 +203,24 @@ static_assert(step_shapes_fit(), "a budget for which the step's block does not f
 // non-mandatory tokens with the largest vouchers (lower position first among equals); exactly one token is then not
 // forced and loses: the one with the smallest utility, the latest position among equals. When the sponsored tokens fit the
 // protected slots, or are one too many, block-wide minima decide; otherwise a radix select on the voucher keys.
+// the units of one launch: layers l0 .. l0 + nl - 1, sequences b0 .. b0 + nb - 1, KV heads g0 .. g0 + ng - 1
+struct StreamPart {
+  int l0, nl, b0, nb, g0, ng;
+  int update;  // the sequences' last launch
+};
+
 template <int E>
 __global__ void __launch_bounds__(step_threads(E), E == 8 ? 1 : 2)
-ta_stream_step_kernel(ta_stream_dev st, const ta_stream_seq_info* info, const float* __restrict__ attn,
-                      int vocab, float alpha, float beta, float gamma, float delta, float lambda, float rho,
+ta_stream_step_kernel(ta_stream_dev st, PatternTable pt, const int32_t* __restrict__ new_ids, const float* __restrict__ attn,
+                      ta_stream_sync sync, StreamPart part, int vocab, float voucher_decay, float alpha, float beta, float gamma, float delta, float lambda, float rho,
                       float budget_decay, int n_sink, int n_recent, int k_protected, int32_t* __restrict__ evicted_pos,
                       ta_dev_status* status) {
   extern __shared__ __align__(16) unsigned char smem[];
-  const int u = blockIdx.x, tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, n_warps = nt >> 5;
-  const int b = (u / st.Hkv) % st.B;
+  // by layer, sequence, head: every sequence's first block comes before those that wait for it
+  const int lb = blockIdx.x / part.ng, g = part.g0 + blockIdx.x - lb * part.ng, bi = lb % part.nb, b = part.b0 + bi;
+  const int u = ((part.l0 + lb / part.nb) * st.B + b) * st.Hkv + g;
+  const bool first = lb < part.nb && g == part.g0;
+  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, n_warps = nt >> 5;
   const int K = st.K, C = K + 1, len = st.len, n = len + 1;
   const size_t base = (size_t)u * C;
   float* s_attn = reinterpret_cast<float*>(smem);  // [C] attention mass by cache row
@@ -190,49 +229,73 @@ ta_stream_step_kernel(ta_stream_dev st, const ta_stream_seq_info* info, const fl
   __shared__ uint32_t hist[256];
   __shared__ int tie_cnt[E * step_warps(E)];  // [entry][warp]
   __shared__ int sel_bin, sel_above, sel_pop;
+  __shared__ ulonglong2 s_seq;
+  __shared__ int s_best;
 
-  // ---- the unit's state (from L2: other blocks wrote it) and its attention masses, all requested before the first is used.
-  // Launched as a programmatic dependent of the per-sequence kernel, which lets this one start when everything before it
-  // is complete.
+  ta_wait_for_prior_grid();
+  // ---- the unit's state (from L2: the step before wrote it) and its attention masses, all requested before the first is used
+  const int x = new_ids[b];
+  if (first && warp == 0) {  // before everything else: the other blocks wait for it
+    const SeqStep seq = sequence_step(st, pt, b, x, vocab, voucher_decay, budget_decay);
+    const ulonglong2 w = seq_words(seq);
+    for (int q = 1 + lane; q < part.nl * part.ng; q += 32) {
+      const int l = q / part.ng;
+      ulonglong2* to = sync.words + ((l * part.nb + bi) * part.ng + q - l * part.ng);
+      *(volatile unsigned long long*)&to->x = w.x;
+      *(volatile unsigned long long*)&to->y = w.y;
+    }
+    if (lane == 0) {
+      s_seq = w;
+      s_best = seq.best;
+    }
+  }
   int pos[E], row[E], id[E], S[E];
   float A[E], P[E], V[E];
 #pragma unroll
   for (int e = 0; e < E; ++e) {
     const int r = tid + e * nt;
     const bool old = r < len;
+    id[e] = old ? __ldcg(&st.tok[base + r]) : r == len ? x : 0;
     pos[e] = old ? __ldcg(&st.pos[base + r]) : 0;
     row[e] = old ? __ldcg(&st.slot[base + r]) : r == len ? __ldcg(&st.next_slot[u]) : -1;
-    id[e] = old ? __ldcg(&st.tok[base + r]) : 0;
     A[e] = old ? __ldcg(&st.A[base + r]) : 0.0f;
     P[e] = old ? __ldcg(&st.P[base + r]) : 0.0f;
     V[e] = old ? __ldcg(&st.V[base + r]) : 0.0f;
     S[e] = old ? __ldcg(&st.S[base + r]) : 0;
     if (r < C) s_attn[r] = attn[base + r];
   }
-  ta_wait_for_prior_grid();
-  // (not through a const __restrict__ pointer: such a load counts as invariant and may be moved above the wait)
-  static_assert(sizeof(ta_stream_seq_info) == 16, "one 16-byte load");
-  const int4 raw = __ldcg(reinterpret_cast<const int4*>(info + b));
-  ta_stream_seq_info si;
-  si.t = raw.x;
-  si.match_len = raw.y;
-  si.v_new = __int_as_float(raw.z);
-  si.id = raw.w;
-  const int t = si.t;
-  const float nf = (float)(t + 1), rn = __frcp_rn(nf);
-  const float omr = __fsub_rn(1.0f, rho);
-  int c[E];
+  // (the first look at the words: not waited for before the counts are requested)
+  unsigned long long* const word = reinterpret_cast<unsigned long long*>(sync.words + blockIdx.x) + (lane & 1);
+  unsigned long long said1 = 0;
+  if (!first && warp == 0) said1 = *(volatile unsigned long long*)word;
+  int c[E];  // occurrences of the entry's id; of the new token's, which the sequence's first unit counts up: from the words
 #pragma unroll
   for (int e = 0; e < E; ++e) {
     const int r = tid + e * nt;
-    if (r == len) {
-      pos[e] = t;
-      id[e] = si.id;
-      V[e] = si.v_new;
+    const bool counted = r < n && id[e] >= 0 && id[e] < vocab;
+    c[e] = counted && id[e] != x ? __ldcg(&st.hist[(size_t)b * vocab + id[e]]) : counted ? -1 : 0;
+  }
+  if (!first && warp == 0) {
+    if (!(said1 & kPublished)) said1 = wait_word(word, sync.wait_limit_ns, status, u);
+    if (lane < 2) {
+      reinterpret_cast<unsigned long long*>(&s_seq)[lane] = said1;
+      *word = 0ull;
     }
-    c[e] = (r < n && id[e] >= 0 && id[e] < vocab) ? __ldcg(&st.hist[(size_t)b * vocab + id[e]]) : 0;
   }
   __syncthreads();
+  const ulonglong2 said = s_seq;
+  const int t = (int)(said.y >> 32) & 0x7fffffff, match_len = (int)(said.x >> 32) & 0xff;
+  const float v_new = __uint_as_float((uint32_t)said.x);
+#pragma unroll
+  for (int e = 0; e < E; ++e) {
+    if (c[e] < 0) c[e] = (int)(uint32_t)said.y + 1;
+    if (tid + e * nt == len) {
+      pos[e] = t;
+      V[e] = v_new;
+    }
+  }
+  const float nf = (float)(t + 1), rn = __frcp_rn(nf);
+  const float omr = __fsub_rn(1.0f, rho);
   // ---- attention update, utility
   uint32_t changed = 0;  // entries whose anchor indicator changed
   uint32_t ku[E];
@@ -246,7 +309,7 @@ ta_stream_step_kernel(ta_stream_dev st, const ta_stream_seq_info* info, const fl
       else report(status, TA_ERR_DEVICE_BOUNDS, 6, u, row[e]);
       A[e] = __fadd_rn(A[e], a);
       P[e] = __fadd_rn(__fmul_rn(rho, P[e]), __fmul_rn(omr, a));
-      if (pos[e] >= t - si.match_len + 1 && !S[e]) {
+      if (pos[e] >= t - match_len + 1 && !S[e]) {
         S[e] = 1;
         changed |= 1u << e;
       }
@@ -415,36 +478,29 @@ ta_stream_step_kernel(ta_stream_dev st, const ta_stream_seq_info* info, const fl
     st.next_slot[u] = n;  // rows fill up in order until the cache is full
     evicted_pos[u] = -1;
   }
+  // ---- the first unit: what the sequence's units share goes on by one token
+  if (first && part.update && tid == 0) {
+    const int x = new_ids[b], t = (int)(s_seq.y >> 32) & 0x7fffffff;
+    st.tok_ring[(size_t)b * TA_MAX_PATTERN_LEN + (t & (TA_MAX_PATTERN_LEN - 1))] = x;
+    if (x >= 0 && x < vocab) st.hist[(size_t)b * vocab + x] = (int)(uint32_t)s_seq.y + 1;
+    else report(status, TA_ERR_DEVICE_BOUNDS, 5, b, x);
+    st.anc_B[(size_t)b * TA_MAX_SPAN + (t & (TA_MAX_SPAN - 1))] = s_best >= 0 ? pt.budget[s_best] : 0.0f;
+    st.anc_L[(size_t)b * TA_MAX_SPAN + (t & (TA_MAX_SPAN - 1))] = s_best >= 0 ? pt.span[s_best] : 0;
+    st.n_seen[b] = t + 1;
+  }
 }
 
 }  // namespace
 
-cudaError_t ta_launch_stream_seq(const ta_stream_dev& st, const ta_patterns* pats, const ta_policy& pol,
-                                 const int32_t* new_ids, ta_stream_seq_info* info, ta_dev_status* status,
-                                 cudaStream_t stream) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)st.B, 1, 1);
-  cfg.blockDim = dim3(32, 1, 1);
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  ta_pdl_attribute(&attr[0]);
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, ta_stream_seq_kernel, st, new_ids, (const int32_t*)pats->d_ids,
-                            (const int32_t*)pats->d_len, (const float*)pats->d_budget, (const int32_t*)pats->d_span,
-                            pats->n_pat, pol.voucher_decay, pol.budget_decay, pol.vocab_size, info, status);
-}
-
-cudaError_t ta_launch_stream_step(const ta_stream_dev& st, const ta_policy& pol, const ta_stream_seq_info* info,
-                                  const float* attn, int32_t* evicted_pos, ta_dev_status* status,
+cudaError_t ta_launch_stream_step(const ta_stream_dev& st, const ta_patterns* pats, const ta_policy& pol, const int32_t* new_ids,
+                                  const float* attn, const ta_stream_sync& sync, int32_t* evicted_pos, ta_dev_status* status,
                                   cudaStream_t stream) {
-  const int U = st.n_layers * st.B * st.Hkv, C = st.K + 1;
+  const int C = st.K + 1;
   const int items = step_items(C), threads = step_block(C, items);
   const size_t smem = (size_t)C * 4;  // at most 16 KB
   auto kern = items == 3 ? ta_stream_step_kernel<3> : items == 4 ? ta_stream_step_kernel<4> : ta_stream_step_kernel<8>;
-  // runs beside the kernel before it on the stream (ta_stream_seq_kernel in ta_stream_step)
+  const PatternTable pt = {pats->d_ids, pats->d_len, pats->d_budget, pats->d_span, pats->n_pat};
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)U, 1, 1);
   cfg.blockDim = dim3((unsigned)threads, 1, 1);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
@@ -452,7 +508,21 @@ cudaError_t ta_launch_stream_step(const ta_stream_dev& st, const ta_policy& pol,
   ta_pdl_attribute(&attr[0]);
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, st, info, attn, pol.vocab_size, pol.alpha, pol.beta, pol.gamma, pol.delta,
-                            pol.lambda, pol.pension_rho, pol.budget_decay, pol.n_sink, pol.n_recent, pol.k_protected,
-                            evicted_pos, status);
+  cudaError_t e = cudaSuccess;
+  // In parts of as many blocks as there are words for, in practice one. The sequences' shared state changes in their last part.
+  const int ng = st.Hkv < kStreamWords ? st.Hkv : kStreamWords;
+  const int nb = st.B < kStreamWords / ng ? st.B : kStreamWords / ng;
+  const int nl = st.n_layers < kStreamWords / (ng * nb) ? st.n_layers : kStreamWords / (ng * nb);
+  for (int b0 = 0; b0 < st.B; b0 += nb)
+    for (int l0 = 0; l0 < st.n_layers; l0 += nl)
+      for (int g0 = 0; g0 < st.Hkv && e == cudaSuccess; g0 += ng) {
+        auto rest = [](int all, int from, int n) { return all - from < n ? all - from : n; };
+        const StreamPart part = {l0, rest(st.n_layers, l0, nl), b0, rest(st.B, b0, nb), g0, rest(st.Hkv, g0, ng),
+                                 l0 + nl >= st.n_layers && g0 + ng >= st.Hkv};
+        cfg.gridDim = dim3((unsigned)(part.nl * part.nb * part.ng), 1, 1);
+        e = cudaLaunchKernelEx(&cfg, kern, st, pt, new_ids, attn, sync, part, pol.vocab_size, pol.voucher_decay, pol.alpha,
+                               pol.beta, pol.gamma, pol.delta, pol.lambda, pol.pension_rho, pol.budget_decay, pol.n_sink,
+                               pol.n_recent, pol.k_protected, evicted_pos, status);
+      }
+  return e;
 }
