@@ -95,21 +95,21 @@ constexpr int kRegsNeeded = (kSoftWarps * kRegsSoftmax + 4 * kRegsOther) * 32;
 #define TA_SCORE_POLY_MB2 2
 #endif
 
-// Of the eight pairs of a 16-element group, this many run on the FMA pipe; pair q2 (elements 2*q2, 2*q2 + 1) does when
-// poly_pair is true (spread evenly).
-template <int MB>
-__host__ __device__ constexpr int poly_pairs() {
-  return MB == 1 ? 1 : TA_SCORE_POLY_MB2 / 2;
-}
-template <int MB>
-__host__ __device__ constexpr bool poly_pair(int q2) {
-  return ((q2 * poly_pairs<MB>()) / 8) != (((q2 + 1) * poly_pairs<MB>()) / 8);
-}
-
 // how pass 2 turns the exponentials of a key into outputs
 constexpr int kOutA = 0;      // A only
 constexpr int kOutAP = 3;     // A and P (per-row pension weights), or their weighted sum
 constexpr int kOutFused = 4;  // alpha*A + delta*P with the positive row weights folded into the exponent
+
+// Of the eight pairs of a 16-element group, this many run on the FMA pipe; pair q2 (elements 2*q2, 2*q2 + 1) does when
+// poly_pair is true (spread evenly). With A and P apart and up to 128 rows none: the registers hold no more.
+template <int MB, int PM>
+__host__ __device__ constexpr int poly_pairs() {
+  return MB == 2 ? TA_SCORE_POLY_MB2 / 2 : PM == kOutAP ? 0 : 1;
+}
+template <int MB, int PM>
+__host__ __device__ constexpr bool poly_pair(int q2) {
+  return ((q2 * poly_pairs<MB, PM>()) / 8) != (((q2 + 1) * poly_pairs<MB, PM>()) / 8);
+}
 
 struct ScoreParams {
   ta_seq_desc seq;
@@ -157,8 +157,9 @@ struct alignas(1024) ScoreSmem {
   static constexpr int kPeers = MB == 1 ? kMaxCluster : 8;  // largest cluster the exchange has room for
   float2 peer[kPeers][kRowsPad];           // row statistics (reference, sum) as the CTAs of the cluster sent them
   // [unit parity][row] pass-2 constant of the row; behind them the form that ex2 takes, for rows whose own is the polynomial's
-  float tab[2][MB == 2 && poly_pairs<MB>() ? 2 * kRowsPad : kRowsPad];
+  float tab[2][2 * kRowsPad];
   float wrow[kRowsPad];                    // pension weight per row
+  float lv[kRowsPad];                      // log2 of the row's output weight (kOutFused), else 0
   int8_t row_t[kRowsPad];                  // window index t of the row, -1 for padding rows
   float psum[kRing][2][128];               // MB 2: [ring slot][A|P][key] partial sums of row block 0
   UnitInfo unit[kUnitRing];
@@ -378,18 +379,21 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
   // pass-2 constant of row r from its log2-domain log-sum-exp (+inf: the row is mute)
   // window index t of score row r = h*W + t, -1 for padding rows
   auto row_index = [&](int r) { return r < p.rows ? (int)((uint32_t)r % (uint32_t)p.W) : -1; };
-  // the tables that pass 2 reads; written before the first row constants are published
+  // the tables that the row constants are formed with and that pass 2 reads; written before the first row constants
   auto put_tables = [&](int r, int t) {
+    const float w = t >= 0 ? p.wrow[t] : 0.0f;  // (1-rho) rho^(W-1-t); also right for W' < W (same exponent)
     sm.row_t[r] = (int8_t)t;
-    sm.wrow[r] = t >= 0 ? p.wrow[t] : 0.0f;  // (1-rho) rho^(W-1-t); also right for W' < W (same exponent)
+    sm.wrow[r] = w;
+    // kOutFused: the row's contribution alpha + delta*w (positive, checked by the host) goes into the exponent
+    sm.lv[r] = PM == kOutFused && t >= 0 ? log2f(fmaf(p.delta, w, p.alpha)) : 0.0f;
   };
-  // kOutFused: log2 of the row's contribution alpha + delta*w (positive, checked by the host), which goes into the exponent
-  auto row_weight = [&](int t) { return PM == kOutFused && t >= 0 ? log2f(fmaf(p.delta, p.wrow[t], p.alpha)) : 0.0f; };
-  auto put_row = [&](int up, int r, float lse2, float lv) {
-    const float beta = lse2 - lv;
-    const bool poly = MB == 2 && poly_pair<MB>((r & 15) / 2);
+  auto put_row = [&](int up, int r, float lse2) {
+    const float beta = lse2 - sm.lv[r];
+    const bool poly = MB == 2 && poly_pair<MB, PM>((r & 15) / 2);
     sm.tab[up][r] = poly ? poly_bias(beta) : -beta;
-    if constexpr (MB == 2 && poly_pairs<MB>() > 0) {
+    // (A and P apart, up to 128 rows: the pension weight stands there, so that one address does for both)
+    if constexpr (MB == 1 && PM == kOutAP) sm.tab[up][kRowsPad + r] = sm.wrow[r];
+    if constexpr (MB == 2 && poly_pairs<MB, PM>() > 0) {
       if (poly) sm.tab[up][kRowsPad + r] = -beta;
     }
   };
@@ -584,12 +588,10 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
       if (*reinterpret_cast<volatile int*>(&p.status->code) == (int)TA_ERR_TIMEOUT) *abort_flag = 1;
       constexpr int kRows = kRowsPad / (32 * kStatWarps);
       int tr[kRows];
-      float lv[kRows];
       if (!p.two_pass) {
 #pragma unroll
         for (int i = 0; i < kRows; ++i) {
           tr[i] = row_index(r0 + 32 * kStatWarps * i);
-          lv[i] = row_weight(tr[i]);
           put_tables(r0 + 32 * kStatWarps * i, tr[i]);
         }
       }
@@ -612,7 +614,7 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
             const float lse = p.lse_obs[(((long long)ui.l * p.seq.batch + ui.b) * p.Hq + (ui.g * p.G + h)) * p.W + t];
             lse2 = lse * 1.4426950408889634f;
           }
-          put_row(up, r, lse2, lv[i]);
+          put_row(up, r, lse2);
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(smem_u32(&sm.tab_full[up]));
@@ -672,16 +674,10 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
       if (lane == 0) mbar_arrive(bar_ae + (J % kAcc) * 8);
     };
 
-    int tr[MB];  // of this thread's rows in pass 1
-    float lv[MB];
+    int tr = -1;  // window index of this thread's row in pass 1
     if (p.two_pass) {
-#pragma unroll
-      for (int h = 0; h < MB; ++h) {
-        const int r = h * 128 + row_in_tile;
-        tr[h] = row_index(r);
-        lv[h] = row_weight(tr[h]);
-        if (grp == 0) put_tables(r, tr[h]);
-      }
+      tr = row_index(block * 128 + row_in_tile);
+      if (grp < MB) put_tables(block * 128 + row_in_tile, tr);
     }
     int J = grp;        // this group's next job
     int jg = 0;         // first job of the current pass
@@ -721,8 +717,8 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
         // before the accumulator stage is released and does not wait for the tile's last exponentials: it uses the sum
         // without the last 16 keys and, for those, their largest score. The polynomial exponentials saturate at 2^126,
         // which the same check catches; so does a row without a reference yet (ref -1e30).
-        const int pos = n - p.W + tr[block];
-        const int lim = (tr[block] >= 0 && pos >= 0) ? (p.causal ? pos : n - 1) : -1;  // last key that the thread's row sees
+        const int pos = n - p.W + tr;
+        const int lim = (tr >= 0 && pos >= 0) ? (p.causal ? pos : n - 1) : -1;  // last key that the thread's row sees
         // rows that see no key (padding) get a reference that turns every exponential into 0
         float ref = lim >= 0 ? -1e30f : 1e30f, zsum = 0.0f;
         constexpr float kSumLimit = 1.0e18f;  // about 2^60
@@ -738,7 +734,7 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
 #pragma unroll
           for (int q = 0; q < 16; q += 2) {
             float e0, e1;
-            if (mix && !masked && poly_pair<MB>(q / 2)) {
+            if (mix && !masked && poly_pair<MB, PM>(q / 2)) {
               if constexpr (MB == 2) {
                 exp2_poly2(e0, e1, v[q], v[q + 1], c252, pbias, pbias);
               } else {
@@ -888,7 +884,7 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
             }
           }
 #pragma unroll
-          for (int h = 0; h < MB; ++h) put_row(up, h * 128 + row_in_tile, log2_sum(m[h], z[h]), lv[h]);
+          for (int h = 0; h < MB; ++h) put_row(up, h * 128 + row_in_tile, log2_sum(m[h], z[h]));
           __syncwarp();
           if (lane == 0) mbar_arrive(smem_u32(&sm.tab_full[up]));
         }
@@ -915,7 +911,7 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
           constexpr bool masked = decltype(masked_tag)::value;
           constexpr int hi = decltype(hi_tag)::value;  // 0: rows row0..row0+15, 1: rows row0+16..row0+31
           const float4* tab4 = reinterpret_cast<const float4*>(&sm.tab[up][row0]) + hi * 4;
-          const float4* w4 = reinterpret_cast<const float4*>(&sm.wrow[row0]) + hi * 4;
+          const float4* w4 = MB == 1 ? tab4 + kRowsPad / 4 : reinterpret_cast<const float4*>(&sm.wrow[row0]) + hi * 4;
           const char4* t4 = reinterpret_cast<const char4*>(&sm.row_t[row0]) + hi * 4;
 #pragma unroll
           for (int q4 = 0; q4 < 4; ++q4) {
@@ -924,7 +920,7 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
             float a[4];
 #pragma unroll
             for (int e = 0; e < 4; e += 2) {
-              if (poly_pair<MB>(2 * q4 + e / 2) && !masked) {
+              if (poly_pair<MB, PM>(2 * q4 + e / 2) && !masked) {
                 if constexpr (MB == 2) {
                   exp2_poly2(a[e], a[e + 1], cur[4 * q4 + e], cur[4 * q4 + e + 1], c252, tbv[e], tbv[e + 1]);
                 } else {
@@ -932,7 +928,7 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
                   exp2_poly5<false>(a[e], a[e + 1], a[e], a[e + 1]);
                 }
               } else {
-                if (MB == 2 && poly_pair<MB>(2 * q4 + e / 2)) {
+                if (MB == 2 && poly_pair<MB, PM>(2 * q4 + e / 2)) {
                   const float2 nb = *reinterpret_cast<const float2*>(&sm.tab[up][kRowsPad + row0 + hi * 16 + 4 * q4 + e]);
                   tbv[e] = nb.x;
                   tbv[e + 1] = nb.y;
