@@ -1043,6 +1043,24 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads) ta_select_kernel(ta
     }
   }
   const int want = r_main[b];
+  // The per-token values, mostly from L2, in groups (registers: a group's loads are in flight together, no more); the first
+  // group's before `want` is known.
+  constexpr int kGroup = ITEMS < 8 ? ITEMS : ITEMS > 16 ? 4 : 8;
+  const uint8_t* f = forced + start + lo;
+  const float* sp = src.u_static + start + lo;
+  const float* pp = !src.u && src.A && src.P ? src.P + unit_off + start + lo : nullptr;
+  float us[CACHED ? kGroup : 1], ps[CACHED ? kGroup : 1];
+  uint8_t ff[CACHED ? kGroup : 1];
+  auto load_group = [&](int g0) {
+#pragma unroll
+    for (int q = 0; q < (CACHED ? kGroup : 0); ++q) {
+      const int i = tid + (g0 + q) * kThreads;
+      us[q] = i < nl ? sp[i] : 0.0f;
+      ff[q] = i < nl ? f[i] : (uint8_t)1;
+      ps[q] = pp && i < nl ? pp[i] : 0.0f;
+    }
+  };
+  if constexpr (CACHED) load_group(0);
   if (want == -2) {  // sequence rejected by ta_forced_kernel
     if (lead) {
       for (int r = tid; r < K; r += kThreads) out[r] = -1;
@@ -1059,29 +1077,16 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads) ta_select_kernel(ta
     if constexpr (GATHER) gather_unit(gd, seq, unit, l, b, g, n, K, out, n, true, sh);
     return;
   }
-  const uint8_t* f = forced + start + lo;
   auto key_of = [&](int il, uint32_t& key) {
     key = sortable_key(unit_utility(src, unit_off, (long long)start + lo + il));
     return f[il] == 0;
   };
   if constexpr (CACHED) {
     split_unit_begin<CL>(sh);
-    const float* sp = src.u_static + start + lo;
-    const float* pp = !src.u && src.A && src.P ? src.P + unit_off + start + lo : nullptr;
     kc.elig = 0;
-    // the per-token values, mostly from L2, in groups (registers: a group's loads are in flight together, no more)
-    constexpr int kGroup = ITEMS < 8 ? ITEMS : ITEMS > 16 ? 4 : 8;
 #pragma unroll
     for (int g0 = 0; g0 < ITEMS; g0 += kGroup) {
-      float us[kGroup], ps[kGroup];
-      uint8_t ff[kGroup];
-#pragma unroll
-      for (int q = 0; q < kGroup; ++q) {
-        const int i = tid + (g0 + q) * kThreads;
-        us[q] = i < nl ? sp[i] : 0.0f;
-        ff[q] = i < nl ? f[i] : (uint8_t)1;
-        ps[q] = pp && i < nl ? pp[i] : 0.0f;
-      }
+      if (g0 > 0) load_group(g0);
 #pragma unroll
       for (int q = 0; q < kGroup; ++q) {
         const int it = g0 + q;
