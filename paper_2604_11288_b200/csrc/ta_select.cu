@@ -225,7 +225,10 @@ cudaError_t ta_launch_select_units(const ta_select_args& a, cudaStream_t stream_
                           a.r_main, a.idx, a.count, gd2, co);
   }
   if (!split_units(units, a.seq.max_n, sms) && a.seq.max_n <= kItemsLong * kThreads) {
-    auto kern = a.seq.max_n <= kItems * kThreads
+    // (the smallest instance that holds the unit: every phase walks over all of a thread's slots)
+    auto kern = a.seq.max_n <= 8 * kThreads
+                    ? (gathers ? ta_select_kernel<true, 1, 8, true> : ta_select_kernel<true, 1, 8, false>)
+                : a.seq.max_n <= kItems * kThreads
                     ? (gathers ? ta_select_kernel<true, 1, kItems, true> : ta_select_kernel<true, 1, kItems, false>)
                     : (gathers ? ta_select_kernel<true, 1, kItemsLong, true> : ta_select_kernel<true, 1, kItemsLong, false>);
     return launch_clustered(kern, units, 1, stream, a.seq, a.n_layers, a.Hkv, a.K, a.fast, src, a.forced, a.r_main, a.idx,
