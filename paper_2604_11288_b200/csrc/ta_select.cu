@@ -22,6 +22,16 @@
 
 namespace cg = cooperative_groups;
 
+#define TA_SEL_THREADS 128
+#define TA_SEL_NS sel128
+#include "ta_select_core.cuh"
+#undef TA_SEL_THREADS
+#undef TA_SEL_NS
+#define TA_SEL_THREADS 256
+#define TA_SEL_NS sel256
+#include "ta_select_core.cuh"
+#undef TA_SEL_THREADS
+#undef TA_SEL_NS
 #define TA_SEL_THREADS 512
 #define TA_SEL_NS sel512
 #include "ta_select_core.cuh"
@@ -188,41 +198,78 @@ bool ta_select_gathers(const ta_select_args& a) {
          !split_units(units, a.seq.max_n, sm_count_of(a));
 }
 
+// the same arguments in the types of every block size
+template <class Src>
+Src unit_src(const ta_select_args& a) {
+  Src s;
+  s.u = a.fast ? nullptr : a.u;
+  s.A = a.fast ? nullptr : a.A;
+  s.P = a.fast ? nullptr : a.P;
+  s.u_static = a.u_static;
+  s.alpha = a.alpha;
+  s.delta = a.delta;
+  return s;
+}
+template <class Dst>
+Dst gather_dst(const ta_select_args& a, bool gathers) {
+  Dst d = {};
+  if (gathers) {
+    d.k = a.gather_k;
+    d.v = a.gather_v;
+    d.k_out = reinterpret_cast<uint4*>(a.gather_k_out);
+    d.v_out = reinterpret_cast<uint4*>(a.gather_v_out);
+  }
+  return d;
+}
+
+// Threads of a selecting block that also gathers, where small ones pay (0: they do not). A block is a chain of latencies around
+// a few barriers, so that more and smaller blocks per SM (eight of 128 threads, four of 256, two of 512) fill one another's gaps
+// as long as the gather is small and there are units enough for them; a large gather wants a block's loads together. Time of
+// ta_compress_scores in us with 512 / 256 / 128 threads, uniform lengths:
+//   2048 units, 4000 tokens: K 16 52 / 35 / 31, K 64 86 / 64 / 62, K 128 96 / 84 / 83, K 256 126 / 124 / 128, K 1000 365 / 379
+//   1024 units, 2000 tokens: K 16 27 / 19 / 14, K 64 42 / 31 / 27, K 128 47 / 41 / 39, K 256 63 / 63 / 64
+//   400 units, 2000 tokens: K 16 15.9 / 12.1 / 11.3, K 64 22.8 / 17.8 / 18.1, K 128 25.6 / 21.9 / 23.2, K 256 33.4 / 31.9 / 32.8
+//   256 units, 4000 tokens: K 16 14.0 / 13.0 / 14.9, K 64 19.0 / 18.9 / 23.8, K 128 20.5 / 21.4 / 27.3
+//   2048 units, 8000 tokens: K 16 66 / 49, K 64 118 / 97, K 256 160 / 158; 256 units: K 64 26.4 / 28.8
+int small_threads(const ta_select_args& a, int units, int sms) {
+  const int n = a.seq.max_n;
+  if (n <= sel128::kItemsLong * sel128::kThreads && units >= 5 * sms && a.K <= 128) return sel128::kThreads;
+  if (n <= sel256::kItemsLong * sel256::kThreads &&
+      ((units > 2 * sms && a.K <= 192) || (units > sms && n <= 16 * sel256::kThreads && a.K <= 64)))
+    return sel256::kThreads;
+  return 0;
+}
+
 cudaError_t ta_launch_select_units(const ta_select_args& a, cudaStream_t stream_) {
   if (a.seq.batch == 0 || a.n_layers == 0) return cudaSuccess;
   const StreamPdl stream = {stream_, a.pdl_units != 0};
-  UnitSrc src;
-  src.u = a.fast ? nullptr : a.u;
-  src.A = a.fast ? nullptr : a.A;
-  src.P = a.fast ? nullptr : a.P;
-  src.u_static = a.u_static;
-  src.alpha = a.alpha;
-  src.delta = a.delta;
+  const UnitSrc src = unit_src<UnitSrc>(a);
   const int units = a.fast ? a.seq.batch : a.n_layers * a.seq.batch * a.Hkv;
   const int32_t* co = a.n_classes > 0 ? a.class_of : nullptr;
   const int sms = sm_count_of(a);
-  GatherDst gd = {};
   const bool gathers = ta_select_gathers(a);
-  if (gathers) {
-    gd.k = a.gather_k;
-    gd.v = a.gather_v;
-    gd.k_out = reinterpret_cast<uint4*>(a.gather_k_out);
-    gd.v_out = reinterpret_cast<uint4*>(a.gather_v_out);
-  }
-  sel1024::UnitSrc src2;  // the same fields for the kernels built for 1024 threads
-  src2.u = src.u;
-  src2.A = src.A;
-  src2.P = src.P;
-  src2.u_static = src.u_static;
-  src2.alpha = src.alpha;
-  src2.delta = src.delta;
-  const sel1024::GatherDst gd2 = {gd.k, gd.v, gd.k_out, gd.v_out};
+  const GatherDst gd = gather_dst<GatherDst>(a, gathers);
+  const sel1024::UnitSrc src2 = unit_src<sel1024::UnitSrc>(a);
+  const sel1024::GatherDst gd2 = gather_dst<sel1024::GatherDst>(a, gathers);
   if (few_short_units(a)) {
     auto kern = a.seq.max_n <= 4 * sel1024::kThreads
                     ? (gathers ? sel1024::ta_select_kernel<true, 1, 4, true> : sel1024::ta_select_kernel<true, 1, 4, false>)
                     : (gathers ? sel1024::ta_select_kernel<true, 1, 8, true> : sel1024::ta_select_kernel<true, 1, 8, false>);
     return launch_threads(sel1024::kThreads, kern, units, 1, stream, a.seq, a.n_layers, a.Hkv, a.K, a.fast, src2, a.forced,
                           a.r_main, a.idx, a.count, gd2, co);
+  }
+  const int small = gathers ? small_threads(a, units, sms) : 0;
+  if (small == sel128::kThreads) {
+    auto kern = a.seq.max_n <= 16 * sel128::kThreads ? sel128::ta_select_kernel<true, 1, 16, true>
+                                                     : sel128::ta_select_kernel<true, 1, sel128::kItemsLong, true>;
+    return launch_threads(small, kern, units, 1, stream, a.seq, a.n_layers, a.Hkv, a.K, a.fast, unit_src<sel128::UnitSrc>(a),
+                          a.forced, a.r_main, a.idx, a.count, gather_dst<sel128::GatherDst>(a, true), co);
+  }
+  if (small == sel256::kThreads) {
+    auto kern = a.seq.max_n <= 16 * sel256::kThreads ? sel256::ta_select_kernel<true, 1, 16, true>
+                                                     : sel256::ta_select_kernel<true, 1, sel256::kItemsLong, true>;
+    return launch_threads(small, kern, units, 1, stream, a.seq, a.n_layers, a.Hkv, a.K, a.fast, unit_src<sel256::UnitSrc>(a),
+                          a.forced, a.r_main, a.idx, a.count, gather_dst<sel256::GatherDst>(a, true), co);
   }
   if (!split_units(units, a.seq.max_n, sms) && a.seq.max_n <= kItemsLong * kThreads) {
     // (the smallest instance that holds the unit: every phase walks over all of a thread's slots)

@@ -1,7 +1,7 @@
 // Core of the budget-K selection (radix select, ordered emit, the two kernels), written against a block size that the
 // including file fixes with TA_SEL_THREADS before each inclusion; everything lives in namespace TA_SEL_NS. The
-// selection kernels are built for 512 threads (two blocks per SM for short units) and for 1024 threads (twice the keys
-// in registers for long units).
+// selection kernels are built for 512 threads (two blocks per SM for short units), for 1024 threads (twice the keys in
+// registers for long units, and few short ones) and for 128 and 256 (many short units with small budgets).
 namespace TA_SEL_NS {
 
 constexpr int kThreads = TA_SEL_THREADS;
@@ -123,9 +123,9 @@ __device__ SelectResult block_radix_select(int n, int want, KeyFn key_of, const 
   if (CL > 1) ghist0 = cg::this_cluster().map_shared_rank(&sh.ghist[0][0], 0);
   for (int pass = 0; pass < 4; ++pass) {
     const int shift = 24 - 8 * pass;
-    if (tid < 256) {
-      sh.hist[tid] = 0;
-      if (CL > 1) sh.ghist[pass & 1][tid] = 0;  // only rank 0's copy is used; its readers of two passes ago are done
+    for (int k = tid; k < 256; k += kThreads) {
+      sh.hist[k] = 0;
+      if (CL > 1) sh.ghist[pass & 1][k] = 0;  // only rank 0's copy is used; its readers of two passes ago are done
     }
     if (CL > 1) cg::this_cluster().sync();
     else __syncthreads();
@@ -146,7 +146,8 @@ __device__ SelectResult block_radix_select(int n, int want, KeyFn key_of, const 
     const uint32_t* hist = sh.hist;
     if (CL > 1) {  // merge the slices' histograms on rank 0, then every CTA takes the same decision from the sum
       uint32_t* gh = ghist0 + (pass & 1) * 256;
-      if (tid < 256 && sh.hist[tid]) atomicAdd(&gh[tid], sh.hist[tid]);
+      for (int k = tid; k < 256; k += kThreads)
+        if (sh.hist[k]) atomicAdd(&gh[k], sh.hist[k]);
       cg::this_cluster().sync();
       hist = gh;
     }
@@ -208,9 +209,9 @@ template <int CL>
 __device__ __forceinline__ void split_unit_begin(SelectShared& sh) {
   if (CL > 1) {
     const int tid = threadIdx.x;
-    if (tid < 256) {
-      sh.ghist[0][tid] = 0;
-      sh.ghist[1][tid] = 0;
+    for (int k = tid; k < 256; k += kThreads) {
+      sh.ghist[0][k] = 0;
+      sh.ghist[1][k] = 0;
     }
     if (tid == 0) sh.cand_n = 0;
     cg::this_cluster().barrier_arrive();
@@ -278,7 +279,7 @@ __device__ __forceinline__ void list_radix_finish(int m, int bits, int done, uin
   while (done < bits) {
     const int width = min(8, bits - done), shift = bits - done - width;
     const uint32_t digit_mask = (1u << width) - 1u;
-    if (tid < 256) sh.hist[tid] = 0;
+    for (int k = tid; k < 256; k += kThreads) sh.hist[k] = 0;
     __syncthreads();
 #pragma unroll
     for (int q = 0; q < kPer; ++q) {
@@ -498,11 +499,11 @@ __device__ SelectResult cached_radix_select(int n, int n_unit, int want, const K
     }
     const int width = min(8, bits - done), shift = bits - done - width;
     const uint32_t digit_mask = (1u << width) - 1u;
-    if (tid < 256) sh.hist[tid] = 0;
+    for (int k = tid; k < 256; k += kThreads) sh.hist[k] = 0;
     if (CL > 1 && pass >= 2) {
       // rank 0's merged histogram alternates between two buffers, both zero at the start; from the third pass on the
       // buffer is cleared again (its readers of two passes ago are done) and the clearing made visible
-      if (tid < 256) sh.ghist[pass & 1][tid] = 0;
+      for (int k = tid; k < 256; k += kThreads) sh.ghist[pass & 1][k] = 0;
       cg::this_cluster().sync();
     } else {
       __syncthreads();
@@ -531,7 +532,8 @@ __device__ SelectResult cached_radix_select(int n, int n_unit, int want, const K
     const uint32_t* hist = sh.hist;
     if (CL > 1) {  // merge the slices' histograms on rank 0, then every CTA takes the same decision from the sum
       uint32_t* gh = ghist0 + (pass & 1) * 256;
-      if (tid < 256 && sh.hist[tid]) atomicAdd(&gh[tid], sh.hist[tid]);
+      for (int k = tid; k < 256; k += kThreads)
+        if (sh.hist[k]) atomicAdd(&gh[k], sh.hist[k]);
       cg::this_cluster().sync();
       hist = gh;
     }
