@@ -251,41 +251,54 @@ cudaError_t ta_launch_select_units(const ta_select_args& a, cudaStream_t stream_
   const GatherDst gd = gather_dst<GatherDst>(a, gathers);
   const sel1024::UnitSrc src2 = unit_src<sel1024::UnitSrc>(a);
   const sel1024::GatherDst gd2 = gather_dst<sel1024::GatherDst>(a, gathers);
+  // The instances that look for few tokens, as long as the budget lets them (see cached_radix_select; us without and with them):
+  // 1024 units of 16000 tokens K 128 107 / 90, 250 123 / 109; 2048 units of 4000 tokens K 64 62 / 53; 256 units of 4000 tokens K 256
+  // 26.4 / 25.3; 8 units of up to 7000 tokens K 128, 32 calls with their scores 773 / 756.
+  const bool few = gathers && a.K <= kThreads / 2, few1024 = gathers && a.K <= sel1024::kThreads / 2;
   if (few_short_units(a)) {
     auto kern = a.seq.max_n <= 4 * sel1024::kThreads
                     ? (gathers ? sel1024::ta_select_kernel<true, 1, 4, true> : sel1024::ta_select_kernel<true, 1, 4, false>)
-                    : (gathers ? sel1024::ta_select_kernel<true, 1, 8, true> : sel1024::ta_select_kernel<true, 1, 8, false>);
+                    : (few1024   ? sel1024::ta_select_kernel<true, 1, 8, true, true>
+                       : gathers ? sel1024::ta_select_kernel<true, 1, 8, true>
+                                 : sel1024::ta_select_kernel<true, 1, 8, false>);
     return launch_threads(sel1024::kThreads, kern, units, 1, stream, a.seq, a.n_layers, a.Hkv, a.K, a.fast, src2, a.forced,
                           a.r_main, a.idx, a.count, gd2, co);
   }
   const int small = gathers ? small_threads(a, units, sms) : 0;
   if (small == sel128::kThreads) {
-    auto kern = a.seq.max_n <= 16 * sel128::kThreads ? sel128::ta_select_kernel<true, 1, 16, true>
-                                                     : sel128::ta_select_kernel<true, 1, sel128::kItemsLong, true>;
+    auto kern = a.seq.max_n <= 16 * sel128::kThreads ? sel128::ta_select_kernel<true, 1, 16, true, true>
+                                                     : sel128::ta_select_kernel<true, 1, sel128::kItemsLong, true, true>;
     return launch_threads(small, kern, units, 1, stream, a.seq, a.n_layers, a.Hkv, a.K, a.fast, unit_src<sel128::UnitSrc>(a),
                           a.forced, a.r_main, a.idx, a.count, gather_dst<sel128::GatherDst>(a, true), co);
   }
   if (small == sel256::kThreads) {
-    auto kern = a.seq.max_n <= 16 * sel256::kThreads ? sel256::ta_select_kernel<true, 1, 16, true>
-                                                     : sel256::ta_select_kernel<true, 1, sel256::kItemsLong, true>;
+    auto kern = a.seq.max_n <= 16 * sel256::kThreads ? sel256::ta_select_kernel<true, 1, 16, true, true>
+                                                     : sel256::ta_select_kernel<true, 1, sel256::kItemsLong, true, true>;
     return launch_threads(small, kern, units, 1, stream, a.seq, a.n_layers, a.Hkv, a.K, a.fast, unit_src<sel256::UnitSrc>(a),
                           a.forced, a.r_main, a.idx, a.count, gather_dst<sel256::GatherDst>(a, true), co);
   }
   if (!split_units(units, a.seq.max_n, sms) && a.seq.max_n <= kItemsLong * kThreads) {
     // (the smallest instance that holds the unit: every phase walks over all of a thread's slots)
     auto kern = a.seq.max_n <= 8 * kThreads
-                    ? (gathers ? ta_select_kernel<true, 1, 8, true> : ta_select_kernel<true, 1, 8, false>)
+                    ? (few       ? ta_select_kernel<true, 1, 8, true, true>
+                       : gathers ? ta_select_kernel<true, 1, 8, true>
+                                 : ta_select_kernel<true, 1, 8, false>)
                 : a.seq.max_n <= kItems * kThreads
-                    ? (gathers ? ta_select_kernel<true, 1, kItems, true> : ta_select_kernel<true, 1, kItems, false>)
-                    : (gathers ? ta_select_kernel<true, 1, kItemsLong, true> : ta_select_kernel<true, 1, kItemsLong, false>);
+                    ? (few       ? ta_select_kernel<true, 1, kItems, true, true>
+                       : gathers ? ta_select_kernel<true, 1, kItems, true>
+                                 : ta_select_kernel<true, 1, kItems, false>)
+                    : (few       ? ta_select_kernel<true, 1, kItemsLong, true, true>
+                       : gathers ? ta_select_kernel<true, 1, kItemsLong, true>
+                                 : ta_select_kernel<true, 1, kItemsLong, false>);
     return launch_clustered(kern, units, 1, stream, a.seq, a.n_layers, a.Hkv, a.K, a.fast, src, a.forced, a.r_main, a.idx,
                             a.count, gd, co);
   }
   if (!split_units(units, a.seq.max_n, sms) && a.seq.max_n <= sel1024::kItemsLong * sel1024::kThreads) {
     // many long units: blocks of 1024 threads hold a unit of up to 32768 keys in registers (read once instead of
     // once per radix pass and once more for the ordered write)
-    auto kern = gathers ? sel1024::ta_select_kernel<true, 1, sel1024::kItemsLong, true>
-                        : sel1024::ta_select_kernel<true, 1, sel1024::kItemsLong, false>;
+    auto kern = few1024   ? sel1024::ta_select_kernel<true, 1, sel1024::kItemsLong, true, true>
+                : gathers ? sel1024::ta_select_kernel<true, 1, sel1024::kItemsLong, true>
+                          : sel1024::ta_select_kernel<true, 1, sel1024::kItemsLong, false>;
     return launch_threads(sel1024::kThreads, kern, units, 1, stream, a.seq, a.n_layers, a.Hkv, a.K, a.fast, src2, a.forced,
                           a.r_main, a.idx, a.count, gd2, co);
   }

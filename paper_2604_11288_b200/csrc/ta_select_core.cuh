@@ -342,9 +342,10 @@ __device__ __forceinline__ uint32_t compare_finish(int m, int remaining, int& ab
 // a float alone would put most of them into two or three bins). The first pass counts every eligible element
 // (match.any merges equal digits of a warp into one shared-memory atomic); from then on each thread keeps a bit mask
 // of its elements that are still candidates, and the passes touch those only. The passes stop as soon as the
-// candidates left are exactly as many as are still to take, or so few that they are compared with one another. n_unit is the length of the whole unit (n is this CTA's
+// candidates left are exactly as many as are still to take, or so few that they are compared with one another. FEW (an instance of
+// its own: the code costs large budgets 0.6 %): few are wanted. n_unit is the length of the whole unit (n is this CTA's
 // slice when CL > 1).
-template <int CL, int ITEMS>
+template <int CL, bool FEW = false, int ITEMS>
 __device__ SelectResult cached_radix_select(int n, int n_unit, int want, const KeyCache<ITEMS>& kc, SelectShared& sh) {
   SelectResult r;
   r.thresh = 0;
@@ -367,23 +368,71 @@ __device__ SelectResult cached_radix_select(int n, int n_unit, int want, const K
       kmax = max(kmax, kc.key[it]);
     }
   }
-  kmin = __reduce_min_sync(0xffffffffu, kmin);
-  kmax = __reduce_max_sync(0xffffffffu, kmax);
-  uint32_t num = __reduce_add_sync(0xffffffffu, (uint32_t)__popc(cand));
-  if (lane == 0) {
-    sh.wmin[warp] = kmin;
-    sh.wmax[warp] = kmax;
-    sh.wnum[warp] = num;
-  }
   if (tid == 0) {
     sh.remaining = want;
     sh.cmp_n = 0;
   }
-  __syncthreads();
   static_assert(kWarps <= 32, "one lane per warp in the second reduction step");
-  kmin = __reduce_min_sync(0xffffffffu, lane < kWarps ? sh.wmin[lane] : 0xffffffffu);
-  kmax = __reduce_max_sync(0xffffffffu, lane < kWarps ? sh.wmax[lane] : 0u);
-  num = __reduce_add_sync(0xffffffffu, lane < kWarps ? sh.wnum[lane] : 0u);
+  uint32_t num = 0;
+  bool bounded = false;
+  if constexpr (FEW) {
+    static_assert(CL == 1, "one block's threads");
+    if (want <= kThreads / 2) {
+      // Few are wanted: the want-th largest of the threads' own largest keys is a lower bound of the threshold, and a digit of
+      // those (one per thread) costs a fraction of a digit of all keys. Few keys are at or above it.
+      const uint32_t mine = kmax;  // (0: no eligible key)
+      const uint32_t lo_w = __reduce_min_sync(0xffffffffu, cand != 0u ? mine : 0xffffffffu);
+      const uint32_t hi_w = __reduce_max_sync(0xffffffffu, mine);
+      const int with = __popc(__ballot_sync(0xffffffffu, cand != 0u));
+      if (lane == 0) {
+        sh.wmin[warp] = lo_w;
+        sh.wmax[warp] = hi_w;
+        sh.wnum[warp] = (uint32_t)with;
+      }
+      for (int k = tid; k < 256; k += kThreads) sh.hist[k] = 0;
+      __syncthreads();
+      const uint32_t lo = __reduce_min_sync(0xffffffffu, lane < kWarps ? sh.wmin[lane] : 0xffffffffu);
+      const uint32_t hi = __reduce_max_sync(0xffffffffu, lane < kWarps ? sh.wmax[lane] : 0u);
+      const uint32_t threads_with = __reduce_add_sync(0xffffffffu, lane < kWarps ? sh.wnum[lane] : 0u);
+      bounded = threads_with >= (uint32_t)want;
+      if (bounded) {
+        uint32_t bound = lo;
+        if (lo != hi) {
+          const int top = 32 - __clz(lo ^ hi), shift = max(top - 8, 0);
+          const uint32_t mask = top == 32 ? 0u : (0xffffffffu << top);
+          if (cand != 0u) atomicAdd(&sh.hist[(mine >> shift) & 255u & ~(mask >> shift)], 1u);
+          __syncthreads();
+          if (tid < 32) radix_walk(sh.hist, shift, 255u, hi & mask, mask, sh);
+          __syncthreads();
+          bound = sh.prefix;
+          if (tid == 0) sh.remaining = want;
+        }
+        uint32_t above = 0;
+#pragma unroll
+        for (int it = 0; it < ITEMS; ++it) above |= kc.key[it] >= bound ? (1u << it) : 0u;
+        cand &= above;
+        kmin = bound;
+        kmax = hi;
+        num = (uint32_t)max(n_unit / 8, kCompareCap + 1);  // (not known; few of n_unit)
+      } else {
+        __syncthreads();  // wmin, wmax and wnum are written again
+      }
+    }
+  }
+  if (!bounded) {
+    kmin = __reduce_min_sync(0xffffffffu, kmin);
+    kmax = __reduce_max_sync(0xffffffffu, kmax);
+    num = __reduce_add_sync(0xffffffffu, (uint32_t)__popc(cand));
+    if (lane == 0) {
+      sh.wmin[warp] = kmin;
+      sh.wmax[warp] = kmax;
+      sh.wnum[warp] = num;
+    }
+    __syncthreads();
+    kmin = __reduce_min_sync(0xffffffffu, lane < kWarps ? sh.wmin[lane] : 0xffffffffu);
+    kmax = __reduce_max_sync(0xffffffffu, lane < kWarps ? sh.wmax[lane] : 0u);
+    num = __reduce_add_sync(0xffffffffu, lane < kWarps ? sh.wnum[lane] : 0u);
+  }
   uint32_t* ghist0 = nullptr;
   if (CL > 1) {
     cg::cluster_group cluster = cg::this_cluster();
@@ -406,7 +455,7 @@ __device__ SelectResult cached_radix_select(int n, int n_unit, int want, const K
       num += sh.cl_range[q][2];
     }
   }
-  if (num < (uint32_t)want) {  // fewer eligible elements than requested: all of them
+  if (!bounded && num < (uint32_t)want) {  // fewer eligible elements than requested: all of them
     r.all = 1;
     return r;
   }
@@ -414,7 +463,7 @@ __device__ SelectResult cached_radix_select(int n, int n_unit, int want, const K
   if (diff == 0u) {  // all eligible keys are equal
     r.thresh = kmin;
     r.ties = want;
-    r.all_ties = num == (uint32_t)want;
+    r.all_ties = !bounded && num == (uint32_t)want;
     return r;
   }
   const int bits = 32 - __clz(diff);  // low bits still to resolve
@@ -508,7 +557,7 @@ __device__ SelectResult cached_radix_select(int n, int n_unit, int want, const K
     } else {
       __syncthreads();
     }
-    if (pass == 0 || ncand * 4 > n_unit) {  // most elements are candidates (uniform over the unit's CTAs)
+    if ((pass == 0 && !bounded) || ncand * 4 > n_unit) {  // most elements are candidates (uniform over the unit's CTAs)
 #pragma unroll
       for (int it = 0; it < ITEMS; ++it) {
         if (it * kThreads < n) {
@@ -998,7 +1047,7 @@ __device__ __forceinline__ void gather_unit(const GatherDst& gd, const ta_seq_de
 }
 
 // grid.x = units. scored: unit = (l*B + b)*Hkv + g; fast: unit = b.
-template <bool CACHED, int CL, int ITEMS = kItems, bool GATHER = false>
+template <bool CACHED, int CL, int ITEMS = kItems, bool GATHER = false, bool FEW = false>
 __global__ void __launch_bounds__(kThreads, 1024 / kThreads) ta_select_kernel(ta_seq_desc seq, int n_layers, int Hkv, int K, int fast,
                                                              UnitSrc src, const uint8_t* forced,
                                                              const int32_t* r_main,
@@ -1104,7 +1153,7 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads) ta_select_kernel(ta
     }
   }
   SelectResult r;
-  if constexpr (CACHED) r = cached_radix_select<CL>(hi - lo, n, want, kc, sh);
+  if constexpr (CACHED) r = cached_radix_select<CL, FEW>(hi - lo, n, want, kc, sh);
   else r = block_radix_select<CACHED, CL>(hi - lo, want, key_of, kc, sh);
   auto classify = [&](int, bool elig, uint32_t key, bool& def, bool& tie) {
     def = !elig || (!r.none && (r.all || key > r.thresh));
