@@ -224,18 +224,21 @@ Dst gather_dst(const ta_select_args& a, bool gathers) {
 
 // Threads of a selecting block that also gathers, where small ones pay (0: they do not). A block is a chain of latencies around
 // a few barriers, so that more and smaller blocks per SM (eight of 128 threads, four of 256, two of 512) fill one another's gaps
-// as long as the gather is small and there are units enough for them; a large gather wants a block's loads together. Time of
+// as long as the gather is small and there are units enough for them; a large gather wants a block's loads together. The budgets
+// are those that half a block's threads bound (see cached_radix_select), and a little more where units are short. Time of
 // ta_compress_scores in us with 512 / 256 / 128 threads, uniform lengths:
-//   2048 units, 4000 tokens: K 16 52 / 35 / 31, K 64 86 / 64 / 62, K 128 96 / 84 / 83, K 256 126 / 124 / 128, K 1000 365 / 379
-//   1024 units, 2000 tokens: K 16 27 / 19 / 14, K 64 42 / 31 / 27, K 128 47 / 41 / 39, K 256 63 / 63 / 64
-//   400 units, 2000 tokens: K 16 15.9 / 12.1 / 11.3, K 64 22.8 / 17.8 / 18.1, K 128 25.6 / 21.9 / 23.2, K 256 33.4 / 31.9 / 32.8
-//   256 units, 4000 tokens: K 16 14.0 / 13.0 / 14.9, K 64 19.0 / 18.9 / 23.8, K 128 20.5 / 21.4 / 27.3
-//   2048 units, 8000 tokens: K 16 66 / 49, K 64 118 / 97, K 256 160 / 158; 256 units: K 64 26.4 / 28.8
+//   2048 units, 4000 tokens: K 16 52 / 36 / 31, K 64 77 / 57 / 53, K 128 88 / 77 / 83, K 192 107 / 105 / 106, K 256 120 / 125 / 128
+//   1024 units, 2000 tokens: K 16 27 / 19 / 14, K 64 40 / 29 / 24, K 128 45 / 39 / 39, K 256 61 / 63 / 65
+//   400 units, 2000 tokens: K 16 15.8 / 11.9 / 11.0, K 64 21.8 / 16.6 / 16.2, K 128 24.7 / 20.9 / 23.0, K 256 32.7 / 31.7 / 32.6
+//   256 units, 4000 tokens: K 16 13.9 / 12.9 / 14.8, K 64 17.5 / 16.9 / 20.0, K 128 19.1 / 19.4 / 27.0
+//   2048 units, 8000 tokens: K 16 66 / 49, K 64 101 / 81, K 128 112 / 99, K 192 131 / 135; 256 units: K 64 23.1 / 23.5
 int small_threads(const ta_select_args& a, int units, int sms) {
   const int n = a.seq.max_n;
-  if (n <= sel128::kItemsLong * sel128::kThreads && units >= 5 * sms && a.K <= 128) return sel128::kThreads;
+  const bool is_short = n <= 16 * sel256::kThreads;  // also what 128 threads hold
+  static_assert(16 * sel256::kThreads == sel128::kItemsLong * sel128::kThreads, "one limit for both");
+  if (is_short && units >= 5 * sms && a.K <= sel128::kThreads / 2) return sel128::kThreads;
   if (n <= sel256::kItemsLong * sel256::kThreads &&
-      ((units > 2 * sms && a.K <= 192) || (units > sms && n <= 16 * sel256::kThreads && a.K <= 64)))
+      ((units > 2 * sms && a.K <= (is_short ? 192 : sel256::kThreads / 2)) || (is_short && units > sms && a.K <= 64)))
     return sel256::kThreads;
   return 0;
 }

@@ -27,8 +27,9 @@ def _run(ctx, pats, pol, lengths, K, ids, score, k, v):
     return [x[:L] for x in (idx, cnt, ko.view(torch.int16), vo.view(torch.int16))]
 
 
-@pytest.mark.parametrize("lengths,K", [([2048] * 10, 64), ([4096, 1, 0, 17, 4095, 2049, 300, 64, 128, 1000], 128), ([4096] * 10, 16),
-                                       ([700] * 10, 1), ([4097, 0, 1, 5000] + [900] * 6, 100), ([8192, 3] + [129] * 8, 192),
+@pytest.mark.parametrize("lengths,K", [([2048] * 10, 64), ([4096, 1, 0, 17, 4095, 2049, 300, 64, 128, 1000], 64), ([4096] * 10, 16),
+                                       ([4096, 1, 0, 17, 4095, 2049, 300, 64, 128, 1000], 65), ([4000] * 10, 193),
+                                       ([700] * 10, 1), ([4097, 0, 1, 5000] + [900] * 6, 100), ([8192, 3] + [129] * 8, 128), ([8192, 3] + [129] * 8, 129),
                                        ([1000] * 10, 129), ([300] * 3, 64), ([4000, 31, 2000], 40)])
 def test_small_blocks_match_large_ones(lengths, K):
     L = 20 if len(lengths) == 10 else 14
