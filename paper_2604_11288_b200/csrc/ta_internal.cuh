@@ -27,7 +27,7 @@ struct ta_patterns {
   uint32_t* d_bloom;  // [32] 1024-bit filter over the last id of every pattern
 };
 
-constexpr int kStreamWords = 65536;  // blocks of one launch of the decode step
+constexpr int kStreamWords = 16384;  // blocks of one launch of the decode step (256 KB: a larger allocation makes a context slow to create)
 struct ta_stream_sync {
   ulonglong2* words;  // device [kStreamWords], 0 between launches: what a sequence's first block tells its others
   unsigned long long wait_limit_ns;
