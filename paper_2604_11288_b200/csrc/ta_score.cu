@@ -30,9 +30,9 @@
 //                       are dealt round-robin to the four groups and to the four accumulator stages. Two groups at work
 //                       keep the special-function unit as busy as it can be (1105 cycles a job against 1095 with three);
 //                       the others hide a group's way from one job to the next: its stage's products (some 800 cycles)
-//                       and the signals around them. Three groups with a stage to spare took 2 to 5 % longer. With
-//                       129..256 score rows (MB 2) a
-//                       tile is two consecutive jobs, one per block of 128 rows; in pass 2 their partial sums meet in a
+//                       and the signals around them. Three groups with a stage to spare took 2 to 5 % longer, two groups
+//                       with 16, 32 or 64 columns per load 10 to 15 %. With 129..256 score rows (MB 2) a tile is two
+//                       consecutive jobs, one per block of 128 rows; in pass 2 their partial sums meet in a
 //                       shared-memory ring. Between the passes the group that ends the first one first merges the row
 //                       statistics, exchanges them over the cluster and forms the row constants for pass 2.
 // The producer's warpgroup gives registers back (setmaxnreg) at its start and the softmax warps take them.
@@ -40,19 +40,24 @@
 // A call of few units is a chain of latencies (one layer of 4096 tokens: 8 units, 8 CTAs each, four tiles and 26 K cycles per
 // CTA, of which the exponentials need 9 K). What the chain waits for is started as early as it can be: the producer requests its
 // first tiles before the CTA's set-up is complete (first scores after 4.8 K cycles instead of 7 K), and nothing but the
-// barriers that it needs itself precedes them. 21.9 -> 20.5 us a call, 32 calls of 8 shorter units 905 -> 865 us.
+// barriers that it needs itself precedes them. 21.9 -> 20.5 us a call, 32 calls of 8 shorter units 905 -> 865 us; 19.2 and 788 with
+// four groups and the polynomial. Between the passes 4.4 K cycles remain (merge, exchange, merge, constants: code that is executed
+// once and fetched for it). Letting the selection's blocks in early, looking at the barriers without suspending and unrolling
+// the sends changed nothing or cost time.
 //
 // What bounds it. With up to 128 rows at full clock (32 layers x 4096 tokens): the softmax warps (two exponentials per score
-// element, 16 per clock and SM on the special-function unit) and the memory system, at about the same time each: the parts
-// alone take 85 us (softmax), 73 us (products: 64 KB of operand reads and 32 KB of copies through shared memory per job) and
-// 72 us (copies), together 107 us; 256 units on 148 CTAs are two rounds where 1.73 would do. With 256 rows (16 x 32768
-// tokens): the special-function unit, 74 % of the active cycles. Back to back the board's power limit (1000 W) adds to that by
-// lowering the clock from 1965 MHz: to 1807 on the first call (8 %), 1455 on 64 ragged sequences of up to 16384 tokens with 128
-// rows (3.82 -> 4.47 ms a call), 1582 with 256 rows (11.2 -> 13.0 ms). Of the first call's 118 mJ (122 mJ with the earlier
-// four groups, single-lane issuer and barriers at every unit border) the copies alone take 71 mJ, the products 55 mJ, the
-// softmax arithmetic 34 mJ, each with its share of the idle power: copies dominate, from L2 as well as from HBM (keeping the
-// keys of all units in flight inside L2 with 4 CTAs per unit costs as much energy). The scale-and-shift and the running sums
-// are taken two at a time (fma.rn.f32x2, add.rn.f32x2: the same roundings as the scalar forms, a third fewer issue slots).
+// element, 16 per clock and SM on the special-function unit, an eighth of them on the FMA pipe) and shared memory, into which
+// 32 KB a tile are copied and from which the products read 64 KB a job. A job takes 0.66 us of the steady state (0.70 with three
+// groups and all exponentials on one unit); of those 0.70 the parts alone took 0.61 (softmax), 0.43 (products), 0.58 (copies),
+// products and copies together 0.67. 256 units on 148 CTAs are two rounds where 1.73 would do. With 256 rows (16 x 32768
+// tokens): the special-function unit. Back to back the board's power limit (1000 W) decides: 32 layers x 4096 tokens take 123 mJ
+// a call (129 mJ before) at 1687 MHz instead of 1965, 64 ragged sequences of up to 16384 tokens 4.40 J (4.55) at 1342 MHz,
+// 16 x 32768 tokens with 256 rows 12.8 J (13.1) at 1560 MHz. The products alone run into it at 1535 TFLOP/s, 5.7 of those
+// 12.8 J; products of 256 columns, which read one operand half as often, would reach 1685, but one for both row blocks of a tile
+// ties two accumulator stages together and the call takes as long. Equal shares of tiles over unit borders for both passes (a
+// cut unit's statistics handed to the next CTA through global memory) save 3 % of a single call and cost 5 % back to back: the
+// cut units' keys are read from HBM twice. The scale-and-shift and the running sums are taken two at a time (fma.rn.f32x2,
+// add.rn.f32x2: the same roundings as the scalar forms, a third fewer issue slots).
 //
 // Every wait on an mbarrier is bounded by wall time; when one runs out the CTA records TA_ERR_TIMEOUT, its producer
 // and MMA warps stop issuing work, the copies and MMAs in flight are drained, and the other warps leave their loops
