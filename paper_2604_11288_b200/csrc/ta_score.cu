@@ -210,13 +210,13 @@ __device__ __forceinline__ void exp2_poly2(float& e0, float& e1, float s0, float
   e1 = __uint_as_float((y1 << 23) + __float_as_uint(p1));
 }
 // Two values of exp2(x) as precise as ex2's: a polynomial of degree 5 for 2^f on [0, 1) (minimax in relative error, 7.5e-8) of
-// the same argument that ex2 would take. Arguments are clamped below at -126; CLAMP: also above at 126.
-// Not a number becomes the largest finite number, which mutes the row in pass 1 as a sum that is none does.
+// the same argument that ex2 would take, and with ex2's results at the ends: zero below -126, infinity from 128 on, not a
+// number for what is none. (The power of two is a factor and not added to the exponent's bits, which would make a number of
+// everything: one more multiplication for two values.)
 constexpr float kQ0 = 0.9999999404f, kQ1 = 0.6931530833f, kQ2 = 0.2401536107f, kQ3 = 0.05582631752f, kQ4 = 0.008989339694f, kQ5 = 0.001877576695f;
-template <bool CLAMP>
 __device__ __forceinline__ void exp2_poly5(float& e0, float& e1, float x0, float x1) {
-  asm("max.NaN.f32 %0, %0, %2;\n\tmax.NaN.f32 %1, %1, %2;" : "+f"(x0), "+f"(x1) : "f"(-126.0f));
-  if (CLAMP) asm("min.NaN.f32 %0, %0, %2;\n\tmin.NaN.f32 %1, %1, %2;" : "+f"(x0), "+f"(x1) : "f"(126.0f));
+  asm("max.NaN.f32 %0, %0, %2;\n\tmax.NaN.f32 %1, %1, %2;" : "+f"(x0), "+f"(x1) : "f"(-127.0f));
+  asm("min.NaN.f32 %0, %0, %2;\n\tmin.NaN.f32 %1, %1, %2;" : "+f"(x0), "+f"(x1) : "f"(128.0f));
   float p0, p1;
   uint32_t y0, y1;
   asm("{\n\t.reg .b64 x, m, y, w, f, p, k;\n\t"
@@ -233,8 +233,11 @@ __device__ __forceinline__ void exp2_poly5(float& e0, float& e1, float x0, float
       "mov.b64 {%0, %1}, p;\n\tmov.b64 {%2, %3}, y;\n\t}"
       : "=f"(p0), "=f"(p1), "=r"(y0), "=r"(y1)
       : "f"(x0), "f"(x1), "f"(12582912.0f), "f"(1.0f), "f"(-1.0f), "f"(kQ5), "f"(kQ4), "f"(kQ3), "f"(kQ2), "f"(kQ1), "f"(kQ0));
-  e0 = __uint_as_float((y0 << 23) + __float_as_uint(p0));
-  e1 = __uint_as_float((y1 << 23) + __float_as_uint(p1));
+  // 2^floor(x): 0 for -127, infinity for 128
+  const float w0 = __uint_as_float((y0 << 23) + 0x3f800000u), w1 = __uint_as_float((y1 << 23) + 0x3f800000u);
+  asm("{\n\t.reg .b64 p, w;\n\tmov.b64 p, {%2, %3};\n\tmov.b64 w, {%4, %5};\n\tmul.rn.f32x2 p, p, w;\n\tmov.b64 {%0, %1}, p;\n\t}"
+      : "=f"(e0), "=f"(e1)
+      : "f"(p0), "f"(p1), "f"(w0), "f"(w1));
 }
 // two multiply-adds / two adds in one instruction (same roundings as the scalar forms)
 __device__ __forceinline__ void fma2(float& d0, float& d1, float a0, float a1, float b, float c0, float c1) {
@@ -720,7 +723,7 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
         // a key costs one multiply-add, one exponential and one add, and no maximum is tracked. A tile whose sum
         // leaves the safe range (a score more than 2^60 above ref) is redone against its own maximum. The check runs
         // before the accumulator stage is released and does not wait for the tile's last exponentials: it uses the sum
-        // without the last 16 keys and, for those, their largest score. The polynomial exponentials saturate at 2^126,
+        // without the last 16 keys and, for those, their largest score. The cubic's exponentials saturate at 2^126,
         // which the same check catches; so does a row without a reference yet (ref -1e30).
         const int pos = n - p.W + tr;
         const int lim = (tr >= 0 && pos >= 0) ? (p.causal ? pos : n - 1) : -1;  // last key that the thread's row sees
@@ -744,7 +747,7 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
                 exp2_poly2(e0, e1, v[q], v[q + 1], c252, pbias, pbias);
               } else {
                 fma2(e0, e1, v[q], v[q + 1], c, -rc, -rc);
-                exp2_poly5<true>(e0, e1, e0, e1);
+                exp2_poly5(e0, e1, e0, e1);
               }
             } else {
               fma2(e0, e1, v[q], v[q + 1], c, -rc, -rc);
@@ -930,7 +933,7 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
                   exp2_poly2(a[e], a[e + 1], cur[4 * q4 + e], cur[4 * q4 + e + 1], c252, tbv[e], tbv[e + 1]);
                 } else {
                   fma2(a[e], a[e + 1], cur[4 * q4 + e], cur[4 * q4 + e + 1], c, tbv[e], tbv[e + 1]);
-                  exp2_poly5<false>(a[e], a[e + 1], a[e], a[e + 1]);
+                  exp2_poly5(a[e], a[e + 1], a[e], a[e + 1]);
                 }
               } else {
                 if (MB == 2 && poly_pair<MB, PM>(2 * q4 + e / 2)) {

@@ -66,21 +66,19 @@ def exp2_poly_model(s, c, beta, coef):
     return (bits & 0xFFFFFFFF).astype(np.uint32).view(f32)
 
 
-def exp2_poly5_model(x, coef, clamp=False):
+def exp2_poly5_model(x, coef):
     """What exp2_poly5(x) computes, step by step in fp32 (numpy): clamp, round-down add onto 1.5 * 2^23, exact fraction, Horner
-    polynomial, exponent splice."""
+    polynomial, times the power of two (0 for -127, infinity for 128)."""
     f32 = np.float32
-    x = np.maximum(np.asarray(x, f32), f32(-126.0))
-    if clamp:
-        x = np.minimum(x, f32(126.0))
+    x = np.minimum(np.maximum(np.asarray(x, f32), f32(-127.0)), f32(128.0))
     y = np.floor(x.astype(np.float64) + 12582912.0)                       # an integer below 2^24: exact in fp32
     f = (x.astype(np.float64) + (12582912.0 - y)).astype(f32)             # exact
     p = f32(coef[5])
     for ci in coef[4::-1]:
         p = (np.asarray(p, np.float64) * f.astype(np.float64) + np.float64(ci)).astype(f32)
+    y = np.where(np.isnan(y), 12582912.0, y)
     j = (y - 12582912.0).astype(np.int64)
-    bits = p.view(np.int32).astype(np.int64) + (j << 23)
-    return (bits & 0xFFFFFFFF).astype(np.uint32).view(f32)
+    return p * (((j + 127) << 23) & 0xFFFFFFFF).astype(np.uint32).view(f32)
 
 
 if __name__ == "__main__":

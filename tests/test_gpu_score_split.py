@@ -84,3 +84,45 @@ def test_128_rows_are_as_precise_as_fp32_sums(n):
     hidden = torch.arange(n, device="cuda").view(1, -1) > torch.arange(n - W, n, device="cuda").view(-1, 1)
     want = (torch.softmax(s.view(L, Hkv, 4, W, n).masked_fill(hidden, float("-inf")), -1) * w).sum((2, 3))
     assert (u.double() - want).norm() / want.norm() < 3e-7
+
+
+def _weighted(q, k, W):
+    """ta_score_weighted of one unit with 128 rows (4 heads, W = 32)."""
+    n = k.shape[0]
+    pol = ta.ta_policy_default(ta.TA_PRESET_THEOREM, 4)
+    batch = ta.make_batch(1, 1, n, n, n)
+    ctx = ta.ta_ctx_create(0, ta.ta_scratch_bytes(batch, 4, 1, 128, 4, pol))
+    try:
+        u = torch.empty((1, 1, n), device="cuda")
+        ta.ta_score_weighted(ctx, pol, batch, 4, 1, 128, ta.view(q.view(1, 1, 4, W, 128)), ta.view(k.view(1, 1, 1, n, 128)),
+                             None, u, torch.cuda.current_stream().cuda_stream)
+        assert ta.ta_ctx_poll(ctx) == ta.TA_OK
+    finally:
+        ta.ta_ctx_destroy(ctx)
+    return u.view(n)
+
+
+def test_keys_far_below_the_largest_score_zero():
+    # Key 5 is 20 * 20 * 128 / sqrt(128) = 4525 above every other key in all rows: their exponentials are 0 in fp32, whichever
+    # row and unit computes them. Key 5 takes all of every row: the sum of the rows' weights.
+    n, W = 700, 32
+    q = torch.full((4 * W, 128), 20.0, dtype=torch.bfloat16, device="cuda")
+    k = torch.zeros((n, 128), dtype=torch.bfloat16, device="cuda")
+    k[5] = 20.0
+    u = _weighted(q, k, W)
+    assert u[5] > 0 and torch.isfinite(u).all()
+    u[5] = 0
+    assert (u == 0).all()
+
+
+@pytest.mark.parametrize("row", [0, 13, 14, 15, 31])
+def test_a_query_that_is_no_number_shows_in_the_keys_it_sees(row):
+    n, W = 700, 32
+    g = torch.Generator(device="cuda")
+    g.manual_seed(row)
+    q = torch.randn((4 * W, 128), generator=g, dtype=torch.bfloat16, device="cuda")
+    k = torch.randn((n, 128), generator=g, dtype=torch.bfloat16, device="cuda")
+    q[row] = float("nan")
+    u = _weighted(q, k, W)
+    assert torch.isnan(u[:n - W + row + 1]).all()
+    assert torch.isfinite(u[n - W + row + 1:]).all()
