@@ -427,7 +427,7 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
       int pre = 0;  // tiles of the first unit that are requested here
       if (p.by_length) {
         set_up();
-        ta_wait_for_prior_grid();
+        if (!p.late_wait) ta_wait_for_prior_grid();
       } else {
         asm volatile("bar.arrive 1, %0;" ::"n"(kThreads) : "memory");
         cluster_arrive_relaxed();
