@@ -264,10 +264,12 @@ ta_stream_step_kernel(ta_stream_dev st, PatternTable pt, const int32_t* __restri
     S[e] = old ? __ldcg(&st.S[base + r]) : 0;
     if (r < C) s_attn[r] = attn[base + r];
   }
-  // (the first look at the words: not waited for before the counts are requested)
-  unsigned long long* const word = reinterpret_cast<unsigned long long*>(sync.words + blockIdx.x) + (lane & 1);
+  // Two threads wait, each for a word that it alone reads and clears: one that read along could miss the word and wait for good.
+  // (The first look at the words: not waited for before the counts are requested.)
+  const bool waits = !first && tid < 2;
+  unsigned long long* const word = reinterpret_cast<unsigned long long*>(sync.words + blockIdx.x) + (tid & 1);
   unsigned long long said1 = 0;
-  if (!first && warp == 0) said1 = *(volatile unsigned long long*)word;
+  if (waits) said1 = *(volatile unsigned long long*)word;
   int c[E];  // occurrences of the entry's id; of the new token's, which the sequence's first unit counts up: from the words
 #pragma unroll
   for (int e = 0; e < E; ++e) {
@@ -275,12 +277,10 @@ ta_stream_step_kernel(ta_stream_dev st, PatternTable pt, const int32_t* __restri
     const bool counted = r < n && id[e] >= 0 && id[e] < vocab;
     c[e] = counted && id[e] != x ? __ldcg(&st.hist[(size_t)b * vocab + id[e]]) : counted ? -1 : 0;
   }
-  if (!first && warp == 0) {
+  if (waits) {
     if (!(said1 & kPublished)) said1 = wait_word(word, sync.wait_limit_ns, status, u);
-    if (lane < 2) {
-      reinterpret_cast<unsigned long long*>(&s_seq)[lane] = said1;
-      *word = 0ull;
-    }
+    reinterpret_cast<unsigned long long*>(&s_seq)[tid] = said1;
+    *word = 0ull;
   }
   __syncthreads();
   const ulonglong2 said = s_seq;
