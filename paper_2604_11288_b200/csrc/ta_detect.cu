@@ -35,8 +35,8 @@ __device__ __forceinline__ float sq2(uint32_t w) {  // sum of squares of a bf16 
 }
 
 __global__ void __launch_bounds__(kWarps * 32, 3)
-ta_embed_conf_kernel(long long total, const __nv_bfloat16* __restrict__ emb, long long stride, int D,
-                     const __nv_bfloat16* __restrict__ concepts, int C, float* __restrict__ conf) {
+ta_embed_conf_kernel(long long total, const __nv_bfloat16* emb, long long stride, int D, const __nv_bfloat16* concepts, int C,
+                     float* __restrict__ conf) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int ld = D + 32;  // padded row: consecutive rows start 64 bytes apart modulo 128 (conflict-free 16-byte loads)
   __nv_bfloat16* s_c = reinterpret_cast<__nv_bfloat16*>(smem);           // [8][D + 32], unused concepts are zero

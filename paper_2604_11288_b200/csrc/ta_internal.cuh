@@ -91,7 +91,8 @@ __host__ __device__ inline int ta_seq_begin(const ta_seq_desc& s, int b, const i
 // on the stream is still draining (its launch latency overlaps that kernel's tail); it must call
 // ta_wait_for_prior_grid() before its first access to memory. The call returns at once in a kernel launched normally. What
 // the kernel before it wrote must not be read through a const __restrict__ pointer: such loads count as invariant, and the
-// compiler may move them above the wait.
+// compiler may move them above the wait. For the first kernel of a call the kernel before it is the caller's own, which may have
+// let its dependents start early: such a kernel reads nothing through one.
 inline void ta_pdl_attribute(cudaLaunchAttribute* attr) {
   attr->id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr->val.programmaticStreamSerializationAllowed = 1;

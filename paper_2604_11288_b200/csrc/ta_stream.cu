@@ -211,10 +211,10 @@ struct StreamPart {
 
 template <int E>
 __global__ void __launch_bounds__(step_threads(E), E == 8 ? 1 : 2)
-ta_stream_step_kernel(ta_stream_dev st, PatternTable pt, const int32_t* __restrict__ new_ids, const float* __restrict__ attn,
-                      ta_stream_sync sync, StreamPart part, int vocab, float voucher_decay, float alpha, float beta, float gamma, float delta, float lambda, float rho,
-                      float budget_decay, int n_sink, int n_recent, int k_protected, int32_t* __restrict__ evicted_pos,
-                      ta_dev_status* status) {
+ta_stream_step_kernel(ta_stream_dev st, PatternTable pt, const int32_t* new_ids, const float* attn, ta_stream_sync sync,
+                      StreamPart part, int vocab, float voucher_decay, float alpha, float beta, float gamma, float delta,
+                      float lambda, float rho, float budget_decay, int n_sink, int n_recent, int k_protected,
+                      int32_t* __restrict__ evicted_pos, ta_dev_status* status) {
   extern __shared__ __align__(16) unsigned char smem[];
   // by layer, sequence, head: every sequence's first block comes before those that wait for it
   const int lb = blockIdx.x / part.ng, g = part.g0 + blockIdx.x - lb * part.ng, bi = lb % part.nb, b = part.b0 + bi;
