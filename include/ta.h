@@ -447,6 +447,16 @@ ta_status ta_stream_scratch_bytes(const ta_stream* st, size_t* out_bytes);
  *   evicted_pos  DEVICE int32 [U] out    position of the evicted token, -1 when nothing was evicted */
 ta_status ta_stream_step(ta_ctx* ctx, const ta_patterns* pats, const ta_policy* policy, ta_stream* st /*HOST*/,
                          const int32_t* new_ids, const float* attn, int32_t* evicted_pos, void* stream);
+/* A sequence's units wait on the device for what the sequence's first unit works out (ta_ctx_set_wait_limit). When such a wait
+ * runs out, a unit has either done the whole step or nothing of it: its state and its entry of evicted_pos are then as
+ * they were before, but the units no longer agree with one another, nor with cache_len. Steps enqueued before the
+ * ta_ctx_poll that reports TA_ERR_TIMEOUT do nothing; after it the context works again, on states that the caller has
+ * set up anew. A time-out that another call of the context left unpolled does not concern the step.
+ * Diagnostic for this: a step whose waits have a limit of limit_ns (at most one second), and whose first units hold back what
+ * they have worked out for twice as long. In sequences of several units only the first one then steps. */
+ta_status ta_ctx_selftest_step_wait(ta_ctx* ctx, const ta_patterns* pats, const ta_policy* policy, ta_stream* st /*HOST*/,
+                                    const int32_t* new_ids, const float* attn, int32_t* evicted_pos, uint64_t limit_ns,
+                                    void* stream);
 
 /* ---- host-buffer variant of ta_compress --------------------------------------------------------------------
  * Same computation with every data pointer on the HOST (pinned memory makes the copies asynchronous):

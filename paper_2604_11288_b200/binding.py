@@ -181,6 +181,7 @@ def lib():
                                           ta_bf16_view, vp, vp, vp, vp, vp]),
             "ta_stream_scratch_bytes": (i32, [C.POINTER(ta_stream), C.POINTER(sz)]),
             "ta_stream_step": (i32, [vp, vp, PP, C.POINTER(ta_stream), vp, vp, vp, vp]),
+            "ta_ctx_selftest_step_wait": (i32, [vp, vp, PP, C.POINTER(ta_stream), vp, vp, vp, u64, vp]),
             "ta_compress_host_workspace_bytes": (i32, [PB, i32, i32, i32, i32, PP, C.POINTER(sz)]),
             "ta_compress_host": (i32, [vp, vp, PP, PB, i32, i32, i32, i32, vp, vp, vp, vp, vp, vp, vp, vp, vp, sz, vp]),
         }
@@ -413,6 +414,11 @@ def ta_stream_scratch_bytes(st: ta_stream) -> int:
 
 def ta_stream_step(ctx, pats, policy, st: ta_stream, new_ids, attn, evicted_pos, stream=None):
     _check((_call or _native()).ta_stream_step(ctx, pats, policy, st, new_ids, attn, evicted_pos, stream), "ta_stream_step")
+
+
+def ta_ctx_selftest_step_wait(ctx, pats, policy, st: ta_stream, new_ids, attn, evicted_pos, limit_ns: int, stream=None):
+    _check(lib().ta_ctx_selftest_step_wait(ctx, pats, C.byref(policy), C.byref(st), _ptr(new_ids), _ptr(attn),
+                                           _ptr(evicted_pos), int(limit_ns), stream), "ta_ctx_selftest_step_wait")
 
 
 def ta_compress_host_workspace_bytes(batch, Hq, Hkv, d, K, policy) -> int:

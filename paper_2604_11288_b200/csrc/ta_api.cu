@@ -993,9 +993,10 @@ ta_status ta_stream_scratch_bytes(const ta_stream* st, size_t* out_bytes) {
   return TA_OK;
 }
 
-ta_status ta_stream_step(ta_ctx* ctx, const ta_patterns* pats, const ta_policy* policy, ta_stream* st,
-                         const int32_t* new_ids, const float* attn, int32_t* evicted_pos, void* stream_v) {
-  Range range("ta_stream_step");
+// test_limit_ns: 0, or the self-test's limit of the step's waits, which then run out
+static ta_status stream_step_impl(ta_ctx* ctx, const ta_patterns* pats, const ta_policy* policy, ta_stream* st,
+                                  const int32_t* new_ids, const float* attn, int32_t* evicted_pos, uint64_t test_limit_ns,
+                                  void* stream_v) {
   if (!ctx || !pats || !new_ids || !attn || !evicted_pos) return TA_ERR_INVALID_ARG;
   ta_status s = check_policy(policy);
   if (s == TA_OK) s = check_stream(st);
@@ -1026,12 +1027,26 @@ ta_status ta_stream_step(ta_ctx* ctx, const ta_patterns* pats, const ta_policy* 
   d.anc_L = st->anc_L;
   const bool evict = st->cache_len + 1 > st->K;
   ta_stream_sync sync = ctx->stream_sync;
-  sync.wait_limit_ns = ctx->wait_limit_ns ? ctx->wait_limit_ns : 2000000000ull;
+  sync.wait_limit_ns = test_limit_ns ? test_limit_ns : ctx->wait_limit_ns ? ctx->wait_limit_ns : 2000000000ull;
+  sync.hold_ns = 2 * test_limit_ns;
 
   cudaError_t e = ta_launch_stream_step(d, pats, *policy, new_ids, attn, sync, evicted_pos, ctx->d_status, stream);
   if (e != cudaSuccess) return cuda_fail(ctx, e);
   st->cache_len = evict ? st->K : st->cache_len + 1;
   return TA_OK;
+}
+
+ta_status ta_stream_step(ta_ctx* ctx, const ta_patterns* pats, const ta_policy* policy, ta_stream* st,
+                         const int32_t* new_ids, const float* attn, int32_t* evicted_pos, void* stream) {
+  Range range("ta_stream_step");
+  return stream_step_impl(ctx, pats, policy, st, new_ids, attn, evicted_pos, 0, stream);
+}
+
+ta_status ta_ctx_selftest_step_wait(ta_ctx* ctx, const ta_patterns* pats, const ta_policy* policy, ta_stream* st,
+                                    const int32_t* new_ids, const float* attn, int32_t* evicted_pos, uint64_t limit_ns,
+                                    void* stream) {
+  if (limit_ns == 0 || limit_ns > 1000000000ull) return TA_ERR_INVALID_ARG;
+  return stream_step_impl(ctx, pats, policy, st, new_ids, attn, evicted_pos, limit_ns, stream);
 }
 
 // ---------------------------------------------------------------------------------------------- host buffers

@@ -6,12 +6,14 @@
 
 #include "ta.h"
 
-// Device status block: word 0 = first error code (ta_status), word 1..3 = detail (where, what).
+// Device status block: word 0 = first error code (ta_status), word 1..3 = detail (where, what), word 4 = a wait of the decode
+// step ran out.
 struct ta_dev_status {
   int code;
   int where;
   int detail0;
   int detail1;
+  int step_gave_up;
 };
 
 struct ta_patterns {
@@ -31,6 +33,7 @@ constexpr int kStreamWords = 16384;  // blocks of one launch of the decode step 
 struct ta_stream_sync {
   ulonglong2* words;  // device [kStreamWords], 0 between launches: what a sequence's first block tells its others
   unsigned long long wait_limit_ns;
+  unsigned long long hold_ns;  // 0; in the self-test: how long the first blocks hold their words back
 };
 
 struct ta_ctx {

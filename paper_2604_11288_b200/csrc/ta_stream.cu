@@ -140,22 +140,35 @@ __device__ __forceinline__ ulonglong2 seq_words(const SeqStep& r) {
   return make_ulonglong2(kPublished | ((unsigned long long)r.match_len << 32) | __float_as_uint(r.v_new),
                          kPublished | ((unsigned long long)r.t << 32) | (uint32_t)r.count);
 }
-// One word, once it is there. (The block that writes it has a lower index than every block that waits for it.)
+__device__ __forceinline__ bool step_gave_up(const ta_dev_status* status) { return *(volatile const int*)&status->step_gave_up != 0; }
+// One word, once it is there; 0 if the wait runs out. (The block that writes it has a lower index than every block that waits
+// for it.) With one wait that ran out the others of this step end too, and no later step of the context touches its state until
+// the host has polled and cleared the words: one that came late must not be taken for the next step's.
 __device__ __forceinline__ unsigned long long wait_word(const unsigned long long* word, unsigned long long limit_ns,
                                                         ta_dev_status* status, int u) {
   unsigned long long w, t0 = 0;
   for (int it = 0; ((w = *(volatile const unsigned long long*)word) & kPublished) == 0; ++it) {
     if ((it & 63) != 63) continue;
+    if (step_gave_up(status)) return 0ull;
     unsigned long long now;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
     if (t0 == 0) t0 = now;
-    // (the step's results are then not to be used; the waits of other blocks end with this one)
-    if (now - t0 > limit_ns || *(volatile int*)&status->code == (int)TA_ERR_TIMEOUT) {
+    if (now - t0 > limit_ns) {
       report(status, TA_ERR_TIMEOUT, 7, u, 0);
-      break;
+      *(volatile int*)&status->step_gave_up = 1;
+      return 0ull;
     }
   }
   return w;
+}
+// The self-test's first units: for longer than the others wait.
+__device__ __forceinline__ void hold_words(unsigned long long ns) {
+  unsigned long long t0, now;
+  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
+  do {
+    __nanosleep(1000);
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
+  } while (now - t0 < ns);
 }
 
 __device__ __forceinline__ uint32_t sortable_key(float f) {
@@ -236,8 +249,10 @@ ta_stream_step_kernel(ta_stream_dev st, PatternTable pt, const int32_t* new_ids,
   // ---- the unit's state (from L2: the step before wrote it) and its attention masses, all requested before the first is used
   const int x = new_ids[b];
   if (first && warp == 0) {  // before everything else: the other blocks wait for it
+    const bool gone = step_gave_up(status);
     const SeqStep seq = sequence_step(st, pt, b, x, vocab, voucher_decay, budget_decay);
-    const ulonglong2 w = seq_words(seq);
+    if (sync.hold_ns) hold_words(sync.hold_ns);
+    const ulonglong2 w = gone ? make_ulonglong2(0ull, 0ull) : seq_words(seq);
     for (int q = 1 + lane; q < part.nl * part.ng; q += 32) {
       const int l = q / part.ng;
       ulonglong2* to = sync.words + ((l * part.nb + bi) * part.ng + q - l * part.ng);
@@ -269,7 +284,11 @@ ta_stream_step_kernel(ta_stream_dev st, PatternTable pt, const int32_t* new_ids,
   const bool waits = !first && tid < 2;
   unsigned long long* const word = reinterpret_cast<unsigned long long*>(sync.words + blockIdx.x) + (tid & 1);
   unsigned long long said1 = 0;
-  if (waits) said1 = *(volatile unsigned long long*)word;
+  bool gone = false;
+  if (waits) {
+    said1 = *(volatile unsigned long long*)word;
+    gone = step_gave_up(status);
+  }
   int c[E];  // occurrences of the entry's id; of the new token's, which the sequence's first unit counts up: from the words
 #pragma unroll
   for (int e = 0; e < E; ++e) {
@@ -278,12 +297,14 @@ ta_stream_step_kernel(ta_stream_dev st, PatternTable pt, const int32_t* new_ids,
     c[e] = counted && id[e] != x ? __ldcg(&st.hist[(size_t)b * vocab + id[e]]) : counted ? -1 : 0;
   }
   if (waits) {
-    if (!(said1 & kPublished)) said1 = wait_word(word, sync.wait_limit_ns, status, u);
+    if (gone) said1 = 0ull;
+    else if (!(said1 & kPublished)) said1 = wait_word(word, sync.wait_limit_ns, status, u);
     reinterpret_cast<unsigned long long*>(&s_seq)[tid] = said1;
-    *word = 0ull;
+    if (said1) *word = 0ull;
   }
   __syncthreads();
   const ulonglong2 said = s_seq;
+  if (!(said.x & said.y & kPublished)) return;  // a wait ran out: the unit's state stays as it is
   const int t = (int)(said.y >> 32) & 0x7fffffff, match_len = (int)(said.x >> 32) & 0xff;
   const float v_new = __uint_as_float((uint32_t)said.x);
 #pragma unroll

@@ -34,3 +34,119 @@ def test_no_wait_runs_out_while_every_word_comes(L, B, Hkv, K):
     finally:
         ta.ta_patterns_destroy(pats)
         ta.ta_ctx_destroy(ctx)
+
+
+class _Streams:
+    """A context and a decode state of 2 layers, 3 sequences and 4 heads, which has run until its units were full."""
+
+    L, B, Hkv, K = 2, 3, 4, 40
+
+    def __init__(self, seed):
+        self.st, self.t = _state(self.L, self.B, self.Hkv, self.K)
+        self.U = self.L * self.B * self.Hkv
+        self.vocab = self.t["hist"].shape[1]
+        self.pol = ta.ta_policy_default(ta.TA_PRESET_SEC33, self.K)
+        self.pol.vocab_size = self.vocab
+        self.ctx = ta.ta_ctx_create(0, ta.ta_stream_scratch_bytes(self.st))
+        self.pats = ta.ta_patterns_create(self.ctx, [[3], [4, 5]])
+        self.g = torch.Generator(device="cuda")
+        self.g.manual_seed(seed)
+        self.ev = torch.full((self.U,), -9, dtype=torch.int32, device="cuda")
+        self.stream = torch.cuda.current_stream().cuda_stream
+        self.first = torch.zeros(self.U, dtype=torch.bool)  # the first unit of every sequence
+        self.first[: self.B * self.Hkv : self.Hkv] = True
+        for _ in range(self.K + 7):
+            self.step(*self.inputs())
+
+    def inputs(self):
+        ids = torch.randint(0, 8, (self.B,), generator=self.g, device="cuda", dtype=torch.int32)
+        return ids, torch.rand((self.U, self.K + 1), generator=self.g, device="cuda")
+
+    def step(self, ids, attn):
+        ta.ta_stream_step(self.ctx, self.pats, self.pol, self.st, ids, attn, self.ev, self.stream)
+
+    def timed_out_step(self, ids, attn):
+        ta.ta_ctx_selftest_step_wait(self.ctx, self.pats, self.pol, self.st, ids, attn, self.ev, 1_000_000, self.stream)
+
+    def state(self):
+        torch.cuda.synchronize()
+        return {**{n: x.cpu().clone() for n, x in self.t.items()}, "ev": self.ev.cpu().clone()}
+
+    def restore(self, s):
+        for n, x in self.t.items():
+            x.copy_(s[n])
+        self.ev.copy_(s["ev"])
+        torch.cuda.synchronize()
+
+    def close(self):
+        ta.ta_patterns_destroy(self.pats)
+        ta.ta_ctx_destroy(self.ctx)
+
+
+def _same(a, b, units=None):
+    for n in a:
+        x, y = a[n], b[n]
+        if units is not None:
+            if n in ("n_seen", "hist", "tok_ring", "anc_B", "anc_L"):
+                continue  # of a sequence, not of a unit
+            x, y = x[units], y[units]
+        if not torch.equal(x, y):
+            return False
+    return True
+
+
+@pytest.fixture
+def streams():
+    s, ref = _Streams(5), _Streams(5)
+    try:
+        yield s, ref
+    finally:
+        s.close()
+        ref.close()
+
+
+def test_a_unit_whose_wait_runs_out_keeps_its_state(streams):
+    s, ref = streams
+    before = s.state()
+    ids, attn = s.inputs()
+    s.timed_out_step(ids, attn)
+    after = s.state()
+    assert _same(before, after, ~s.first)
+    ref.step(*ref.inputs())
+    assert _same(ref.state(), after, s.first)  # the first units had all that they need
+    # until the context is polled nothing more happens to any unit
+    s.step(*s.inputs())
+    assert _same(after, s.state())
+    assert ta.ta_ctx_poll(s.ctx) == ta.TA_ERR_TIMEOUT
+    assert ta.ta_ctx_poll(s.ctx) == ta.TA_OK
+
+
+def test_words_that_came_late_are_not_taken_for_the_next_steps(streams):
+    s, ref = streams
+    before = s.state()
+    s.timed_out_step(*s.inputs())
+    assert ta.ta_ctx_poll(s.ctx) == ta.TA_ERR_TIMEOUT
+    s.restore(before)
+    s.g.manual_seed(77), ref.g.manual_seed(77)
+    for _ in range(5):
+        s.step(*s.inputs()), ref.step(*ref.inputs())
+        assert _same(ref.state(), s.state())
+    assert ta.ta_ctx_poll(s.ctx) == ta.TA_OK
+
+
+def test_a_time_out_of_another_call_does_not_concern_the_step(streams):
+    s, ref = streams
+    ta.ta_ctx_selftest_wait(s.ctx, 1_000_000, torch.zeros(1, dtype=torch.int32, device="cuda"), s.stream)
+    for _ in range(5):
+        s.step(*s.inputs()), ref.step(*ref.inputs())
+    assert _same(ref.state(), s.state())
+    assert ta.ta_ctx_poll(s.ctx) == ta.TA_ERR_TIMEOUT
+    assert ta.ta_ctx_poll(ref.ctx) == ta.TA_OK
+
+
+@pytest.mark.parametrize("limit", [0, 1_000_000_001])
+def test_the_self_tests_limit_is_checked(streams, limit):
+    s, _ = streams
+    with pytest.raises(ta.TAError) as e:
+        ta.ta_ctx_selftest_step_wait(s.ctx, s.pats, s.pol, s.st, s.ev, s.ev, s.ev, limit, s.stream)
+    assert e.value.status == ta.TA_ERR_INVALID_ARG
