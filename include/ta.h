@@ -146,7 +146,8 @@ void ta_ctx_destroy(ta_ctx* ctx);
 ta_status ta_scratch_bytes(const ta_batch* batch, int Hq, int Hkv, int d, int K, const ta_policy* policy,
                            size_t* out_bytes);
 
-/* Synchronises the context's device, then returns and clears the first device-detected error (TA_OK if none). */
+/* Synchronises the context's device, then returns and clears the first device-detected error (TA_OK if none). When a wait of
+ * ta_stream_step ran out, that is TA_ERR_TIMEOUT, whatever was detected before it. */
 ta_status ta_ctx_poll(ta_ctx* ctx);
 int ta_ctx_last_cuda_error(const ta_ctx* ctx);
 const char* ta_status_string(ta_status s);

@@ -298,10 +298,10 @@ ta_status ta_ctx_poll(ta_ctx* ctx) {
   if (e != cudaSuccess) return cuda_fail(ctx, e);
   if (st.code != 0) {
     cudaMemset(ctx->d_status, 0, sizeof st);
-    if (st.code == TA_ERR_TIMEOUT)  // a block that gave up waiting for its word may have left it to come
+    if (st.step_gave_up)  // a block that gave up waiting for its word may have left it to come
       cudaMemset(ctx->stream_sync.words, 0, kStreamWords * sizeof(ulonglong2));
     ctx->cached_epoch = 0;
-    return (ta_status)st.code;
+    return st.step_gave_up ? TA_ERR_TIMEOUT : (ta_status)st.code;
   }
   return TA_OK;
 }

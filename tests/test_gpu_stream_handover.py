@@ -134,6 +134,21 @@ def test_words_that_came_late_are_not_taken_for_the_next_steps(streams):
     assert ta.ta_ctx_poll(s.ctx) == ta.TA_OK
 
 
+def test_late_words_are_cleared_whatever_was_reported_first(streams):
+    s, ref = streams
+    before = s.state()
+    ids, attn = s.inputs()
+    s.step(torch.full_like(ids, s.vocab), attn)  # outside the vocabulary: the first thing that is reported
+    s.timed_out_step(ids, attn)
+    assert ta.ta_ctx_poll(s.ctx) == ta.TA_ERR_TIMEOUT  # what has cost the state comes before what has not
+    s.restore(before)
+    s.g.manual_seed(78), ref.g.manual_seed(78)
+    for _ in range(5):
+        s.step(*s.inputs()), ref.step(*ref.inputs())
+        assert _same(ref.state(), s.state())
+    assert ta.ta_ctx_poll(s.ctx) == ta.TA_OK
+
+
 def test_a_time_out_of_another_call_does_not_concern_the_step(streams):
     s, ref = streams
     ta.ta_ctx_selftest_wait(s.ctx, 1_000_000, torch.zeros(1, dtype=torch.int32, device="cuda"), s.stream)
