@@ -228,7 +228,6 @@ ta_status ta_ctx_create(int device, size_t scratch_bytes, ta_ctx** out) {
   // the status block and, behind it, the decode step's words
   constexpr size_t kWords = 256, kSyncBytes = kWords + kStreamWords * sizeof(ulonglong2);
   cudaError_t e = cudaMalloc(&c->d_status, kSyncBytes);
-  if (e == cudaSuccess) e = cudaMemset(c->d_status, 0, kSyncBytes);
   c->stream_sync.words = reinterpret_cast<ulonglong2*>(reinterpret_cast<uint8_t*>(c->d_status) + kWords);
   if (e == cudaSuccess && scratch_bytes) e = cudaMalloc(&c->scratch, scratch_bytes);
   for (int i = 0; e == cudaSuccess && i < 8; ++i) e = cudaEventCreate(&c->ev[i]);
@@ -241,6 +240,9 @@ ta_status ta_ctx_create(int device, size_t scratch_bytes, ta_ctx** out) {
     e = cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &c->encode_tiled, cudaEnableDefault, &q);
     if (e == cudaSuccess && (q != cudaDriverEntryPointSuccess || !c->encode_tiled)) e = cudaErrorNotSupported;
   }
+  // complete before the first call, which may be on any stream
+  if (e == cudaSuccess) e = cudaMemsetAsync(c->d_status, 0, kSyncBytes, c->copy_in);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(c->copy_in);
   if (e != cudaSuccess) {
     ta_ctx_destroy(c);
     return TA_ERR_CUDA;
@@ -297,10 +299,13 @@ ta_status ta_ctx_poll(ta_ctx* ctx) {
   e = cudaMemcpy(&st, ctx->d_status, sizeof st, cudaMemcpyDeviceToHost);
   if (e != cudaSuccess) return cuda_fail(ctx, e);
   if (st.code != 0) {
-    cudaMemset(ctx->d_status, 0, sizeof st);
-    if (st.step_gave_up)  // a block that gave up waiting for its word may have left it to come
-      cudaMemset(ctx->stream_sync.words, 0, kStreamWords * sizeof(ulonglong2));
     ctx->cached_epoch = 0;
+    // (complete before this returns: the next call may be on any stream)
+    e = cudaMemsetAsync(ctx->d_status, 0, sizeof st, ctx->copy_in);
+    if (e == cudaSuccess && st.step_gave_up)  // a block that gave up waiting for its word may have left it to come
+      e = cudaMemsetAsync(ctx->stream_sync.words, 0, kStreamWords * sizeof(ulonglong2), ctx->copy_in);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->copy_in);
+    if (e != cudaSuccess) return cuda_fail(ctx, e);
     return st.step_gave_up ? TA_ERR_TIMEOUT : (ta_status)st.code;
   }
   return TA_OK;

@@ -149,6 +149,26 @@ def test_late_words_are_cleared_whatever_was_reported_first(streams):
     assert ta.ta_ctx_poll(s.ctx) == ta.TA_OK
 
 
+def test_a_poll_returns_when_its_clearing_is_complete(streams):
+    # the step after it is on a stream that does not wait for the legacy stream's work
+    s, ref = streams
+    own = torch.cuda.Stream()
+    s.stream = own.cuda_stream
+    for i in range(30):
+        before = s.state()
+        s.timed_out_step(*s.inputs())
+        torch.cuda.synchronize()
+        s.restore(before)
+        s.g.manual_seed(100 + i), ref.g.manual_seed(100 + i)
+        inputs = s.inputs()
+        polled, idle = ta.ta_ctx_poll(s.ctx), torch.cuda.default_stream().query()
+        s.step(*inputs)
+        assert polled == ta.TA_ERR_TIMEOUT and idle
+        ref.step(*ref.inputs())
+        assert _same(ref.state(), s.state())
+    assert ta.ta_ctx_poll(s.ctx) == ta.TA_OK
+
+
 def test_a_time_out_of_another_call_does_not_concern_the_step(streams):
     s, ref = streams
     ta.ta_ctx_selftest_wait(s.ctx, 1_000_000, torch.zeros(1, dtype=torch.int32, device="cuda"), s.stream)
