@@ -1009,7 +1009,6 @@ static ta_status stream_step_impl(ta_ctx* ctx, const ta_patterns* pats, const ta
   if (pats->device != ctx->device) return TA_ERR_INVALID_ARG;
   if (stream_scratch(*st) > ctx->scratch_bytes) return TA_ERR_SCRATCH_TOO_SMALL;
   DeviceGuard guard(ctx->device);
-  ctx->cached_epoch = 0;  // the scratch is shared with ta_compress's per-sequence cache
   cudaStream_t stream = (cudaStream_t)stream_v;
   ta_stream_dev d = {};
   d.n_layers = st->n_layers;
