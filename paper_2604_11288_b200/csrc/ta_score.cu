@@ -375,7 +375,7 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     __syncwarp();
   };
-  bool cluster_known = false, cluster_left = false;  // this warp knows its peers to run / will touch no peer any more
+  bool cluster_known = false;  // this warp knows its peers to run
   // The end of the set-up. Every CTA of the cluster must be running (barriers initialised) before a peer writes to its shared
   // memory or arrives on its barriers: warps that do wait for that before the first time, the others only when they leave.
   auto set_up = [&] {
@@ -902,11 +902,6 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
       // ---- pass 2: for key row_in_tile of each tile, the sum over the job's rows of exp2(s*c - beta_row)
       {
         mbar_wait(smem_u32(&sm.tab_full[up]), ph, abort_flag, p.status, 39, limit);
-        if (one_round && p.cluster > 1) {  // nothing will be sent to a peer any more: said early, so that no CTA waits for it at its end
-          if (!cluster_known) cluster_wait();
-          cluster_arrive_relaxed();
-          cluster_known = cluster_left = true;
-        }
         // every valid row sees keys up to here; key i beyond it is seen by the rows with t >= i - (n - W)
         const int min_lim = p.causal ? n - min(p.W, n) : n - 1;
         const long long out0 = ((long long)ui.l * p.Hkv + ui.g) * p.seq.total + ui.tok0;
@@ -1044,7 +1039,7 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
   }
   // no CTA may leave while a peer can still write to its shared memory or arrive on its barriers
   if (!cluster_known) cluster_wait();  // the set-up's arrival
-  if (!cluster_left) cluster_arrive();
+  cluster_arrive();
   cluster_wait();
   // (after a wait that ran out, statistics that this CTA did not wait for may still be on their way to it)
   if (*abort_flag) __nanosleep(50000);
