@@ -384,7 +384,6 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
     tc_fence_after();
     cluster_arrive_relaxed();
   };
-  // pass-2 constant of row r from its log2-domain log-sum-exp (+inf: the row is mute)
   // window index t of score row r = h*W + t, -1 for padding rows
   auto row_index = [&](int r) { return r < p.rows ? (int)((uint32_t)r % (uint32_t)p.W) : -1; };
   // the tables that the row constants are formed with and that pass 2 reads; written before the first row constants
@@ -395,6 +394,7 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
     // kOutFused: the row's contribution alpha + delta*w (positive, checked by the host) goes into the exponent
     sm.lv[r] = PM == kOutFused && t >= 0 ? log2f(fmaf(p.delta, w, p.alpha)) : 0.0f;
   };
+  // pass-2 constant of row r from its log2-domain log-sum-exp (+inf: the row is mute)
   auto put_row = [&](int up, int r, float lse2) {
     const float beta = lse2 - sm.lv[r];
     const bool poly = MB == 2 && poly_pair<MB, PM>((r & 15) / 2);
