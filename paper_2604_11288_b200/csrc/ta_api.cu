@@ -1141,7 +1141,8 @@ ta_status ta_compress_host(ta_ctx* ctx, const ta_patterns* pats, const ta_policy
 
   // The layers are independent of one another: their caches are copied, compressed and copied back in a few groups, so that
   // the copies of one group run beside the kernels of another and both directions of the bus are busy (8 layers of 2 x 3000
-  // tokens: 2.20 -> 2.06 ms, 107 MB to the device at 55 GB/s being 1.95 ms). A group's cache is at least kGroupBytes, below which its copy is no longer worth the launches.
+  // tokens: 2.20 -> 2.06 ms, 107 MB to the device at 55 GB/s being 1.95 ms). A group's cache is at least kGroupBytes,
+  // below which its copy is no longer worth the launches.
   constexpr size_t kGroupBytes = 8u << 20;
   constexpr int kMaxGroups = 16;
   const int n_layers = batch->n_layers;

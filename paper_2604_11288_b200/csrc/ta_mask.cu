@@ -6,7 +6,8 @@
 // is embarrassingly parallel and HBM traffic is 4 B read + 5 B written per token.
 //   phase a  token ids of tile + halo -> shared memory; per-sequence token histogram via global atomics
 //   phase b  warp-parallel multi-pattern match: every lane tests one end position; a 1024-bit filter on the last
-//            id of all patterns rejects almost every position before the pattern table is walked; one ballot per 32 positions leaves a bitmap of the anchors
+//            id of all patterns rejects almost every position before the pattern table is walked; one ballot per 32
+//            positions leaves a bitmap of the anchors
 //   phase c  span spread: the bitmap's 64 bits before a token, cut off at its sequence's start, name the anchors that can
 //            reach it; their vouchers are added nearest anchor first, in fp32 with one rounding per operation (bit-exact by
 //            construction)

@@ -256,7 +256,9 @@ cudaError_t ta_launch_select_units(const ta_select_args& a, cudaStream_t stream_
   const sel1024::GatherDst gd2 = gather_dst<sel1024::GatherDst>(a, gathers);
   // The instances that look for few tokens, as long as the budget lets them (see cached_radix_select; us without and with them):
   // 1024 units of 16000 tokens K 128 107 / 90, 250 123 / 109; 2048 units of 4000 tokens K 64 62 / 53; 256 units of 4000 tokens K 256
-  // 26.4 / 25.3; 8 units of up to 7000 tokens K 128, 32 calls with their scores 773 / 756.
+  // 26.4 / 25.3; 8 units of up to 7000 tokens K 128, 32 calls with their scores 773 / 756. There is none with 4 keys per thread of
+  // 1024: 8 units K 16 and 64 take as long with one, K 128, 256, 512 of 4000 tokens 16.7, 18.1, 21.5 without and 15.7, 17.4, 20.7
+  // with it, K 256 and 512 of 1000 tokens 14.7 and 17.6 without, 15.0 and 18.0 with it.
   const bool few = gathers && a.K <= kThreads / 2, few1024 = gathers && a.K <= sel1024::kThreads / 2;
   if (few_short_units(a)) {
     auto kern = a.seq.max_n <= 4 * sel1024::kThreads

@@ -6,10 +6,11 @@
 // the lowest index; the new token's voucher from the anchors of the last TA_MAX_SPAN positions, Eq. 2 with budgets that decayed
 // once per step since detection: a lane per anchor), tells the blocks of the sequence's other units, in two words that each of
 // them clears again (a counter of those that have read took 0.8 ns a block), and brings the state that they share (histogram,
-// last ids, anchors, tokens seen) up to date: they read none of it but counts of other ids than the new one. Every block appends the new token to its unit's position-ordered state, adds this step's attention mass to A,
-// updates the pension average P, forms the utility of Eq. 1, applies the budget partition of Section 3.3 to the K+1 cached
-// tokens (exactly one token loses), removes it from the ordered state (4-byte entries move; key/value rows never do: the freed
-// cache row is handed to the next token) and decays every voucher by budget_decay (Algorithm 1 step 10).
+// last ids, anchors, tokens seen) up to date: they read none of it but counts of other ids than the new one. Every block appends
+// the new token to its unit's position-ordered state, adds this step's attention mass to A, updates the pension average P, forms
+// the utility of Eq. 1, applies the budget partition of Section 3.3 to the K+1 cached tokens (exactly one token loses), removes it
+// from the ordered state (4-byte entries move; key/value rows never do: the freed cache row is handed to the next token) and
+// decays every voucher by budget_decay (Algorithm 1 step 10). A block whose words do not come in time leaves its unit as it is.
 // (A kernel of its own for the sequences, in front of this one, cost its launch and tail: 256 units of 257 tokens 11.7 us a step,
 // now 9.5; 4096 units 18.5, now 17.9, alone 38 and 35.5; 2048 units of 1001 tokens 35.4, now 33.7.)
 // What bounds it: latency at few units, the state's bytes (25 read, 12 to 25 written per cached token, 4 of attention
@@ -211,17 +212,17 @@ constexpr bool step_shapes_fit() {
 }
 static_assert(step_shapes_fit(), "a budget for which the step's block does not fit its kernel");
 
-// One block per unit; thread tid holds the entries tid, tid + nt, .. (E of them) in registers for the whole step.
-// Selection (Section 3.3 on the K+1 cached tokens): mandatory sinks and recents; the protected pool = the sponsored,
-// non-mandatory tokens with the largest vouchers (lower position first among equals); exactly one token is then not
-// forced and loses: the one with the smallest utility, the latest position among equals. When the sponsored tokens fit the
-// protected slots, or are one too many, block-wide minima decide; otherwise a radix select on the voucher keys.
 // the units of one launch: layers l0 .. l0 + nl - 1, sequences b0 .. b0 + nb - 1, KV heads g0 .. g0 + ng - 1
 struct StreamPart {
   int l0, nl, b0, nb, g0, ng;
   int update;  // the sequences' last launch
 };
 
+// One block per unit; thread tid holds the entries tid, tid + nt, .. (E of them) in registers for the whole step.
+// Selection (Section 3.3 on the K+1 cached tokens): mandatory sinks and recents; the protected pool = the sponsored,
+// non-mandatory tokens with the largest vouchers (lower position first among equals); exactly one token is then not
+// forced and loses: the one with the smallest utility, the latest position among equals. When the sponsored tokens fit the
+// protected slots, or are one too many, block-wide minima decide; otherwise a radix select on the voucher keys.
 template <int E>
 __global__ void __launch_bounds__(step_threads(E), E == 8 ? 1 : 2)
 ta_stream_step_kernel(ta_stream_dev st, PatternTable pt, const int32_t* new_ids, const float* attn, ta_stream_sync sync,
