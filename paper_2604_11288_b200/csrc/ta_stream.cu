@@ -11,8 +11,11 @@
 // the utility of Eq. 1, applies the budget partition of Section 3.3 to the K+1 cached tokens (exactly one token loses), removes it
 // from the ordered state (4-byte entries move; key/value rows never do: the freed cache row is handed to the next token) and
 // decays every voucher by budget_decay (Algorithm 1 step 10). A block whose words do not come in time leaves its unit as it is.
-// (A kernel of its own for the sequences, in front of this one, cost its launch and tail: 256 units of 257 tokens 11.7 us a step,
-// now 9.5; 4096 units 18.5, now 17.9, alone 38 and 35.5; 2048 units of 1001 tokens 35.4, now 33.7.)
+// The attention masses go to shared memory by asynchronous copies, which hold no registers and which nothing waits for before the
+// block's first barrier (loads that a store to shared memory follows held the loads of the next entry back).
+// (A kernel of its own for the sequences, in front of this one, cost its launch and tail. GPU time of a step in us with it / as one
+// kernel that loads the masses / now: 8 units of 17 tokens 4.9 / 5.4 / 4.6, of 257 5.5 / 6.0 / 5.0, of 1001 6.4 / 6.7 / 5.9; 1024
+// units of 257 7.7 / 7.4 / 6.2, of 1001 19.5 / 17.5 / 16.2; 4096 of 257 19.0 / 17.6 / 16.7.)
 // What bounds it: latency at few units, the state's bytes (25 read, 12 to 25 written per cached token, 4 of attention
 // mass read) at many. 4096 units of 257 tokens, three states in turn (180 MB: more than L2), where the tokens with a voucher fit
 // the protected slots, and where all compete for a quarter of the slots (the extremes of what a generation meets): 31 and 70 us
@@ -172,6 +175,12 @@ __device__ __forceinline__ void hold_words(unsigned long long ns) {
   } while (now - t0 < ns);
 }
 
+// four bytes to shared memory without a register and without waiting for them
+__device__ __forceinline__ void copy_async4(float* to_shared, const float* from) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(to_shared)), "l"(from));
+}
+__device__ __forceinline__ void copy_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
 __device__ __forceinline__ uint32_t sortable_key(float f) {
   uint32_t b = __float_as_uint(f);
   if ((b << 1) == 0u) b = 0u;  // -0 == +0
@@ -187,20 +196,22 @@ __device__ __forceinline__ uint32_t sortable_key(float f) {
 //     1001   71.6   65.5   80.8   82.8   68.1   74.2   71.9   62.5   77.0
 //     1501      -      -      -   94.4   97.8  106.8  101.5  106.9  107.2
 //     2041      -      -      -      -      -      -  183.4  123.5  156.1
-__host__ __device__ constexpr int step_threads(int e) { return e == 3 ? 576 : e == 4 ? 512 : 544; }
+__host__ __device__ constexpr int step_threads(int e) { return e == 3 ? 576 : e == 4 ? 512 : 480; }
 constexpr int step_regs(int e) { return e == 3 ? 56 : 64; }
 // warps of the largest block: what the shared arrays are sized for
 __host__ __device__ constexpr int step_warps(int e) { return step_threads(e) / 32; }
 
 // Entries per thread for units of C cached tokens: three or four, whichever lets an SM hold more blocks (three when equal:
-// fewer spills); eight where a block would have to be larger than those kernels allow.
+// fewer spills); nine where a block would have to be larger than those kernels allow: the largest unit, of 4097 tokens, then has
+// 480 threads, which leaves them the registers that eight entries in 544 did not have (104 bytes spilled; us with eight / nine:
+// 8 units of 2049 tokens 11.3 / 8.1, of 4001 13.0 / 10.9; 1024 units 60.7 / 41.6 and 111 / 79.7).
 constexpr int step_block(int C, int e) { return ((C + e - 1) / e + 31) / 32 * 32; }
 constexpr int step_resident(int C, int e) {
   return step_block(C, e) <= step_threads(e) ? 65536 / (step_block(C, e) * step_regs(e)) : 0;
 }
 constexpr int step_items(int C) {
   const int r3 = step_resident(C, 3), r4 = step_resident(C, 4);
-  return r3 == 0 && r4 == 0 ? 8 : r3 >= r4 ? 3 : 4;
+  return r3 == 0 && r4 == 0 ? 9 : r3 >= r4 ? 3 : 4;
 }
 // every block that the rule can choose holds its unit and is no larger than its kernel's arrays and launch bounds
 constexpr bool step_shapes_fit() {
@@ -224,7 +235,7 @@ struct StreamPart {
 // forced and loses: the one with the smallest utility, the latest position among equals. When the sponsored tokens fit the
 // protected slots, or are one too many, block-wide minima decide; otherwise a radix select on the voucher keys.
 template <int E>
-__global__ void __launch_bounds__(step_threads(E), E == 8 ? 1 : 2)
+__global__ void __launch_bounds__(step_threads(E), E == 9 ? 1 : 2)
 ta_stream_step_kernel(ta_stream_dev st, PatternTable pt, const int32_t* new_ids, const float* attn, ta_stream_sync sync,
                       StreamPart part, int vocab, float voucher_decay, float alpha, float beta, float gamma, float delta,
                       float lambda, float rho, float budget_decay, int n_sink, int n_recent, int k_protected,
@@ -278,7 +289,7 @@ ta_stream_step_kernel(ta_stream_dev st, PatternTable pt, const int32_t* new_ids,
     P[e] = old ? __ldcg(&st.P[base + r]) : 0.0f;
     V[e] = old ? __ldcg(&st.V[base + r]) : 0.0f;
     S[e] = old ? __ldcg(&st.S[base + r]) : 0;
-    if (r < C) s_attn[r] = attn[base + r];
+    if (r < C) copy_async4(&s_attn[r], &attn[base + r]);
   }
   // Two threads wait, each for a word that it alone reads and clears: one that read along could miss the word and wait for good.
   // (The first look at the words: not waited for before the counts are requested.)
@@ -303,6 +314,7 @@ ta_stream_step_kernel(ta_stream_dev st, PatternTable pt, const int32_t* new_ids,
     reinterpret_cast<unsigned long long*>(&s_seq)[tid] = said1;
     if (said1) *word = 0ull;
   }
+  copy_async_wait();
   __syncthreads();
   const ulonglong2 said = s_seq;
   if (!(said.x & said.y & kPublished)) return;  // a wait ran out: the unit's state stays as it is
@@ -520,7 +532,7 @@ cudaError_t ta_launch_stream_step(const ta_stream_dev& st, const ta_patterns* pa
   const int C = st.K + 1;
   const int items = step_items(C), threads = step_block(C, items);
   const size_t smem = (size_t)C * 4;  // at most 16 KB
-  auto kern = items == 3 ? ta_stream_step_kernel<3> : items == 4 ? ta_stream_step_kernel<4> : ta_stream_step_kernel<8>;
+  auto kern = items == 3 ? ta_stream_step_kernel<3> : items == 4 ? ta_stream_step_kernel<4> : ta_stream_step_kernel<9>;
   const PatternTable pt = {pats->d_ids, pats->d_len, pats->d_budget, pats->d_span, pats->n_pat};
   cudaLaunchConfig_t cfg = {};
   cfg.blockDim = dim3((unsigned)threads, 1, 1);

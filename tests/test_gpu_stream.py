@@ -144,7 +144,7 @@ def test_stream_no_patterns_tiny_budget():
                                             (2047, "SEC33", 2060), (2048, "SEC33", 2070)])
 def test_stream_more_sponsored_tokens_than_protected_slots(K, preset, steps):
     # anchors every few tokens: most cached tokens are sponsored, below K = 64 many with equal vouchers (no decay); three, four
-    # and eight cached tokens per thread at the edges of their ranges
+    # and nine cached tokens per thread at the edges of their ranges
     pats = oracle.Patterns([[5], [6, 7]], budget=[15.0, 2.0], span=[3, 8])
     pol = oracle.preset(preset, K, vocab_size=64, budget_decay=1.0 if K < 64 else 0.9)
     _run(K=K, L=1, B=1, Hkv=2 if K < 100 else 1, steps=steps, pats=pats, pol=pol, seed=K, check_every=97)
@@ -154,7 +154,7 @@ def test_stream_more_sponsored_tokens_than_protected_slots(K, preset, steps):
 def test_stream_equal_vouchers_at_the_threshold_in_the_largest_block(K):
     # vouchers that never decay: a few distinct values shared by hundreds of tokens, so that the last protected slots go to
     # the earliest of equal ones; K + 1 entries in the largest blocks of the kernel with three entries per thread (18 warps) and
-    # with four, and in the smallest with eight
+    # with four, and in the smallest with nine
     pats = oracle.Patterns([[5], [6, 7]], budget=[15.0, 2.0], span=[3, 8])
     pol = oracle.preset("SEC33", K, vocab_size=64, budget_decay=1.0)
     ora = _run(K=K, L=1, B=1, Hkv=1, steps=K + 12, pats=pats, pol=pol, seed=K, check_every=97)
