@@ -20,7 +20,7 @@
 // mass read) at many. 4096 units of 257 tokens, three states in turn (180 MB: more than L2), where the tokens with a voucher fit
 // the protected slots, and where all compete for a quarter of the slots (the extremes of what a generation meets): 31 and 70 us
 // with serial scans by one thread in the pool selection, one lane per sequence for the voucher and all entries through shared
-// memory; 22 with two entries in 64 registers, of which an SM held 6 blocks; 18.5 and 25.6 with three in 56.
+// memory; 22 with two entries in 64 registers, of which an SM held 6 blocks; 18.5 and 25.6 with three in 56; 16.5 and 24 now.
 // All arithmetic that decides the selection is fp32 with one rounding per operation, in the order the CPU oracle uses.
 #include "ta_internal.cuh"
 
