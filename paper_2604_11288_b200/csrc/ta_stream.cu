@@ -263,7 +263,7 @@ ta_stream_step_kernel(ta_stream_dev st, PatternTable pt, const int32_t* new_ids,
   if (first && warp == 0) {  // before everything else: the other blocks wait for it
     const bool gone = step_gave_up(status);
     const SeqStep seq = sequence_step(st, pt, b, x, vocab, voucher_decay, budget_decay);
-    if (sync.hold_ns) hold_words(sync.hold_ns);
+    if (sync.hold_ns && !gone && part.nl * part.ng > 1) hold_words(sync.hold_ns);
     const ulonglong2 w = gone ? make_ulonglong2(0ull, 0ull) : seq_words(seq);
     for (int q = 1 + lane; q < part.nl * part.ng; q += 32) {
       const int l = q / part.ng;

@@ -185,3 +185,26 @@ def test_the_self_tests_limit_is_checked(streams, limit):
     with pytest.raises(ta.TAError) as e:
         ta.ta_ctx_selftest_step_wait(s.ctx, s.pats, s.pol, s.st, s.ev, s.ev, s.ev, limit, s.stream)
     assert e.value.status == ta.TA_ERR_INVALID_ARG
+
+
+def test_the_self_test_holds_no_longer_than_the_units_wait():
+    # a call of several launches, and one in which nobody waits: held once, or not at all
+    for L, B, Hkv, expect in ((2, 9000, 2, ta.TA_ERR_TIMEOUT), (1, 20000, 1, ta.TA_OK)):
+        st, t = _state(L, B, Hkv, 4)
+        pol = ta.ta_policy_default(ta.TA_PRESET_THEOREM, 4)
+        pol.vocab_size = t["hist"].shape[1]
+        ctx = ta.ta_ctx_create(0, ta.ta_stream_scratch_bytes(st))
+        pats = ta.ta_patterns_create(ctx, [[3]])
+        stream = torch.cuda.current_stream().cuda_stream
+        ids = torch.randint(0, 8, (B,), device="cuda", dtype=torch.int32)
+        try:
+            e0, e1 = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            e0.record()
+            ta.ta_ctx_selftest_step_wait(ctx, pats, pol, st, ids, torch.rand((L * B * Hkv, 5), device="cuda"),
+                                         torch.empty(L * B * Hkv, dtype=torch.int32, device="cuda"), 50_000_000, stream)
+            e1.record()
+            assert ta.ta_ctx_poll(ctx) == expect
+            assert e0.elapsed_time(e1) < (300 if expect else 50)
+        finally:
+            ta.ta_patterns_destroy(pats)
+            ta.ta_ctx_destroy(ctx)
