@@ -726,6 +726,7 @@ ta_status compress_impl(ta_ctx* ctx, const ta_patterns* pats, const ta_policy* p
   sel.k_protected = policy->k_protected;
   sel.fast = fast;
   sel.sm_count = ctx->sm_count;
+  sel.status = ctx->d_status;
   sel.alpha = policy->alpha;
   sel.delta = policy->delta;
   sel.flags = flags;

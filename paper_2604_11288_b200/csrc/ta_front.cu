@@ -1,10 +1,11 @@
-// Steps 1 and (per-sequence part of) 3 in one kernel, for sequences of up to 16384 tokens: anchor detection, vouchers, the
+// Steps 1 and (per-sequence part of) 3 in one kernel, for sequences of up to 262144 tokens: anchor detection, vouchers, the
 // attention-free utility (Section 3.2; Eq. 2; Eq. 3; Algorithm 1 steps 1-7 without the attention terms), the forced set of
 // Section 3.3 (mandatory tokens and the protected pool) and, in fast mode, the whole selection.
 //
-// One block of 1024 threads per sequence; token i belongs to thread i mod 1024 in every phase. Everything a phase needs from
-// another token sits in shared memory: the ids, the pattern that ends at each position, a bitmap of those positions, and
-// the sequence's token histogram (16-bit counters, two per word; in global memory when the vocabulary does not fit).
+// One block of 1024 threads per sequence, or a cluster of them with a slice of the sequence each; token i of a slice belongs to
+// thread i mod 1024 in every phase. Everything a phase needs from another token sits in shared memory: the ids (and the ids
+// around the slice), the pattern that ends at each position, a bitmap of those positions, and one block's token histogram (16-bit
+// counters, two per word; in global memory when the vocabulary does not fit or the sequence is split).
 //   a  ids -> shared memory; counters cleared
 //   b  histogram; which pattern (longest, then lowest index) ends at each position, behind a 1024-bit filter on the
 //      patterns' last ids; one ballot per 32 positions fills the bitmap
@@ -12,14 +13,18 @@
 //   d  forced set (radix select over the vouchers only when there are more sponsored tokens than protected slots)
 //   e  fast mode: main pool by utility and the ordered write
 // What bounds it: latency (a few barriers, one trip to memory). The same results took a memset and three to five kernels
-// (ta_mask.cu, ta_select.cu: still the path for longer sequences, where one block per sequence would be too few), each
-// with its own launch, trip to memory and tail: one sequence of 4096 tokens 25.6 -> 11.7 us between events around the stage,
-// fast mode with the selection 35.3 -> 12.8 us.
+// (ta_mask.cu, ta_select.cu: still the path for longer sequences and for budgets per layer and head), each with its own launch,
+// trip to memory and tail: one sequence of 4096 tokens 25.6 -> 11.7 us between events around the stage, fast mode with the
+// selection 35.3 -> 12.8 us; four of 131072 tokens 57 -> 35 us a call of one layer with one KV head, 60 of 32768 145 -> 45.
+// A slice of 8192 tokens takes 10 K cycles each for the counts with the matches and for the vouchers with the utilities, the search
+// among 16 slices 17 K, the rest 16 K. The slices' counts meet in global memory: added up through distributed shared memory (every
+// block a share of the vocabulary, the sums handed to all) they took 16 K cycles in place of 5.
 #include <cooperative_groups.h>
 
 #include <atomic>
 
 #include "ta_internal.cuh"
+#include "ta_sm100.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -36,7 +41,8 @@ using namespace front1024;
 constexpr int kPad = TA_MAX_PATTERN_LEN;  // ids before the sequence (never part of a match)
 constexpr int kMaxItems = 16;             // tokens per thread
 constexpr int kListCap = 256;             // so few sponsored tokens are ranked by comparing them with one another
-constexpr int kMaxDynamicSmem = 187 * 1024;  // beside 40 KB of static shared memory (a block may use 227 KB)
+constexpr int kMaxDynamicSmem = 211 * 1024;  // beside at most 16 KB of static shared memory (a block may use 227 KB)
+constexpr int kMaxCluster = 16;
 
 struct FrontParams {
   ta_seq_desc seq;
@@ -62,69 +68,86 @@ struct FrontParams {
 
 // Dynamic shared memory for sequences of up to `items` * 1024 tokens.
 struct FrontSmem {
-  int ids, apat, bits, hist, end;  // byte offsets
+  int select, ids, apat, bits, hist, end;  // byte offsets
 };
-__host__ __device__ inline FrontSmem front_smem(int items, int vocab, bool smem_hist) {
-  const int n = items * kThreads;
+__host__ __device__ constexpr int front_halo(int cl) { return cl > 1 ? TA_MAX_SPAN : 0; }
+__host__ __device__ inline FrontSmem front_smem(int items, int vocab, bool smem_hist, int cl, size_t select_bytes) {
+  const int n = items * kThreads + (cl > 1 ? 32 : 0), halo = front_halo(cl);
   FrontSmem f;
-  f.ids = 0;
-  f.bits = f.ids + (kPad + n) * 4;
+  f.select = 0;
+  f.ids = (int)(select_bytes + 15) / 16 * 16;
+  f.bits = f.ids + (kPad + halo + n) * 4;
   f.apat = f.bits + (n / 32 + 4) * 4;  // two words of zeros before and after
-  f.hist = f.apat + n * 2;
-  f.end = f.hist + (smem_hist ? (vocab + 1) / 2 * 4 : 0);
+  f.hist = (f.apat + (halo + n) * 2 + 15) / 16 * 16;
+  f.end = f.hist + (smem_hist ? (vocab + 7) / 8 * 16 : 0);
   return f;
 }
 
-template <int ITEMS, bool FAST, bool SMEM_HIST>
+template <int ITEMS, bool FAST, bool SMEM_HIST, int CL>
 __global__ void __launch_bounds__(kThreads, 1) ta_front_kernel(const __grid_constant__ FrontParams p) {
   extern __shared__ __align__(16) unsigned char dyn[];
-  __shared__ SelectShared sh;
   __shared__ int32_t s_pid[TA_MAX_PATTERNS * TA_MAX_PATTERN_LEN];
   __shared__ int32_t s_plen[TA_MAX_PATTERNS], s_pspan[TA_MAX_PATTERNS];
   __shared__ float s_pbud[TA_MAX_PATTERNS];
   __shared__ uint32_t s_bloom[32];
   __shared__ float s_w[TA_MAX_SPAN + 1];
   __shared__ uint32_t s_fbits[kMaxItems * kWarps];  // bit of every token: forced
-  __shared__ int s_count;
   __shared__ __align__(8) uint2 s_list[kListCap];  // key and position of sponsored, not mandatory tokens
+  __shared__ __align__(8) int s_sponsored[CL][2];     // CL > 1: sponsored, not mandatory tokens of every slice
   __shared__ int s_listed;                            // how many there are (also beyond the capacity of the list)
-  const FrontSmem L = front_smem(ITEMS, p.vocab, SMEM_HIST);
-  int32_t* s_id = reinterpret_cast<int32_t*>(dyn + L.ids) + kPad;       // s_id[-kPad .. n)
-  uint32_t* s_bits = reinterpret_cast<uint32_t*>(dyn + L.bits) + 2;     // s_bits[-2 .. n/32 + 2)
-  int16_t* s_apat = reinterpret_cast<int16_t*>(dyn + L.apat);
+  constexpr int kHalo = front_halo(CL);  // positions before the slice whose matches reach into it
+  const FrontSmem L = front_smem(ITEMS, p.vocab, SMEM_HIST, CL, sizeof(SelectShared<CL>));
+  SelectShared<CL>& sh = *reinterpret_cast<SelectShared<CL>*>(dyn + L.select);
+  int32_t* s_id = reinterpret_cast<int32_t*>(dyn + L.ids) + kPad + kHalo;  // s_id[-kPad - kHalo .. n)
+  uint32_t* s_bits = reinterpret_cast<uint32_t*>(dyn + L.bits) + 2;        // s_bits[-2 .. n/32 + 2)
+  int16_t* s_apat = reinterpret_cast<int16_t*>(dyn + L.apat) + kHalo;
   uint32_t* s_hist = reinterpret_cast<uint32_t*>(dyn + L.hist);
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int b = blockIdx.x;
+  const int b = blockIdx.x / CL;
   // decay^k by repeated multiplication (one rounding per step), thread k on its own
   if (tid <= TA_MAX_SPAN) {
     float w = 1.0f;
     for (int k = 0; k < tid; ++k) w = __fmul_rn(w, p.voucher_decay);
     s_w[tid] = w;
   }
-  if (tid < kPad) s_id[tid - kPad] = -1;
+  if (CL == 1 && tid < kPad) s_id[tid - kPad] = -1;
   if (tid < ITEMS * kWarps + 4) s_bits[tid - 2] = 0u;  // also the words of positions behind the sequence
-  if (tid == 0) s_count = s_listed = 0;
+  if (tid == 0) s_listed = 0;
   if (tid < ITEMS * kWarps) s_fbits[tid] = 0u;
   if (SMEM_HIST)
 #pragma unroll 4
-    for (int i = tid; i < (p.vocab + 1) / 2; i += kThreads) s_hist[i] = 0u;
+    for (int i = tid; i < (p.vocab + 7) / 8; i += kThreads) reinterpret_cast<uint4*>(s_hist)[i] = make_uint4(0u, 0u, 0u, 0u);
+  Exchange<CL> ex;
+  ex.status = p.status;
+  if constexpr (CL > 1) ex.set_up(sh);
   ta_wait_for_prior_grid();
   ta_launch_dependents();
 
   // ---- a: every load is requested before the first is used
   const SeqInfo s = seq_info(p.seq, b, p.K, p.n_sink, p.n_recent, p.k_protected);
   const int n = s.n;
+  // this CTA's slice: tokens [lo, lo + nl); local index i <-> position lo + i. Whole words of the bitmap.
+  const int per = CL == 1 ? n : ((n + CL - 1) / CL + 31) / 32 * 32;
+  const int rank = CL == 1 ? 0 : (int)cg::this_cluster().block_rank();
+  const int lo = min(n, rank * per), nl = min(n - lo, per);
+  const int nx = CL == 1 ? n : min(nl + TA_MAX_PATTERN_LEN, n - lo);  // with the tokens whose matches can cover the slice's last
   int32_t* hist = p.hist + (size_t)b * p.vocab;
+  const int32_t* ids = p.ids + (long long)s.start + lo;
   int id[ITEMS];
 #pragma unroll
   for (int it = 0; it < ITEMS; ++it) {
     const int i = tid + it * kThreads;
-    id[it] = i < n ? p.ids[(long long)s.start + i] : -1;
+    id[it] = i < nx ? ids[i] : -1;
   }
+  // the tokens before the slice that can match into it, and those behind it that do not fit the threads' slots
+  const int i_halo = tid < kPad + kHalo ? tid - kPad - kHalo : ITEMS * kThreads + tid - kPad - kHalo;
+  int id_halo = -1;
+  if (CL > 1 && tid < kPad + kHalo + kPad && lo + i_halo >= 0 && i_halo < nx) id_halo = ids[i_halo];
   int32_t r_pid[2];
 #pragma unroll
   for (int q = 0; q < 2; ++q) r_pid[q] = tid + q * kThreads < p.n_pat * TA_MAX_PATTERN_LEN ? p.p_ids[tid + q * kThreads] : 0;
+  static_assert(CL == 1 || !SMEM_HIST, "the counters of one block");
   static_assert(TA_MAX_PATTERNS * TA_MAX_PATTERN_LEN <= 2 * kThreads, "two table entries per thread");
   int32_t r_len = 0, r_span = 0;
   float r_bud = 0.0f;
@@ -148,9 +171,16 @@ __global__ void __launch_bounds__(kThreads, 1) ta_front_kernel(const __grid_cons
   for (int it = 0; it < ITEMS; ++it) {
     const int i = tid + it * kThreads;
     s_id[i] = id[it];
-    if (!SMEM_HIST && id[it] >= 0 && id[it] < p.vocab) hist[id[it]] = 0;
+    if (CL == 1 && !SMEM_HIST && id[it] >= 0 && id[it] < p.vocab) hist[id[it]] = 0;
   }
-  __syncthreads();
+  if (CL > 1 && tid < kPad + kHalo + kPad) s_id[i_halo] = id_halo;
+  if constexpr (CL > 1) {  // every CTA clears its share of the sequence's counters
+    const int share = (p.vocab + CL - 1) / CL, end = min(p.vocab, (rank + 1) * share);
+    for (int i = rank * share + tid; i < end; i += kThreads) hist[i] = 0;
+    cg::this_cluster().sync();
+  } else {
+    __syncthreads();
+  }
   if (s.bad) {
     if (tid == 0) {
       if (atomicCAS(&p.status->code, 0, (int)TA_ERR_DEVICE_BOUNDS) == 0) {
@@ -161,7 +191,7 @@ __global__ void __launch_bounds__(kThreads, 1) ta_front_kernel(const __grid_cons
       if (FAST) p.count[b] = 0;
       else p.r_main[b] = -2;  // poisoned: the selection writes an empty result
     }
-    if (FAST)
+    if (FAST && rank == 0)
       for (int r = tid; r < p.K; r += kThreads) p.idx[(long long)b * p.K + r] = -1;
     return;
   }
@@ -171,18 +201,21 @@ __global__ void __launch_bounds__(kThreads, 1) ta_front_kernel(const __grid_cons
   // sponsored tokens).
   // ---- b: histogram and matches
 #pragma unroll 1
-  for (int it = 0; it * kThreads < n; ++it) {
+  for (int it = CL == 1 ? 0 : -1; it * kThreads < nx; ++it) {  // (chunk -1: the positions before a slice)
     const int i = tid + it * kThreads;
-    const int x = s_id[i];
+    if (CL > 1 && (i - lane < -kHalo || i - lane >= nx)) continue;  // (whole warps; the words behind the slice are zero)
+    const int x = i < nx ? s_id[i] : -1;
     int best = -1;
     bool may_end = false;
-    if (i < n) {
-      if (x >= 0 && x < p.vocab) {
+    if (i < nx) {
+      if (CL > 1 && (i < 0 || i >= nl)) {
+        // another CTA counts it
+      } else if (x >= 0 && x < p.vocab) {
         if (SMEM_HIST) atomicAdd(&s_hist[x >> 1], (x & 1) ? 0x10000u : 1u);
         else atomicAdd(&hist[x], 1);
       } else if (atomicCAS(&p.status->code, 0, (int)TA_ERR_DEVICE_BOUNDS) == 0) {
         p.status->where = 1;
-        p.status->detail0 = s.start + i;
+        p.status->detail0 = s.start + lo + i;
         p.status->detail1 = x;
       }
       const uint32_t h = ((uint32_t)x * 2654435761u) >> 22;
@@ -194,7 +227,7 @@ __global__ void __launch_bounds__(kThreads, 1) ta_front_kernel(const __grid_cons
     for (unsigned left = __ballot_sync(0xffffffffu, may_end); left != 0u; left &= left - 1u) {
       const int src = __ffs((int)left) - 1, end = i - lane + src;
       const int y = __shfl_sync(0xffffffffu, x, src);
-      const int avail = min(TA_MAX_PATTERN_LEN, end + 1);  // matches never cross the start of the sequence
+      const int avail = min(TA_MAX_PATTERN_LEN, lo + end + 1);  // matches never cross the start of the sequence
       uint32_t mine = 0;                                   // length, then the complement of the index: the largest wins
 #pragma unroll 1
       for (int q = lane; q < p.n_pat; q += 32) {
@@ -213,7 +246,11 @@ __global__ void __launch_bounds__(kThreads, 1) ta_front_kernel(const __grid_cons
     if (word) s_apat[i] = (int16_t)best;  // read only where a bit of `word` is set
     if (lane == 0) s_bits[it * kWarps + warp] = word;
   }
-  __syncthreads();
+  if constexpr (CL == 1) {
+    __syncthreads();
+  } else {
+    cg::this_cluster().sync();  // the sequence's counts are complete
+  }
 
   // ---- c: vouchers and static utilities. From here on a thread reads its own ids only: fast mode leaves the utilities in
   // their place.
@@ -237,7 +274,7 @@ __global__ void __launch_bounds__(kThreads, 1) ta_front_kernel(const __grid_cons
     return V;
   };
 #pragma unroll 1
-  for (int it = 0; it * kThreads < n; ++it) {
+  for (int it = 0; it * kThreads < nl; ++it) {
     const int i = tid + it * kThreads;
     const int x = s_id[i];
     const uint32_t* w = s_bits + (i >> 5);  // the same for the whole warp
@@ -254,24 +291,32 @@ __global__ void __launch_bounds__(kThreads, 1) ta_front_kernel(const __grid_cons
         anchor_token = anchor_token || s_plen[s_apat[i + k]] > k;
       }
     }
-    if (i < n) {
+    if (i < nl) {
       int c = 0;
       if (x >= 0 && x < p.vocab) {
         if (SMEM_HIST) c = (int)((s_hist[x >> 1] >> ((x & 1) * 16)) & 0xffffu);
         else c = __ldcg(&hist[x]);
       }
-      const float u = ta_static_utility(i, n, c, anchor_token, V, p.beta, p.gamma, p.lambda);
+      const float u = ta_static_utility(lo + i, n, c, anchor_token, V, p.beta, p.gamma, p.lambda);
       if (FAST) s_u[i] = u;
-      else p.u_static[(long long)s.start + i] = u;
-      if (V > 0.0f && !mandatory(i)) {
+      else p.u_static[(long long)s.start + lo + i] = u;
+      if (CL == 1 && V > 0.0f && !mandatory(i)) {
         const int slot = atomicAdd(&s_listed, 1);
         if (slot < kListCap) s_list[slot] = make_uint2(sortable_key(V), (uint32_t)i);
+      }
+    }
+    if (CL > 1) {  // the sponsored, not mandatory tokens as bits: forced if the cluster's fit the protected slots
+      const unsigned sponsored = __ballot_sync(0xffffffffu, i < nl && V > 0.0f && !mandatory(lo + i));
+      if (lane == 0 && sponsored != 0u) {
+        s_fbits[it * kWarps + warp] = sponsored;
+        atomicAdd(&s_listed, __popc(sponsored));
       }
     }
   }
   __syncthreads();
 
   if (s.K_eff == n) {  // keep everything
+    if (rank != 0) return;
     if (FAST) {
       for (int r = tid; r < p.K; r += kThreads) p.idx[(long long)b * p.K + r] = r < n ? r : -1;
       if (tid == 0) p.count[b] = n;
@@ -283,9 +328,19 @@ __global__ void __launch_bounds__(kThreads, 1) ta_front_kernel(const __grid_cons
 
   // ---- d: the forced set, as bits: the mandatory tokens and the s.p largest vouchers, lower positions first among equals
   KeyCache<ITEMS> kc;
-  const int m = s_listed;
+  int m = s_listed;
   int taken = s.s_take + s.r_take;
-  if (m <= kListCap) {
+  if constexpr (CL > 1) {
+    if (tid < CL) ex.send2(sh, s_sponsored[rank], tid, (uint32_t)m, 0u);
+    const bool ok = ex.wait(sh, CL * 8);
+    m = 0;
+#pragma unroll
+    for (int q = 0; q < CL; ++q) m += s_sponsored[q][0];
+    if (!ok) m = 0;
+  }
+  if (CL > 1 && m <= s.p) {
+    taken += m;  // (the bits are there)
+  } else if (CL == 1 && m <= kListCap) {
     if (tid < m) {
       const uint2 mine = s_list[tid];
       int before = 0;  // listed tokens that come first
@@ -304,27 +359,28 @@ __global__ void __launch_bounds__(kThreads, 1) ta_front_kernel(const __grid_cons
     for (int it = 0; it < ITEMS; ++it) {
       const int i = tid + it * kThreads;
       kc.key[it] = 0u;
-      if (i < n) {
+      if (i < nl) {
         const float V = voucher(s_bits + (i >> 5), i);
         kc.key[it] = sortable_key(V);
-        if (mandatory(i)) always |= 1u << it;
+        if (mandatory(lo + i)) always |= 1u << it;
         else if (V > 0.0f) kc.elig |= 1u << it;
       }
     }
-    const SelectResult r = cached_radix_select<1>(n, n, s.p, kc, sh);
-    taken = cached_ordered_emit<1>(n, r, kc, always, [&](int i, int) { atomicOr(&s_fbits[i >> 5], 1u << (i & 31)); }, sh);
+    if (CL > 1 && tid < ITEMS * kWarps) s_fbits[tid] = 0u;  // (set again below, several barriers later)
+    const SelectResult r = cached_radix_select<CL>(nl, n, s.p, kc, sh, ex);
+    taken = cached_ordered_emit<CL>(nl, r, kc, always, [&](int i, int) { atomicOr(&s_fbits[i >> 5], 1u << (i & 31)); }, sh, ex);
   }
   __syncthreads();
   uint32_t fmask = 0;  // bit it: this thread's token of chunk it is forced
 #pragma unroll
   for (int it = 0; it < ITEMS; ++it) {
     const int i = tid + it * kThreads;
-    const bool f = i < n && (((s_fbits[it * kWarps + warp] >> lane) & 1u) != 0 || mandatory(i));
+    const bool f = i < nl && (((s_fbits[it * kWarps + warp] >> lane) & 1u) != 0 || mandatory(lo + i));
     if (FAST) fmask |= f ? 1u << it : 0u;
-    else if (i < n) p.forced[(long long)s.start + i] = f ? 1 : 0;
+    else if (i < nl) p.forced[(long long)s.start + lo + i] = f ? 1 : 0;
   }
   if (!FAST) {
-    if (tid == 0) p.r_main[b] = s.K_eff - taken;
+    if (tid == 0 && rank == 0) p.r_main[b] = s.K_eff - taken;
     return;
   }
 
@@ -333,23 +389,25 @@ __global__ void __launch_bounds__(kThreads, 1) ta_front_kernel(const __grid_cons
 #pragma unroll
   for (int it = 0; it < ITEMS; ++it) {
     const int i = tid + it * kThreads;
-    kc.key[it] = i < n ? sortable_key(s_u[i]) : 0u;
+    kc.key[it] = i < nl ? sortable_key(s_u[i]) : 0u;
   }
-  kc.elig = exist_mask(n) & ~fmask;
+  kc.elig = exist_mask(nl) & ~fmask;
   __syncthreads();  // the select state is used a second time
-  const SelectResult r2 = cached_radix_select<1>(n, n, s.K_eff - taken, kc, sh);
-  const int got = cached_ordered_emit<1>(n, r2, kc, fmask, [&](int i, int rank) {
-    if (rank < p.K) out[rank] = i;
-  }, sh);
+  const SelectResult r2 = cached_radix_select<CL>(nl, n, s.K_eff - taken, kc, sh, ex);
+  const int got = cached_ordered_emit<CL>(nl, r2, kc, fmask, [&](int i, int place) {
+    if (place < p.K) out[place] = lo + i;
+  }, sh, ex);
+  if (rank != 0) return;
   for (int q = got + tid; q < p.K; q += kThreads) out[q] = -1;
   if (tid == 0) p.count[b] = got;
 }
 
-template <int ITEMS, bool FAST>
-cudaError_t launch_front(const FrontParams& p, bool smem_hist, cudaStream_t stream) {
-  auto kern = smem_hist ? ta_front_kernel<ITEMS, FAST, true> : ta_front_kernel<ITEMS, FAST, false>;
-  const int smem = front_smem(ITEMS, p.vocab, smem_hist).end;
-  // per device; setting the (sticky) attribute twice from two threads is harmless, the flag only saves the call
+template <int ITEMS, bool FAST, int CL>
+cudaError_t launch_front(const FrontParams& p, cudaStream_t stream) {
+  const bool smem_hist = CL == 1 && front_smem(ITEMS, p.vocab, true, CL, sizeof(SelectShared<CL>)).end <= kMaxDynamicSmem;
+  auto kern = smem_hist ? ta_front_kernel<ITEMS, FAST, CL == 1, CL> : ta_front_kernel<ITEMS, FAST, false, CL>;
+  const int smem = front_smem(ITEMS, p.vocab, smem_hist, CL, sizeof(SelectShared<CL>)).end;
+  // per device; setting the (sticky) attributes twice from two threads is harmless, the flag only saves the calls
   static std::atomic<bool> attr_set[2][64];
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
@@ -357,24 +415,69 @@ cudaError_t launch_front(const FrontParams& p, bool smem_hist, cudaStream_t stre
   std::atomic<bool>& set = attr_set[smem_hist ? 1 : 0][dev & 63];
   if (!set.load(std::memory_order_acquire)) {
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynamicSmem);
+    if (e == cudaSuccess && CL > 8) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
     set.store(true, std::memory_order_release);
   }
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)p.seq.batch, 1, 1);
+  cfg.gridDim = dim3((unsigned)(p.seq.batch * CL), 1, 1);
   cfg.blockDim = dim3(kThreads, 1, 1);
   cfg.dynamicSmemBytes = (size_t)smem;
   cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   ta_pdl_attribute(&attr[0]);
   cfg.attrs = attr;
   cfg.numAttrs = 1;
+  if (CL > 1) {
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)CL;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
+    cfg.numAttrs = 2;
+  }
   return cudaLaunchKernelEx(&cfg, kern, p);
+}
+
+// Blocks per sequence. One holds up to 16384 tokens; more are worth their exchanges where a thread of one block would have more
+// than 12 tokens, or has to. Of the sizes that hold the longest sequence the largest of which all sequences' clusters fit at once
+// (148 SMs: 7 of 16 blocks, 15 of 8, 35 of 4, 74 of 2), else the smallest. us per call of TA-Fast (one layer, one KV head) with
+// separate kernels for mask, forced set and selection / 2 / 4 / 8 / 16 blocks:
+//   1 x 131072 K 64 38.1 / - / - / 41.2 / 29.7; 4 x 131072 K 4096 57.1 / - / - / 46.1 / 35.4; 16 x 131072 109.6 / - / - / 78.5 / 82.6
+//   4 x 65536 42.2 / - / 40.5 / 28.5 / 24.5; 8 x 32768 37.7 / 41.4 / 28.5 / 23.6 / 44.0; 60 x 32768 144.6 / 45.4 / 57.9 / 87.5 / 190
+// and with one block / 2 / 4 / 8: 1 x 16384 26.3 / 25.7 / 19.3 / 16.9, 8 x 16384 27.5 / 26.8 / 20.5 / 18.2, 60 x 16384 31.7 / 31.1 /
+// 41.6 / 66; 4 x 12000 18.5 / 25.6 / 19.4 / 17.6, 1 x 8192 14.7 / 21.7 / 18.0 / 16.6. Beside a score kernel, which hides it, one
+// block leaves it the most SMs.
+int front_blocks(int n, int batch, int sms, bool hidden) {
+  if (n <= (hidden ? kMaxItems : 12) * kThreads) return 1;
+  const int fit[] = {7, 15, 35, 74}, least = (n + kMaxItems * kThreads - 1) / (kMaxItems * kThreads);
+  for (int i = 0, cl = kMaxCluster; cl > 1 && cl >= least; ++i, cl /= 2)
+    if (batch <= fit[i] * sms / 148) return cl;
+  return least <= 1 ? 1 : least <= 2 ? 2 : least <= 4 ? 4 : least <= 8 ? 8 : kMaxCluster;
+}
+
+template <bool FAST, int CL>
+cudaError_t launch_items(const FrontParams& p, cudaStream_t stream) {
+  // the smallest instance that holds the slices: unused slots cost issue time in every phase
+  const int items = (p.seq.max_n + CL * kThreads - 1) / (CL * kThreads);
+  if (CL != 2 && items <= 4) return launch_front<CL == 2 ? kMaxItems : 4, FAST, CL>(p, stream);
+  if (CL != 2 && items <= 8) return launch_front<CL == 2 ? kMaxItems : 8, FAST, CL>(p, stream);
+  return launch_front<kMaxItems, FAST, CL>(p, stream);
+}
+
+template <bool FAST>
+cudaError_t launch_split(const FrontParams& p, int sms, bool hidden, cudaStream_t stream) {
+  switch (front_blocks(p.seq.max_n, p.seq.batch, sms, hidden)) {
+    case 1: return launch_items<FAST, 1>(p, stream);
+    case 2: return launch_items<FAST, 2>(p, stream);
+    case 4: return launch_items<FAST, 4>(p, stream);
+    case 8: return launch_items<FAST, 8>(p, stream);
+    default: return launch_items<FAST, kMaxCluster>(p, stream);
+  }
 }
 
 }  // namespace
 
-bool ta_front_fits(const ta_seq_desc& seq) { return seq.max_n <= kMaxItems * kThreads; }
+bool ta_front_fits(const ta_seq_desc& seq) { return seq.max_n <= kMaxCluster * kMaxItems * kThreads; }
 
 cudaError_t ta_launch_front(const ta_patterns* pats, const ta_policy& pol, const ta_select_args& a, const int32_t* ids,
                             int32_t* hist, ta_dev_status* status, cudaStream_t stream) {
@@ -408,15 +511,6 @@ cudaError_t ta_launch_front(const ta_patterns* pats, const ta_policy& pol, const
   p.idx = a.idx;
   p.count = a.count;
   p.status = status;
-  // the smallest instance that holds the sequences: unused slots cost issue time in every phase
-  const int items = a.seq.max_n <= 4 * kThreads ? 4 : a.seq.max_n <= 8 * kThreads ? 8 : 16;
-  const bool smem_hist = front_smem(items, pol.vocab_size, true).end <= kMaxDynamicSmem;
-  if (a.fast) {
-    if (items == 4) return launch_front<4, true>(p, smem_hist, stream);
-    if (items == 8) return launch_front<8, true>(p, smem_hist, stream);
-    return launch_front<16, true>(p, smem_hist, stream);
-  }
-  if (items == 4) return launch_front<4, false>(p, smem_hist, stream);
-  if (items == 8) return launch_front<8, false>(p, smem_hist, stream);
-  return launch_front<16, false>(p, smem_hist, stream);
+  const int sms = a.sm_count > 0 ? a.sm_count : 148;
+  return a.fast ? launch_split<true>(p, sms, false, stream) : launch_split<false>(p, sms, a.u != nullptr, stream);
 }

@@ -209,6 +209,7 @@ struct ta_select_args {
   int fast;
   int sm_count;  // of the device the launch goes to (0: ask the runtime about the current device)
   float alpha, delta;
+  ta_dev_status* status;  // of ta_launch_select_units (nullable)
   const uint8_t* flags;
   const float* voucher;
   const float* u_static;
@@ -239,9 +240,10 @@ struct ta_select_args {
   float beta, gamma, lambda;
 };
 bool ta_select_gathers(const ta_select_args& a);  // whether ta_launch_select_units will do the gather itself
-// Steps 1 and the per-sequence part of 3 in one kernel for sequences that fit one block (ta_front.cu): static utilities, forced
+// Steps 1 and the per-sequence part of 3 in one kernel for sequences that fit a cluster of blocks (ta_front.cu): static utilities, forced
 // set and r_main as ta_launch_mask and ta_launch_forced leave them (without flags and vouchers); fast mode: idx and count
-// per sequence, and nothing else. hist is used only for vocabularies that do not fit in shared memory; needs no clearing.
+// per sequence, and nothing else. hist is used for vocabularies that do not fit in shared memory and for sequences beyond one
+// block; needs no clearing.
 // The kernel lets its programmatic dependent start as soon as it runs itself.
 bool ta_front_fits(const ta_seq_desc& seq);
 cudaError_t ta_launch_front(const ta_patterns* pats, const ta_policy& pol, const ta_select_args& a, const int32_t* ids,

@@ -19,6 +19,7 @@
 #include <cooperative_groups.h>
 
 #include "ta_internal.cuh"
+#include "ta_sm100.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -208,6 +209,7 @@ Src unit_src(const ta_select_args& a) {
   s.u_static = a.u_static;
   s.alpha = a.alpha;
   s.delta = a.delta;
+  s.status = a.status;
   return s;
 }
 template <class Dst>
@@ -328,7 +330,9 @@ cudaError_t ta_launch_select_units(const ta_select_args& a, cudaStream_t stream_
 cudaError_t ta_launch_select(const ta_select_args& a, ta_dev_status* status, cudaStream_t stream) {
   cudaError_t e = ta_launch_forced(a, status, stream);
   if (e != cudaSuccess) return e;
-  return ta_launch_select_units(a, stream);
+  ta_select_args with_status = a;
+  with_status.status = status;
+  return ta_launch_select_units(with_status, stream);
 }
 
 cudaError_t ta_launch_broadcast_idx(int B, int Hkv, int K, int n_layers, const int32_t* idx_seq,

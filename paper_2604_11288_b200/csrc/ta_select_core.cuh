@@ -26,8 +26,9 @@ struct SelectResult {
 constexpr int kCandCap = 2048;  // candidates a split unit finishes locally
 constexpr int kCompareCap = 32;  // so few candidates are compared with one another instead of counted by digits
 
+template <int CL>  // CTAs that share a unit
 struct SelectShared {
-  uint32_t hist[256];
+  __align__(16) uint32_t hist[256];
   uint32_t prefix, mask;
   int remaining;
   int done_all;
@@ -35,11 +36,12 @@ struct SelectShared {
   __align__(16) uint32_t warp_cnt[kWarps];  // per warp: definite count (low 16 bits) | tie count (high 16 bits)
   // range of the eligible keys: per warp (smallest, largest, how many), and per CTA of a cluster
   uint32_t wmin[kWarps], wmax[kWarps], wnum[kWarps];
-  uint32_t cl_range[8][4];
-  // long sequences are split over the CTAs of a cluster: histogram of the whole unit (on rank 0, two buffers
-  // alternating by pass) and every CTA's (definite, tie) totals
-  uint32_t ghist[2][256];
-  int totals[8][2];
+  __align__(16) uint32_t cl_range[CL][4];
+  // long sequences are split over the CTAs of a cluster: every CTA's histogram, two counts to a word, as it sent them to all
+  // (two buffers alternating by pass), and every CTA's (definite, tie) totals
+  __align__(16) uint32_t ghist[CL > 1 ? 2 : 1][CL][CL > 1 ? 128 : 1];
+  __align__(8) int totals[2][CL][2];        // (by the exchange's number)
+  __align__(8) unsigned long long arrived[2];  // mbarriers of the exchanges between the CTAs, taken in turn
   // ordered write of a unit whose keys sit in registers: bitmaps of the definite and of the tie elements in position
   // order (word e covers positions 32e .. 32e+31 of this CTA's slice)
   // (a row of kWarps words per chunk, padded by one word so that the 32 rows a warp writes fall into 32 banks)
@@ -47,8 +49,8 @@ struct SelectShared {
   uint32_t wtot[kWarps];
   uint32_t before[kThreads];  // definite (low 16 bits) and tie elements before every word
   uint32_t total;
-  // a unit split over a cluster: once few candidates are left, their keys are collected (on rank 0, then copied by
-  // every CTA) and the remaining passes run on that list inside each CTA, without cluster barriers
+  // a unit split over a cluster: once few candidates are left, every CTA sends its own to all and the remaining passes run on
+  // that list inside each CTA, without cluster barriers
   uint32_t cand_n;
   __align__(16) uint32_t cand_keys[kCandCap];
   uint32_t cmp_n, cmp_thresh;  // the same inside one CTA, for at most kCompareCap candidates
@@ -104,7 +106,7 @@ __device__ __forceinline__ void sweep(int n, KeyFn key_of, const KeyCache<ITEMS>
 // Top-`want` of the eligible elements of [0, n) by key. All threads of the block must call it; the result is uniform
 // across the block.
 template <bool CACHED, int CL, class KeyFn, int ITEMS>
-__device__ SelectResult block_radix_select(int n, int want, KeyFn key_of, const KeyCache<ITEMS>& kc, SelectShared& sh) {
+__device__ SelectResult block_radix_select(int n, int want, KeyFn key_of, const KeyCache<ITEMS>& kc, SelectShared<CL>& sh) {
   SelectResult r;
   r.thresh = 0;
   r.ties = 0;
@@ -120,12 +122,12 @@ __device__ SelectResult block_radix_select(int n, int want, KeyFn key_of, const 
     sh.done_all = 0;
   }
   uint32_t* ghist0 = nullptr;
-  if (CL > 1) ghist0 = cg::this_cluster().map_shared_rank(&sh.ghist[0][0], 0);
+  if (CL > 1) ghist0 = cg::this_cluster().map_shared_rank(&sh.ghist[0][0][0], 0);
   for (int pass = 0; pass < 4; ++pass) {
     const int shift = 24 - 8 * pass;
     for (int k = tid; k < 256; k += kThreads) {
       sh.hist[k] = 0;
-      if (CL > 1) sh.ghist[pass & 1][k] = 0;  // only rank 0's copy is used; its readers of two passes ago are done
+      if (CL > 1) (&sh.ghist[pass & 1][0][0])[k] = 0;  // only rank 0's copy is used; its readers of two passes ago are done
     }
     if (CL > 1) cg::this_cluster().sync();
     else __syncthreads();
@@ -145,7 +147,7 @@ __device__ SelectResult block_radix_select(int n, int want, KeyFn key_of, const 
     __syncthreads();
     const uint32_t* hist = sh.hist;
     if (CL > 1) {  // merge the slices' histograms on rank 0, then every CTA takes the same decision from the sum
-      uint32_t* gh = ghist0 + (pass & 1) * 256;
+      uint32_t* gh = ghist0 + (pass & 1) * (CL * 128);
       for (int k = tid; k < 256; k += kThreads)
         if (sh.hist[k]) atomicAdd(&gh[k], sh.hist[k]);
       cg::this_cluster().sync();
@@ -203,31 +205,77 @@ __device__ SelectResult block_radix_select(int n, int want, KeyFn key_of, const 
   return r;
 }
 
-// A unit split over a cluster, keys in registers: clears the state that peers will add to and arrives at the
-// cluster barrier whose wait opens cached_radix_select(); the loads of the keys run in between.
+// A unit split over a cluster, keys in registers: the CTAs exchange what they found with stores that count on the receiver's
+// mbarrier when they land. (A cluster barrier of 1024 threads after plain remote stores costs 1.5 to 3 K cycles, most of it the
+// release of everything that the threads wrote; a search has five exchanges.) Every CTA sends to all and waits for all, so that
+// none can be two exchanges ahead of another: two mbarriers and two buffers, taken in turn, are enough, and no CTA leaves while
+// something is on its way to it. What is read after an exchange is read before the block barrier in front of the next one's sends.
 template <int CL>
-__device__ __forceinline__ void split_unit_begin(SelectShared& sh) {
-  if (CL > 1) {
-    const int tid = threadIdx.x;
-    for (int k = tid; k < 256; k += kThreads) {
-      sh.ghist[0][k] = 0;
-      sh.ghist[1][k] = 0;
+struct Exchange {
+  int k = 0;                        // exchanges begun
+  ta_dev_status* status = nullptr;
+  static __device__ __forceinline__ void set_up(SelectShared<CL>& sh) {  // before a barrier of the cluster
+    if (threadIdx.x == 0) {
+      ta_sm100::mbar_init(ta_sm100::smem_u32(&sh.arrived[0]), 1);
+      ta_sm100::mbar_init(ta_sm100::smem_u32(&sh.arrived[1]), 1);
+      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (tid == 0) sh.cand_n = 0;
-    cg::this_cluster().barrier_arrive();
   }
-}
+  // words to the same place in CTA q's shared memory
+  __device__ __forceinline__ void send1(SelectShared<CL>& sh, const void* to, int q, uint32_t a) {
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(at(to, q)), "r"(a),
+                 "r"(at(&sh.arrived[k & 1], q))
+                 : "memory");
+  }
+  __device__ __forceinline__ void send2(SelectShared<CL>& sh, const void* to, int q, uint32_t a, uint32_t b) {
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.b32 [%0], {%1, %2}, [%3];" ::"r"(at(to, q)), "r"(a),
+                 "r"(b), "r"(at(&sh.arrived[k & 1], q))
+                 : "memory");
+  }
+  __device__ __forceinline__ void send4(SelectShared<CL>& sh, const void* to, int q, uint4 v) {
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(at(to, q)),
+                 "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w), "r"(at(&sh.arrived[k & 1], q))
+                 : "memory");
+  }
+  // All threads, after the sends: `bytes` have arrived. A barrier of the block. False: they did not come within a limit that CTAs which run together
+  // do not reach (reported; what was to be received must not be used).
+  __device__ __forceinline__ bool wait(SelectShared<CL>& sh, uint32_t bytes) {
+    const uint32_t bar = ta_sm100::smem_u32(&sh.arrived[k & 1]), parity = (uint32_t)(k >> 1) & 1u;
+    if (threadIdx.x == 0) ta_sm100::mbar_expect_tx(bar, bytes);
+    ++k;
+    bool ok = true;
+    unsigned long long began = 0;
+    for (int tries = 0; !ta_sm100::mbar_try_wait_cluster(bar, parity); ++tries) {
+      if ((tries & 63) != 63) continue;
+      const unsigned long long now = ta_sm100::globaltimer_ns();
+      if (began == 0) began = now;
+      if (now - began > ta_sm100::kWaitLimitNs) {
+        if (status && atomicCAS(&status->code, 0, (int)TA_ERR_TIMEOUT) == 0) status->where = 8;
+        ok = false;
+        break;
+      }
+    }
+    return __syncthreads_and(ok) != 0;
+  }
+
+ private:
+  static __device__ __forceinline__ uint32_t at(const void* p, int q) {
+    return ta_sm100::map_peer(ta_sm100::smem_u32(p), (uint32_t)q);
+  }
+};
+template <>
+struct Exchange<1> {
+  int k = 0;
+  ta_dev_status* status = nullptr;
+};
 
 // Shared step of the radix passes: warp 0 walks the 256-bin histogram from the top bin down until `remaining`
 // elements are covered and publishes the bin it stops in (sh.prefix gets the digit at `shift`, sh.remaining what is
 // still to take inside that bin, sh.ncand the bin's population). Called by all threads of warp 0.
-__device__ __forceinline__ void radix_walk(const uint32_t* hist, int shift, uint32_t digit_mask, uint32_t prefix,
-                                           uint32_t mask, SelectShared& sh) {
-  const int lane = threadIdx.x & 31;
-  // lane l owns bins [8l, 8l+8)
-  uint32_t hl[8];
-#pragma unroll
-  for (int k = 0; k < 8; ++k) hl[k] = hist[8 * lane + k];
+template <int CL>
+__device__ __forceinline__ void radix_walk(const uint32_t (&hl)[8], int shift, uint32_t digit_mask, uint32_t prefix,
+                                           uint32_t mask, SelectShared<CL>& sh) {
+  const int lane = threadIdx.x & 31;  // lane l owns bins [8l, 8l+8): hl
   uint32_t tot = 0;
 #pragma unroll
   for (int k = 0; k < 8; ++k) tot += hl[k];
@@ -261,10 +309,20 @@ __device__ __forceinline__ void radix_walk(const uint32_t* hist, int shift, uint
   }
 }
 
+template <int CL>
+__device__ __forceinline__ void radix_walk(const uint32_t* hist, int shift, uint32_t digit_mask, uint32_t prefix,
+                                           uint32_t mask, SelectShared<CL>& sh) {
+  uint32_t hl[8];
+#pragma unroll
+  for (int k = 0; k < 8; ++k) hl[k] = hist[8 * (threadIdx.x & 31) + k];
+  radix_walk(hl, shift, digit_mask, prefix, mask, sh);
+}
+
 // The remaining radix passes over the m candidate keys in sh.cand_keys (all of them match `prefix` under `mask`),
 // with block barriers only. On return prefix/remaining describe the threshold as at the end of the register passes.
+template <int CL>
 __device__ __forceinline__ void list_radix_finish(int m, int bits, int done, uint32_t& prefix, uint32_t& mask,
-                                                  int& remaining, SelectShared& sh) {
+                                                  int& remaining, SelectShared<CL>& sh) {
   const int tid = threadIdx.x;
   constexpr int kPer = (kCandCap + kThreads - 1) / kThreads;
   uint32_t lk[kPer];
@@ -305,11 +363,13 @@ __device__ __forceinline__ void list_radix_finish(int m, int bits, int done, uin
 // it / equal to it. One warp, a key per lane: beyond 32 keys another digit is cheaper, integer compares run at half rate (256
 // keys among 4096: 3.6 K cycles shared out over 32 warps, 1.7 K for a digit and the comparison of what it leaves).
 // compare_begin() runs before the barrier that publishes the keys.
-__device__ __forceinline__ void compare_begin(int m, SelectShared& sh) {
+template <int CL>
+__device__ __forceinline__ void compare_begin(int m, SelectShared<CL>& sh) {
   const int tid = threadIdx.x;
   if (tid >= m && tid < (m + 3) / 4 * 4) sh.cand_keys[tid] = 0u;  // above no key
 }
-__device__ __forceinline__ uint32_t compare_finish(int m, int remaining, int& above, int& equal, SelectShared& sh) {
+template <int CL>
+__device__ __forceinline__ uint32_t compare_finish(int m, int remaining, int& above, int& equal, SelectShared<CL>& sh) {
   const int tid = threadIdx.x;
   static_assert(kCompareCap == 32, "a key per lane");
   if (tid < 32) {
@@ -346,16 +406,14 @@ __device__ __forceinline__ uint32_t compare_finish(int m, int remaining, int& ab
 // its own: the code costs large budgets 0.6 %): few are wanted. n_unit is the length of the whole unit (n is this CTA's
 // slice when CL > 1).
 template <int CL, bool FEW = false, int ITEMS>
-__device__ SelectResult cached_radix_select(int n, int n_unit, int want, const KeyCache<ITEMS>& kc, SelectShared& sh) {
+__device__ SelectResult cached_radix_select(int n, int n_unit, int want, const KeyCache<ITEMS>& kc, SelectShared<CL>& sh,
+                                            Exchange<CL>& ex) {
   SelectResult r;
   r.thresh = 0;
   r.ties = 0;
   r.all = 0;
   r.all_ties = 0;
   r.none = (want <= 0);
-  // the cluster barrier that split_unit_begin() arrived at before the keys were loaded: from here on every CTA of the
-  // cluster is known to run (its shared memory may be written) and to have zeroed its ghist and cand_n
-  if (CL > 1) cg::this_cluster().barrier_wait();
   if (r.none) return r;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const unsigned lt = (1u << lane) - 1u;
@@ -371,6 +429,7 @@ __device__ SelectResult cached_radix_select(int n, int n_unit, int want, const K
   if (tid == 0) {
     sh.remaining = want;
     sh.cmp_n = 0;
+    sh.cand_n = 0;
   }
   static_assert(kWarps <= 32, "one lane per warp in the second reduction step");
   uint32_t num = 0;
@@ -433,18 +492,12 @@ __device__ SelectResult cached_radix_select(int n, int n_unit, int want, const K
     kmax = __reduce_max_sync(0xffffffffu, lane < kWarps ? sh.wmax[lane] : 0u);
     num = __reduce_add_sync(0xffffffffu, lane < kWarps ? sh.wnum[lane] : 0u);
   }
-  uint32_t* ghist0 = nullptr;
-  if (CL > 1) {
-    cg::cluster_group cluster = cg::this_cluster();
-    const int rank = (int)cluster.block_rank();
-    ghist0 = cluster.map_shared_rank(&sh.ghist[0][0], 0);
-    if (tid < CL) {
-      uint32_t* peer = cluster.map_shared_rank(&sh.cl_range[0][0], tid);
-      peer[rank * 4 + 0] = kmin;
-      peer[rank * 4 + 1] = kmax;
-      peer[rank * 4 + 2] = num;
-    }
-    cluster.sync();
+  int first = 0;  // CL > 1: how many of the unit's candidates belong to the CTAs before this one, and how many are its own
+  int own = 0;
+  if constexpr (CL > 1) {
+    const int rank = (int)cg::this_cluster().block_rank();
+    if (tid < CL) ex.send4(sh, sh.cl_range[rank], tid, make_uint4(kmin, kmax, num, 0u));
+    const bool ok = ex.wait(sh, CL * 16);
     kmin = 0xffffffffu;
     kmax = 0u;
     num = 0u;
@@ -452,8 +505,11 @@ __device__ SelectResult cached_radix_select(int n, int n_unit, int want, const K
     for (int q = 0; q < CL; ++q) {
       kmin = min(kmin, sh.cl_range[q][0]);
       kmax = max(kmax, sh.cl_range[q][1]);
+      if (q < rank) first += (int)sh.cl_range[q][2];
+      if (q == rank) own = (int)sh.cl_range[q][2];
       num += sh.cl_range[q][2];
     }
+    if (!ok) num = 0u;
   }
   if (!bounded && num < (uint32_t)want) {  // fewer eligible elements than requested: all of them
     r.all = 1;
@@ -503,60 +559,45 @@ __device__ SelectResult cached_radix_select(int n, int n_unit, int want, const K
       r.all_ties = r.ties == equal;
       return r;
     }
-    if (CL > 1 && ncand <= kCandCap) {
-      // Few candidates left (uniform over the cluster: ncand comes from the merged histogram, or is the number of
-      // eligible elements before the first pass). Every CTA appends its own to the list on rank 0; after one cluster
-      // barrier every CTA copies the list and finishes alone. The list's order does not matter: only the multiset of
-      // keys decides the threshold, so all CTAs arrive at the same one.
-      cg::cluster_group cluster = cg::this_cluster();
-      uint32_t* list0 = cluster.map_shared_rank(&sh.cand_keys[0], 0);
-      uint32_t* count0 = cluster.map_shared_rank(&sh.cand_n, 0);
+    if constexpr (CL > 1) if (ncand <= kCandCap) {
+      // Few candidates left (uniform over the cluster: every CTA knows how many each of them has). Every CTA sends its own to
+      // the lists of all, behind those of the CTAs before it; after one cluster barrier every CTA finishes alone. Only the
+      // multiset of keys decides the threshold, so that all arrive at the same one.
       uint32_t mine = 0;
       if (cand != 0u) {
 #pragma unroll
         for (int it = 0; it < ITEMS; ++it)
           if (((cand >> it) & 1u) && (kc.key[it] & mask) == prefix) mine |= 1u << it;
       }
-      // one remote atomic per warp reserves the warp's range of the list
-      const uint32_t cnt = (uint32_t)__popc(mine);
-      uint32_t incl = cnt;
+      if (__any_sync(0xffffffffu, mine != 0u)) {
+        const uint32_t cnt = (uint32_t)__popc(mine);
+        uint32_t incl = cnt;
 #pragma unroll
-      for (int off = 1; off < 32; off <<= 1) {
-        const uint32_t o = __shfl_up_sync(0xffffffffu, incl, off);
-        if (lane >= off) incl += o;
-      }
-      const uint32_t warp_n = __shfl_sync(0xffffffffu, incl, 31);
-      uint32_t base = 0;
-      if (lane == 0 && warp_n != 0u) base = atomicAdd(count0, warp_n);
-      base = __shfl_sync(0xffffffffu, base, 0);
-      uint32_t slot = base + incl - cnt;
-      if (mine != 0u) {
-#pragma unroll
-        for (int it = 0; it < ITEMS; ++it) {
-          if ((mine >> it) & 1u) {
-            if (slot < (uint32_t)kCandCap) list0[slot] = kc.key[it];
-            ++slot;
-          }
+        for (int off = 1; off < 32; off <<= 1) {
+          const uint32_t o = __shfl_up_sync(0xffffffffu, incl, off);
+          if (lane >= off) incl += o;
         }
+        uint32_t slot = 0;
+        if (lane == 31) slot = atomicAdd(&sh.cand_n, incl);
+        slot = (uint32_t)first + __shfl_sync(0xffffffffu, slot, 31) + incl - cnt;
+#pragma unroll
+        for (int it = 0; it < ITEMS; ++it)
+          if ((mine >> it) & 1u) sh.cand_keys[min(slot++, (uint32_t)kCandCap - 1u)] = kc.key[it];
       }
-      cluster.sync();
-      if (cluster.block_rank() != 0)
-        for (int j = tid; j < ncand; j += kThreads) sh.cand_keys[j] = list0[j];
       __syncthreads();
+      const int rank = (int)cg::this_cluster().block_rank();
+      for (int j = tid; j < own * CL; j += kThreads) {
+        const int q = j / own, at = min(first + j - q * own, kCandCap - 1);
+        if (q != rank) ex.send1(sh, &sh.cand_keys[at], q, sh.cand_keys[at]);
+      }
+      ex.wait(sh, (uint32_t)(ncand - own) * 4u);
       list_radix_finish(ncand, bits, done, prefix, mask, remaining, sh);
       break;
     }
     const int width = min(8, bits - done), shift = bits - done - width;
     const uint32_t digit_mask = (1u << width) - 1u;
     for (int k = tid; k < 256; k += kThreads) sh.hist[k] = 0;
-    if (CL > 1 && pass >= 2) {
-      // rank 0's merged histogram alternates between two buffers, both zero at the start; from the third pass on the
-      // buffer is cleared again (its readers of two passes ago are done) and the clearing made visible
-      for (int k = tid; k < 256; k += kThreads) sh.ghist[pass & 1][k] = 0;
-      cg::this_cluster().sync();
-    } else {
-      __syncthreads();
-    }
+    __syncthreads();
     if ((pass == 0 && !bounded) || ncand * 4 > n_unit) {  // most elements are candidates (uniform over the unit's CTAs)
 #pragma unroll
       for (int it = 0; it < ITEMS; ++it) {
@@ -578,20 +619,46 @@ __device__ SelectResult cached_radix_select(int n, int n_unit, int want, const K
       }
     }
     __syncthreads();
-    const uint32_t* hist = sh.hist;
-    if (CL > 1) {  // merge the slices' histograms on rank 0, then every CTA takes the same decision from the sum
-      uint32_t* gh = ghist0 + (pass & 1) * 256;
-      for (int k = tid; k < 256; k += kThreads)
-        if (sh.hist[k]) atomicAdd(&gh[k], sh.hist[k]);
-      cg::this_cluster().sync();
-      hist = gh;
+    if constexpr (CL > 1) {
+      // Every CTA sends its histogram to all and takes the same decision from the sum. (Added up by remote atomics on one CTA
+      // and read from there, a search among 16 CTAs took 25 K cycles: distributed shared memory moves some 10 bytes a clock.)
+      const int rank = (int)cg::this_cluster().block_rank();
+      for (int j = tid; j < 32 * CL; j += kThreads) {
+        const int q = j / 32, k = j % 32;  // bins 8k .. 8k + 7 (at most 32768 keys a CTA: 16 bits hold a count)
+        const uint4 a = reinterpret_cast<const uint4*>(sh.hist)[2 * k], b = reinterpret_cast<const uint4*>(sh.hist)[2 * k + 1];
+        ex.send4(sh, &sh.ghist[pass & 1][rank][4 * k], q,
+                 make_uint4(a.x | (a.y << 16), a.z | (a.w << 16), b.x | (b.y << 16), b.z | (b.w << 16)));
+      }
+      ex.wait(sh, CL * 512);
+      if (tid < 32) {
+        uint32_t hl[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
+#pragma unroll 4
+        for (int q = 0; q < CL; ++q) {
+          const uint4 v = reinterpret_cast<const uint4*>(&sh.ghist[pass & 1][q][0])[lane];
+          const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            hl[2 * k] += w[k] & 0xffffu;
+            hl[2 * k + 1] += w[k] >> 16;
+          }
+        }
+        radix_walk(hl, shift, digit_mask, prefix, mask, sh);
+      }
+    } else if (tid < 32) {
+      radix_walk(sh.hist, shift, digit_mask, prefix, mask, sh);
     }
-    if (tid < 32) radix_walk(hist, shift, digit_mask, prefix, mask, sh);
     __syncthreads();
     prefix = sh.prefix;
     mask = sh.mask;
     remaining = sh.remaining;
     ncand = sh.ncand;
+    if constexpr (CL > 1) {  // who has how many of the bin that the threshold fell into
+      const int rank = (int)cg::this_cluster().block_rank();
+      const uint32_t bin = (prefix >> shift) & digit_mask;
+      const uint32_t n_q = lane < CL ? (sh.ghist[pass & 1][lane & (CL - 1)][bin >> 1] >> (16 * (bin & 1))) & 0xffffu : 0u;
+      first = (int)__reduce_add_sync(0xffffffffu, lane < rank ? n_q : 0u);
+      own = (int)__shfl_sync(0xffffffffu, n_q, rank);
+    }
     done += width;
     ++pass;
     if (ncand == remaining) {  // every candidate left is taken: the low bits need no pass
@@ -607,9 +674,9 @@ __device__ SelectResult cached_radix_select(int n, int n_unit, int want, const K
 // Ordered pass over [0, n): classify(i, eligible, key, def, tie) marks element i `definite` (taken for sure) or a
 // `tie` (taken while ties last). Calls emit(i, rank) for every taken element with its rank in ascending position
 // order. Returns the number taken.
-template <bool CACHED, class KeyFn, class ClassFn, class EmitFn, int ITEMS>
+template <bool CACHED, class KeyFn, class ClassFn, class EmitFn, int ITEMS, int CL>
 __device__ int block_ordered_emit(int n, int ties_allowed, KeyFn key_of, const KeyCache<ITEMS>& kc, ClassFn classify,
-                                  EmitFn emit, SelectShared& sh, int def_base = 0, int tie_base = 0,
+                                  EmitFn emit, SelectShared<CL>& sh, int def_base = 0, int tie_base = 0,
                                   int* def_total_out = nullptr, int* tie_total_out = nullptr) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int def0 = def_base, tie0 = tie_base;
@@ -676,7 +743,7 @@ __device__ __forceinline__ uint32_t warp_transpose32(uint32_t x, int lane) {
 // ranks). emit may run on another thread than the one that holds the element's key.
 template <int CL, class EmitFn, int ITEMS>
 __device__ int cached_ordered_emit(int n, const SelectResult& r, const KeyCache<ITEMS>& kc, uint32_t always,
-                                   EmitFn emit, SelectShared& sh) {
+                                   EmitFn emit, SelectShared<CL>& sh, Exchange<CL>& ex) {
   static_assert(ITEMS <= kItemsLong && ITEMS <= 32, "per-thread masks hold one bit per chunk");
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int chunks = (n + kThreads - 1) / kThreads;
@@ -736,40 +803,35 @@ __device__ int cached_ordered_emit(int n, const SelectResult& r, const KeyCache<
   const uint32_t wt_l = lane < kWarps ? sh.wtot[lane] : 0u;  // (no carry between the halves: at most 32768 elements)
   const uint32_t before = __reduce_add_sync(0xffffffffu, lane < warp ? wt_l : 0u);
   const uint32_t all = __reduce_add_sync(0xffffffffu, wt_l);
-  const uint32_t ex = before + run - mine;
+  const uint32_t upto = before + run - mine;
   int def_base = 0, tie_base = 0;
   const int def_mine = (int)(all & 0xffffu), tie_mine = (int)(all >> 16);
   int def_all = def_mine, tie_all = tie_mine;
-  if (CL > 1) {
-    cg::cluster_group cluster = cg::this_cluster();
-    const int rank = (int)cluster.block_rank();
-    if (tid < CL) {
-      int* peer = cluster.map_shared_rank(&sh.totals[0][0], tid);
-      peer[rank * 2 + 0] = def_all;
-      peer[rank * 2 + 1] = tie_all;
-    }
-    cluster.sync();
+  if constexpr (CL > 1) {
+    const int rank = (int)cg::this_cluster().block_rank(), turn = ex.k & 1;
+    if (tid < CL) ex.send2(sh, sh.totals[turn][rank], tid, (uint32_t)def_all, (uint32_t)tie_all);
+    if (!ex.wait(sh, CL * 8)) return 0;
     def_all = 0;
     tie_all = 0;
 #pragma unroll
     for (int r = 0; r < CL; ++r) {
       if (r < rank) {
-        def_base += sh.totals[r][0];
-        tie_base += sh.totals[r][1];
+        def_base += sh.totals[turn][r][0];
+        tie_base += sh.totals[turn][r][1];
       }
-      def_all += sh.totals[r][0];
-      tie_all += sh.totals[r][1];
+      def_all += sh.totals[turn][r][0];
+      tie_all += sh.totals[turn][r][1];
     }
   }
-  int def_before = def_base + (int)(ex & 0xffffu);
-  int ties_seen = tie_base + (int)(ex >> 16);
+  int def_before = def_base + (int)(upto & 0xffffu);
+  int ties_seen = tie_base + (int)(upto >> 16);
   uint32_t m = wd | wt;
   // Sparse words: every thread walks its own word. Dense ones (recency makes runs of neighbours win together, so that a few
   // words hold most of what is taken): the warps of the block share the words, a lane per position (TA-Fast, 1024 of 4096
   // tokens, with the search above: 58.2 -> 55.8 us a call). A warp meets at most `chunks` words that are not empty that
   // way, a thread up to `most` positions the other way.
   if (most > min(chunks, (def_mine + tie_mine) / kWarps + 1) + 2) {
-    sh.before[tid] = ex;
+    sh.before[tid] = upto;
     __syncthreads();
     const unsigned lt = (1u << lane) - 1u;
     const int row = lane * (kWarps + 1) + warp;
@@ -804,7 +866,7 @@ __device__ int cached_ordered_emit(int n, const SelectResult& r, const KeyCache<
 // emitting sweep starts from the sums of the lower ranks. Returns the number taken over the whole unit.
 template <bool CACHED, int CL, class KeyFn, class ClassFn, class EmitFn, int ITEMS>
 __device__ int cluster_ordered_emit(int n, int ties_allowed, KeyFn key_of, const KeyCache<ITEMS>& kc, ClassFn classify,
-                                    EmitFn emit, SelectShared& sh) {
+                                    EmitFn emit, SelectShared<CL>& sh) {
   static_assert(!CACHED, "keys in registers: call cached_ordered_emit");
   if (CL == 1) return block_ordered_emit<CACHED>(n, ties_allowed, key_of, kc, classify, emit, sh);
   cg::cluster_group cluster = cg::this_cluster();
@@ -812,7 +874,7 @@ __device__ int cluster_ordered_emit(int n, int ties_allowed, KeyFn key_of, const
   int dt = 0, tt = 0;
   block_ordered_emit<CACHED>(n, 0, key_of, kc, classify, [](int, int) {}, sh, 0, 0, &dt, &tt);
   if (threadIdx.x < CL) {
-    int* peer = cluster.map_shared_rank(&sh.totals[0][0], threadIdx.x);
+    int* peer = cluster.map_shared_rank(&sh.totals[0][0][0], threadIdx.x);
     peer[rank * 2 + 0] = dt;
     peer[rank * 2 + 1] = tt;
   }
@@ -821,11 +883,11 @@ __device__ int cluster_ordered_emit(int n, int ties_allowed, KeyFn key_of, const
 #pragma unroll
   for (int r = 0; r < CL; ++r) {
     if (r < rank) {
-      def_base += sh.totals[r][0];
-      tie_base += sh.totals[r][1];
+      def_base += sh.totals[0][r][0];
+      tie_base += sh.totals[0][r][1];
     }
-    def_all += sh.totals[r][0];
-    tie_all += sh.totals[r][1];
+    def_all += sh.totals[0][r][0];
+    tie_all += sh.totals[0][r][1];
   }
   block_ordered_emit<CACHED>(n, ties_allowed, key_of, kc, classify, emit, sh, def_base, tie_base);
   return def_all + min(tie_all, ties_allowed);
@@ -877,7 +939,7 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads) ta_forced_kernel(ta
                                                              uint8_t* __restrict__ forced,
                                                              int32_t* __restrict__ r_main, ta_dev_status* status,
                                                              const int32_t* __restrict__ class_K, ta_static_out so) {
-  __shared__ SelectShared sh;
+  __shared__ SelectShared<CL> sh;
   ta_launch_dependents();  // its dependent does not start before every block of the kernel before it runs
   ta_wait_for_prior_grid();
   // grid.x = classes * sequences * CL; without budget classes there is one class and K is the argument
@@ -941,7 +1003,12 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads) ta_forced_kernel(ta
     return v > 0.0f && !mandatory(lo + il);
   };
   KeyCache<ITEMS> kc;
-  if constexpr (CACHED) split_unit_begin<CL>(sh);
+  Exchange<CL> ex;
+  ex.status = status;
+  if constexpr (CACHED && CL > 1) {
+    ex.set_up(sh);
+    cg::this_cluster().barrier_arrive();
+  }
   if constexpr (CACHED) {  // loads as selects, never under a branch: nothing keeps them from being in flight together
     float v[ITEMS];
 #pragma unroll
@@ -958,7 +1025,8 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads) ta_forced_kernel(ta
     }
   }
   SelectResult r;
-  if constexpr (CACHED) r = cached_radix_select<CL>(hi - lo, s.n, s.p, kc, sh);
+  if constexpr (CACHED && CL > 1) cg::this_cluster().barrier_wait();
+  if constexpr (CACHED) r = cached_radix_select<CL>(hi - lo, s.n, s.p, kc, sh, ex);
   else r = block_radix_select<CACHED, CL>(hi - lo, s.p, key_of, kc, sh);
   uint8_t* f = forced + s.start + lo;
   // ordered pass: mandatory tokens and vouchers above the threshold are forced for sure; vouchers equal to the
@@ -980,7 +1048,7 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads) ta_forced_kernel(ta
         if (mandatory(lo + il)) always |= 1u << it;
       }
     }
-    taken = cached_ordered_emit<CL>(hi - lo, r, kc, always, emit, sh);
+    taken = cached_ordered_emit<CL>(hi - lo, r, kc, always, emit, sh, ex);
   } else {
     taken = cluster_ordered_emit<CACHED, CL>(hi - lo, r.ties, key_of, kc, classify, emit, sh);
   }
@@ -993,6 +1061,7 @@ struct UnitSrc {  // where a unit's utility comes from
   const float* P;
   const float* u_static;  // per token
   float alpha, delta;
+  ta_dev_status* status;
 };
 
 __device__ __forceinline__ float unit_utility(const UnitSrc& src, long long unit_off, long long tok) {
@@ -1053,7 +1122,7 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads) ta_select_kernel(ta
                                                              const int32_t* r_main,
                                                              int32_t* __restrict__ idx, int32_t* __restrict__ count,
                                                              GatherDst gd, const int32_t* __restrict__ class_of) {
-  __shared__ SelectShared sh;
+  __shared__ SelectShared<CL> sh;
   ta_wait_for_prior_grid();
   ta_launch_dependents();
   const int unit = blockIdx.x / CL;
@@ -1128,12 +1197,17 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads) ta_select_kernel(ta
     if constexpr (GATHER) gather_unit(gd, seq, unit, l, b, g, n, K, out, n, true, sh);
     return;
   }
+  Exchange<CL> ex;
+  ex.status = src.status;
   auto key_of = [&](int il, uint32_t& key) {
     key = sortable_key(unit_utility(src, unit_off, (long long)start + lo + il));
     return f[il] == 0;
   };
   if constexpr (CACHED) {
-    split_unit_begin<CL>(sh);
+    if constexpr (CL > 1) {
+      ex.set_up(sh);
+      cg::this_cluster().barrier_arrive();
+    }
     kc.elig = 0;
 #pragma unroll
     for (int g0 = 0; g0 < ITEMS; g0 += kGroup) {
@@ -1153,7 +1227,8 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads) ta_select_kernel(ta
     }
   }
   SelectResult r;
-  if constexpr (CACHED) r = cached_radix_select<CL, FEW>(hi - lo, n, want, kc, sh);
+  if constexpr (CACHED && CL > 1) cg::this_cluster().barrier_wait();
+  if constexpr (CACHED) r = cached_radix_select<CL, FEW>(hi - lo, n, want, kc, sh, ex);
   else r = block_radix_select<CACHED, CL>(hi - lo, want, key_of, kc, sh);
   auto classify = [&](int, bool elig, uint32_t key, bool& def, bool& tie) {
     def = !elig || (!r.none && (r.all || key > r.thresh));
@@ -1165,7 +1240,7 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads) ta_select_kernel(ta
   };
   int taken;
   if constexpr (CACHED)  // forced tokens (not eligible, inside the unit) are taken whatever their key
-    taken = cached_ordered_emit<CL>(hi - lo, r, kc, exist_mask(hi - lo) & ~kc.elig, emit, sh);
+    taken = cached_ordered_emit<CL>(hi - lo, r, kc, exist_mask(hi - lo) & ~kc.elig, emit, sh, ex);
   else
     taken = cluster_ordered_emit<CACHED, CL>(hi - lo, r.ties, key_of, kc, classify, emit, sh);
   if (!lead) return;
