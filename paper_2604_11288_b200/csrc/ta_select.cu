@@ -263,6 +263,17 @@ cudaError_t ta_launch_select_units(const ta_select_args& a, cudaStream_t stream_
   // with it, K 256 and 512 of 1000 tokens 14.7 and 17.6 without, 15.0 and 18.0 with it.
   const bool few = gathers && a.K <= kThreads / 2, few1024 = gathers && a.K <= sel1024::kThreads / 2;
   if (few_short_units(a)) {
+    // A large gather by a cluster of blocks per unit, of which the first selects: one block reads a unit's rows one round trip
+    // after another. us per call without / with 4 / 8 blocks: 8 units K 256 23.9 / 24.2 / 24.5, K 512 30.3 / 28.9 / 28.8, K 1024 33.3 /
+    // 26.6 / 25.6; 16 units K 606 34.0 / 30.7 / 40.6 (15 clusters of 8 fit at once, 35 of 4); K 128 25.6 / 27.8 / 27.7.
+    const int help = a.K >= 512 && units <= 35 * sms / 148 ? 4 : 1;
+    if (gathers && help > 1) {
+      auto kern = a.seq.max_n <= 4 * sel1024::kThreads ? sel1024::ta_select_kernel<true, 1, 4, true, false, true>
+                  : few1024                            ? sel1024::ta_select_kernel<true, 1, 8, true, true, true>
+                                                       : sel1024::ta_select_kernel<true, 1, 8, true, false, true>;
+      return launch_threads(sel1024::kThreads, kern, units, help, stream, a.seq, a.n_layers, a.Hkv, a.K, a.fast, src2, a.forced,
+                            a.r_main, a.idx, a.count, gd2, co);
+    }
     auto kern = a.seq.max_n <= 4 * sel1024::kThreads
                     ? (gathers ? sel1024::ta_select_kernel<true, 1, 4, true> : sel1024::ta_select_kernel<true, 1, 4, false>)
                     : (few1024   ? sel1024::ta_select_kernel<true, 1, 8, true, true>

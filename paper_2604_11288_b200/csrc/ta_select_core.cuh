@@ -1084,9 +1084,11 @@ struct GatherDst {
   uint4* v_out;
 };
 
-// Rows are listed in sh.cand_keys (the first kCandCap of them) and in `out`; all: row r is position r.
+// Rows are listed in `list` (the first kCandCap of them) and in `out`; all: row r is position r. Of `blocks` blocks that share
+// the unit's rows this is number `block`.
 __device__ __forceinline__ void gather_unit(const GatherDst& gd, const ta_seq_desc& seq, int unit, int l, int b, int g,
-                                            int n, int K, const int32_t* out, int taken, bool all, const SelectShared& sh) {
+                                            int n, int K, const int32_t* out, int taken, bool all, const uint32_t* list,
+                                            int block = 0, int blocks = 1) {
   constexpr int kLanesPerRow = TA_HEAD_DIM * 2 / 16;  // a warp moves the K and the V row of one position at a time
   constexpr int kUnroll = 8;
   static_assert(2 * kLanesPerRow == 32, "one lane per 16-byte piece of a K row and a V row");
@@ -1098,25 +1100,27 @@ __device__ __forceinline__ void gather_unit(const GatherDst& gd, const ta_seq_de
   const uint4* from = reinterpret_cast<const uint4*>(reinterpret_cast<const uint16_t*>(src.ptr) + base) + piece;
   uint4* to = (which ? gd.v_out : gd.k_out) + (long long)unit * K * kLanesPerRow + piece;
   const long long row_pieces = src.stride_n / 8;
-  for (int r0 = threadIdx.x / 32; r0 < K; r0 += kUnroll * kWarps) {
+  const int step = kWarps * blocks;
+  for (int r0 = block * kWarps + threadIdx.x / 32; r0 < K; r0 += kUnroll * step) {
     uint4 val[kUnroll];
 #pragma unroll
     for (int j = 0; j < kUnroll; ++j) {
-      const int r = r0 + j * kWarps;
-      int i = all ? r : (int)sh.cand_keys[min(r, kCandCap - 1)];
+      const int r = r0 + j * step;
+      int i = all ? r : (int)list[min(r, kCandCap - 1)];
       if (r >= kCandCap && r < taken && !all) i = out[r];
       val[j] = ta_ld_stream_if(from + i * row_pieces, r < taken && i >= 0 && i < n);
     }
 #pragma unroll
     for (int j = 0; j < kUnroll; ++j) {
-      const int r = r0 + j * kWarps;
+      const int r = r0 + j * step;
       if (r < K) ta_st_stream(to + (long long)r * kLanesPerRow, val[j]);
     }
   }
 }
 
-// grid.x = units. scored: unit = (l*B + b)*Hkv + g; fast: unit = b.
-template <bool CACHED, int CL, int ITEMS = kItems, bool GATHER = false, bool FEW = false>
+// grid.x = units. scored: unit = (l*B + b)*Hkv + g; fast: unit = b. HELP: the unit has a cluster of blocks, of which the first
+// selects and all move rows.
+template <bool CACHED, int CL, int ITEMS = kItems, bool GATHER = false, bool FEW = false, bool HELP = false>
 __global__ void __launch_bounds__(kThreads, 1024 / kThreads) ta_select_kernel(ta_seq_desc seq, int n_layers, int Hkv, int K, int fast,
                                                              UnitSrc src, const uint8_t* forced,
                                                              const int32_t* r_main,
@@ -1125,8 +1129,10 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads) ta_select_kernel(ta
   __shared__ SelectShared<CL> sh;
   ta_wait_for_prior_grid();
   ta_launch_dependents();
-  const int unit = blockIdx.x / CL;
-  const bool lead = blockIdx.x % CL == 0;
+  static_assert(!HELP || (GATHER && CL == 1), "helpers move rows and nothing else");
+  const int blocks = HELP ? (int)cg::this_cluster().num_blocks() : CL;
+  const int unit = blockIdx.x / blocks;
+  const bool lead = blockIdx.x % blocks == 0;
   int b, l = 0, g = 0;
   if (fast) {
     b = unit;
@@ -1145,6 +1151,26 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads) ta_select_kernel(ta
   int32_t* out = idx + (long long)unit * K;
   const int tid = threadIdx.x;
   const long long unit_off = fast ? 0 : ((long long)l * Hkv + g) * seq.total;
+  // the unit's rows, once the selecting block has listed them
+  auto gather = [&](int taken, bool all) {
+    if constexpr (GATHER && !HELP) gather_unit(gd, seq, unit, l, b, g, n, K, out, taken, all, sh.cand_keys);
+    if constexpr (HELP) {
+      cg::cluster_group cluster = cg::this_cluster();
+      if (lead && tid == 0) {
+        sh.totals[0][0][0] = taken;
+        sh.totals[0][0][1] = all;
+      }
+      cluster.sync();
+      const int* said = cluster.map_shared_rank(&sh.totals[0][0][0], 0);
+      gather_unit(gd, seq, unit, l, b, g, n, K, out, said[0], said[1] != 0, cluster.map_shared_rank(&sh.cand_keys[0], 0),
+                  (int)cluster.block_rank(), blocks);
+      cluster.sync();  // the selecting block's list has been read
+    }
+  };
+  if (HELP && !lead) {
+    gather(0, false);
+    return;
+  }
   // a sequence that does not lie inside the token arrays (want -2 below) is not read
   const bool inside = n >= 0 && n <= seq.max_n && start >= 0 && (long long)start + n <= seq.total;
   int lo, hi;
@@ -1186,7 +1212,7 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads) ta_select_kernel(ta
       for (int r = tid; r < K; r += kThreads) out[r] = -1;
       if (tid == 0) count[unit] = 0;
     }
-    if constexpr (GATHER) gather_unit(gd, seq, unit, l, b, g, n, K, out, 0, true, sh);
+    gather(0, true);
     return;
   }
   if (want == -1) {  // K >= n: keep everything
@@ -1194,7 +1220,7 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads) ta_select_kernel(ta
       for (int r = tid; r < K; r += kThreads) out[r] = r < n ? r : -1;
       if (tid == 0) count[unit] = n;
     }
-    if constexpr (GATHER) gather_unit(gd, seq, unit, l, b, g, n, K, out, n, true, sh);
+    gather(n, true);
     return;
   }
   Exchange<CL> ex;
@@ -1246,7 +1272,7 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads) ta_select_kernel(ta
   if (!lead) return;
   for (int q = taken + tid; q < K; q += kThreads) out[q] = -1;
   if (tid == 0) count[unit] = taken;
-  if constexpr (GATHER) gather_unit(gd, seq, unit, l, b, g, n, K, out, min(taken, K), false, sh);
+  gather(min(taken, K), false);
 }
 
 }  // namespace TA_SEL_NS
