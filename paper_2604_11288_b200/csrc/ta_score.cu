@@ -10,7 +10,7 @@
 // Both passes use the same shared-memory operand tiles (both K-major, 128-byte swizzle); only the roles in the
 // instruction descriptor swap, which puts the reduction axis of each pass along a thread's own registers.
 // A unit is handled by a cluster of 1, 2, 4 or 8 CTAs (chosen per launch: one CTA when there are many units, more when there
-// are few, 9 to 16 for a handful of units of up to 128 rows, where all of them fit at once: a cluster stays inside a group of
+// are few, 9 to 16 for a handful of units, where all of them fit at once: a cluster stays inside a group of
 // SMs, 148 SMs hold 8 clusters of 9 or 10 CTAs and 7 of 11 to 16); each CTA owns a contiguous range of 128-key tiles. Between
 // the passes every CTA stores its per-row (reference, sum) pairs into the shared memory of all its peers with stores that count
 // on the receiver's mbarrier when they land (reading the peers' pairs over the cluster took 1.9 us of a 15 us kernel, plain
@@ -147,20 +147,19 @@ struct alignas(16) UnitInfo {
 };
 constexpr int kUnitRing = 4;  // unit descriptions in flight between the producer and the other warps
 constexpr int kAcc = 4;       // accumulator stages of 128 tensor-memory columns (512 columns in all)
-constexpr int kStages = 4;    // ring of key tiles
 constexpr int kRing = 4;      // MB 2: partial column sums in flight between the groups
 
 template <int MB>
 struct alignas(1024) ScoreSmem {
   static constexpr int kQBufs = MB == 1 ? 2 : 1;  // query tiles in flight (next unit's tile loads early)
   static constexpr int kRowsPad = MB * 128;
+  static constexpr int kStages = MB == 1 ? 4 : 3;  // ring of key tiles (256 rows: a fourth leaves no room for 16 peers)
   uint8_t q[kQBufs][MB * 2 * kHalfBytes];  // [buffer][half][MB*128 rows][128 B]
   uint8_t k[kStages][kKTileBytes];         // [stage][half][128 rows][128 B]
   // [softmax group][row of its block]: reference and sum of the group's keys (one unit's at a time: a softmax warp waits for
   // the row constants that are formed from them before it goes on to the next unit)
   float part_m[kGroups][128], part_z[kGroups][128];
-  static constexpr int kPeers = MB == 1 ? kMaxCluster : 8;  // largest cluster the exchange has room for
-  float2 peer[kPeers][kRowsPad];           // row statistics (reference, sum) as the CTAs of the cluster sent them
+  float2 peer[kMaxCluster][kRowsPad];           // row statistics (reference, sum) as the CTAs of the cluster sent them
   // [unit parity][row] pass-2 constant of the row; behind them the form that ex2 takes, for rows whose own is the polynomial's
   float tab[2][2 * kRowsPad];
   float wrow[kRowsPad];                    // pension weight per row
@@ -283,7 +282,7 @@ ta_score_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
   using Smem = ScoreSmem<MB>;
   constexpr int kWarpTma = kSoftWarps, kWarpMma = kSoftWarps + 1, kWarpStat = kSoftWarps + 2;
   constexpr int kStatWarps = 2;
-  constexpr int kQBufs = Smem::kQBufs, kRowsPad = Smem::kRowsPad;
+  constexpr int kQBufs = Smem::kQBufs, kRowsPad = Smem::kRowsPad, kStages = Smem::kStages;
   constexpr uint32_t kTmemCols = 512;  // kAcc accumulator stages of 128 columns
   extern __shared__ uint8_t smem_raw[];
   Smem& sm = *reinterpret_cast<Smem*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -1109,11 +1108,15 @@ cudaError_t launch_variant(ta_ctx* ctx, const CUtensorMap& mq, const CUtensorMap
   // (128) slower on average than the best, at most 4.1 % and 0.2 % (152 units of 2048 tokens with 256 rows: 98 us with 1 CTA,
   // 83 us with 2; 320 units of 4096 tokens with 128 rows: 149 us with 1, 134 us with 2). Jobs are not rounded up to whole
   // rounds of the softmax groups: fewer than four at work take little longer per job.
+  // With 256 rows 9 to 16 CTAs need the peers' 32 KB, for which one of four stages of key tiles made room (16 x 32768 tokens take as
+  // long: 12.63 and 12.61 ms). us a layer with 8 and with up to 16 CTAs: 2 units of 14714 tokens 61.4 / 42.8, of 16000 64.3 / 44.0, of
+  // 5000 30.8 / 26.2; 8 units of 8000 39.5 / 37.4, of 6000 34.5 / 32.6.
   // (Choosing more CTAs per unit so that the keys of all units in flight fit in L2 was measured and lost: 16 x 32768
-  // tokens, 8 CTAs per unit 2.02 ms against 1.63 ms.)
+  // tokens, 8 CTAs per unit 2.02 ms against 1.63 ms. With 16 or 32 rows, where the second read is what bounds it, too: 1296 units of
+  // 5634 tokens 555, 539, 634, 815 us with 1, 2, 4 and 8 CTAs, 1024 of 12000 912, 927, 999, 1213.)
   int best_cl = ctx->score_force_cluster;
   long long best_cost = best_cl > 0 ? 0 : -1;
-  for (int cl = 1; cl <= ScoreSmem<MB>::kPeers; cl = cl < 8 ? 2 * cl : cl + 1) {
+  for (int cl = 1; cl <= kMaxCluster; cl = cl < 8 ? 2 * cl : cl + 1) {
     if (ctx->score_force_cluster > 0 && cl != ctx->score_force_cluster) continue;
     if (cl > 1 && tiles_max < 2 * cl && ctx->score_force_cluster <= 0) break;
     if (cl > 8 && sp.units > max_clusters[8]) break;  // only for a single round of few units

@@ -58,6 +58,14 @@ def test_more_than_eight_ctas_for_a_handful_of_units(L, Hkv, n):
     np.testing.assert_allclose(got, ref, rtol=SCORE_RTOL, atol=SCORE_ATOL)
 
 
+@pytest.mark.parametrize("L,Hkv,n", [(1, 1, 16384), (1, 2, 9001), (1, 4, 6000), (7, 1, 4090)])
+def test_more_than_eight_ctas_with_256_rows(L, Hkv, n):
+    got, size = _score(L, 1, Hkv, n, 64, 0)
+    assert 8 < size <= 16
+    ref, _ = _score(L, 1, Hkv, n, 64, 1)
+    np.testing.assert_allclose(got, ref, rtol=SCORE_RTOL, atol=SCORE_ATOL)
+
+
 @pytest.mark.parametrize("n", [1000, 4096])
 def test_128_rows_are_as_precise_as_fp32_sums(n):
     # Every term carries the rounding of its exponent (|x| < 32: 2^-20 absolute, 0.7 of it relative) and of its exponential
