@@ -37,6 +37,7 @@ struct SelectShared {
   // range of the eligible keys: per warp (smallest, largest, how many), and per CTA of a cluster
   uint32_t wmin[kWarps], wmax[kWarps], wnum[kWarps];
   __align__(16) uint32_t cl_range[CL][4];
+  uint32_t took_part[CL];  // of the exchange of candidates (never read: what counts is that the words arrive)
   // long sequences are split over the CTAs of a cluster: every CTA's histogram, two counts to a word, as it sent them to all
   // (two buffers alternating by pass), and every CTA's (definite, tie) totals
   __align__(16) uint32_t ghist[CL > 1 ? 2 : 1][CL][CL > 1 ? 128 : 1];
@@ -561,8 +562,10 @@ __device__ SelectResult cached_radix_select(int n, int n_unit, int want, const K
     }
     if constexpr (CL > 1) if (ncand <= kCandCap) {
       // Few candidates left (uniform over the cluster: every CTA knows how many each of them has). Every CTA sends its own to
-      // the lists of all, behind those of the CTAs before it; after one cluster barrier every CTA finishes alone. Only the
-      // multiset of keys decides the threshold, so that all arrive at the same one.
+      // the lists of all, behind those of the CTAs before it; when all have arrived every CTA finishes alone. Only the
+      // multiset of keys decides the threshold, so that all arrive at the same one. Every CTA also sends a word to all: one
+      // that has all the candidates would wait for nobody without it, and its next exchange could reach a CTA that is still
+      // in the one before this.
       uint32_t mine = 0;
       if (cand != 0u) {
 #pragma unroll
@@ -586,11 +589,12 @@ __device__ SelectResult cached_radix_select(int n, int n_unit, int want, const K
       }
       __syncthreads();
       const int rank = (int)cg::this_cluster().block_rank();
+      if (tid < CL) ex.send1(sh, &sh.took_part[rank], tid, 0u);
       for (int j = tid; j < own * CL; j += kThreads) {
         const int q = j / own, at = min(first + j - q * own, kCandCap - 1);
         if (q != rank) ex.send1(sh, &sh.cand_keys[at], q, sh.cand_keys[at]);
       }
-      ex.wait(sh, (uint32_t)(ncand - own) * 4u);
+      ex.wait(sh, (uint32_t)(CL + ncand - own) * 4u);
       list_radix_finish(ncand, bits, done, prefix, mask, remaining, sh);
       break;
     }
