@@ -594,6 +594,7 @@ ta_status ta_select_topk(ta_ctx* ctx, const ta_policy* policy, const ta_batch* b
   a.A = A;
   a.P = P;
   a.u = nullptr;
+  a.wait_limit_ns = ctx->wait_limit_ns;
   a.forced = forced;
   a.r_main = r_main;
   a.idx = fast ? idx_seq : idx;
@@ -727,6 +728,7 @@ ta_status compress_impl(ta_ctx* ctx, const ta_patterns* pats, const ta_policy* p
   sel.fast = fast;
   sel.sm_count = ctx->sm_count;
   sel.status = ctx->d_status;
+  sel.wait_limit_ns = ctx->wait_limit_ns;
   sel.alpha = policy->alpha;
   sel.delta = policy->delta;
   sel.flags = flags;
@@ -1032,7 +1034,7 @@ static ta_status stream_step_impl(ta_ctx* ctx, const ta_patterns* pats, const ta
   d.anc_L = st->anc_L;
   const bool evict = st->cache_len + 1 > st->K;
   ta_stream_sync sync = ctx->stream_sync;
-  sync.wait_limit_ns = test_limit_ns ? test_limit_ns : ctx->wait_limit_ns ? ctx->wait_limit_ns : 2000000000ull;
+  sync.wait_limit_ns = test_limit_ns ? test_limit_ns : ta_wait_limit(ctx->wait_limit_ns);
   sync.hold_ns = 2 * test_limit_ns;
 
   cudaError_t e = ta_launch_stream_step(d, pats, *policy, new_ids, attn, sync, evicted_pos, ctx->d_status, stream);

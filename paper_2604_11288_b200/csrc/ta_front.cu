@@ -63,7 +63,7 @@ struct FrontParams {
   int32_t* r_main;    // out (scored)
   int32_t* idx;       // out (fast) [B][K]
   int32_t* count;     // out (fast) [B]
-  ta_dev_status* status;
+  ta_waits waits;
 };
 
 // Dynamic shared memory for sequences of up to `items` * 1024 tokens.
@@ -118,8 +118,7 @@ __global__ void __launch_bounds__(kThreads, 1) ta_front_kernel(const __grid_cons
   if (SMEM_HIST)
 #pragma unroll 4
     for (int i = tid; i < (p.vocab + 7) / 8; i += kThreads) reinterpret_cast<uint4*>(s_hist)[i] = make_uint4(0u, 0u, 0u, 0u);
-  Exchange<CL> ex;
-  ex.status = p.status;
+  Exchange<CL> ex{p.waits};
   if constexpr (CL > 1) ex.set_up(sh);
   ta_wait_for_prior_grid();
   ta_launch_dependents();
@@ -183,10 +182,10 @@ __global__ void __launch_bounds__(kThreads, 1) ta_front_kernel(const __grid_cons
   }
   if (s.bad) {
     if (tid == 0) {
-      if (atomicCAS(&p.status->code, 0, (int)TA_ERR_DEVICE_BOUNDS) == 0) {
-        p.status->where = 3;
-        p.status->detail0 = b;
-        p.status->detail1 = s.start;
+      if (atomicCAS(&p.waits.status->code, 0, (int)TA_ERR_DEVICE_BOUNDS) == 0) {
+        p.waits.status->where = 3;
+        p.waits.status->detail0 = b;
+        p.waits.status->detail1 = s.start;
       }
       if (FAST) p.count[b] = 0;
       else p.r_main[b] = -2;  // poisoned: the selection writes an empty result
@@ -213,10 +212,10 @@ __global__ void __launch_bounds__(kThreads, 1) ta_front_kernel(const __grid_cons
       } else if (x >= 0 && x < p.vocab) {
         if (SMEM_HIST) atomicAdd(&s_hist[x >> 1], (x & 1) ? 0x10000u : 1u);
         else atomicAdd(&hist[x], 1);
-      } else if (atomicCAS(&p.status->code, 0, (int)TA_ERR_DEVICE_BOUNDS) == 0) {
-        p.status->where = 1;
-        p.status->detail0 = s.start + lo + i;
-        p.status->detail1 = x;
+      } else if (atomicCAS(&p.waits.status->code, 0, (int)TA_ERR_DEVICE_BOUNDS) == 0) {
+        p.waits.status->where = 1;
+        p.waits.status->detail0 = s.start + lo + i;
+        p.waits.status->detail1 = x;
       }
       const uint32_t h = ((uint32_t)x * 2654435761u) >> 22;
       may_end = x >= 0 && ((s_bloom[h >> 5] >> (h & 31)) & 1u);
@@ -510,7 +509,7 @@ cudaError_t ta_launch_front(const ta_patterns* pats, const ta_policy& pol, const
   p.r_main = a.r_main;
   p.idx = a.idx;
   p.count = a.count;
-  p.status = status;
+  p.waits = {status, ta_wait_limit(a.wait_limit_ns)};
   const int sms = a.sm_count > 0 ? a.sm_count : 148;
   return a.fast ? launch_split<true>(p, sms, false, stream) : launch_split<false>(p, sms, a.u != nullptr, stream);
 }

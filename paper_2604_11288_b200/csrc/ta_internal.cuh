@@ -16,6 +16,15 @@ struct ta_dev_status {
   int step_gave_up;
 };
 
+// Limit of a device-side wait for callers without a context and for contexts that set none: 2 s.
+constexpr unsigned long long kDefaultWaitLimitNs = 2000000000ull;
+inline unsigned long long ta_wait_limit(unsigned long long set_ns) { return set_ns ? set_ns : kDefaultWaitLimitNs; }
+
+struct ta_waits {  // what a kernel with bounded waits is told
+  ta_dev_status* status;  // where a wait that runs out is reported (nullable)
+  unsigned long long limit_ns;
+};
+
 struct ta_patterns {
   int device;
   int n_pat;
@@ -71,7 +80,7 @@ struct ta_ctx {
   // pension weights of the window rows for the (rho, W) they were last formed for
   float wrow_rho, wrow[TA_MAX_WINDOW];
   int wrow_W;
-  unsigned long long wait_limit_ns;   // 0: default limit of device-side waits
+  unsigned long long wait_limit_ns;   // 0: default limit of device-side waits (ta_wait_limit)
   // driver entry point for tensor-map encoding (resolved at create time)
   void* encode_tiled;
 };
@@ -210,6 +219,7 @@ struct ta_select_args {
   int sm_count;  // of the device the launch goes to (0: ask the runtime about the current device)
   float alpha, delta;
   ta_dev_status* status;  // of ta_launch_select_units (nullable)
+  unsigned long long wait_limit_ns;  // of clustered searches; 0: the default
   const uint8_t* flags;
   const float* voucher;
   const float* u_static;

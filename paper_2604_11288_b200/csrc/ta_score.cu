@@ -1237,7 +1237,7 @@ cudaError_t ta_launch_score(ta_ctx* ctx, const ta_score_args& a, ta_dev_status* 
   sp.P = a.P;
   sp.u = a.u;
   sp.status = status;
-  sp.wait_limit_ns = ctx->wait_limit_ns ? ctx->wait_limit_ns : kWaitLimitNs;
+  sp.wait_limit_ns = ta_wait_limit(ctx->wait_limit_ns);
   if (ctx->wrow_W != a.W || ctx->wrow_rho != a.rho) {  // 32 calls of pow() are a microsecond of host time
     for (int t = 0; t < a.W; ++t)
       ctx->wrow[t] = (float)((1.0 - (double)a.rho) * pow((double)a.rho, (double)(a.W - 1 - t)));

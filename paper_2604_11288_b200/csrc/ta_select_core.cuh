@@ -213,8 +213,8 @@ __device__ SelectResult block_radix_select(int n, int want, KeyFn key_of, const 
 // something is on its way to it. What is read after an exchange is read before the block barrier in front of the next one's sends.
 template <int CL>
 struct Exchange {
-  int k = 0;                        // exchanges begun
-  ta_dev_status* status = nullptr;
+  const ta_waits waits;
+  int k = 0;  // exchanges begun
   static __device__ __forceinline__ void set_up(SelectShared<CL>& sh) {  // before a barrier of the cluster
     if (threadIdx.x == 0) {
       ta_sm100::mbar_init(ta_sm100::smem_u32(&sh.arrived[0]), 1);
@@ -250,8 +250,8 @@ struct Exchange {
       if ((tries & 63) != 63) continue;
       const unsigned long long now = ta_sm100::globaltimer_ns();
       if (began == 0) began = now;
-      if (now - began > ta_sm100::kWaitLimitNs) {
-        if (status && atomicCAS(&status->code, 0, (int)TA_ERR_TIMEOUT) == 0) status->where = 8;
+      if (now - began > waits.limit_ns) {
+        if (waits.status && atomicCAS(&waits.status->code, 0, (int)TA_ERR_TIMEOUT) == 0) waits.status->where = 8;
         ok = false;
         break;
       }
@@ -266,8 +266,8 @@ struct Exchange {
 };
 template <>
 struct Exchange<1> {
+  const ta_waits waits;
   int k = 0;
-  ta_dev_status* status = nullptr;
 };
 
 // Shared step of the radix passes: warp 0 walks the 256-bin histogram from the top bin down until `remaining`
@@ -941,7 +941,7 @@ template <bool CACHED, int CL, int ITEMS = kItems>
 __global__ void __launch_bounds__(kThreads, 1024 / kThreads) ta_forced_kernel(ta_seq_desc seq, int K, int n_sink, int n_recent,
                                                              int k_protected, const float* voucher,
                                                              uint8_t* __restrict__ forced,
-                                                             int32_t* __restrict__ r_main, ta_dev_status* status,
+                                                             int32_t* __restrict__ r_main, ta_waits waits,
                                                              const int32_t* __restrict__ class_K, ta_static_out so) {
   __shared__ SelectShared<CL> sh;
   ta_launch_dependents();  // its dependent does not start before every block of the kernel before it runs
@@ -984,10 +984,10 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads) ta_forced_kernel(ta
   }
   if (s.bad) {
     if (threadIdx.x == 0) {
-      if (atomicCAS(&status->code, 0, (int)TA_ERR_DEVICE_BOUNDS) == 0) {
-        status->where = 3;
-        status->detail0 = b;
-        status->detail1 = s.start;
+      if (atomicCAS(&waits.status->code, 0, (int)TA_ERR_DEVICE_BOUNDS) == 0) {
+        waits.status->where = 3;
+        waits.status->detail0 = b;
+        waits.status->detail1 = s.start;
       }
       r_main[b] = -2;  // poisoned: the select kernel writes an empty result
     }
@@ -1007,8 +1007,7 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads) ta_forced_kernel(ta
     return v > 0.0f && !mandatory(lo + il);
   };
   KeyCache<ITEMS> kc;
-  Exchange<CL> ex;
-  ex.status = status;
+  Exchange<CL> ex{waits};
   if constexpr (CACHED && CL > 1) {
     ex.set_up(sh);
     cg::this_cluster().barrier_arrive();
@@ -1065,7 +1064,7 @@ struct UnitSrc {  // where a unit's utility comes from
   const float* P;
   const float* u_static;  // per token
   float alpha, delta;
-  ta_dev_status* status;
+  ta_waits waits;
 };
 
 __device__ __forceinline__ float unit_utility(const UnitSrc& src, long long unit_off, long long tok) {
@@ -1227,8 +1226,7 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads) ta_select_kernel(ta
     gather(n, true);
     return;
   }
-  Exchange<CL> ex;
-  ex.status = src.status;
+  Exchange<CL> ex{src.waits};
   auto key_of = [&](int il, uint32_t& key) {
     key = sortable_key(unit_utility(src, unit_off, (long long)start + lo + il));
     return f[il] == 0;

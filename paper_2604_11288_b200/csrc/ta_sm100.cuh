@@ -9,8 +9,6 @@
 
 namespace ta_sm100 {
 
-constexpr unsigned long long kWaitLimitNs = 2000000000ull;  // default limit of a device-side wait: 2 s
-
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {

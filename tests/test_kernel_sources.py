@@ -35,3 +35,14 @@ def test_kernels_launched_early_read_no_callers_data_as_invariant():
         assert not invariant or name in BEHIND_OWN_KERNEL, (name, invariant)
     first = {"ta_stream_step_kernel", "ta_embed_conf_kernel", "ta_compact_kernel", "ta_score_kernel", "ta_front_kernel"}
     assert first | BEHIND_OWN_KERNEL <= seen
+
+
+def test_every_wait_takes_the_contexts_limit():
+    # one place knows the default, no other file a limit of its own, and whoever has a context hands its limit on
+    for path in sorted(glob.glob(os.path.join(CSRC, "*.cu")) + glob.glob(os.path.join(CSRC, "*.cuh"))):
+        src = re.sub(r"//[^\n]*", "", open(path).read())
+        if os.path.basename(path) != "ta_internal.cuh":
+            assert not re.search(r"WaitLimitNs\b|\b2000000000", src), path
+        if os.path.basename(path) == "ta_api.cu":
+            made = re.findall(r"ta_select_args (\w+) = \{\};", src)
+            assert made and all(f"{m}.wait_limit_ns = ctx->wait_limit_ns;" in src for m in made), made
