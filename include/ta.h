@@ -162,6 +162,10 @@ ta_status ta_ctx_set_wait_limit(ta_ctx* ctx, uint64_t nanoseconds);
  * when the limit is reached, sets bit 2 of *outcome (DEVICE int32; bits 0 and 1 would mean a wait succeeded), and
  * the next ta_ctx_poll reports TA_ERR_TIMEOUT once. The context stays usable. */
 ta_status ta_ctx_selftest_wait(ta_ctx* ctx, uint64_t limit_ns, int32_t* outcome, void* stream);
+/* The same for the searches that several CTAs share (long sequences): two CTAs search together, and the second stops taking part
+ * after `stop` of four exchanges (0..3; 4: it takes part in all). *outcome (DEVICE int32) gets how many of 100 wanted keys were taken;
+ * it keeps its value when a wait ran out, which the next ta_ctx_poll reports as TA_ERR_TIMEOUT once. */
+ta_status ta_ctx_selftest_exchange(ta_ctx* ctx, uint64_t limit_ns, int stop, int32_t* outcome, void* stream);
 /* Tuning: CTAs that share one (layer, sequence, KV head) unit in the score kernel: 1, 2, 4 or 8; 0 (default) lets
  * the library choose per launch from the unit count, the sequence length and the L2 size. */
 ta_status ta_ctx_set_score_cluster(ta_ctx* ctx, int ctas_per_unit);

@@ -159,6 +159,7 @@ def lib():
             "ta_ctx_set_wait_limit": (i32, [vp, u64]),
             "ta_ctx_set_score_cluster": (i32, [vp, i32]),
             "ta_ctx_selftest_wait": (i32, [vp, u64, vp, vp]),
+            "ta_ctx_selftest_exchange": (i32, [vp, u64, i32, vp, vp]),
             "ta_ctx_last_launch_info": (i32, [vp, C.POINTER(C.c_int32)]),
             "ta_select_topk": (i32, [vp, PP, PB, i32, i32, vp, vp, vp, vp, vp, vp, vp, vp]),
             "ta_select_topk_static": (i32, [PP, PB, i32, i32, vp, vp, vp, vp, vp, vp, vp, vp]),
@@ -340,6 +341,10 @@ def ta_ctx_last_launch_info(ctx):
 
 def ta_ctx_selftest_wait(ctx, limit_ns: int, outcome, stream=None):
     _check(lib().ta_ctx_selftest_wait(ctx, int(limit_ns), _ptr(outcome), stream), "ta_ctx_selftest_wait")
+
+
+def ta_ctx_selftest_exchange(ctx, limit_ns: int, stop: int, outcome, stream=None):
+    _check(lib().ta_ctx_selftest_exchange(ctx, int(limit_ns), int(stop), _ptr(outcome), stream), "ta_ctx_selftest_exchange")
 
 
 def ta_ctx_set_score_cluster(ctx, ctas_per_unit: int):

@@ -334,6 +334,13 @@ ta_status ta_ctx_selftest_wait(ta_ctx* ctx, uint64_t limit_ns, int32_t* outcome,
   return e == cudaSuccess ? TA_OK : cuda_fail(ctx, e);
 }
 
+ta_status ta_ctx_selftest_exchange(ta_ctx* ctx, uint64_t limit_ns, int stop, int32_t* outcome, void* stream) {
+  if (!ctx || !outcome || limit_ns == 0 || limit_ns > 1000000000ull || stop < 0 || stop > 4) return TA_ERR_INVALID_ARG;
+  DeviceGuard guard(ctx->device);
+  cudaError_t e = ta_launch_exchange_selftest(ctx->d_status, limit_ns, stop, outcome, (cudaStream_t)stream);
+  return e == cudaSuccess ? TA_OK : cuda_fail(ctx, e);
+}
+
 ta_status ta_ctx_last_launch_info(const ta_ctx* ctx, int32_t out[4]) {
   if (!ctx || !out) return TA_ERR_INVALID_ARG;
   out[0] = ctx->score_cluster;

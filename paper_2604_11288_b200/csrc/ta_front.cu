@@ -330,12 +330,15 @@ __global__ void __launch_bounds__(kThreads, 1) ta_front_kernel(const __grid_cons
   int m = s_listed;
   int taken = s.s_take + s.r_take;
   if constexpr (CL > 1) {
+    if (tid == 0 && rank == 0) {  // what a wait that runs out leaves: an empty result
+      if (FAST) p.count[b] = 0;
+      else p.r_main[b] = -2;
+    }
     if (tid < CL) ex.send2(sh, s_sponsored[rank], tid, (uint32_t)m, 0u);
-    const bool ok = ex.wait(sh, CL * 8);
+    ex.wait(sh, CL * 8);
     m = 0;
 #pragma unroll
     for (int q = 0; q < CL; ++q) m += s_sponsored[q][0];
-    if (!ok) m = 0;
   }
   if (CL > 1 && m <= s.p) {
     taken += m;  // (the bits are there)
@@ -398,7 +401,7 @@ __global__ void __launch_bounds__(kThreads, 1) ta_front_kernel(const __grid_cons
   }, sh, ex);
   if (rank != 0) return;
   for (int q = got + tid; q < p.K; q += kThreads) out[q] = -1;
-  if (tid == 0) p.count[b] = got;
+  if (tid == 0) p.count[b] = min(got, p.K);
 }
 
 template <int ITEMS, bool FAST, int CL>

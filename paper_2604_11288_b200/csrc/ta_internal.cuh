@@ -249,6 +249,9 @@ struct ta_select_args {
   int static_vocab;
   float beta, gamma, lambda;
 };
+// diagnostic: a search shared by two CTAs of which the second stops taking part (ta_exchange_selftest_kernel)
+cudaError_t ta_launch_exchange_selftest(ta_dev_status* status, unsigned long long limit_ns, int stop, int32_t* outcome,
+                                        cudaStream_t stream);
 bool ta_select_gathers(const ta_select_args& a);  // whether ta_launch_select_units will do the gather itself
 // Steps 1 and the per-sequence part of 3 in one kernel for sequences that fit a cluster of blocks (ta_front.cu): static utilities, forced
 // set and r_main as ta_launch_mask and ta_launch_forced leave them (without flags and vouchers); fast mode: idx and count

@@ -89,7 +89,53 @@ __global__ void ta_broadcast_heads_kernel(long long units_lb, int Hkv, int K, co
   }
 }
 
+// Two CTAs search 2 x 512 keys together (stop 2: 2 x 2048), and the second stops after what its first `stop` exchanges need: 0
+// nothing, 1 and 2 the range of its keys (then candidates or a histogram are missing), 3 also its candidates (then its totals are);
+// 4: it stays to the end. *outcome: the keys taken, unless a wait ran out.
+__global__ void __launch_bounds__(kThreads) ta_exchange_selftest_kernel(ta_waits waits, int stop, int32_t* outcome) {
+  __shared__ SelectShared<2> sh;
+  constexpr int kPer = 4, kSent = 8;
+  const int tid = threadIdx.x, rank = (int)cg::this_cluster().block_rank();
+  const int n = stop == 2 ? kPer * kThreads : kThreads;
+  const uint32_t lo = 1u << 20;  // the keys: lo .. lo + 2n - 1, every other one of each CTA
+  KeyCache<kPer> kc;
+#pragma unroll
+  for (int it = 0; it < kPer; ++it) kc.key[it] = lo + 2u * (uint32_t)(tid + it * kThreads) + (uint32_t)rank;
+  kc.elig = stop == 2 ? (1u << kPer) - 1u : 1u;
+  Exchange<2> ex{waits};
+  ex.set_up(sh);
+  cg::this_cluster().sync();
+  if (rank == 0 || stop >= 4) {
+    const SelectResult r = cached_radix_select<2>(n, 2 * n, 100, kc, sh, ex);
+    const int taken = cached_ordered_emit<2>(n, r, kc, 0u, [](int, int) {}, sh, ex);
+    if (rank == 0 && tid == 0) *outcome = taken;
+  } else {
+    if (stop >= 1 && tid < 2)
+      ex.send4(sh, sh.cl_range[1], tid, make_uint4(lo + 1u, lo + 2u * (uint32_t)n - 1u, stop == 2 ? (uint32_t)n : (uint32_t)kSent, 0u));
+    ex.k = 1;
+    if (stop >= 3 && tid < 2) ex.send1(sh, &sh.took_part[1], tid, 0u);
+    if (stop >= 3 && tid < kSent) ex.send1(sh, &sh.cand_keys[n + tid], 0, lo + 2u * (uint32_t)(n - tid) - 1u);
+    ex.stay();  // the first one sends to it
+  }
+}
+
 }  // namespace
+
+cudaError_t ta_launch_exchange_selftest(ta_dev_status* status, unsigned long long limit_ns, int stop, int32_t* outcome,
+                                        cudaStream_t stream) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(2, 1, 1);
+  cfg.blockDim = dim3(kThreads, 1, 1);
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = 2;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, ta_exchange_selftest_kernel, ta_waits{status, limit_ns}, stop, outcome);
+}
 
 // Scratch layout used by the launcher (the caller carves it): forced [total] bytes, r_main [B] ints; fast mode
 // additionally idx_seq [B][K] and count_seq [B] (passed through a.idx / a.count by the caller when it wants the

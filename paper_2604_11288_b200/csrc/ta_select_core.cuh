@@ -209,8 +209,12 @@ __device__ SelectResult block_radix_select(int n, int want, KeyFn key_of, const 
 // A unit split over a cluster, keys in registers: the CTAs exchange what they found with stores that count on the receiver's
 // mbarrier when they land. (A cluster barrier of 1024 threads after plain remote stores costs 1.5 to 3 K cycles, most of it the
 // release of everything that the threads wrote; a search has five exchanges.) Every CTA sends to all and waits for all, so that
-// none can be two exchanges ahead of another: two mbarriers and two buffers, taken in turn, are enough, and no CTA leaves while
-// something is on its way to it. What is read after an exchange is read before the block barrier in front of the next one's sends.
+// none can be two exchanges ahead of another: two mbarriers and two buffers, taken in turn, are enough. What is read after an exchange
+// is read before the block barrier in front of the next one's sends. A CTA that has been through all exchanges has received all that
+// was ever sent to it and may leave. A wait that ran out ends its CTA: what the kernel leaves behind then has to be there before. Its
+// peers' next waits run out in turn, and since they may send to it until then it stays until they have all left or given up as well
+// (the cluster's barrier counts CTAs that have left. With all CTAs in that barrier 1 x 131072 tokens took 1 us more; with a search
+// that returns in place of ending its CTA as much, for registers that it spilled).
 template <int CL>
 struct Exchange {
   const ta_waits waits;
@@ -238,9 +242,9 @@ struct Exchange {
                  "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w), "r"(at(&sh.arrived[k & 1], q))
                  : "memory");
   }
-  // All threads, after the sends: `bytes` have arrived. A barrier of the block. False: they did not come within a limit that CTAs which run together
-  // do not reach (reported; what was to be received must not be used).
-  __device__ __forceinline__ bool wait(SelectShared<CL>& sh, uint32_t bytes) {
+  // All threads, after the sends: `bytes` have arrived. A barrier of the block. Does not return when they did not come within a limit
+  // that CTAs which run together do not reach (reported).
+  __device__ __forceinline__ void wait(SelectShared<CL>& sh, uint32_t bytes) {
     const uint32_t bar = ta_sm100::smem_u32(&sh.arrived[k & 1]), parity = (uint32_t)(k >> 1) & 1u;
     if (threadIdx.x == 0) ta_sm100::mbar_expect_tx(bar, bytes);
     ++k;
@@ -256,7 +260,16 @@ struct Exchange {
         break;
       }
     }
-    return __syncthreads_and(ok) != 0;
+    if (__syncthreads_and(ok) == 0) {
+      stay();
+      asm volatile("exit;");
+      __builtin_unreachable();
+    }
+  }
+  static __device__ __forceinline__ void stay() {
+    ta_sm100::cluster_arrive();
+    ta_sm100::cluster_wait();
+    __nanosleep(50000);  // what its peers sent before they arrived has landed
   }
 
  private:
@@ -498,7 +511,7 @@ __device__ SelectResult cached_radix_select(int n, int n_unit, int want, const K
   if constexpr (CL > 1) {
     const int rank = (int)cg::this_cluster().block_rank();
     if (tid < CL) ex.send4(sh, sh.cl_range[rank], tid, make_uint4(kmin, kmax, num, 0u));
-    const bool ok = ex.wait(sh, CL * 16);
+    ex.wait(sh, CL * 16);
     kmin = 0xffffffffu;
     kmax = 0u;
     num = 0u;
@@ -510,7 +523,6 @@ __device__ SelectResult cached_radix_select(int n, int n_unit, int want, const K
       if (q == rank) own = (int)sh.cl_range[q][2];
       num += sh.cl_range[q][2];
     }
-    if (!ok) num = 0u;
   }
   if (!bounded && num < (uint32_t)want) {  // fewer eligible elements than requested: all of them
     r.all = 1;
@@ -814,7 +826,7 @@ __device__ int cached_ordered_emit(int n, const SelectResult& r, const KeyCache<
   if constexpr (CL > 1) {
     const int rank = (int)cg::this_cluster().block_rank(), turn = ex.k & 1;
     if (tid < CL) ex.send2(sh, sh.totals[turn][rank], tid, (uint32_t)def_all, (uint32_t)tie_all);
-    if (!ex.wait(sh, CL * 8)) return 0;
+    ex.wait(sh, CL * 8);
     def_all = 0;
     tie_all = 0;
 #pragma unroll
@@ -1009,6 +1021,7 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads) ta_forced_kernel(ta
   KeyCache<ITEMS> kc;
   Exchange<CL> ex{waits};
   if constexpr (CACHED && CL > 1) {
+    if (threadIdx.x == 0 && blockIdx.x % CL == 0) r_main[b] = -2;  // what a wait that runs out leaves: an empty result
     ex.set_up(sh);
     cg::this_cluster().barrier_arrive();
   }
@@ -1233,6 +1246,7 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads) ta_select_kernel(ta
   };
   if constexpr (CACHED) {
     if constexpr (CL > 1) {
+      if (lead && tid == 0) count[unit] = 0;  // what a wait that runs out leaves
       ex.set_up(sh);
       cg::this_cluster().barrier_arrive();
     }
@@ -1273,7 +1287,7 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads) ta_select_kernel(ta
     taken = cluster_ordered_emit<CACHED, CL>(hi - lo, r.ties, key_of, kc, classify, emit, sh);
   if (!lead) return;
   for (int q = taken + tid; q < K; q += kThreads) out[q] = -1;
-  if (tid == 0) count[unit] = taken;
+  if (tid == 0) count[unit] = min(taken, K);
   gather(min(taken, K), false);
 }
 
