@@ -793,8 +793,9 @@ ta_status compress_impl(ta_ctx* ctx, const ta_patterns* pats, const ta_policy* p
   bool beside = false;  // the kernel before the score kernel is one that lets it start at once
   if (!reuse) {
     if (timing && e == cudaSuccess) e = cudaEventRecord(ctx->ev[5], stream);
-    if (!budgets && ta_front_fits(seq)) {
-      if (e == cudaSuccess) e = ta_launch_front(pats, *policy, sel, token_ids, hist, ctx->d_status, stream);
+    bool front = false;
+    if (e == cudaSuccess && !budgets) e = ta_launch_front(pats, *policy, sel, token_ids, hist, ctx->d_status, &front, stream);
+    if (front) {
       launches += 1;
     } else {
       if (e == cudaSuccess)

@@ -23,6 +23,7 @@
 
 #include <atomic>
 
+#include "ta_front_rule.h"
 #include "ta_internal.cuh"
 #include "ta_sm100.cuh"
 
@@ -39,10 +40,11 @@ namespace {
 using namespace front1024;
 
 constexpr int kPad = TA_MAX_PATTERN_LEN;  // ids before the sequence (never part of a match)
-constexpr int kMaxItems = 16;             // tokens per thread
+constexpr int kMaxItems = kFrontMaxItems;
+static_assert(kThreads == kFrontThreads, "the rule's block");
 constexpr int kListCap = 256;             // so few sponsored tokens are ranked by comparing them with one another
 constexpr int kMaxDynamicSmem = 211 * 1024;  // beside at most 16 KB of static shared memory (a block may use 227 KB)
-constexpr int kMaxCluster = 16;
+constexpr int kMaxCluster = kFrontMaxCluster;
 
 struct FrontParams {
   ta_seq_desc seq;
@@ -404,85 +406,113 @@ __global__ void __launch_bounds__(kThreads, 1) ta_front_kernel(const __grid_cons
   if (tid == 0) p.count[b] = min(got, p.K);
 }
 
+// An instance made ready for launching, and how many of its clusters the current device holds at once (0: none).
 template <int ITEMS, bool FAST, int CL>
-cudaError_t launch_front(const FrontParams& p, cudaStream_t stream) {
-  const bool smem_hist = CL == 1 && front_smem(ITEMS, p.vocab, true, CL, sizeof(SelectShared<CL>)).end <= kMaxDynamicSmem;
-  auto kern = smem_hist ? ta_front_kernel<ITEMS, FAST, CL == 1, CL> : ta_front_kernel<ITEMS, FAST, false, CL>;
-  const int smem = front_smem(ITEMS, p.vocab, smem_hist, CL, sizeof(SelectShared<CL>)).end;
-  // per device; setting the (sticky) attributes twice from two threads is harmless, the flag only saves the calls
-  static std::atomic<bool> attr_set[2][64];
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  std::atomic<bool>& set = attr_set[smem_hist ? 1 : 0][dev & 63];
-  if (!set.load(std::memory_order_acquire)) {
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynamicSmem);
-    if (e == cudaSuccess && CL > 8) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+struct FrontInstance {
+  bool smem_hist;
+  int smem;
+  using Kernel = void (*)(const FrontParams);
+  Kernel kern;
+
+  explicit FrontInstance(int vocab) {
+    smem_hist = CL == 1 && front_smem(ITEMS, vocab, true, CL, sizeof(SelectShared<CL>)).end <= kMaxDynamicSmem;
+    kern = smem_hist ? ta_front_kernel<ITEMS, FAST, CL == 1, CL> : ta_front_kernel<ITEMS, FAST, false, CL>;
+    smem = front_smem(ITEMS, vocab, smem_hist, CL, sizeof(SelectShared<CL>)).end;
+  }
+  void configure(cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr) const {  // room for one attribute
+    cfg->blockDim = dim3(kThreads, 1, 1);
+    cfg->dynamicSmemBytes = (size_t)smem;
+    cfg->attrs = attr;
+    cfg->numAttrs = 0;
+    if (CL > 1) {
+      attr[0].id = cudaLaunchAttributeClusterDimension;
+      attr[0].val.clusterDim.x = (unsigned)CL;
+      attr[0].val.clusterDim.y = 1;
+      attr[0].val.clusterDim.z = 1;
+      cfg->numAttrs = 1;
+    }
+  }
+  // per device; doing it twice from two threads is harmless (the attributes are sticky), what is kept only saves the calls
+  cudaError_t ready(int* clusters) const {
+    static std::atomic<int> known[2][64];  // 1 + clusters
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    set.store(true, std::memory_order_release);
+    std::atomic<int>& k = known[smem_hist ? 1 : 0][dev & 63];
+    int have = k.load(std::memory_order_acquire);
+    if (have == 0) {
+      e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynamicSmem);
+      if (e == cudaSuccess && CL > 8) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+      if (e != cudaSuccess) return e;
+      int n = 1;
+      if (CL > 1) {
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute attr[1];
+        configure(&cfg, attr);
+        cfg.gridDim = dim3(CL, 1, 1);
+        if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess) {
+          cudaGetLastError();  // a size that the device does not have
+          n = 0;
+        }
+      }
+      have = 1 + n;
+      k.store(have, std::memory_order_release);
+    }
+    *clusters = have - 1;
+    return cudaSuccess;
   }
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(p.seq.batch * CL), 1, 1);
-  cfg.blockDim = dim3(kThreads, 1, 1);
-  cfg.dynamicSmemBytes = (size_t)smem;
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[2];
-  ta_pdl_attribute(&attr[0]);
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  if (CL > 1) {
-    attr[1].id = cudaLaunchAttributeClusterDimension;
-    attr[1].val.clusterDim.x = (unsigned)CL;
-    attr[1].val.clusterDim.y = 1;
-    attr[1].val.clusterDim.z = 1;
-    cfg.numAttrs = 2;
+  cudaError_t launch(const FrontParams& p, cudaStream_t stream) const {
+    int clusters = 0;
+    cudaError_t e = ready(&clusters);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[2];
+    configure(&cfg, attr);
+    cfg.gridDim = dim3((unsigned)(p.seq.batch * CL), 1, 1);
+    cfg.stream = stream;
+    ta_pdl_attribute(&attr[cfg.numAttrs++]);
+    return cudaLaunchKernelEx(&cfg, kern, p);
   }
-  return cudaLaunchKernelEx(&cfg, kern, p);
-}
+};
 
-// Blocks per sequence. One holds up to 16384 tokens; more are worth their exchanges where a thread of one block would have more
-// than 12 tokens, or has to. Of the sizes that hold the longest sequence the largest of which all sequences' clusters fit at once
-// (148 SMs: 7 of 16 blocks, 15 of 8, 35 of 4, 74 of 2), else the smallest. us per call of TA-Fast (one layer, one KV head) with
-// separate kernels for mask, forced set and selection / 2 / 4 / 8 / 16 blocks:
-//   1 x 131072 K 64 38.1 / - / - / 41.2 / 29.7; 4 x 131072 K 4096 57.1 / - / - / 46.1 / 35.4; 16 x 131072 109.6 / - / - / 78.5 / 82.6
-//   4 x 65536 42.2 / - / 40.5 / 28.5 / 24.5; 8 x 32768 37.7 / 41.4 / 28.5 / 23.6 / 44.0; 60 x 32768 144.6 / 45.4 / 57.9 / 87.5 / 190
-// and with one block / 2 / 4 / 8: 1 x 16384 26.3 / 25.7 / 19.3 / 16.9, 8 x 16384 27.5 / 26.8 / 20.5 / 18.2, 60 x 16384 31.7 / 31.1 /
-// 41.6 / 66; 4 x 12000 18.5 / 25.6 / 19.4 / 17.6, 1 x 8192 14.7 / 21.7 / 18.0 / 16.6. Beside a score kernel, which hides it, one
-// block leaves it the most SMs.
-int front_blocks(int n, int batch, int sms, bool hidden) {
-  if (n <= (hidden ? kMaxItems : 12) * kThreads) return 1;
-  const int fit[] = {7, 15, 35, 74}, least = (n + kMaxItems * kThreads - 1) / (kMaxItems * kThreads);
-  for (int i = 0, cl = kMaxCluster; cl > 1 && cl >= least; ++i, cl /= 2)
-    if (batch <= fit[i] * sms / 148) return cl;
-  return least <= 1 ? 1 : least <= 2 ? 2 : least <= 4 ? 4 : least <= 8 ? 8 : kMaxCluster;
-}
-
-template <bool FAST, int CL>
-cudaError_t launch_items(const FrontParams& p, cudaStream_t stream) {
-  // the smallest instance that holds the slices: unused slots cost issue time in every phase
+// f(the smallest instance that holds the slices): unused slots cost issue time in every phase
+template <bool FAST, int CL, class F>
+cudaError_t with_items(const FrontParams& p, F f) {
   const int items = (p.seq.max_n + CL * kThreads - 1) / (CL * kThreads);
-  if (CL != 2 && items <= 4) return launch_front<CL == 2 ? kMaxItems : 4, FAST, CL>(p, stream);
-  if (CL != 2 && items <= 8) return launch_front<CL == 2 ? kMaxItems : 8, FAST, CL>(p, stream);
-  return launch_front<kMaxItems, FAST, CL>(p, stream);
+  if (CL != 2 && items <= 4) return f(FrontInstance<CL == 2 ? kMaxItems : 4, FAST, CL>(p.vocab));
+  if (CL != 2 && items <= 8) return f(FrontInstance<CL == 2 ? kMaxItems : 8, FAST, CL>(p.vocab));
+  return f(FrontInstance<kMaxItems, FAST, CL>(p.vocab));
+}
+template <bool FAST, class F>
+cudaError_t with_instance(const FrontParams& p, int blocks, F f) {
+  switch (blocks) {
+    case 1: return with_items<FAST, 1>(p, f);
+    case 2: return with_items<FAST, 2>(p, f);
+    case 4: return with_items<FAST, 4>(p, f);
+    case 8: return with_items<FAST, 8>(p, f);
+    default: return with_items<FAST, kMaxCluster>(p, f);
+  }
 }
 
 template <bool FAST>
-cudaError_t launch_split(const FrontParams& p, int sms, bool hidden, cudaStream_t stream) {
-  switch (front_blocks(p.seq.max_n, p.seq.batch, sms, hidden)) {
-    case 1: return launch_items<FAST, 1>(p, stream);
-    case 2: return launch_items<FAST, 2>(p, stream);
-    case 4: return launch_items<FAST, 4>(p, stream);
-    case 8: return launch_items<FAST, 8>(p, stream);
-    default: return launch_items<FAST, kMaxCluster>(p, stream);
-  }
+cudaError_t launch_split(const FrontParams& p, int sms, bool hidden, bool* launched, cudaStream_t stream) {
+  cudaError_t e = cudaSuccess;
+  const int blocks = ta_front_blocks(p.seq.max_n, p.seq.batch, sms, hidden, [&](int cl) {
+    int clusters = 0;
+    const cudaError_t r = with_instance<FAST>(p, cl, [&](const auto& inst) { return inst.ready(&clusters); });
+    if (r != cudaSuccess) e = r;
+    return r == cudaSuccess ? clusters : 0;
+  });
+  *launched = blocks > 0;
+  if (e != cudaSuccess || blocks == 0) return e;
+  return with_instance<FAST>(p, blocks, [&](const auto& inst) { return inst.launch(p, stream); });
 }
 
 }  // namespace
 
-bool ta_front_fits(const ta_seq_desc& seq) { return seq.max_n <= kMaxCluster * kMaxItems * kThreads; }
-
 cudaError_t ta_launch_front(const ta_patterns* pats, const ta_policy& pol, const ta_select_args& a, const int32_t* ids,
-                            int32_t* hist, ta_dev_status* status, cudaStream_t stream) {
+                            int32_t* hist, ta_dev_status* status, bool* launched, cudaStream_t stream) {
+  *launched = true;
   if (a.seq.batch == 0) return cudaSuccess;
   FrontParams p = {};
   p.seq = a.seq;
@@ -514,5 +544,6 @@ cudaError_t ta_launch_front(const ta_patterns* pats, const ta_policy& pol, const
   p.count = a.count;
   p.waits = {status, ta_wait_limit(a.wait_limit_ns)};
   const int sms = a.sm_count > 0 ? a.sm_count : 148;
-  return a.fast ? launch_split<true>(p, sms, false, stream) : launch_split<false>(p, sms, a.u != nullptr, stream);
+  return a.fast ? launch_split<true>(p, sms, false, launched, stream)
+                : launch_split<false>(p, sms, a.u != nullptr, launched, stream);
 }

@@ -258,9 +258,9 @@ bool ta_select_gathers(const ta_select_args& a);  // whether ta_launch_select_un
 // per sequence, and nothing else. hist is used for vocabularies that do not fit in shared memory and for sequences beyond one
 // block; needs no clearing.
 // The kernel lets its programmatic dependent start as soon as it runs itself.
-bool ta_front_fits(const ta_seq_desc& seq);
+// launched: false, and nothing was done, when the sequences are too long or the device holds no cluster of blocks that they need.
 cudaError_t ta_launch_front(const ta_patterns* pats, const ta_policy& pol, const ta_select_args& a, const int32_t* ids,
-                            int32_t* hist /*[B][vocab]*/, ta_dev_status* status, cudaStream_t stream);
+                            int32_t* hist /*[B][vocab]*/, ta_dev_status* status, bool* launched, cudaStream_t stream);
 cudaError_t ta_launch_select(const ta_select_args& a, ta_dev_status* status, cudaStream_t stream);  // both below
 cudaError_t ta_launch_forced(const ta_select_args& a, ta_dev_status* status, cudaStream_t stream);
 cudaError_t ta_launch_select_units(const ta_select_args& a, cudaStream_t stream);

@@ -1,0 +1,52 @@
+"""How many blocks of the per-sequence kernel share a sequence, and that a device which holds no such cluster is given one kernel per
+step: the rule is host code, compiled here by itself."""
+import ctypes
+import os
+import subprocess
+
+import pytest
+
+import paper_2604_11288_b200 as ta
+
+SOURCE = r"""
+#include "ta_front_rule.h"
+extern "C" int blocks(int n, int batch, int sms, int hidden, const int* fits) {
+  return ta_front_blocks(n, batch, sms, hidden != 0, [&](int cl) { return cl == 16 ? fits[3] : cl == 8 ? fits[2] : cl == 4 ? fits[1] : fits[0]; });
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def rule(tmp_path_factory):
+    d = tmp_path_factory.mktemp("rule")
+    (d / "rule.cpp").write_text(SOURCE)
+    csrc = os.path.join(os.path.dirname(ta.__file__), "csrc")
+    subprocess.run([os.environ.get("CXX", "g++"), "-std=c++17", "-O1", "-fPIC", "-shared", "-I", csrc, str(d / "rule.cpp"), "-o",
+                    str(d / "rule.so")], check=True)
+    f = ctypes.CDLL(str(d / "rule.so")).blocks
+
+    def blocks(n, batch, fits, hidden=False, sms=148):
+        return f(n, batch, sms, int(hidden), (ctypes.c_int * 4)(*fits))
+    return blocks
+
+
+B200 = (74, 33, 15, 7)  # clusters of 2, 4, 8, 16 blocks
+SIZES = [1, 12288, 12289, 16384, 16385, 32768, 32769, 65536, 65537, 131072, 131073, 262144, 262145]
+
+
+@pytest.mark.parametrize("hidden", [False, True])
+@pytest.mark.parametrize("fits", [B200, (0, 0, 0, 0), (74, 0, 0, 0), (74, 33, 15, 0), (0, 0, 3, 1), (9, 4, 0, 0)])
+def test_only_sizes_that_hold_the_sequence_and_that_the_device_holds(rule, fits, hidden):
+    for n in SIZES:
+        for batch in (1, 2, 7, 8, 15, 16, 33, 34, 74, 75, 1000):
+            cl = rule(n, batch, fits, hidden)
+            able = [c for c, f in zip((1, 2, 4, 8, 16), (1,) + fits) if c * 16384 >= n and f > 0]
+            assert cl in able or (cl == 0 and (not able or n > 131072)), (n, batch, cl)
+            if n <= 12288:
+                assert cl == 1
+
+
+def test_all_clusters_at_once_where_they_fit(rule):
+    assert [rule(20000, b, B200) for b in (15, 16, 33, 34, 74, 75)] == [8, 4, 4, 2, 2, 2]
+    assert rule(200000, 3, (74, 33, 15, 0)) == 0
+    assert rule(20000, 20, (0, 0, 0, 0)) == 0
