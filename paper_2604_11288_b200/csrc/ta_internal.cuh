@@ -252,6 +252,14 @@ struct ta_select_args {
 // diagnostic: a search shared by two CTAs of which the second stops taking part (ta_exchange_selftest_kernel)
 cudaError_t ta_launch_exchange_selftest(ta_dev_status* status, unsigned long long limit_ns, int stop, int32_t* outcome,
                                         cudaStream_t stream);
+// Whether a cluster of kHelpBlocks blocks per unit, of which the first selects, moves the rows of few short units: one block reads a
+// unit's rows one round trip after another. Only where all units' clusters run at once (held: how many the device holds). us per
+// call (given scores) without / with 4 blocks: 1 to 33 units of 4096 tokens K 512 20.7 to 22.0 / 18.5 to 19.8, K 1024 28.3 to 29.4 /
+// 22.3 to 22.9, K 4000 57.9 to 63.1 / 29.7 to 32.5; on a GPU that holds 33 clusters 34 units K 600 23.3 / 31.9, 35 units of 8000
+// tokens K 1024 34.2 / 44.1. Smaller budgets: 8 units K 128 25.6 / 27.8, K 256 23.9 / 24.2. 8 blocks: 8 units K 1024 33.3 / 25.6 (4: 26.6),
+// 16 units K 606 34.0 / 40.6 (4: 30.7).
+constexpr int kHelpBlocks = 4, kHelpedBudget = 512;
+inline bool ta_select_helped(int K, int units, int held) { return K >= kHelpedBudget && units <= held; }
 bool ta_select_gathers(const ta_select_args& a);  // whether ta_launch_select_units will do the gather itself
 // Steps 1 and the per-sequence part of 3 in one kernel for sequences that fit a cluster of blocks (ta_front.cu): static utilities, forced
 // set and r_main as ta_launch_mask and ta_launch_forced leave them (without flags and vouchers); fast mode: idx and count

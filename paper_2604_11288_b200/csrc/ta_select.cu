@@ -18,6 +18,8 @@
 //                      result is copied to every head.
 #include <cooperative_groups.h>
 
+#include <atomic>
+
 #include "ta_internal.cuh"
 #include "ta_sm100.cuh"
 
@@ -186,6 +188,33 @@ cudaError_t launch_threads(int threads, Kern kern, int units, int cl, StreamPdl 
   cfg.numAttrs = n;
   return cudaLaunchKernelEx(&cfg, kern, args...);
 }
+// How many clusters of cl such blocks the current device holds at once; known: what earlier calls found, 1 + clusters per device.
+constexpr int kMaxDevices = 64;
+template <class Kern>
+int clusters_held(Kern kern, int threads, int cl, std::atomic<int>* known) {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+  std::atomic<int>& k = known[dev % kMaxDevices];
+  const int have = k.load(std::memory_order_relaxed);
+  if (have > 0) return have - 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)cl, 1, 1);
+  cfg.blockDim = dim3((unsigned)threads, 1, 1);
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)cl;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  int n = 0;
+  if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess) {
+    cudaGetLastError();  // a size that the device does not have
+    n = 0;
+  }
+  k.store(1 + n, std::memory_order_relaxed);
+  return n;
+}
 template <class Kern, class... Args>
 cudaError_t launch_clustered(Kern kern, int units, int cl, StreamPdl sp, Args... args) {
   return launch_threads(kThreads, kern, units, cl, sp, args...);
@@ -310,17 +339,17 @@ cudaError_t ta_launch_select_units(const ta_select_args& a, cudaStream_t stream_
   // with it, K 256 and 512 of 1000 tokens 14.7 and 17.6 without, 15.0 and 18.0 with it.
   const bool few = gathers && a.K <= kThreads / 2, few1024 = gathers && a.K <= sel1024::kThreads / 2;
   if (few_short_units(a)) {
-    // A large gather by a cluster of blocks per unit, of which the first selects: one block reads a unit's rows one round trip
-    // after another. us per call without / with 4 / 8 blocks: 8 units K 256 23.9 / 24.2 / 24.5, K 512 30.3 / 28.9 / 28.8, K 1024 33.3 /
-    // 26.6 / 25.6; 16 units K 606 34.0 / 30.7 / 40.6 (15 clusters of 8 fit at once, 35 of 4); K 128 25.6 / 27.8 / 27.7.
-    const int help = a.K >= 512 && units <= 35 * sms / 148 ? 4 : 1;
-    if (gathers && help > 1) {
-      auto kern = a.seq.max_n <= 4 * sel1024::kThreads ? sel1024::ta_select_kernel<true, 1, 4, true, false, true>
-                  : few1024                            ? sel1024::ta_select_kernel<true, 1, 8, true, true, true>
-                                                       : sel1024::ta_select_kernel<true, 1, 8, true, false, true>;
-      return launch_threads(sel1024::kThreads, kern, units, help, stream, a.seq, a.n_layers, a.Hkv, a.K, a.fast, src2, a.forced,
-                            a.r_main, a.idx, a.count, gd2, co);
-    }
+    // (the instance for few wanted tokens at the one budget that both rules take: 8 units of 5000, 6000, 8000 tokens K 512 22.0, 22.9,
+    // 24.1 with it, 22.5, 23.5, 25.2 without)
+    const int which = a.seq.max_n <= 4 * sel1024::kThreads ? 0 : few1024 ? 1 : 2;
+    auto helped = which == 0   ? sel1024::ta_select_kernel<true, 1, 4, true, false, true>
+                  : which == 1 ? sel1024::ta_select_kernel<true, 1, 8, true, true, true>
+                               : sel1024::ta_select_kernel<true, 1, 8, true, false, true>;
+    static std::atomic<int> held[3][kMaxDevices];
+    if (gathers && a.K >= kHelpedBudget && units <= sms / kHelpBlocks &&
+        ta_select_helped(a.K, units, clusters_held(helped, sel1024::kThreads, kHelpBlocks, held[which])))
+      return launch_threads(sel1024::kThreads, helped, units, kHelpBlocks, stream, a.seq, a.n_layers, a.Hkv, a.K, a.fast, src2,
+                            a.forced, a.r_main, a.idx, a.count, gd2, co);
     auto kern = a.seq.max_n <= 4 * sel1024::kThreads
                     ? (gathers ? sel1024::ta_select_kernel<true, 1, 4, true> : sel1024::ta_select_kernel<true, 1, 4, false>)
                     : (few1024   ? sel1024::ta_select_kernel<true, 1, 8, true, true>
@@ -433,7 +462,6 @@ cudaError_t ta_launch_broadcast_heads(int n_layers, int B, int Hkv, int K, const
 static __device__ __align__(256) unsigned char g_ta_static_scratch[TA_STATIC_SCRATCH_BYTES];
 
 namespace {
-constexpr int kMaxDevices = 64;
 std::mutex g_static_mutex;
 unsigned char* g_static_ptr[kMaxDevices] = {};  // device address of g_ta_static_scratch, per device ordinal
 

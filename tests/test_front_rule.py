@@ -1,5 +1,5 @@
-"""How many blocks of the per-sequence kernel share a sequence, and that a device which holds no such cluster is given one kernel per
-step: the rule is host code, compiled here by itself."""
+"""How many blocks share a sequence or a unit, and that a device which does not hold their clusters at once is given something else:
+the rules are host code, compiled here by themselves."""
 import ctypes
 import os
 import subprocess
@@ -8,8 +8,11 @@ import pytest
 
 import paper_2604_11288_b200 as ta
 
+INCLUDE = os.path.join(os.path.dirname(os.path.dirname(os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc"))), "include")
 SOURCE = r"""
 #include "ta_front_rule.h"
+#include "ta_internal.cuh"
+extern "C" int helped(int K, int units, int held) { return ta_select_helped(K, units, held); }
 extern "C" int blocks(int n, int batch, int sms, int hidden, const int* fits) {
   return ta_front_blocks(n, batch, sms, hidden != 0, [&](int cl) { return cl == 16 ? fits[3] : cl == 8 ? fits[2] : cl == 4 ? fits[1] : fits[0]; });
 }
@@ -21,12 +24,14 @@ def rule(tmp_path_factory):
     d = tmp_path_factory.mktemp("rule")
     (d / "rule.cpp").write_text(SOURCE)
     csrc = os.path.join(os.path.dirname(ta.__file__), "csrc")
-    subprocess.run([os.environ.get("CXX", "g++"), "-std=c++17", "-O1", "-fPIC", "-shared", "-I", csrc, str(d / "rule.cpp"), "-o",
+    subprocess.run([os.environ.get("CXX", "g++"), "-std=c++17", "-O1", "-fPIC", "-shared", "-I", csrc, "-I", INCLUDE,
+                    "-I", os.path.join(os.path.dirname(os.path.dirname(ta.__file__)), "include"), str(d / "rule.cpp"), "-o",
                     str(d / "rule.so")], check=True)
-    f = ctypes.CDLL(str(d / "rule.so")).blocks
+    lib = ctypes.CDLL(str(d / "rule.so"))
 
     def blocks(n, batch, fits, hidden=False, sms=148):
-        return f(n, batch, sms, int(hidden), (ctypes.c_int * 4)(*fits))
+        return lib.blocks(n, batch, sms, int(hidden), (ctypes.c_int * 4)(*fits))
+    blocks.helped = lib.helped
     return blocks
 
 
@@ -50,3 +55,8 @@ def test_all_clusters_at_once_where_they_fit(rule):
     assert [rule(20000, b, B200) for b in (15, 16, 33, 34, 74, 75)] == [8, 4, 4, 2, 2, 2]
     assert rule(200000, 3, (74, 33, 15, 0)) == 0
     assert rule(20000, 20, (0, 0, 0, 0)) == 0
+
+
+def test_helping_blocks_only_where_all_clusters_run_at_once(rule):
+    assert [rule.helped(512, u, 33) for u in (1, 33, 34, 35)] == [1, 1, 0, 0]
+    assert rule.helped(511, 8, 33) == 0 and rule.helped(4096, 1, 0) == 0
