@@ -301,6 +301,7 @@ __global__ void __launch_bounds__(kThreads, 1) ta_front_kernel(const __grid_cons
       const float u = ta_static_utility(lo + i, n, c, anchor_token, V, p.beta, p.gamma, p.lambda);
       if (FAST) s_u[i] = u;
       else p.u_static[(long long)s.start + lo + i] = u;
+      if (CL > 1 && !FAST) p.forced[(long long)s.start + lo + i] = 0;  // what a wait that runs out leaves: no flags of an earlier call
       if (CL == 1 && V > 0.0f && !mandatory(i)) {
         const int slot = atomicAdd(&s_listed, 1);
         if (slot < kListCap) s_list[slot] = make_uint2(sortable_key(V), (uint32_t)i);

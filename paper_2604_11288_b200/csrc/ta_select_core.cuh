@@ -37,7 +37,6 @@ struct SelectShared {
   // range of the eligible keys: per warp (smallest, largest, how many), and per CTA of a cluster
   uint32_t wmin[kWarps], wmax[kWarps], wnum[kWarps];
   __align__(16) uint32_t cl_range[CL][4];
-  uint32_t took_part[CL];  // of the exchange of candidates (never read: what counts is that the words arrive)
   // long sequences are split over the CTAs of a cluster: every CTA's histogram, two counts to a word, as it sent them to all
   // (two buffers alternating by pass), and every CTA's (definite, tie) totals
   __align__(16) uint32_t ghist[CL > 1 ? 2 : 1][CL][CL > 1 ? 128 : 1];
@@ -56,6 +55,7 @@ struct SelectShared {
   __align__(16) uint32_t cand_keys[kCandCap];
   uint32_t cmp_n, cmp_thresh;  // the same inside one CTA, for at most kCompareCap candidates
   int cmp_above, cmp_equal;
+  uint32_t took_part[CL];  // in the exchange of candidates (never read: what counts is that the words arrive)
 };
 constexpr int kSelectCluster = 8;  // CTAs per unit when a sequence is longer than kItems * kThreads
 
@@ -1031,6 +1031,7 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads) ta_forced_kernel(ta
     for (int it = 0; it < ITEMS; ++it) {
       const int il = (int)threadIdx.x + it * kThreads;
       v[it] = il < hi - lo ? V[il] : 0.0f;
+      if (CL > 1 && il < hi - lo) forced[s.start + lo + il] = 0;  // before a wait can run out: no flags of an earlier call are left
     }
     kc.elig = 0;
 #pragma unroll
@@ -1060,7 +1061,7 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads) ta_forced_kernel(ta
     for (int it = 0; it < ITEMS; ++it) {
       const int il = (int)threadIdx.x + it * kThreads;
       if (il < hi - lo) {
-        f[il] = 0;
+        if (CL == 1) f[il] = 0;
         if (mandatory(lo + il)) always |= 1u << it;
       }
     }
@@ -1287,7 +1288,7 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads) ta_select_kernel(ta
     taken = cluster_ordered_emit<CACHED, CL>(hi - lo, r.ties, key_of, kc, classify, emit, sh);
   if (!lead) return;
   for (int q = taken + tid; q < K; q += kThreads) out[q] = -1;
-  if (tid == 0) count[unit] = min(taken, K);
+  if (tid == 0) count[unit] = CL > 1 ? min(taken, K) : taken;
   gather(min(taken, K), false);
 }
 
