@@ -732,6 +732,7 @@ ta_status compress_impl(ta_ctx* ctx, const ta_patterns* pats, const ta_policy* p
   sel.n_sink = policy->n_sink;
   sel.n_recent = policy->n_recent;
   sel.k_protected = policy->k_protected;
+  sel.score_units = fast || external ? 0 : batch->n_layers * batch->batch * Hkv;
   sel.fast = fast;
   sel.sm_count = ctx->sm_count;
   sel.status = ctx->d_status;

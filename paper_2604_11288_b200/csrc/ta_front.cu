@@ -496,9 +496,9 @@ cudaError_t with_instance(const FrontParams& p, int blocks, F f) {
 }
 
 template <bool FAST>
-cudaError_t launch_split(const FrontParams& p, int sms, bool hidden, bool* launched, cudaStream_t stream) {
+cudaError_t launch_split(const FrontParams& p, int sms, int score_units, bool* launched, cudaStream_t stream) {
   cudaError_t e = cudaSuccess;
-  const int blocks = ta_front_blocks(p.seq.max_n, p.seq.batch, sms, hidden, [&](int cl) {
+  const int blocks = ta_front_blocks(p.seq.max_n, p.seq.batch, sms, score_units, [&](int cl) {
     int clusters = 0;
     const cudaError_t r = with_instance<FAST>(p, cl, [&](const auto& inst) { return inst.ready(&clusters); });
     if (r != cudaSuccess) e = r;
@@ -545,6 +545,5 @@ cudaError_t ta_launch_front(const ta_patterns* pats, const ta_policy& pol, const
   p.count = a.count;
   p.waits = {status, ta_wait_limit(a.wait_limit_ns)};
   const int sms = a.sm_count > 0 ? a.sm_count : 148;
-  return a.fast ? launch_split<true>(p, sms, false, launched, stream)
-                : launch_split<false>(p, sms, a.u != nullptr, launched, stream);
+  return a.fast ? launch_split<true>(p, sms, 0, launched, stream) : launch_split<false>(p, sms, a.score_units, launched, stream);
 }

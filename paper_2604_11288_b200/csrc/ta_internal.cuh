@@ -214,6 +214,7 @@ struct ta_static_out {  // what ta_forced_kernel needs to write the static utili
 struct ta_select_args {
   ta_seq_desc seq;
   int n_layers, Hkv, K;
+  int score_units;  // units of the score kernel that runs beside the per-sequence kernel (0: none does)
   int n_sink, n_recent, k_protected;
   int fast;
   int sm_count;  // of the device the launch goes to (0: ask the runtime about the current device)
