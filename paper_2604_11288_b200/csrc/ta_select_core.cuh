@@ -50,7 +50,7 @@ struct SelectShared {
   uint32_t before[kThreads];  // definite (low 16 bits) and tie elements before every word
   uint32_t total;
   // a unit split over a cluster: once few candidates are left, every CTA sends its own to all and the remaining passes run on
-  // that list inside each CTA, without cluster barriers
+  // that list inside each CTA
   uint32_t cand_n;
   __align__(16) uint32_t cand_keys[kCandCap];
   uint32_t cmp_n, cmp_thresh;  // the same inside one CTA, for at most kCompareCap candidates
@@ -755,8 +755,7 @@ __device__ __forceinline__ uint32_t warp_transpose32(uint32_t x, int lane) {
 // order: the bits of warp w in chunk it are word it*kWarps + w and cover positions 32 * word .. + 31.
 // From there on thread j owns word j: a block-wide exclusive scan over the words' populations gives it the number
 // of definite and of tie elements before its 32 positions, and the taken positions are written from the words alone
-// (no key is needed for that). Three or four block barriers (and one cluster barrier for the totals of the lower
-// ranks). emit may run on another thread than the one that holds the element's key.
+// (no key is needed for that). Three or four block barriers (and one exchange of the CTAs' totals). emit may run on another thread than the one that holds the element's key.
 template <int CL, class EmitFn, int ITEMS>
 __device__ int cached_ordered_emit(int n, const SelectResult& r, const KeyCache<ITEMS>& kc, uint32_t always,
                                    EmitFn emit, SelectShared<CL>& sh, Exchange<CL>& ex) {
