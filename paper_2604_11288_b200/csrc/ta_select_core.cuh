@@ -1055,7 +1055,7 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads) ta_forced_kernel(ta
   auto emit = [&](int il, int rank) { f[il] = 1; };
   int taken;
   if constexpr (CACHED) {
-    uint32_t always = 0;  // the mandatory tokens; every flag is cleared here and set by emit after a block barrier
+    uint32_t always = 0;  // the mandatory tokens; every flag is cleared (here or above) and set by emit after a block barrier
 #pragma unroll
     for (int it = 0; it < ITEMS; ++it) {
       const int il = (int)threadIdx.x + it * kThreads;
