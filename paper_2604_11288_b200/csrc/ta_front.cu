@@ -131,7 +131,7 @@ __global__ void __launch_bounds__(kThreads, 1) ta_front_kernel(const __grid_cons
   // this CTA's slice: tokens [lo, lo + nl); local index i <-> position lo + i. Whole words of the bitmap.
   const int per = CL == 1 ? n : ((n + CL - 1) / CL + 31) / 32 * 32;
   const int rank = CL == 1 ? 0 : (int)cg::this_cluster().block_rank();
-  const int lo = min(n, rank * per), nl = min(n - lo, per);
+  const int lo = CL == 1 ? 0 : min(n, rank * per), nl = CL == 1 ? n : min(n - lo, per);
   const int nx = CL == 1 ? n : min(nl + TA_MAX_PATTERN_LEN, n - lo);  // with the tokens whose matches can cover the slice's last
   int32_t* hist = p.hist + (size_t)b * p.vocab;
   const int32_t* ids = p.ids + (long long)s.start + lo;
@@ -205,7 +205,7 @@ __global__ void __launch_bounds__(kThreads, 1) ta_front_kernel(const __grid_cons
   for (int it = CL == 1 ? 0 : -1; it * kThreads < nx; ++it) {  // (chunk -1: the positions before a slice)
     const int i = tid + it * kThreads;
     if (CL > 1 && (i - lane < -kHalo || i - lane >= nx)) continue;  // (whole warps; the words behind the slice are zero)
-    const int x = i < nx ? s_id[i] : -1;
+    const int x = CL == 1 || i < nx ? s_id[i] : -1;
     int best = -1;
     bool may_end = false;
     if (i < nx) {
