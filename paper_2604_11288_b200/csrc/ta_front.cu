@@ -498,7 +498,7 @@ cudaError_t with_instance(const FrontParams& p, int blocks, F f) {
 template <bool FAST>
 cudaError_t launch_split(const FrontParams& p, int sms, int score_units, bool* launched, cudaStream_t stream) {
   cudaError_t e = cudaSuccess;
-  const int blocks = ta_front_blocks(p.seq.max_n, p.seq.batch, sms, score_units, [&](int cl) {
+  const int blocks = ta_front_blocks(p.seq.max_n, p.seq.batch, sms, score_units, FAST, [&](int cl) {
     int clusters = 0;
     const cudaError_t r = with_instance<FAST>(p, cl, [&](const auto& inst) { return inst.ready(&clusters); });
     if (r != cudaSuccess) e = r;

@@ -6,7 +6,7 @@ constexpr int kFrontMaxItems = 16;    // tokens per thread
 constexpr int kFrontMaxCluster = 16;  // blocks per sequence
 
 // fit(cl): how many clusters of cl blocks the device holds at once, 0 when it holds none. score_units: units of the score kernel that
-// runs beside, 0 without one. 0: one kernel per step instead.
+// runs beside, 0 without one. selects: the kernel also searches the main pool (TA-Fast). 0: one kernel per step instead.
 // One block holds up to 16384 tokens; more are worth their exchanges where a thread of one block would have more than 12 tokens, or
 // has to. Of the sizes that hold the longest sequence the largest of which all sequences' clusters fit at once, else the smallest. How
 // many fit depends on the GPU: B200s with 148 SMs hold 7 clusters of 16 blocks, 15 of 8, 33 or 35 of 4, 74 of 2. us per call of
@@ -16,7 +16,8 @@ constexpr int kFrontMaxCluster = 16;  // blocks per sequence
 // and with one block / 2 / 4 / 8: 1 x 16384 26.3 / 25.7 / 19.3 / 16.9, 8 x 16384 27.5 / 26.8 / 20.5 / 18.2, 60 x 16384 31.7 / 31.1 /
 // 41.6 / 66; 4 x 12000 18.5 / 25.6 / 19.4 / 17.6, 1 x 8192 14.7 / 21.7 / 18.0 / 16.6.
 // 16 blocks where 8 leave a thread more than 4 tokens (8 / 16 blocks: 4 x 14000 17.7 / 18.2, 7 x 20000 19.8 / 20.4, 7 x 30000 22.3 /
-// 23.4, 7 x 70000 31.7 / 25.6).
+// 23.4, 7 x 70000 31.7 / 25.6; beside a score kernel 4 x 20000, 8 units 44.3 / 49.1) or where nothing is searched and nothing runs
+// beside (given scores, 8 units a sequence: 1 x 13000 20.2 / 19.2, 1 x 20000 22.2 / 20.8, 4 x 30000 32.0 / 29.5).
 // Beside a score kernel, which hides the one block of up to 16384 tokens, that leaves it the most SMs. Longer ones gain there too: 1
 // to 100 sequences, 20000 to 131072 tokens, 1 to 384 units, 205 sizes with separate kernels and with this: 33 % faster to 1.5 % slower
 // (4 x 40000, 8 units 73.9 / 66.6; 12 x 131072, 24 units 461.7 / 443.6; 4 layers of 4 x 40000 640 / 634).
@@ -27,7 +28,7 @@ constexpr int kFrontMaxCluster = 16;  // blocks per sequence
 // 8 units 243.4 / 268.2; with fewer or more sequences or units it is the other way round: 7 x 140000, 14 units 275.4 / 247.6; 4 x
 // 140000, 16 units 413.0 / 406.2; 3 x 140000, 6 units 170.8 / 145.6).
 template <class Fit>
-inline int ta_front_blocks(int n, int batch, int sms, int score_units, Fit fit) {
+inline int ta_front_blocks(int n, int batch, int sms, int score_units, bool selects, Fit fit) {
   if (n > kFrontMaxCluster * kFrontMaxItems * kFrontThreads) return 0;
   if (n <= (score_units > 0 ? kFrontMaxItems : 12) * kFrontThreads) return 1;
   int least = 1;
@@ -38,7 +39,7 @@ inline int ta_front_blocks(int n, int batch, int sms, int score_units, Fit fit) 
     const bool crowded = 2 * batch >= at_once - 1 && 2 * batch <= at_once + 1 && score_units >= 8 && score_units <= (2 * batch < at_once ? 24 : 12);
     return at_once < 1 || lone || crowded ? 0 : least;
   }
-  for (int cl = n <= 8 * 4 * kFrontThreads ? 8 : kFrontMaxCluster; cl > 1 && cl >= least; cl /= 2)
+  for (int cl = n <= 8 * 4 * kFrontThreads && (selects || score_units > 0) ? 8 : kFrontMaxCluster; cl > 1 && cl >= least; cl /= 2)
     if (batch <= sms / cl && batch <= fit(cl)) return cl;
   for (int cl = least; cl <= kFrontMaxCluster; cl *= 2)
     if (cl == 1 || fit(cl) > 0) return cl;

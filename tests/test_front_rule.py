@@ -13,8 +13,8 @@ SOURCE = r"""
 #include "ta_front_rule.h"
 #include "ta_internal.cuh"
 extern "C" int helped(int K, int units, int held) { return ta_select_helped(K, units, held); }
-extern "C" int blocks(int n, int batch, int sms, int score_units, const int* fits) {
-  return ta_front_blocks(n, batch, sms, score_units, [&](int cl) { return cl == 16 ? fits[3] : cl == 8 ? fits[2] : cl == 4 ? fits[1] : fits[0]; });
+extern "C" int blocks(int n, int batch, int sms, int score_units, int selects, const int* fits) {
+  return ta_front_blocks(n, batch, sms, score_units, selects != 0, [&](int cl) { return cl == 16 ? fits[3] : cl == 8 ? fits[2] : cl == 4 ? fits[1] : fits[0]; });
 }
 """
 
@@ -29,8 +29,8 @@ def rule(tmp_path_factory):
                     str(d / "rule.so")], check=True)
     lib = ctypes.CDLL(str(d / "rule.so"))
 
-    def blocks(n, batch, fits, score_units=0, sms=148):
-        return lib.blocks(n, batch, sms, score_units, (ctypes.c_int * 4)(*fits))
+    def blocks(n, batch, fits, score_units=0, selects=True, sms=148):
+        return lib.blocks(n, batch, sms, score_units, int(selects), (ctypes.c_int * 4)(*fits))
     blocks.helped = lib.helped
     return blocks
 
@@ -73,4 +73,6 @@ def test_sequences_that_need_the_largest_clusters(rule):
 
 def test_blocks_beside_a_score_kernel_and_without(rule):
     assert [rule(n, 4, B200) for n in (12288, 12289, 32768, 32769)] == [1, 8, 8, 16]
-    assert [rule(n, 4, B200, 32) for n in (16384, 16385, 32768, 32769, 131072)] == [1, 8, 8, 16, 16]
+    assert [rule(n, 4, B200, 0, False) for n in (12288, 12289, 32769)] == [1, 16, 16]
+    assert [rule(n, 8, B200, 0, False) for n in (12289, 32768, 32769)] == [8, 8, 8]
+    assert [rule(n, 4, B200, 32, False) for n in (16384, 16385, 32768, 32769, 131072)] == [1, 8, 8, 16, 16]
