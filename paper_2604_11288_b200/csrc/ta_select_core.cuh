@@ -248,23 +248,27 @@ struct Exchange {
     const uint32_t bar = ta_sm100::smem_u32(&sh.arrived[k & 1]), parity = (uint32_t)(k >> 1) & 1u;
     if (threadIdx.x == 0) ta_sm100::mbar_expect_tx(bar, bytes);
     ++k;
-    bool ok = true;
-    unsigned long long began = 0;
-    for (int tries = 0; !ta_sm100::mbar_try_wait_cluster(bar, parity); ++tries) {
-      if ((tries & 63) != 63) continue;
-      const unsigned long long now = ta_sm100::globaltimer_ns();
-      if (began == 0) began = now;
-      if (now - began > waits.limit_ns) {
-        if (waits.status && atomicCAS(&waits.status->code, 0, (int)TA_ERR_TIMEOUT) == 0) waits.status->where = 8;
-        ok = false;
-        break;
-      }
-    }
+    bool ok = ta_sm100::mbar_try_wait_cluster(bar, parity);
+    if (!ok) ok = wait_slow(bar, parity, waits.limit_ns, waits.status);
     if (__syncthreads_and(ok) == 0) {
       stay();
       asm volatile("exit;");
       __builtin_unreachable();
     }
+  }
+  // Out of line: with the five waits' loops in a kernel 1 x 60000 tokens of 8 units with their scores took 92.1 us, with this 91.0.
+  static __device__ __noinline__ bool wait_slow(uint32_t bar, uint32_t parity, unsigned long long limit_ns, ta_dev_status* status) {
+    unsigned long long began = 0;
+    for (int tries = 0; !ta_sm100::mbar_try_wait_cluster(bar, parity); ++tries) {
+      if ((tries & 63) != 63) continue;
+      const unsigned long long now = ta_sm100::globaltimer_ns();
+      if (began == 0) began = now;
+      if (now - began > limit_ns) {
+        if (status && atomicCAS(&status->code, 0, (int)TA_ERR_TIMEOUT) == 0) status->where = 8;
+        return false;
+      }
+    }
+    return true;
   }
   static __device__ __forceinline__ void stay() {
     ta_sm100::cluster_arrive();
