@@ -21,12 +21,16 @@ def sources():
     return sorted(glob.glob(os.path.join(_HERE, "csrc", "*.cu")))
 
 
+def headers():
+    return glob.glob(os.path.join(_HERE, "csrc", "*.cuh")) + glob.glob(os.path.join(_HERE, "csrc", "*.h")) + glob.glob(
+        os.path.join(_ROOT, "include", "*.h"))
+
+
 def _stale():
     if not os.path.exists(LIB_PATH):
         return True
     t = os.path.getmtime(LIB_PATH)
-    deps = sources() + glob.glob(os.path.join(_HERE, "csrc", "*.cuh")) + glob.glob(os.path.join(_ROOT, "include", "*.h"))
-    return any(os.path.getmtime(d) > t for d in deps)
+    return any(os.path.getmtime(d) > t for d in sources() + headers())
 
 
 def _build_call(force: bool) -> None:

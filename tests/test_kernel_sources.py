@@ -46,3 +46,11 @@ def test_every_wait_takes_the_contexts_limit():
         if os.path.basename(path) == "ta_api.cu":
             made = re.findall(r"ta_select_args (\w+) = \{\};", src)
             assert made and all(f"{m}.wait_limit_ns = ctx->wait_limit_ns;" in src for m in made), made
+
+
+def test_the_build_watches_every_header_that_a_source_includes():
+    from paper_2604_11288_b200 import build
+    watched = {os.path.basename(h) for h in build.headers()}
+    for path in build.sources() + build.headers():
+        for name in re.findall(r'#include "([^"]+)"', open(path).read()):
+            assert os.path.basename(name) in watched, (path, name)
