@@ -16,9 +16,10 @@ constexpr int kFrontMaxCluster = 16;  // blocks per sequence
 // and with one block / 2 / 4 / 8: 1 x 16384 26.3 / 25.7 / 19.3 / 16.9, 8 x 16384 27.5 / 26.8 / 20.5 / 18.2, 60 x 16384 31.7 / 31.1 /
 // 41.6 / 66; 4 x 12000 18.5 / 25.6 / 19.4 / 17.6, 1 x 8192 14.7 / 21.7 / 18.0 / 16.6.
 // 16 blocks where 8 leave a thread more than 4 tokens (8 / 16 blocks: 4 x 14000 17.7 / 18.2, 7 x 20000 19.8 / 20.4, 7 x 30000 22.3 /
-// 23.4, 7 x 70000 31.7 / 25.6) or where the kernel does not search the main pool (given scores, 8 units a sequence: 1 x 13000 20.2 /
-// 19.2, 1 x 20000 22.2 / 20.8, 4 x 30000 32.0 / 29.5; beside a score kernel 3 x 20000, 6 units 45.0 / 44.1, 1 x 30000, 16 units 106.8 /
-// 103.7, but 4 x 20000, 8 units 44.3 / 49.1).
+// 23.4, 7 x 70000 31.7 / 25.6; beside a score kernel, 72 sizes of 1 to 7 sequences of 17000 to 32768 tokens, 1 to 112 units: 17 % faster
+// to 4 % slower, 3 % faster on average: 4 x 17000, 8 units 41.5 / 46.1, 5 x 24000, 10 units 48.6 / 56.0, 1 x 17000, 8 units 41.2 / 42.9, 3 x
+// 32768, 6 units 52.7 / 52.5, 2 x 24000, 16 units 91.3 / 87.4), or where nothing is searched and nothing runs beside (given scores, 8
+// units a sequence: 1 x 13000 20.2 / 19.2, 1 x 20000 22.2 / 20.8, 4 x 30000 32.0 / 29.5).
 // Beside a score kernel, which hides the one block of up to 16384 tokens, that leaves it the most SMs. Longer ones gain there too: 1
 // to 100 sequences, 20000 to 131072 tokens, 1 to 384 units, 205 sizes with separate kernels and with this: 33 % faster to 1.5 % slower
 // (4 x 40000, 8 units 73.9 / 66.6; 12 x 131072, 24 units 461.7 / 443.6; 4 layers of 4 x 40000 640 / 634).
@@ -40,7 +41,7 @@ inline int ta_front_blocks(int n, int batch, int sms, int score_units, bool sele
     const bool crowded = 2 * batch >= at_once - 1 && 2 * batch <= at_once + 1 && score_units >= 8 && score_units <= (2 * batch < at_once ? 24 : 12);
     return at_once < 1 || lone || crowded ? 0 : least;
   }
-  for (int cl = n <= 8 * 4 * kFrontThreads && selects ? 8 : kFrontMaxCluster; cl > 1 && cl >= least; cl /= 2)
+  for (int cl = n <= 8 * 4 * kFrontThreads && (selects || score_units > 0) ? 8 : kFrontMaxCluster; cl > 1 && cl >= least; cl /= 2)
     if (batch <= sms / cl && batch <= fit(cl)) return cl;
   for (int cl = least; cl <= kFrontMaxCluster; cl *= 2)
     if (cl == 1 || fit(cl) > 0) return cl;

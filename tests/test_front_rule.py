@@ -75,4 +75,4 @@ def test_blocks_beside_a_score_kernel_and_without(rule):
     assert [rule(n, 4, B200) for n in (12288, 12289, 32768, 32769)] == [1, 8, 8, 16]
     assert [rule(n, 4, B200, 0, False) for n in (12288, 12289, 32769)] == [1, 16, 16]
     assert [rule(n, 8, B200, 0, False) for n in (12289, 32768, 32769)] == [8, 8, 8]
-    assert [rule(n, 4, B200, 32, False) for n in (16384, 16385, 32768, 32769, 131072)] == [1, 16, 16, 16, 16]
+    assert [rule(n, 4, B200, 32, False) for n in (16384, 16385, 32768, 32769, 131072)] == [1, 8, 8, 16, 16]
